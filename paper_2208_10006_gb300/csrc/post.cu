@@ -10,14 +10,15 @@
 // C to zero at realistic path loss; the reading used is the Frobenius
 // normalisation W_f = (Nr Nt / Qbar) H_f H_f^H (H_f^H H_f when Nt < Nr),
 // Qbar = mean_f ||H_f||_F^2. W_f is formed in FP32 on CUDA cores, then
-// log2 det(I + SNR/Nt W_f) by an FP64 complex Cholesky in shared memory, one
-// block per frequency; the per-(f, SNR) log-determinants are averaged over f
-// in a fixed order.
+// log2 det(I + SNR/Nt W_f) from a complex L D L^H factorisation in registers
+// (double-float, or FP64 at high SNR); the per-(f, SNR) log-determinants are
+// averaged over f in a fixed order.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
 #include <vector>
 
+#include "dfloat.cuh"
 #include "sbr_internal.cuh"
 
 namespace sbr {
@@ -121,132 +122,361 @@ k_pdp(const int32_t* __restrict__ rx_off, const double* __restrict__ L, const do
 // ---------------------------------------------------------------- capacity
 constexpr int kCapThreads = 256;
 constexpr int kMaxSnr = 32;        // SNR values per capacity call
-
-__global__ void k_frob(const float2* __restrict__ H, int64_t per_f, double* __restrict__ qf) {
-    __shared__ double sh[33];
-    const float2* h = H + (int64_t)blockIdx.x * per_f;
-    double v = 0.0;
-    for (int64_t i = threadIdx.x; i < per_f; i += blockDim.x) {
-        float2 x = h[i];
-        v += (double)x.x * x.x + (double)x.y * x.y;
-    }
-    v = block_sum(v, sh);
-    if (threadIdx.x == 0) qf[blockIdx.x] = v;
-}
-
-__global__ void k_qbar(const double* __restrict__ qf, int32_t F, double* __restrict__ qbar) {
-    double s = 0.0;
-    for (int32_t f = 0; f < F; ++f) s += qf[f];
-    *qbar = s / F;
-}
-
-// one block per frequency; n = min(Nr, Nt) <= 64
-__global__ void __launch_bounds__(kCapThreads)
-k_capacity(const float2* __restrict__ H, int32_t Nr, int32_t Nt, const double* __restrict__ snr_lin,
-           int32_t n_snr, const double* __restrict__ qbar, double* __restrict__ ld) {
-    extern __shared__ unsigned char smem[];
-    const int n = Nr < Nt ? Nr : Nt;
-    float2* W = reinterpret_cast<float2*>(smem);                           // [n*n]
-    double2* A = reinterpret_cast<double2*>(smem + sizeof(float2) * ((n * n + 1) & ~1));  // [n*n]
-    __shared__ double s_ld;
-    __shared__ int s_bad;
-    const int f = blockIdx.x;
-    const float2* h = H + (int64_t)f * Nr * Nt;
-    // W[a][b] = sum_p H[a][p] conj(H[b][p])  (Nt >= Nr)  or  sum_q conj(H[q][a]) H[q][b]
-    // Blocked summation: FP32 partial sums over runs of kCapRun terms, added
-    // into FP64 totals, so the rounding error of an entry grows with the run
-    // length rather than with the array size (16,384 terms at a 128 x 128 UPA)
-    constexpr int kCapRun = 32;
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-        int a = e / n, b = e - a * n;
-        double sre = 0.0, sim = 0.0;
-        if (Nt >= Nr) {
-            for (int p0 = 0; p0 < Nt; p0 += kCapRun) {
-                const int p1 = min(Nt, p0 + kCapRun);
-                float re = 0.f, im = 0.f;
-                for (int p = p0; p < p1; ++p) {
-                    float2 x = h[(int64_t)a * Nt + p], y = h[(int64_t)b * Nt + p];
-                    re += x.x * y.x + x.y * y.y;
-                    im += x.y * y.x - x.x * y.y;
-                }
-                sre += re;
-                sim += im;
-            }
-        } else {
-            for (int q0 = 0; q0 < Nr; q0 += kCapRun) {
-                const int q1 = min(Nr, q0 + kCapRun);
-                float re = 0.f, im = 0.f;
-                for (int q = q0; q < q1; ++q) {
-                    float2 x = h[(int64_t)q * Nt + a], y = h[(int64_t)q * Nt + b];
-                    re += x.x * y.x + x.y * y.y;
-                    im += x.x * y.y - x.y * y.x;
-                }
-                sre += re;
-                sim += im;
-            }
-        }
-        W[e] = make_float2((float)sre, (float)sim);
-    }
-    __syncthreads();
-    const double scale = (double)Nr * Nt / *qbar;
-    for (int si = 0; si < n_snr; ++si) {
-        const double c = snr_lin[si] / Nt * scale;
-        for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-            int a = e / n, b = e - a * n;
-            A[e] = make_double2((a == b ? 1.0 : 0.0) + c * W[e].x, c * W[e].y);
-        }
-        if (threadIdx.x == 0) { s_ld = 0.0; s_bad = 0; }
-        __syncthreads();
-        for (int j = 0; j < n; ++j) {
-            if (threadIdx.x == 0) {
-                double d = A[j * n + j].x;
-                if (!(d > 0.0)) { s_bad = 1; d = 1.0; }
-                double l = sqrt(d);
-                A[j * n + j] = make_double2(l, 0.0);
-                s_ld += 2.0 * log(l);
-            }
-            __syncthreads();
-            const double inv = 1.0 / A[j * n + j].x;
-            for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) {
-                double2 v = A[i * n + j];
-                A[i * n + j] = make_double2(v.x * inv, v.y * inv);
-            }
-            __syncthreads();
-            const int m = n - j - 1;
-            for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-                int i = j + 1 + e / m, k = j + 1 + e % m;
-                if (k > i) continue;
-                double2 lij = A[i * n + j], lkj = A[k * n + j];
-                double2 v = A[i * n + k];
-                // A[i][k] -= L[i][j] conj(L[k][j])
-                v.x -= lij.x * lkj.x + lij.y * lkj.y;
-                v.y -= lij.y * lkj.x - lij.x * lkj.y;
-                A[i * n + k] = v;
-            }
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) ld[(int64_t)f * n_snr + si] = s_bad ? NAN : s_ld;
-        __syncthreads();
-    }
-}
-
-__global__ void k_cap_reduce(const double* __restrict__ ld, int32_t F, int32_t n_snr,
-                             double* __restrict__ C) {
-    int si = threadIdx.x;
-    if (si >= n_snr) return;
-    double s = 0.0;
-    for (int32_t f = 0; f < F; ++f) s += ld[(int64_t)f * n_snr + si];
-    C[si] = s / F / log(2.0);
-}
+constexpr int kFrobBlocks = 512;   // most partial sums of ||H||^2
 
 // linear SNR values of one capacity call, passed by value in the launch
 struct SnrList {
     double lin[kMaxSnr];
 };
 
-__global__ void k_snr_store(const __grid_constant__ SnrList snr, int32_t n, double* __restrict__ out) {
-    int i = threadIdx.x;
-    if (i < n) out[i] = snr.lin[i];
+// sum of |h|^2 over this block's share of H, in double-float: an FP64 addition
+// costs some 70 FP32 ones on this GPU, a double-float one about ten, so the
+// pass runs at memory speed (H [1024, 64, 256]: 167 us with FP64 sums, 28 us).
+// A share with an entry that is not finite, above 2^60, or with none above
+// 2^-40 (where an FP32 product could leave the normal range) is summed in FP64.
+__global__ void __launch_bounds__(kCapThreads)
+k_frob(const float2* __restrict__ H, int64_t n, double* __restrict__ part) {
+    ::sbr::pdl_wait();
+    __shared__ double sh[33];
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    df s{0.f, 0.f};
+    float top = 0.f;
+    bool wild = false;
+    auto add = [&](float x) {
+        const df p = two_prod(x, x);
+        const df t = two_sum(s.hi, p.hi);
+        s = fast_two_sum(t.hi, __fadd_rn(s.lo, __fadd_rn(t.lo, p.lo)));
+        top = fmaxf(top, fabsf(x));
+        wild |= !(fabsf(x) < 1.1529215e18f);
+    };
+    // 16-byte loads of two entries where H starts on 16 bytes
+    const bool pairs = (reinterpret_cast<uintptr_t>(H) & 15) == 0;
+    const int64_t np = pairs ? n / 2 : 0;
+    const float4* H4 = reinterpret_cast<const float4*>(H);
+    int64_t i = first;
+    for (; i + 3 * step < np; i += 4 * step) {   // four loads in flight
+        float4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = __ldg(H4 + i + u * step);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { add(v[u].x); add(v[u].y); add(v[u].z); add(v[u].w); }
+    }
+    for (; i < np; i += step) {
+        const float4 v = __ldg(H4 + i);
+        add(v.x); add(v.y); add(v.z); add(v.w);
+    }
+    for (i = 2 * np + first; i < n; i += step) { add(H[i].x); add(H[i].y); }
+    const bool plain = !__syncthreads_or(wild) && __syncthreads_or(top > 9.094947e-13f);
+    double v = df_to_double(s);
+    if (!plain) {
+        v = 0.0;
+        for (i = first; i < n; i += step) v += (double)H[i].x * H[i].x + (double)H[i].y * H[i].y;
+    }
+    v = block_sum(v, sh);
+    if (threadIdx.x == 0) part[blockIdx.x] = v;
+}
+
+// Complex entries of the matrix that is factorised, as double-float pairs
+// (.x real, .y imaginary; packed FP32 instructions) or in FP64. Both take 16 bytes.
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 dup(float x) { return make_float2(x, x); }
+
+struct EntryDf {
+    float2 h, l;
+    struct Row { float2 h, l, sh, sl; };   // u and (Im u, -Re u)
+    // c w + one
+    __device__ __forceinline__ void set(double c, float2 w, float one) {
+        const df cd = df_from_double(c);
+        const df r = df_add(df{one, 0.f}, df_mul_f(cd, w.x)), m = df_mul_f(cd, w.y);
+        h = make_float2(r.hi, m.hi);
+        l = make_float2(r.lo, m.lo);
+    }
+    __device__ __forceinline__ double real() const { return (double)h.x + (double)l.x; }
+    // 1 / Re of the pivot: the reciprocal of the high word and a second-order correction
+    struct Inv { df v; };
+    __device__ __forceinline__ Inv inverse() const {
+        const float x = __frcp_rn(h.x);
+        const float r = __fmaf_rn(-l.x, x, __fmaf_rn(-h.x, x, 1.f));
+        return Inv{fast_two_sum(x, x * __fmaf_rn(r, r, r))};
+    }
+    __device__ __forceinline__ Row row(const Inv& inv) const {
+        const df r = df_mul(df{h.x, l.x}, inv.v), m = df_mul(df{h.y, l.y}, inv.v);
+        return Row{make_float2(r.hi, m.hi), make_float2(r.lo, m.lo), make_float2(m.hi, -r.hi), make_float2(m.lo, -r.lo)};
+    }
+    // this -= u conj(k): the two products and the two sums of each part error-free
+    // on the high words, everything below gathered in the low word
+    __device__ __forceinline__ void update(const Row& u, const EntryDf& k) {
+        const float2 kr = dup(k.h.x), ki = dup(k.h.y), nr = dup(-k.h.x), ni = dup(-k.h.y);
+        const float2 n1 = __fmul2_rn(u.h, nr), n2 = __fmul2_rn(u.sh, ni);
+        float2 e = __ffma2_rn(u.h, kr, n1);
+        e = __ffma2_rn(u.h, dup(k.l.x), e);
+        e = __ffma2_rn(u.l, kr, e);
+        e = __ffma2_rn(u.sh, dup(k.l.y), e);
+        e = __ffma2_rn(u.sl, ki, e);
+        e = __fadd2_rn(e, __ffma2_rn(u.sh, ki, n2));
+        const float2 s1 = __fadd2_rn(h, n1), b1 = sub2(s1, h);
+        const float2 t1 = __fadd2_rn(sub2(h, sub2(s1, b1)), sub2(n1, b1));
+        const float2 s2 = __fadd2_rn(s1, n2), b2 = sub2(s2, s1);
+        const float2 t2 = __fadd2_rn(sub2(s1, sub2(s2, b2)), sub2(n2, b2));
+        const float2 lo = sub2(__fadd2_rn(l, __fadd2_rn(t1, t2)), e);
+        h = __fadd2_rn(s2, lo);
+        l = sub2(lo, sub2(h, s2));
+    }
+};
+
+struct EntryF64 {
+    double re, im;
+    struct Row { double re, im; };
+    struct Inv { double v; };
+    __device__ __forceinline__ void set(double c, float2 w, float one) { re = one + c * w.x; im = c * w.y; }
+    __device__ __forceinline__ double real() const { return re; }
+    __device__ __forceinline__ Inv inverse() const { return Inv{1.0 / re}; }
+    __device__ __forceinline__ Row row(const Inv& inv) const { return Row{re * inv.v, im * inv.v}; }
+    __device__ __forceinline__ void update(const Row& u, const EntryF64& k) {
+        re -= u.re * k.re + u.im * k.im;
+        im -= u.im * k.re - u.re * k.im;
+    }
+};
+static_assert(sizeof(EntryDf) == 16 && sizeof(EntryF64) == 16, "one shared-memory column of 16-byte entries");
+
+__host__ __device__ constexpr int cap_blk(int a, int b) { return a * (a + 1) / 2 + b; }   // block (a, b), a >= b
+
+// the columns of block jb (16 jb ...), then those of the blocks after it
+template <int NB, int jb, class E>
+__device__ __forceinline__ void ldl_block(int n, E (&A)[cap_blk(NB, 0)], E* s_col, double* piv) {
+    constexpr int N = 16 * NB;
+    const int ti = threadIdx.x >> 4, tk = threadIdx.x & 15;
+    for (int jj = 0; jj < 16 && 16 * jb + jj < n; ++jj) {
+        const int j = 16 * jb + jj;
+        const E* col = s_col + (j & 1) * N;
+        E* next = s_col + ((j + 1) & 1) * N;
+        const E d = col[j];
+        if (threadIdx.x == 0) piv[j] = d.real();
+        const typename E::Inv inv = d.inverse();
+        typename E::Row u[NB];
+#pragma unroll
+        for (int a = jb; a < NB; ++a) u[a] = col[ti + 16 * a].row(inv);
+#pragma unroll
+        for (int b = jb; b < NB; ++b) {
+            const E k = col[tk + 16 * b];
+#pragma unroll
+            for (int a = b; a < NB; ++a) A[cap_blk(a, b)].update(u[a], k);
+        }
+        if (tk == ((jj + 1) & 15)) {
+            if (jj < 15) {
+#pragma unroll
+                for (int a = jb; a < NB; ++a) next[ti + 16 * a] = A[cap_blk(a, jb)];
+            } else if constexpr (jb + 1 < NB) {
+#pragma unroll
+                for (int a = jb + 1; a < NB; ++a) next[ti + 16 * a] = A[cap_blk(a, jb + 1)];
+            }
+        }
+        __syncthreads();
+    }
+    if constexpr (jb + 1 < NB) ldl_block<NB, jb + 1, E>(n, A, s_col, piv);
+}
+
+// Pivots of the L D L^H factorisation of I + c W into piv[0 .. n). Thread
+// (ti, tk) of 16 x 16 holds entries (ti + 16 a, tk + 16 b), a >= b, in
+// registers; per column one barrier, after which every thread reads the column
+// and updates its entries (those left of the column or above the diagonal are
+// updated too: nothing reads them).
+template <int NB, class E>
+__device__ __forceinline__ void ldl_pivots(int n, double c, const float2* s_w, E* s_col, double* piv) {
+    constexpr int N = 16 * NB;
+    const int ti = threadIdx.x >> 4, tk = threadIdx.x & 15;
+    E A[cap_blk(NB, 0)];
+#pragma unroll
+    for (int a = 0; a < NB; ++a)
+#pragma unroll
+        for (int b = 0; b <= a; ++b)
+            A[cap_blk(a, b)].set(c, s_w[cap_blk(a, b) * kCapThreads + threadIdx.x], a == b && ti == tk ? 1.f : 0.f);
+    if (tk == 0)
+#pragma unroll
+        for (int a = 0; a < NB; ++a) s_col[ti + 16 * a] = A[cap_blk(a, 0)];
+    __syncthreads();
+    ldl_block<NB, 0>(n, A, s_col, piv);
+}
+
+// Log-determinants ln det(I + SNR/Nt W_f) of one frequency, n = min(Nr, Nt) <=
+// 16 NB <= 64. grid (F, splits): block (f, y) forms W_f and takes the SNRs y,
+// y + splits, ...
+//
+// W[a][b] = sum_p H[a][p] conj(H[b][p])  (Nt >= Nr)  or  sum_q conj(H[q][a]) H[q][b].
+// Blocked summation: FP32 partial sums over runs of kCapRun terms, their totals
+// in double-float, so the rounding error of an entry grows with the run length
+// rather than with the array size (16,384 terms at a 128 x 128 UPA). Each
+// thread forms the entries that it later factorises, from a run of H staged in
+// shared memory. The factorisation is bound by the FP32 pipe (27 packed
+// instructions per entry and column in place of 4 FP64 ones at 1/71 of the FP32
+// rate); it runs in double-float (about 2^-46 relative) while the largest
+// diagonal entry of I + c W is at most 2^16: rounding then stays below 2^-28 of
+// the smallest pivot (>= 1), far inside what the FP32 entries of W carry. Above
+// (SNRs beyond about 45 dB) it runs in FP64.
+// H [1024, 64, 256], seven SNRs, the whole call: 15.4 ms with an FP64 Cholesky
+// in shared memory (three barriers per column), 1.87 ms so; the packed
+// instructions alone take 1.1 ms.
+constexpr int kCapRun = 32;
+
+template <int NB>
+struct CapShared {
+    float2 h[kCapRun][16 * NB + 1];
+    float4 col[2 * 16 * NB];
+    float2 w[cap_blk(NB, 0) * kCapThreads];
+    double piv[16 * NB];
+    double scale;
+};
+
+// W_f's entries of this thread (rounded to FP32) into sh.w, in the order of ldl_pivots
+template <int NB, bool kWide>
+__device__ __forceinline__ void gram(const float2* __restrict__ h, int Nt, int n, int len, CapShared<NB>& sh) {
+    constexpr int N = 16 * NB, kBlk = cap_blk(NB, 0), kLoad = kCapRun * N / kCapThreads;
+    const int tid = threadIdx.x, ti = tid >> 4, tk = tid & 15;
+    // entry e of a run is (p, row), consecutive threads along the rows of H
+    float2 v[kLoad];
+    auto load = [&](int p0) {
+#pragma unroll
+        for (int k = 0; k < kLoad; ++k) {
+            const int e = tid + k * kCapThreads;
+            const int r = kWide ? e / kCapRun : e % N, p = p0 + (kWide ? e % kCapRun : e / N);
+            v[k] = r < n && p < len ? __ldg(h + (kWide ? (int64_t)r * Nt + p : (int64_t)p * Nt + r)) : make_float2(0.f, 0.f);
+        }
+    };
+    df re[kBlk], im[kBlk];
+#pragma unroll
+    for (int k = 0; k < kBlk; ++k) re[k] = im[k] = df{0.f, 0.f};
+    load(0);
+    for (int p0 = 0; p0 < len; p0 += kCapRun) {
+#pragma unroll
+        for (int k = 0; k < kLoad; ++k) {
+            const int e = tid + k * kCapThreads;
+            sh.h[kWide ? e % kCapRun : e / N][kWide ? e / kCapRun : e % N] = v[k];
+        }
+        __syncthreads();
+        if (p0 + kCapRun < len) load(p0 + kCapRun);
+        float sr[kBlk], si[kBlk];
+#pragma unroll
+        for (int k = 0; k < kBlk; ++k) sr[k] = si[k] = 0.f;
+#pragma unroll 4
+        for (int p = 0; p < kCapRun; ++p) {
+            float2 x[NB], y[NB];
+#pragma unroll
+            for (int a = 0; a < NB; ++a) {
+                x[a] = sh.h[p][ti + 16 * a];
+                y[a] = sh.h[p][tk + 16 * a];
+            }
+#pragma unroll
+            for (int a = 0; a < NB; ++a)
+#pragma unroll
+                for (int b = 0; b <= a; ++b) {
+                    sr[cap_blk(a, b)] += x[a].x * y[b].x + x[a].y * y[b].y;
+                    si[cap_blk(a, b)] += kWide ? x[a].y * y[b].x - x[a].x * y[b].y : x[a].x * y[b].y - x[a].y * y[b].x;
+                }
+        }
+#pragma unroll
+        for (int k = 0; k < kBlk; ++k) {
+            re[k] = df_add(re[k], df{sr[k], 0.f});
+            im[k] = df_add(im[k], df{si[k], 0.f});
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int k = 0; k < kBlk; ++k) sh.w[k * kCapThreads + tid] = make_float2(re[k].hi, im[k].hi);
+}
+
+template <int NB>
+__global__ void __launch_bounds__(kCapThreads, 2)
+k_capacity(const float2* __restrict__ H, int32_t Nr, int32_t Nt, const __grid_constant__ SnrList snr, int32_t n_snr,
+           const double* __restrict__ part, int32_t n_part, double* __restrict__ ld) {
+    ::sbr::pdl_wait();
+    extern __shared__ __align__(16) unsigned char smem[];
+    CapShared<NB>& sh = *reinterpret_cast<CapShared<NB>*>(smem);
+    const int tid = threadIdx.x, ti = tid >> 4, tk = tid & 15;
+    const int n = min(Nr, Nt);
+    const float2* h = H + (int64_t)blockIdx.x * Nr * Nt;
+    if (tid < 32) {   // Qbar = mean over f of ||H_f||^2, from the partial sums of all of H
+        double q = 0.0;
+        for (int i = tid; i < n_part; i += 32) q += part[i];
+        for (int o = 16; o; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        if (tid == 0) sh.scale = (double)Nr * Nt / (q / gridDim.x);
+    }
+    if (Nt >= Nr) gram<NB, true>(h, Nt, n, Nt, sh);
+    else gram<NB, false>(h, Nt, n, Nr, sh);
+    __syncthreads();
+    const double scale = sh.scale;
+    for (int si = blockIdx.y; si < n_snr; si += gridDim.y) {
+        const double c = snr.lin[si] / Nt * scale;
+        bool large = false;
+        if (ti == tk)
+#pragma unroll
+            for (int a = 0; a < NB; ++a)
+                large |= ti + 16 * a < n && !(1.0 + c * sh.w[cap_blk(a, a) * kCapThreads + tid].x <= 65536.0);
+        if (__syncthreads_or(large))
+            ldl_pivots<NB>(n, c, sh.w, reinterpret_cast<EntryF64*>(sh.col), sh.piv);
+        else
+            ldl_pivots<NB>(n, c, sh.w, reinterpret_cast<EntryDf*>(sh.col), sh.piv);
+        // thread 0 alone writes piv, and its warp alone reads it
+        if (tid < 32) {
+            __syncwarp();
+            double s = 0.0;
+            bool bad = false;
+            for (int j = tid; j < n; j += 32) {
+                const double d = sh.piv[j];
+                bad |= !(d > 0.0);
+                s += log(d);
+            }
+            for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            bad = __any_sync(0xffffffffu, bad);
+            if (tid == 0) ld[(int64_t)blockIdx.x * n_snr + si] = bad ? NAN : s;
+        }
+    }
+}
+
+// one block per SNR: the mean over frequencies, in bit/s/Hz
+__global__ void __launch_bounds__(kCapThreads)
+k_cap_reduce(const double* __restrict__ ld, int32_t F, int32_t n_snr, double* __restrict__ C) {
+    ::sbr::pdl_wait();
+    __shared__ double sh[33];
+    double s = 0.0;
+    for (int32_t f = threadIdx.x; f < F; f += blockDim.x) s += ld[(int64_t)f * n_snr + blockIdx.x];
+    s = block_sum(s, sh);
+    if (threadIdx.x == 0) C[blockIdx.x] = s / F / log(2.0);
+}
+
+template <int NB>
+sbr_status capacity_launch(const float2* H, int32_t F, int32_t Nr, int32_t Nt, const SnrList& snr, int32_t n_snr,
+                           const double* part, int32_t n_part, double* ld, cudaStream_t s) {
+    static std::atomic<unsigned long long> attr{0};
+    SBR_TRY(set_smem_once((const void*)k_capacity<NB>, (int)sizeof(CapShared<NB>), &attr));
+    // one block per frequency while these fill the chip twice over; below, the
+    // SNRs of a frequency go to blocks of their own, each of which forms W_f again
+    const int splits = std::max(1, std::min<int>(n_snr, 4 * sm_count() / std::max(1, F)));
+    ::sbr::note_launch();
+    SBR_TRY_CUDA(::sbr::launch_pdl(k_capacity<NB>, dim3((unsigned)F, (unsigned)splits), dim3(kCapThreads),
+                                   sizeof(CapShared<NB>), s, H, Nr, Nt, snr, n_snr, part, n_part, ld));
+    return SBR_OK;
+}
+
+// the three launches of a capacity call: part [kFrobBlocks] and ld [F * n_snr] are scratch
+sbr_status capacity_kernels(const float2* H, int32_t F, int32_t Nr, int32_t Nt, const double* snr_db, int32_t n_snr,
+                            double* part, double* ld, double* C, cudaStream_t s) {
+    // the linear SNR list travels by value in the launch, so the call returns as
+    // soon as its work is enqueued (no host table has to outlive it)
+    SnrList snr{};
+    for (int i = 0; i < n_snr; ++i) snr.lin[i] = std::pow(10.0, snr_db[i] / 10.0);
+    const int64_t total = (int64_t)F * Nr * Nt;
+    const int n_part = (int)std::min<int64_t>(kFrobBlocks, (total + 2 * kCapThreads - 1) / (2 * kCapThreads));
+    ::sbr::note_launch();
+    SBR_TRY_CUDA(::sbr::launch_pdl(k_frob, dim3(n_part), dim3(kCapThreads), 0, s, H, total, part));
+    const int n = std::min(Nr, Nt);
+    if (n <= 16) SBR_TRY(capacity_launch<1>(H, F, Nr, Nt, snr, n_snr, part, n_part, ld, s));
+    else if (n <= 32) SBR_TRY(capacity_launch<2>(H, F, Nr, Nt, snr, n_snr, part, n_part, ld, s));
+    else if (n <= 48) SBR_TRY(capacity_launch<3>(H, F, Nr, Nt, snr, n_snr, part, n_part, ld, s));
+    else SBR_TRY(capacity_launch<4>(H, F, Nr, Nt, snr, n_snr, part, n_part, ld, s));
+    ::sbr::note_launch();
+    SBR_TRY_CUDA(::sbr::launch_pdl(k_cap_reduce, dim3(n_snr), dim3(kCapThreads), 0, s, ld, F, n_snr, C));
+    return SBR_OK;
 }
 
 // surrogate targets: one warp per (receiver, frequency); FP64 sums over the
@@ -315,11 +545,6 @@ sbr_status pdp_run(const sbr_path_list* pl, const float2* g, int32_t F, int32_t 
     return SBR_OK;
 }
 
-size_t capacity_smem(int32_t Nr, int32_t Nt) {
-    int n = std::min(Nr, Nt);
-    return sizeof(float2) * (size_t)((n * n + 1) & ~1) + sizeof(double2) * (size_t)n * n;
-}
-
 sbr_status surrogate_targets_run(const sbr_path_list* pl, const float2* g, int32_t F, int32_t n_taps,
                                 double tap_s, double floor_db, float* out, cudaStream_t s) {
     if (pl->n_rx == 0) return SBR_OK;
@@ -332,25 +557,15 @@ sbr_status surrogate_targets_run(const sbr_path_list* pl, const float2* g, int32
 
 sbr_status capacity_run(const float2* H, int32_t F, int32_t Nr, int32_t Nt, const double* snr_db,
                         int32_t n_snr, double* C, cudaStream_t s) {
-    // the linear SNR list travels by value in the first launch, so the call
-    // returns as soon as its work is enqueued (no host table has to outlive it)
-    SnrList snr{};
-    for (int i = 0; i < n_snr; ++i) snr.lin[i] = std::pow(10.0, snr_db[i] / 10.0);
-    double *d_lin, *qf, *qbar, *ld;
-    SBR_TRY(dalloc_n(&d_lin, n_snr, s));
-    SBR_TRY(dalloc_n(&qf, F, s));
-    SBR_TRY(dalloc_n(&qbar, 1, s));
-    SBR_TRY(dalloc_n(&ld, (size_t)F * n_snr, s));
-    ::sbr::note_launch(), k_snr_store<<<1, kMaxSnr, 0, s>>>(snr, n_snr, d_lin);
-    ::sbr::note_launch(), k_frob<<<F, kCapThreads, 0, s>>>(H, (int64_t)Nr * Nt, qf);
-    ::sbr::note_launch(), k_qbar<<<1, 1, 0, s>>>(qf, F, qbar);
-    size_t smem = capacity_smem(Nr, Nt);
-    SBR_TRY_CUDA(cudaFuncSetAttribute(k_capacity, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    ::sbr::note_launch(), k_capacity<<<F, kCapThreads, smem, s>>>(H, Nr, Nt, d_lin, n_snr, qbar, ld);
-    ::sbr::note_launch(), k_cap_reduce<<<1, 32, 0, s>>>(ld, F, n_snr, C);
-    SBR_TRY_CUDA(cudaGetLastError());
-    dfree(d_lin, s); dfree(qf, s); dfree(qbar, s); dfree(ld, s);
-    return SBR_OK;
+    double *part, *ld;
+    SBR_TRY(dalloc_n(&part, kFrobBlocks, s));
+    sbr_status st = dalloc_n(&ld, (size_t)F * n_snr, s);
+    if (st == SBR_OK) {
+        st = capacity_kernels(H, F, Nr, Nt, snr_db, n_snr, part, ld, C, s);
+        dfree(ld, s);
+    }
+    dfree(part, s);
+    return st;
 }
 
 
@@ -366,9 +581,7 @@ constexpr int kNoAllocMaxF = 4096;    // frequencies per call
 constexpr int kNoAllocMaxSnr = kMaxSnr;  // SNR values per call
 
 struct CapacityScratch {
-    double qf[kNoAllocMaxF];                     // ||H_f||_F^2
-    double qbar;                                 // mean over f
-    double snr_lin[kNoAllocMaxSnr];              // 10^(dB/10)
+    double part[kFrobBlocks];                    // partial sums of ||H||_F^2
     double ld[kNoAllocMaxF * kNoAllocMaxSnr];    // ln det per (f, SNR)
 };
 static __device__ __align__(256) CapacityScratch g_capacity_scratch;
@@ -412,20 +625,9 @@ sbr_status capacity_noalloc_run(const float2* H, int32_t F, int32_t Nr, int32_t 
     }
     CapacityScratch* scr = nullptr;
     SBR_TRY(capacity_scratch(&scr));
-    // every scratch field read below is first written by this call, so nothing
-    // has to be cleared; the SNR list travels by value in the launch itself
-    SnrList snr{};
-    for (int i = 0; i < n_snr; ++i) snr.lin[i] = std::pow(10.0, snr_db[i] / 10.0);
-    ::sbr::note_launch(), k_snr_store<<<1, kMaxSnr, 0, s>>>(snr, n_snr, scr->snr_lin);
-    ::sbr::note_launch(), k_frob<<<F, kCapThreads, 0, s>>>(H, (int64_t)Nr * Nt, scr->qf);
-    ::sbr::note_launch(), k_qbar<<<1, 1, 0, s>>>(scr->qf, F, &scr->qbar);
-    size_t smem = capacity_smem(Nr, Nt);
-    SBR_TRY_CUDA(cudaFuncSetAttribute(k_capacity, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    ::sbr::note_launch(), k_capacity<<<F, kCapThreads, smem, s>>>(H, Nr, Nt, scr->snr_lin, n_snr, &scr->qbar,
-                                                                   scr->ld);
-    ::sbr::note_launch(), k_cap_reduce<<<1, 32, 0, s>>>(scr->ld, F, n_snr, C);
-    SBR_TRY_CUDA(cudaGetLastError());
-    return SBR_OK;
+    // every scratch field read is first written by this call, so nothing has to
+    // be cleared
+    return capacity_kernels(H, F, Nr, Nt, snr_db, n_snr, scr->part, scr->ld, C, s);
 }
 
 }  // namespace sbr
