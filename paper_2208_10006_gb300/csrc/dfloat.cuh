@@ -24,6 +24,24 @@ __host__ __device__ __forceinline__ df df_from_double(double x) {
 }
 __device__ __forceinline__ double df_to_double(df a) { return (double)a.hi + (double)a.lo; }
 
+#ifdef __CUDACC__
+// the same split by integer operations (a double-precision conversion or
+// subtraction takes some 70 FP32 slots on this GPU): the upper 24 significant
+// bits by shifting, the lower 29 through an integer conversion. Values outside
+// [2^-74, 2^127) keep their FP32 rounding only.
+__device__ __forceinline__ df df_split(double x) {
+    const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+    const unsigned e = (h >> 20) & 0x7ffu;
+    if (e - 949u >= 201u) return df{__double2float_rn(x), 0.f};
+    const unsigned sign = h & 0x80000000u;
+    const float hi = __uint_as_float(((__funnelshift_l(l, h, 3) ^ 0x40000000u) & 0x7fffffffu) | sign);
+    const float scale = __uint_as_float(((e - 948u) << 23) | sign);
+    const float lo = __fmul_rn(__uint2float_rn(l & 0x1fffffffu), scale);
+    const float s = __fadd_rn(hi, lo);
+    return df{s, __fsub_rn(lo, __fsub_rn(s, hi))};
+}
+#endif
+
 __device__ __forceinline__ df two_sum(float a, float b) {
     float s = __fadd_rn(a, b);
     float bb = __fsub_rn(s, a);
@@ -77,6 +95,52 @@ __device__ __forceinline__ df df_div(df a, df b) {
     float q3 = r.hi * ib;
     df q = fast_two_sum(q1, q2);
     return df_add(q, df{q3, 0.f});
+}
+// a b + c d, error-free on the high words, the rest gathered in one float
+__device__ __forceinline__ df df_dot2(df a, df b, df c, df d) {
+    const df p = two_prod(a.hi, b.hi), q = two_prod(c.hi, d.hi);
+    const df s = two_sum(p.hi, q.hi);
+    float e = __fadd_rn(__fadd_rn(p.lo, q.lo), s.lo);
+    e = __fmaf_rn(a.hi, b.lo, e);
+    e = __fmaf_rn(a.lo, b.hi, e);
+    e = __fmaf_rn(c.hi, d.lo, e);
+    e = __fmaf_rn(c.lo, d.hi, e);
+    return two_sum(s.hi, e);
+}
+// 1 / a and sqrt(a) for normal a (a > 0 under the root): the hardware
+// approximation x and one correction from its exact residual, 1 / a with the
+// second-order term (relative error about 2^-45)
+__device__ __forceinline__ df df_rcp(df a) {
+    float x;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(a.hi));
+    const float r = __fmaf_rn(-a.lo, x, __fmaf_rn(-a.hi, x, 1.f));
+    return fast_two_sum(x, __fmul_rn(x, __fmaf_rn(r, r, r)));
+}
+__device__ __forceinline__ df df_sqrt(df a) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(a.hi));
+    const float s = __fmul_rn(a.hi, y);
+    const float r = __fadd_rn(__fmaf_rn(-s, s, a.hi), a.lo);
+    return fast_two_sum(s, __fmul_rn(__fmul_rn(0.5f, y), r));
+}
+// log2 of a positive normal double: exponent and 2 atanh((m - 1) / (m + 1)) of
+// the mantissa m in [0.71, 1.42); absolute error below 1e-9
+__device__ __forceinline__ df df_log2(double x) {
+    const int h = __double2hiint(x);
+    const bool up = (h & 0xfffff) >= 0x6a09e;   // m >= sqrt 2
+    const float e = (float)((h >> 20) - 1023 + (up ? 1 : 0));
+    const df m = df_split(__hiloint2double((h & 0xfffff) | (up ? 0x3fe00000 : 0x3ff00000), __double2loint(x)));
+    const df one{1.f, 0.f};
+    const df s = df_mul(df_sub(m, one), df_rcp(df_add(m, one)));
+    const float t = __fmul_rn(s.hi, s.hi);
+    float q = __fmaf_rn(1.f / 13.f, t, 1.f / 11.f);
+    q = __fmaf_rn(q, t, 1.f / 9.f);
+    q = __fmaf_rn(q, t, 1.f / 7.f);
+    q = __fmaf_rn(q, t, 1.f / 5.f);
+    q = __fmul_rn(__fmaf_rn(q, t, 1.f / 3.f), t);
+    df y = fast_two_sum(s.hi, __fmul_rn(s.hi, q));
+    y.lo = __fadd_rn(y.lo, s.lo);
+    return df_add(df{e, 0.f}, df_mul(y, df{2.88539004f, 3.85192598e-8f}));   // 2 / ln 2
 }
 // a < b, a <= b on the represented values
 __device__ __forceinline__ bool df_lt(df a, df b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }

@@ -277,21 +277,23 @@ __device__ __forceinline__ void ldl_block(int n, E (&A)[cap_blk(NB, 0)], E* s_co
     if constexpr (jb + 1 < NB) ldl_block<NB, jb + 1, E>(n, A, s_col, piv);
 }
 
-// Pivots of the L D L^H factorisation of I + c W into piv[0 .. n). Thread
+// Pivots of the L D L^H factorisation of I + c ws W into piv[0 .. n). Thread
 // (ti, tk) of 16 x 16 holds entries (ti + 16 a, tk + 16 b), a >= b, in
 // registers; per column one barrier, after which every thread reads the column
 // and updates its entries (those left of the column or above the diagonal are
 // updated too: nothing reads them).
 template <int NB, class E>
-__device__ __forceinline__ void ldl_pivots(int n, double c, const float2* s_w, E* s_col, double* piv) {
+__device__ __forceinline__ void ldl_pivots(int n, double c, const float2* s_w, float ws, E* s_col, double* piv) {
     constexpr int N = 16 * NB;
     const int ti = threadIdx.x >> 4, tk = threadIdx.x & 15;
     E A[cap_blk(NB, 0)];
 #pragma unroll
     for (int a = 0; a < NB; ++a)
 #pragma unroll
-        for (int b = 0; b <= a; ++b)
-            A[cap_blk(a, b)].set(c, s_w[cap_blk(a, b) * kCapThreads + threadIdx.x], a == b && ti == tk ? 1.f : 0.f);
+        for (int b = 0; b <= a; ++b) {
+            const float2 w = s_w[cap_blk(a, b) * kCapThreads + threadIdx.x];
+            A[cap_blk(a, b)].set(c, make_float2(w.x * ws, w.y * ws), a == b && ti == tk ? 1.f : 0.f);
+        }
     if (tk == 0)
 #pragma unroll
         for (int a = 0; a < NB; ++a) s_col[ti + 16 * a] = A[cap_blk(a, 0)];
@@ -326,6 +328,7 @@ struct CapShared {
     float2 w[cap_blk(NB, 0) * kCapThreads];
     double piv[16 * NB];
     double scale;
+    unsigned top;   // bits of the largest diagonal entry of W
 };
 
 // W_f's entries of this thread (rounded to FP32) into sh.w, in the order of ldl_pivots
@@ -399,23 +402,33 @@ k_capacity(const float2* __restrict__ H, int32_t Nr, int32_t Nt, const __grid_co
         double q = 0.0;
         for (int i = tid; i < n_part; i += 32) q += part[i];
         for (int o = 16; o; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-        if (tid == 0) sh.scale = (double)Nr * Nt / (q / gridDim.x);
+        if (tid == 0) {
+            sh.scale = (double)Nr * Nt / (q / gridDim.x);
+            sh.top = 0u;
+        }
     }
     if (Nt >= Nr) gram<NB, true>(h, Nt, n, Nt, sh);
-    else gram<NB, false>(h, Nt, n, Nr, sh);
+    else gram<NB, false>(h, Nt, n, Nr, sh);   // at least one barrier in either
+    if (ti == tk)
+#pragma unroll
+        for (int a = 0; a < NB; ++a) atomicMax(&sh.top, __float_as_uint(sh.w[cap_blk(a, a) * kCapThreads + tid].x));
     __syncthreads();
+    // W in units of 2^e, its largest entry in [1, 2), so that neither it nor the
+    // factor of an SNR leaves the normal FP32 range whatever the scale of H
+    const int e = (int)((sh.top >> 23) & 0xffu) - 127;
+    const float ws = e > -127 && e < 127 ? ldexpf(1.f, -e) : 1.f;
     const double scale = sh.scale;
     for (int si = blockIdx.y; si < n_snr; si += gridDim.y) {
-        const double c = snr.lin[si] / Nt * scale;
+        const double c = snr.lin[si] / Nt * scale / ws;
         bool large = false;
         if (ti == tk)
 #pragma unroll
             for (int a = 0; a < NB; ++a)
-                large |= ti + 16 * a < n && !(1.0 + c * sh.w[cap_blk(a, a) * kCapThreads + tid].x <= 65536.0);
+                large |= ti + 16 * a < n && !(1.0 + c * (sh.w[cap_blk(a, a) * kCapThreads + tid].x * ws) <= 65536.0);
         if (__syncthreads_or(large))
-            ldl_pivots<NB>(n, c, sh.w, reinterpret_cast<EntryF64*>(sh.col), sh.piv);
+            ldl_pivots<NB>(n, c, sh.w, ws, reinterpret_cast<EntryF64*>(sh.col), sh.piv);
         else
-            ldl_pivots<NB>(n, c, sh.w, reinterpret_cast<EntryDf*>(sh.col), sh.piv);
+            ldl_pivots<NB>(n, c, sh.w, ws, reinterpret_cast<EntryDf*>(sh.col), sh.piv);
         // thread 0 alone writes piv, and its warp alone reads it
         if (tid < 32) {
             __syncwarp();
@@ -479,55 +492,99 @@ sbr_status capacity_kernels(const float2* H, int32_t F, int32_t Nr, int32_t Nt, 
     return SBR_OK;
 }
 
-// surrogate targets: one warp per (receiver, frequency); FP64 sums over the
-// receiver's paths of P_n = |g_n(f)|^2, tau_n = L_n / c, relative to the first
-// arrival for the delay spread and the taps
-__global__ void k_surrogate_targets(const int32_t* __restrict__ rx_off, int32_t n_rx, const float2* __restrict__ g,
-                                    const double* __restrict__ L, int32_t F, int32_t n_taps, double tap_s,
-                                    double floor_db, float* __restrict__ out) {
-    const int lane = threadIdx.x & 31;
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (w >= (int64_t)n_rx * F) return;
-    const int r = (int)(w / F), f = (int)(w - (int64_t)r * F);
+// 10 log10 of a / b for powers (a > 0): in double-float, one FP64 logarithm costs
+// some 3000 FP32 slots on this GPU; FP64 where a or b is zero, subnormal or not finite
+__device__ __forceinline__ float ratio_db(double a, double b) {
+    auto plain = [](double x) { return (unsigned)(__double2hiint(x) - 0x00100000) < 0x7fe00000u; };
+    if (!plain(a) || !plain(b)) return (float)(10.0 * log10(a / b));
+    return df_mul(df_sub(df_log2(a), df_log2(b)), df{3.01029992f, 3.56040455e-8f}).hi;   // 10 log10 2
+}
+
+// surrogate targets of P_n = |g_n(f)|^2, tau_n = L_n / c relative to the first
+// arrival: one warp per receiver. Its lanes first compute the delay and the tap
+// of one path each (FP64, once for all frequencies), then stand for (slice,
+// frequency): nf = the power of two at or above F (at most 32) frequencies and
+// 32 / nf slices of the paths, each lane with sums of its own and a column of
+// taps in shared memory; the slices are added at the end. Bound by the FP64 pipe
+// (nine operations per path and frequency). 4096 receivers x 25 paths x 8
+// frequencies: 1436 us with a warp per (receiver, frequency) and butterflies
+// over 35 FP64 sums; with the gains of the same paths (2517 us more) the two
+// take 100 us now.
+constexpr int kTgtWarps = 4;
+
+__global__ void __launch_bounds__(32 * kTgtWarps)
+k_surrogate_targets(const int32_t* __restrict__ rx_off, int32_t n_rx, const float2* __restrict__ g,
+                    const double* __restrict__ L, int32_t F, int nf, int32_t n_taps, double tap_s, double floor_db,
+                    float* __restrict__ out) {
+    ::sbr::pdl_wait();
+    extern __shared__ double tgt_smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double* s_tap = tgt_smem + warp * (32 * n_taps + 48);   // [n_taps][32]
+    double* s_t = s_tap + 32 * n_taps;                      // [32]
+    int* s_b = reinterpret_cast<int*>(s_t + 32);            // [32]
+    const int r = blockIdx.x * kTgtWarps + warp;
+    if (r >= n_rx) return;
     const int p0 = rx_off[r], p1 = rx_off[r + 1];
     const int stride = 2 + n_taps;
-    float* o = out + w * stride;
+    float* o = out + (int64_t)r * F * stride;
     if (p1 == p0) {
-        for (int k = lane; k < stride; k += 32) o[k] = NAN;
+        for (int64_t k = lane; k < (int64_t)F * stride; k += 32) o[k] = NAN;
         return;
     }
-    double tmin = INFINITY;
-    for (int p = p0 + lane; p < p1; p += 32) tmin = fmin(tmin, L[p] / kC0);
-    for (int s = 16; s; s >>= 1) tmin = fmin(tmin, __shfl_xor_sync(0xffffffffu, tmin, s));
-    double sp = 0.0, st = 0.0, st2 = 0.0;
-    double tap[32];
-    for (int k = 0; k < 32; ++k) tap[k] = 0.0;
-    for (int p = p0 + lane; p < p1; p += 32) {
-        float2 gg = g[(int64_t)p * F + f];
-        double pw = (double)gg.x * gg.x + (double)gg.y * gg.y;
-        double t = L[p] / kC0 - tmin;
-        sp += pw;
-        st += pw * t;
-        st2 += pw * t * t;
-        double b = floor(t / tap_s);
-        if (b >= 0.0 && b < n_taps) {
-            int bi = (int)b;
-            for (int k = 0; k < 32; ++k) tap[k] += k == bi ? pw : 0.0;
+    // lengths are not negative: their bit patterns are ordered as they are
+    unsigned long long lmin = ~0ull;
+    for (int p = p0 + lane; p < p1; p += 32) lmin = min(lmin, (unsigned long long)__double_as_longlong(L[p]));
+    for (int s = 16; s; s >>= 1) lmin = min(lmin, __shfl_xor_sync(0xffffffffu, lmin, s));
+    const double tmin = __longlong_as_double((long long)lmin) / kC0;
+    const int slices = 32 / nf, fl = lane & (nf - 1), sl = lane / nf;
+    for (int f0 = 0; f0 < F; f0 += nf) {
+        const int f = f0 + fl;
+        for (int k = 0; k < n_taps; ++k) s_tap[32 * k + lane] = 0.0;
+        double sp = 0.0, st = 0.0, st2 = 0.0;
+        for (int c0 = p0; c0 < p1; c0 += 32) {
+            __syncwarp();
+            if (c0 + lane < p1) {
+                const double t = L[c0 + lane] / kC0 - tmin;
+                const double b = floor(t / tap_s);
+                s_t[lane] = t;
+                s_b[lane] = b >= 0.0 && b < n_taps ? (int)b : -1;
+            }
+            __syncwarp();
+            const int cnt = min(32, p1 - c0);
+            if (f < F) {
+                for (int k = sl; k < cnt; k += slices) {
+                    const float2 gg = __ldg(g + (int64_t)(c0 + k) * F + f);
+                    const double pw = (double)gg.x * gg.x + (double)gg.y * gg.y;
+                    const double t = s_t[k];
+                    const int b = s_b[k];
+                    sp += pw;
+                    st += pw * t;
+                    st2 += pw * t * t;
+                    if (b >= 0) s_tap[32 * b + lane] += pw;
+                }
+            }
         }
-    }
-    for (int s = 16; s; s >>= 1) {
-        sp += __shfl_xor_sync(0xffffffffu, sp, s);
-        st += __shfl_xor_sync(0xffffffffu, st, s);
-        st2 += __shfl_xor_sync(0xffffffffu, st2, s);
-        for (int k = 0; k < 32; ++k) tap[k] += __shfl_xor_sync(0xffffffffu, tap[k], s);
-    }
-    if (lane != 0) return;
-    o[0] = (float)(-10.0 * log10(sp));
-    double mean = st / sp;
-    o[1] = (float)sqrt(fmax(st2 / sp - mean * mean, 0.0));
-    for (int k = 0; k < n_taps; ++k) {
-        double db = tap[k] > 0.0 ? 10.0 * log10(tap[k] / sp) : floor_db;
-        o[2 + k] = (float)fmax(db, floor_db);
+        for (int s = nf; s < 32; s <<= 1) {
+            sp += __shfl_xor_sync(0xffffffffu, sp, s);
+            st += __shfl_xor_sync(0xffffffffu, st, s);
+            st2 += __shfl_xor_sync(0xffffffffu, st2, s);
+        }
+        __syncwarp();
+        // slice sl of frequency f: taps sl, sl + slices, ...
+        if (f < F) {
+            float* of = o + (int64_t)f * stride;
+            if (sl == 0) {
+                of[0] = -ratio_db(sp, 1.0);
+                const double mean = st / sp;
+                of[1] = (float)sqrt(fmax(st2 / sp - mean * mean, 0.0));
+            }
+            for (int k = sl; k < n_taps; k += slices) {
+                double v = 0.0;
+                for (int q = 0; q < slices; ++q) v += s_tap[32 * k + q * nf + fl];
+                of[2 + k] = fmaxf(v > 0.0 ? ratio_db(v, sp) : (float)floor_db, (float)floor_db);
+            }
+        }
+        __syncwarp();
     }
 }
 
@@ -548,9 +605,12 @@ sbr_status pdp_run(const sbr_path_list* pl, const float2* g, int32_t F, int32_t 
 sbr_status surrogate_targets_run(const sbr_path_list* pl, const float2* g, int32_t F, int32_t n_taps,
                                 double tap_s, double floor_db, float* out, cudaStream_t s) {
     if (pl->n_rx == 0) return SBR_OK;
-    int64_t threads = (int64_t)pl->n_rx * F * 32;
-    ::sbr::note_launch(), k_surrogate_targets<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(
-        pl->rx_off, pl->n_rx, g, pl->L, F, n_taps, tap_s, floor_db, out);
+    int nf = 1;
+    while (nf < F && nf < 32) nf *= 2;
+    const size_t smem = sizeof(double) * kTgtWarps * (32 * (size_t)n_taps + 48);   // n_taps <= 32: below 48 KB
+    ::sbr::note_launch(), (void)::sbr::launch_pdl(
+        k_surrogate_targets, dim3((unsigned)((pl->n_rx + kTgtWarps - 1) / kTgtWarps)), dim3(32 * kTgtWarps), smem, s,
+        pl->rx_off, pl->n_rx, g, pl->L, F, nf, n_taps, tap_s, floor_db, out);
     SBR_TRY_CUDA(cudaGetLastError());
     return SBR_OK;
 }
