@@ -314,7 +314,8 @@ sbr_status sbr_path_gains(const sbr_path_list* pl, const sbr_material* mats, int
  * T_0 = the trace's tx, R_0 = rx_xyz[rx_index]; a LoS path uses the exact
  * |T_p - R_q| in its phase. gains: dev complex64 [P*F] from sbr_path_gains (NULL when P = 0).
  * tx_elem: dev double [Nt*3]; rx_elem: dev double [Nr*3].
- * precision: SBR_SYNTH_FP64 / FP32 (CUDA cores) or SBR_SYNTH_BF16X3 /
+ * precision: SBR_SYNTH_FP64 / FP32 (CUDA cores; the FP64 form sums in
+ * double-float, 48 bits: its error is the rounding of H) or SBR_SYNTH_BF16X3 /
  * SBR_SYNTH_FP16X3 (tcgen05 tensor cores, U diag(w) V^T contraction, FP32
  * accumulation; FP16X3 keeps ~2^-22 of each operand where BF16X3 keeps ~2^-16).
  * H: dev complex64 [F*Nr*Nt], element (f, q, p) at (f*Nr + q)*Nt + p.
@@ -334,10 +335,10 @@ sbr_status sbr_synthesize_H(const sbr_path_list* pl, const void* gains, const do
  * Unlike sbr_synthesize_H no Rx-side correction is applied: the element is
  * the traced point. gains: dev complex64 [P*F] (NULL when P = 0);
  * freqs_hz: dev double [F]; tx_elem: dev double [Nt*3].
- * precision: SBR_SYNTH_FP64 or SBR_SYNTH_FP32 (summation type; element
- * delays and the reduced phase f L_n / c are always FP64).
+ * precision: SBR_SYNTH_FP64 (sums in double-float, 48 bits) or SBR_SYNTH_FP32;
+ * element delays are double-float in both.
  * H: dev complex64 [F*n_rx*Nt], element (f, q, p) at (f*n_rx + q)*Nt + p.
- * F, n_rx <= 65535. Device scratch: P*(Nt+F) doubles (plus the FP32 copies).
+ * F, n_rx <= 65535. Device scratch: P*Nt pairs of floats.
  */
 sbr_status sbr_synthesize_H_elements(const sbr_path_list* pl, const void* gains, const double* freqs_hz,
                                      int32_t F, const double* tx_elem, int32_t Nt, int32_t precision,

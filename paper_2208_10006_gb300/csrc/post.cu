@@ -179,50 +179,22 @@ k_frob(const float2* __restrict__ H, int64_t n, double* __restrict__ part) {
 
 // Complex entries of the matrix that is factorised, as double-float pairs
 // (.x real, .y imaginary; packed FP32 instructions) or in FP64. Both take 16 bytes.
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-__device__ __forceinline__ float2 dup(float x) { return make_float2(x, x); }
-
 struct EntryDf {
-    float2 h, l;
-    struct Row { float2 h, l, sh, sl; };   // u and (Im u, -Re u)
+    cdf2 v;
+    struct Row { cdf2 u, ju; };   // -u and its product with the conjugation's sign: acc + u k_re + ju k_im = acc - u conj(k)
     // c w + one
     __device__ __forceinline__ void set(double c, float2 w, float one) {
         const df cd = df_from_double(c);
-        const df r = df_add(df{one, 0.f}, df_mul_f(cd, w.x)), m = df_mul_f(cd, w.y);
-        h = make_float2(r.hi, m.hi);
-        l = make_float2(r.lo, m.lo);
+        v = cdf2_make(df_add(df{one, 0.f}, df_mul_f(cd, w.x)), df_mul_f(cd, w.y));
     }
-    __device__ __forceinline__ double real() const { return (double)h.x + (double)l.x; }
-    // 1 / Re of the pivot: the reciprocal of the high word and a second-order correction
+    __device__ __forceinline__ double real() const { return (double)v.h.x + (double)v.l.x; }
     struct Inv { df v; };
-    __device__ __forceinline__ Inv inverse() const {
-        const float x = __frcp_rn(h.x);
-        const float r = __fmaf_rn(-l.x, x, __fmaf_rn(-h.x, x, 1.f));
-        return Inv{fast_two_sum(x, x * __fmaf_rn(r, r, r))};
-    }
+    __device__ __forceinline__ Inv inverse() const { return Inv{df_rcp(df{v.h.x, v.l.x})}; }
     __device__ __forceinline__ Row row(const Inv& inv) const {
-        const df r = df_mul(df{h.x, l.x}, inv.v), m = df_mul(df{h.y, l.y}, inv.v);
-        return Row{make_float2(r.hi, m.hi), make_float2(r.lo, m.lo), make_float2(m.hi, -r.hi), make_float2(m.lo, -r.lo)};
+        const df r = df_mul(df{v.h.x, v.l.x}, inv.v), m = df_mul(df{v.h.y, v.l.y}, inv.v);
+        return Row{cdf2_make(df_neg(r), df_neg(m)), cdf2_make(df_neg(m), r)};
     }
-    // this -= u conj(k): the two products and the two sums of each part error-free
-    // on the high words, everything below gathered in the low word
-    __device__ __forceinline__ void update(const Row& u, const EntryDf& k) {
-        const float2 kr = dup(k.h.x), ki = dup(k.h.y), nr = dup(-k.h.x), ni = dup(-k.h.y);
-        const float2 n1 = __fmul2_rn(u.h, nr), n2 = __fmul2_rn(u.sh, ni);
-        float2 e = __ffma2_rn(u.h, kr, n1);
-        e = __ffma2_rn(u.h, dup(k.l.x), e);
-        e = __ffma2_rn(u.l, kr, e);
-        e = __ffma2_rn(u.sh, dup(k.l.y), e);
-        e = __ffma2_rn(u.sl, ki, e);
-        e = __fadd2_rn(e, __ffma2_rn(u.sh, ki, n2));
-        const float2 s1 = __fadd2_rn(h, n1), b1 = sub2(s1, h);
-        const float2 t1 = __fadd2_rn(sub2(h, sub2(s1, b1)), sub2(n1, b1));
-        const float2 s2 = __fadd2_rn(s1, n2), b2 = sub2(s2, s1);
-        const float2 t2 = __fadd2_rn(sub2(s1, sub2(s2, b2)), sub2(n2, b2));
-        const float2 lo = sub2(__fadd2_rn(l, __fadd2_rn(t1, t2)), e);
-        h = __fadd2_rn(s2, lo);
-        l = sub2(lo, sub2(h, s2));
-    }
+    __device__ __forceinline__ void update(const Row& u, const EntryDf& k) { cdf2_mac(v, u.u, u.ju, k.v); }
 };
 
 struct EntryF64 {

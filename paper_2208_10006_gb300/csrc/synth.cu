@@ -1,299 +1,623 @@
 // MIMO H(f) synthesis on CUDA cores (Eq. 11-14, near-field spherical
-// wavefront of Sec. I), the plain FP32 and FP64 forms.
+// wavefront of Sec. I), the FP32 and FP64 forms.
 //
 // For the paths of one receiver, with first/last interaction points P1/Pm,
 //   H[f,q,p] = sum_n w_n(f) exp(-j 2 pi f (dt_pn + dr_qn) / c),
 //   w_n(f)   = g_n(f) exp(-j 2 pi frac(f L_n / c)),
 //   dt_pn    = |T_p - P1| - |T_0 - P1|,  dr_qn = |R_q - Pm| - |R_0 - Pm|;
 // a LoS path uses dlos_qp = |T_p - R_q| - |T_0 - R_0| instead of dt + dr.
-// The prologue computes the element delays and w in FP64 (the large phase
-// f L / c is reduced there); the summation then runs in FP32 or FP64.
+// The phasor of a term is the product of one per (path, receive element) and one
+// per (path, transmit element), so that a tile of H costs (Nr + Nt) sines and
+// cosines per path and one complex multiply-add per term.
+//
+// The FP32 form computes in FP32 with phases reduced from double-float
+// frequencies. The FP64 form computes in double-float (48 bits): an FP64
+// operation takes as long as 71 FP32 ones on this GPU, and the result is rounded
+// to FP32 (its error against 64 bits, 4e-8, is that rounding in either
+// arithmetic).
 #include <algorithm>
 
+#include "dfloat.cuh"
 #include "sbr_internal.cuh"
-#include "synth_common.cuh"
+#include "synth_ops.cuh"
 
 namespace sbr {
 
 namespace {
 
-__global__ void k_prep_delays(int32_t Pr, const int32_t* __restrict__ nb, const double* __restrict__ pts,
-                              d3 T0, const double* __restrict__ R0p, const double* __restrict__ tx_elem,
-                              int32_t Nt, const double* __restrict__ rx_elem, int32_t Nr,
-                              double* __restrict__ dt, double* __restrict__ dr) {
-    const d3 R0 = ld3(R0p);
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int64_t ne = (int64_t)Nt + Nr;
-    if (t >= (int64_t)Pr * ne) return;
-    int64_t n = t / ne;
-    int32_t e = (int32_t)(t - n * ne);
-    int m = nb[n];
-    double v = 0.0;
-    if (m > 0) {
-        if (e < Nt) {
-            d3 P1 = ld3(pts + (n * kKmax) * 3);
-            v = norm(ld3(tx_elem + 3 * e) - P1) - norm(T0 - P1);
-        } else {
-            d3 Pm = ld3(pts + (n * kKmax + m - 1) * 3);
-            v = norm(ld3(rx_elem + 3 * (e - Nt)) - Pm) - norm(R0 - Pm);
+// ---------------------------------------------------------------- delays
+// |b + e| - |b| = e . (2 b + e) / (|b + e| + |b|) without the cancellation of the
+// difference; e and b in double-float
+__device__ __forceinline__ df length_change(const df3& b, df b_norm, const df3& e) {
+    const df3 a = df3_add(b, e), s = df3_add(a, b);
+    const df n2 = df3_dot(a, a);
+    const df n = n2.hi > 0.f ? df_sqrt(n2) : df{0.f, 0.f};
+    const df den = df_add(n, b_norm);
+    return den.hi > 0.f ? df_mul(df3_dot(e, s), df_rcp(den)) : df{0.f, 0.f};
+}
+__device__ __forceinline__ df3 df3_from(d3 v) { return df3{df_split(v.x), df_split(v.y), df_split(v.z)}; }
+__device__ __forceinline__ df df3_norm(const df3& v) {
+    const df n2 = df3_dot(v, v);
+    return n2.hi > 0.f ? df_sqrt(n2) : df{0.f, 0.f};
+}
+
+// Element delays of the paths as (hi, lo): an FP32 delay alone would carry 6e-8 of
+// its cycles into the phase. Thread per element over kDelayPaths paths: the element's offset from its array's reference
+// and each path's vector from the reference to its point are differences taken in
+// FP64, the rest is double-float.
+struct DelayArgs {
+    int64_t P;                // paths
+    const int32_t* nb;
+    const double* pts;
+    const double* R0;         // reference-point form: receiver reference; else null
+    const int32_t* rx;        // per-element form: receiver of each path
+    const double* rx_xyz;
+    d3 T0;
+    const double* tx_elem;
+    const double* rx_elem;    // reference-point form
+    int32_t Nt, Nr;
+    float2 *dt, *dr, *dlos;   // [P][Nt], [P][Nr], [Nr][Nt]
+};
+constexpr int kDelayThreads = 128, kDelayPaths = 2;
+
+// path blocks in y (then, reference-point form, receive elements in groups of
+// kDelayPaths for dlos), elements (transmit, then receive) in x
+__global__ void __launch_bounds__(kDelayThreads) k_delays(const __grid_constant__ DelayArgs a) {
+    ::sbr::pdl_wait();
+    __shared__ df3 s_b[2][kDelayPaths];
+    __shared__ df s_n[2][kDelayPaths];
+    const int64_t blocks = (a.P + kDelayPaths - 1) / kDelayPaths;
+    const bool los = (int64_t)blockIdx.y >= blocks;
+    const int64_t n0 = ((int64_t)blockIdx.y - (los ? blocks : 0)) * kDelayPaths;
+    const d3 R0 = a.R0 ? ld3(a.R0) : mk3(0, 0, 0);
+    if (!los && threadIdx.x < 2 * kDelayPaths) {
+        const int k = threadIdx.x % kDelayPaths, rx_side = threadIdx.x / kDelayPaths;
+        const int64_t n = n0 + k;
+        if (n < a.P) {
+            const int m = a.nb[n];
+            d3 b = mk3(0, 0, 0);
+            if (m > 0) b = rx_side ? R0 - ld3(a.pts + (n * kKmax + m - 1) * 3) : a.T0 - ld3(a.pts + n * kKmax * 3);
+            else if (a.rx) b = a.T0 - ld3(a.rx_xyz + 3 * (int64_t)a.rx[n]);   // LoS of the path's own receiver
+            s_b[rx_side][k] = df3_from(b);
+            s_n[rx_side][k] = df3_norm(s_b[rx_side][k]);
         }
     }
-    if (e < Nt) dt[n * Nt + e] = v;
-    else dr[n * Nr + (e - Nt)] = v;
-}
-
-__global__ void k_prep_w(int32_t Pr, int32_t F, const float2* __restrict__ g,
-                         const double* __restrict__ L, const double* __restrict__ freqs,
-                         double2* __restrict__ w) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (int64_t)Pr * F) return;
-    int64_t f = t / Pr;
-    int64_t n = t - f * Pr;
-    double cyc = freqs[f] * L[n] / kC0;
-    double fr = cyc - floor(cyc);
-    double s, c;
-    sincospi(-2.0 * fr, &s, &c);
-    float2 gg = g[n * F + f];
-    w[f * Pr + n] = make_double2(gg.x * c - gg.y * s, gg.x * s + gg.y * c);
-}
-
-__global__ void k_prep_los(d3 T0, const double* __restrict__ R0p, const double* __restrict__ tx_elem,
-                           int32_t Nt, const double* __restrict__ rx_elem, int32_t Nr,
-                           double* __restrict__ dlos) {
-    const d3 R0 = ld3(R0p);
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (int64_t)Nr * Nt) return;
-    int64_t q = t / Nt, p = t - q * Nt;
-    dlos[t] = norm(ld3(tx_elem + 3 * p) - ld3(rx_elem + 3 * q)) - norm(T0 - R0);
-}
-
-template <class R>
-struct Cplx;
-template <>
-struct Cplx<float> { using T = float2; };
-template <>
-struct Cplx<double> { using T = double2; };
-
-__device__ __forceinline__ void sincospi_(float x, float* s, float* c) { sincospif(x, s, c); }
-__device__ __forceinline__ void sincospi_(double x, double* s, double* c) { sincospi(x, s, c); }
-
-template <class R>
-__global__ void k_convert(const double* __restrict__ in, R* __restrict__ out, int64_t n) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = (R)in[i];
-}
-
-template <class R>
-__global__ void k_convert2(const double2* __restrict__ in, typename Cplx<R>::T* __restrict__ out,
-                           int64_t n) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) { out[i].x = (R)in[i].x; out[i].y = (R)in[i].y; }
-}
-
-constexpr int kSynthThreads = 128;
-
-template <class R>
-__global__ void __launch_bounds__(kSynthThreads)
-k_synth(int32_t F, int32_t Nr, int32_t Nt, int32_t Pr, const int32_t* __restrict__ nb0,
-        const double* __restrict__ freqs,
-        const typename Cplx<R>::T* __restrict__ w, const R* __restrict__ dt, const R* __restrict__ dr,
-        const R* __restrict__ dlos, float2* __restrict__ H) {
-    using C2 = typename Cplx<R>::T;
-    __shared__ C2 s_w[kSynthThreads];
-    __shared__ R s_dr[kSynthThreads];
-    const int32_t p = blockIdx.x * kSynthThreads + threadIdx.x;
-    const int32_t q = blockIdx.y;
-    const int32_t f = blockIdx.z;
-    const R foc = (R)(freqs[f] / kC0);
-    const int32_t los = (Pr > 0 && *nb0 == 0) ? 0 : -1;
-    const bool act = p < Nt;
-    R acc_re = 0, acc_im = 0;
-    for (int32_t n0 = 0; n0 < Pr; n0 += kSynthThreads) {
-        int32_t n = n0 + threadIdx.x;
-        if (n < Pr) {
-            s_w[threadIdx.x] = w[(int64_t)f * Pr + n];
-            s_dr[threadIdx.x] = dr[(int64_t)n * Nr + q];
+    __syncthreads();
+    const int64_t e = (int64_t)blockIdx.x * kDelayThreads + threadIdx.x;
+    const bool rx_side = e >= a.Nt;
+    if (e >= (int64_t)a.Nt + (a.R0 && !los ? a.Nr : 0)) return;
+    const df3 off = df3_from(rx_side ? ld3(a.rx_elem + 3 * (e - a.Nt)) - R0 : ld3(a.tx_elem + 3 * e) - a.T0);
+    if (los) {   // |T_p - R_q| - |T_0 - R_0|
+        const df3 b = df3_from(a.T0 - R0);
+        const df bn = df3_norm(b);
+        for (int64_t q = n0; q < n0 + kDelayPaths && q < a.Nr; ++q) {
+            const df v = length_change(b, bn, df3_sub(off, df3_from(ld3(a.rx_elem + 3 * q) - R0)));
+            a.dlos[q * a.Nt + e] = make_float2(v.hi, v.lo);
         }
+        return;
+    }
+    for (int k = 0; k < kDelayPaths && n0 + k < a.P; ++k) {
+        // a LoS path of the reference-point form takes its delay from dlos
+        const df v = a.nb[n0 + k] > 0 || a.rx ? length_change(s_b[rx_side][k], s_n[rx_side][k], off) : df{0.f, 0.f};
+        (rx_side ? a.dr + (n0 + k) * a.Nr + (e - a.Nt) : a.dt + (n0 + k) * a.Nt + e)[0] = make_float2(v.hi, v.lo);
+    }
+}
+
+sbr_status delays_run(const DelayArgs& a, cudaStream_t s) {
+    const int64_t e = (int64_t)a.Nt + (a.R0 ? a.Nr : 0);
+    const int64_t y = (a.P + kDelayPaths - 1) / kDelayPaths + (a.R0 ? (a.Nr + kDelayPaths - 1) / kDelayPaths : 0);
+    if (y == 0) return SBR_OK;
+    // path groups in slices of at most 65535 (P up to 2^31)
+    if (y > 65535) {
+        DelayArgs part = a;
+        const int64_t step = 32768 * (int64_t)kDelayPaths;
+        const double* r0 = a.R0;
+        for (int64_t n = 0; n < a.P; n += step) {
+            part.P = std::min(step, a.P - n);
+            part.nb = a.nb + n;
+            part.pts = a.pts + n * kKmax * 3;
+            part.rx = a.rx ? a.rx + n : nullptr;
+            part.dt = a.dt + n * a.Nt;
+            part.dr = a.dr + n * a.Nr;
+            part.R0 = r0;
+            SBR_TRY(delays_run(part, s));   // (writes dlos again: the same values)
+        }
+        return SBR_OK;
+    }
+    ::sbr::note_launch();
+    SBR_TRY_CUDA(::sbr::launch_pdl(k_delays, dim3((unsigned)((e + kDelayThreads - 1) / kDelayThreads), (unsigned)y),
+                                   dim3(kDelayThreads), 0, s, a));
+    return SBR_OK;
+}
+
+// ---------------------------------------------------------------- phasors
+// exp(-j 2 pi x) for x = foc d cycles (foc = f / c), FP32: the nearest multiple of
+// a quarter turn is removed exactly (foc d - k / 4 in one fused operation, plus the
+// terms of the low words), sine and cosine of the rest (|z| <= pi / 4) from their Taylor
+// series (remainders below 2e-9). Phases beyond 2^19 turns take sincospif.
+__device__ __forceinline__ float2 phasor32(df foc, float2 d) {
+    const float x4 = 4.f * __fmul_rn(foc.hi, d.x);
+    if (!(fabsf(x4) < 2097152.f)) {
+        float s, c;
+        sincospif(-2.f * (foc.hi * d.x), &s, &c);
+        return make_float2(c, s);
+    }
+    const float m = __fadd_rn(x4, 12582912.f);   // 1.5 2^23: the sum's low bits are the integer
+    const float k = __fsub_rn(m, 12582912.f);
+    const float r = __fmaf_rn(foc.hi, d.y, __fmaf_rn(foc.lo, d.x, __fmaf_rn(foc.hi, d.x, -0.25f * k)));
+    const float z = 6.28318531f * r, z2 = z * z;
+    float s = fmaf(z2, 2.75573192e-6f, -1.98412698e-4f);
+    s = fmaf(s, z2, 8.33333333e-3f);
+    s = fmaf(s, z2, -1.66666667e-1f);
+    s = fmaf(s * z2, z, z);
+    float c = fmaf(z2, -2.75573192e-7f, 2.48015873e-5f);
+    c = fmaf(c, z2, -1.38888889e-3f);
+    c = fmaf(c, z2, 4.16666667e-2f);
+    c = fmaf(c, z2, -0.5f);
+    c = fmaf(c, z2, 1.f);
+    const int q = __float_as_int(m);
+    // exp(-j (z + q pi / 2)): swap for odd q, then the signs
+    const float a = (q & 1) ? s : c, b = (q & 1) ? c : s;
+    const float re = __int_as_float(__float_as_int(a) ^ (((q + 1) & 2) << 30));
+    const float im = __int_as_float(__float_as_int(b) ^ ((~q & 2) << 30));
+    return make_float2(re, im);
+}
+
+// the same in double-float: the leading terms of the series in double-float, the
+// later ones (below 4e-7 of the sum) in FP32
+__device__ __forceinline__ cdf2 phasor_df(df x) {
+    const float k = rintf(4.f * x.hi);
+    const df r = df_add(df{__fmaf_rn(-0.25f, k, x.hi), 0.f}, df{x.lo, 0.f});
+    const df z = df_mul(r, df{6.28318548f, -1.74845560e-7f});
+    const df z2 = df_mul(z, z);
+    const float t = z2.hi;
+    float u = fmaf(t, 1.60590438e-10f, -2.50521084e-8f);   // 1/13!, 1/11!
+    u = fmaf(u, t, 2.75573192e-6f);                        // 1/9!
+    df s = df_fma(df{-1.98412701e-4f, 2.7255969e-12f}, z2, df{u, 0.f});       // 1/7!
+    s = df_fma(df{8.33333377e-3f, -4.34617203e-10f}, z2, s);                  // 1/5!
+    s = df_fma(df{-0.166666672f, 4.96705379e-9f}, z2, s);                     // 1/3!
+    s = df_fma(z, df_mul(z, z2), s);
+    u = fmaf(t, -1.14707456e-11f, 2.08767570e-9f);         // 1/14!, 1/12!
+    u = fmaf(u, t, -2.75573192e-7f);                       // 1/10!
+    df c = df_fma(df{2.48015876e-5f, -3.40699612e-13f}, z2, df{u, 0.f});      // 1/8!
+    c = df_fma(df{-1.38888892e-3f, 3.36310929e-11f}, z2, c);                  // 1/6!
+    c = df_fma(df{4.16666679e-2f, -1.24176345e-9f}, z2, c);                   // 1/4!
+    c = df_fma(df{-0.5f, 0.f}, z2, c);
+    c = df_fma(df{1.f, 0.f}, z2, c);
+    const int q = (int)k;
+    df a = (q & 1) ? s : c, b = (q & 1) ? c : s;
+    if ((q + 1) & 2) a = df_neg(a);
+    if (~q & 2) b = df_neg(b);
+    return cdf2_make(a, b);
+}
+
+// cycles f L / c modulo 1 from double-float factors, in [-0.5, 0.5] and a bit:
+// absolute error about 4e-15 of the product (1e6 cycles: 4e-9)
+__device__ __forceinline__ float cycles_mod1(df f, df t) {
+    const df p = two_prod(f.hi, t.hi);
+    const float k = rintf(p.hi);
+    return __fadd_rn(__fsub_rn(p.hi, k), __fmaf_rn(f.hi, t.lo, __fmaf_rn(f.lo, t.hi, p.lo)));
+}
+__device__ __forceinline__ float2 cmul32(float2 a, float2 b) {
+    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+}
+
+// the arithmetic of the two forms: C a complex value
+struct Form32 {
+    using C = float2;
+    struct Freq { df f, foc; };
+    static __device__ __forceinline__ Freq freq(double f) { return Freq{df_split(f), df_split(f * kInvC0)}; }
+    static __device__ __forceinline__ C phasor(const Freq& f, float2 d) { return phasor32(f.foc, d); }
+    // g exp(-j 2 pi f L / c)
+    static __device__ __forceinline__ C weight(float2 g, const Freq& f, double, double L) {
+        return cmul32(g, phasor32(df{1.f, 0.f}, make_float2(cycles_mod1(f.f, df_split(L * kInvC0)), 0.f)));
+    }
+    static __device__ __forceinline__ C mul(C a, C b) { return cmul32(a, b); }
+    static __device__ __forceinline__ void mac(C& acc, const C& a, const C&, const C& v) {
+        acc.x = fmaf(a.x, v.x, fmaf(-a.y, v.y, acc.x));
+        acc.y = fmaf(a.x, v.y, fmaf(a.y, v.x, acc.y));
+    }
+    static __device__ __forceinline__ C zero() { return make_float2(0.f, 0.f); }
+    static __device__ __forceinline__ C add(C a, C b) { return make_float2(a.x + b.x, a.y + b.y); }
+    static __device__ __forceinline__ C turned(const C& a) { return a; }
+    static __device__ __forceinline__ float2 out(const C& a) { return a; }
+};
+struct FormDf {
+    using C = cdf2;
+    struct Freq { df foc; };
+    static __device__ __forceinline__ Freq freq(double f) { return Freq{df_split(f / kC0)}; }
+    static __device__ __forceinline__ C phasor(const Freq& f, float2 d) { return phasor_df(df_mul(f.foc, df{d.x, d.y})); }
+    static __device__ __forceinline__ C weight(float2 g, const Freq&, double f, double L) {
+        const double cyc = f * L / kC0;
+        return mul(C{g, make_float2(0.f, 0.f)}, phasor_df(df_split(cyc - floor(cyc))));
+    }
+    static __device__ __forceinline__ C mul(const C& a, const C& b) {
+        C r = zero();
+        cdf2_mac(r, a, cdf2_j(a), b);
+        return r;
+    }
+    static __device__ __forceinline__ void mac(C& acc, const C& a, const C& ja, const C& v) { cdf2_mac(acc, a, ja, v); }
+    static __device__ __forceinline__ C zero() { return C{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
+    static __device__ __forceinline__ C add(const C& a, const C& b) {
+        return cdf2_make(df_add(df{a.h.x, a.l.x}, df{b.h.x, b.l.x}), df_add(df{a.h.y, a.l.y}, df{b.h.y, b.l.y}));
+    }
+    static __device__ __forceinline__ C turned(const C& a) { return cdf2_j(a); }
+    static __device__ __forceinline__ float2 out(const C& a) { return a.h; }
+};
+
+// ---------------------------------------------------------------- reference-point form
+// Block: one frequency, 8 RQ receive x 64 transmit elements; G groups of 128
+// threads of RQ x 4 outputs each. Paths in chunks of G NC: all threads fill the
+// chunk's weighted receive phasors and transmit phasors in shared memory (their
+// delays were requested while the previous chunk was summed), then group g runs
+// the outer products of its NC paths; the groups' sums are added at the end. The
+// LoS path (if any, the first) is added per output. Bound by the FP32 pipe: 4
+// operations a term in FP32, 54 in double-float. RQ follows Nr (the smallest of 1,
+// 2, 4, 8 that covers it: rows past Nr are computed for nothing, and a block
+// shares its transmit phasors among 8 RQ rows); G follows the number of blocks, up
+// to 4, so that few frequencies still fill the SMs with warps.
+// Measured: FP32, F 600, 13 x 63, 129 paths: 156 us with a sine and cosine per
+// term and eight launches, 33 us so; FP64, F 128, 16 x 64, 63 paths: 572 us in
+// FP64, 32 us so.
+constexpr int kSynthThreads = 128, kSynthPT = 64;
+
+struct SynthArgs {
+    int32_t F, Nr, Nt, Pr;
+    const int32_t* nb0;       // reflections of the first path (0: it is the LoS path)
+    const double* freqs;
+    const float2* g;          // [Pr][F]
+    const double* L;
+    const float2 *dt, *dr, *dlos;
+    float2* H;
+};
+
+template <class M, int RQ, int G>
+__global__ void __launch_bounds__(kSynthThreads* G) k_synth(const __grid_constant__ SynthArgs a) {
+    ::sbr::pdl_wait();
+    using C = typename M::C;
+    constexpr int QT = 8 * RQ, NC = sizeof(C) == 8 ? 16 : 8, NT = kSynthThreads * G, NCG = NC * G;
+    constexpr int kV = NCG * kSynthPT / NT, kA = (NCG * QT + NT - 1) / NT, kW = 128;   // per thread; NCG divides kW
+    constexpr int kPhasors = NCG * (QT + kSynthPT), kSums = G > 1 ? QT * kSynthPT : 0;
+    __shared__ C s_mem[kPhasors > kSums ? kPhasors : kSums], s_w[kW];
+    C* s_a = s_mem;                    // [NCG][QT]
+    C* s_v = s_mem + NCG * QT;         // [NCG][kSynthPT]
+    const int tid = threadIdx.x, tp = tid & 15, tq = (tid >> 4) & 7, grp = tid / kSynthThreads;
+    const int32_t f = blockIdx.x, p0 = blockIdx.y * kSynthPT, q0 = blockIdx.z * QT;
+    const double fr = a.freqs[f];
+    const typename M::Freq fq = M::freq(fr);
+    const int los = a.Pr > 0 && *a.nb0 == 0 ? 1 : 0;
+    C acc[RQ][4];
+#pragma unroll
+    for (int i = 0; i < RQ; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = M::zero();
+    float2 dv[kV], da[kA];   // delays of the chunk
+    auto request = [&](int n0) {
+#pragma unroll
+        for (int i = 0; i < kV; ++i) {
+            const int e = tid + i * NT, n = n0 + e / kSynthPT, p = p0 + e % kSynthPT;
+            dv[i] = n < a.Pr && p < a.Nt ? __ldg(a.dt + (int64_t)n * a.Nt + p) : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int i = 0; i < kA; ++i) {
+            const int e = tid + i * NT, n = n0 + e / QT, q = q0 + e % QT;
+            da[i] = e < NCG * QT && n < a.Pr && q < a.Nr ? __ldg(a.dr + (int64_t)n * a.Nr + q) : make_float2(0.f, 0.f);
+        }
+    };
+    request(los);
+    for (int n0 = los; n0 < a.Pr; n0 += NCG) {
+        const int cnt = min(NCG, a.Pr - n0), w0 = (n0 - los) % kW;
+        if (w0 == 0) {   // the weights of the next kW paths
+            if (n0 > los) __syncthreads();
+            if (tid < kW && n0 + tid < a.Pr) s_w[tid] = M::weight(a.g[(int64_t)(n0 + tid) * a.F + f], fq, fr, a.L[n0 + tid]);
+        }
+        if (n0 == los || w0 == 0) __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kV; ++i)
+            if ((tid + i * NT) / kSynthPT < cnt) s_v[tid + i * NT] = M::phasor(fq, dv[i]);
+#pragma unroll
+        for (int i = 0; i < kA; ++i)
+            if ((tid + i * NT) / QT < cnt) s_a[tid + i * NT] = M::mul(s_w[w0 + (tid + i * NT) / QT], M::phasor(fq, da[i]));
         __syncthreads();
-        int32_t cnt = min(kSynthThreads, Pr - n0);
-        if (act) {
-            for (int32_t k = 0; k < cnt; ++k) {
-                int32_t nn = n0 + k;
-                R delay = nn == los ? dlos[(int64_t)q * Nt + p] : dt[(int64_t)nn * Nt + p] + s_dr[k];
-                R s, c;
-                sincospi_((R)-2 * foc * delay, &s, &c);
-                C2 ww = s_w[k];
-                acc_re += ww.x * c - ww.y * s;
-                acc_im += ww.x * s + ww.y * c;
+        if (n0 + NCG < a.Pr) request(n0 + NCG);
+        for (int k = grp * NC; k < min(cnt, grp * NC + NC); ++k) {
+            C v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = s_v[k * kSynthPT + tp + 16 * j];
+#pragma unroll
+            for (int i = 0; i < RQ; ++i) {
+                const C x = s_a[k * QT + tq + 8 * i], jx = M::turned(x);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) M::mac(acc[i][j], x, jx, v[j]);
             }
         }
         __syncthreads();
     }
-    if (act) H[((int64_t)f * Nr + q) * Nt + p] = make_float2((float)acc_re, (float)acc_im);
-}
-
-inline unsigned nb256(int64_t n) { return (unsigned)std::max<int64_t>(1, (n + 255) / 256); }
-
-// per-element reception: element delays of every path (FP64),
-//   dt_np = |T_p - R_q| - L_n for the LoS path of element q (so that L_n + dt_np
-//   is the exact element-pair distance), |T_p - P1| - |T_0 - P1| otherwise
-__global__ void k_el_delays(int64_t P, const int32_t* __restrict__ rx, const int32_t* __restrict__ nb,
-                            const double* __restrict__ pts, const double* __restrict__ L, d3 T0,
-                            const double* __restrict__ rx_xyz, const double* __restrict__ tx_elem, int32_t Nt,
-                            double* __restrict__ dt) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= P * Nt) return;
-    int64_t n = t / Nt;
-    int32_t p = (int32_t)(t - n * Nt);
-    d3 Tp = ld3(tx_elem + 3 * p);
-    double v;
-    if (nb[n] == 0) {
-        v = norm(Tp - ld3(rx_xyz + 3 * rx[n])) - L[n];
-    } else {
-        d3 P1 = ld3(pts + (n * kKmax) * 3);
-        v = norm(Tp - P1) - norm(T0 - P1);
+    if (G > 1) {   // the sums of groups 1 .. G - 1 into group 0
+        for (int h = 1; h < G; ++h) {
+            if (grp == h)
+#pragma unroll
+                for (int i = 0; i < RQ; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) s_mem[(4 * i + j) * kSynthThreads + tid % kSynthThreads] = acc[i][j];
+            __syncthreads();
+            if (grp == 0)
+#pragma unroll
+                for (int i = 0; i < RQ; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[i][j] = M::add(acc[i][j], s_mem[(4 * i + j) * kSynthThreads + tid]);
+            __syncthreads();
+        }
+        if (grp > 0) return;
     }
-    dt[t] = v;
+    if (los) {
+        const C w = M::weight(a.g[f], fq, fr, a.L[0]), jw = M::turned(w);
+#pragma unroll
+        for (int i = 0; i < RQ; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int q = q0 + tq + 8 * i, p = p0 + tp + 16 * j;
+                if (q < a.Nr && p < a.Nt)
+                    M::mac(acc[i][j], w, jw, M::phasor(fq, __ldg(a.dlos + (int64_t)q * a.Nt + p)));
+            }
+    }
+#pragma unroll
+    for (int i = 0; i < RQ; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int q = q0 + tq + 8 * i, p = p0 + tp + 16 * j;
+            if (q < a.Nr && p < a.Nt) a.H[((int64_t)f * a.Nr + q) * a.Nt + p] = M::out(acc[i][j]);
+        }
 }
 
-// H[f, q, :] = sum over element q's own paths n of w_n(f) exp(-j 2 pi f dt_np / c)
-template <class R>
-__global__ void __launch_bounds__(kSynthThreads)
-k_synth_el(int32_t F, int32_t Nq, int32_t Nt, int64_t P, const int32_t* __restrict__ rx_off,
-           const double* __restrict__ freqs, const typename Cplx<R>::T* __restrict__ w,
-           const R* __restrict__ dt, float2* __restrict__ H) {
-    using C2 = typename Cplx<R>::T;
-    __shared__ C2 s_w[kSynthThreads];
-    const int32_t p = blockIdx.x * kSynthThreads + threadIdx.x;
-    const int32_t q = blockIdx.y;
-    const int32_t f = blockIdx.z;
-    const R foc = (R)(freqs[f] / kC0);
-    const bool act = p < Nt;
-    const int32_t a0 = rx_off[q], a1 = rx_off[q + 1];
-    R acc_re = 0, acc_im = 0;
+template <class M, int RQ>
+sbr_status synth_launch(const SynthArgs& a, cudaStream_t s) {
+    const dim3 grid((unsigned)a.F, (unsigned)((a.Nt + kSynthPT - 1) / kSynthPT), (unsigned)((a.Nr + 8 * RQ - 1) / (8 * RQ)));
+    // groups: 32 warps per SM are wanted, a block of one group has four
+    const int64_t want = 8 * (int64_t)sm_count() / ((int64_t)grid.x * grid.y * grid.z);
+    ::sbr::note_launch();
+    if constexpr (RQ <= 2) {   // (48 KB of shared memory)
+        if (want >= 4) {
+            SBR_TRY_CUDA(::sbr::launch_pdl(k_synth<M, RQ, 4>, grid, dim3(4 * kSynthThreads), 0, s, a));
+            return SBR_OK;
+        }
+    }
+    if (want >= 2) SBR_TRY_CUDA(::sbr::launch_pdl(k_synth<M, RQ, 2>, grid, dim3(2 * kSynthThreads), 0, s, a));
+    else SBR_TRY_CUDA(::sbr::launch_pdl(k_synth<M, RQ, 1>, grid, dim3(kSynthThreads), 0, s, a));
+    return SBR_OK;
+}
+
+// ---------------------------------------------------------------- per-element form
+// H[f, q, :] = sum over element q's own paths n of w_n(f) exp(-j 2 pi f dt_np / c):
+// nothing is shared between receive elements, so the phasor of every term is
+// needed. FP32: a thread holds two transmit elements (so that their phasors
+// turn in packed operations: half the issue slots) at kElF consecutive frequencies; the phasor
+// at the middle one comes from phasor32, the others by rotating it with
+// exp(-j 2 pi df d / c) - 1 (precise for the small step between subcarriers, at
+// most eight rotations), four operations each instead of a sine and a cosine. That
+// needs equally spaced frequencies (to 2^-28 of a cycle over the delay) and a step
+// of at most 1/16 cycle, tested per path and element; other grids take phasor32
+// per term. The paths are summed from the last to the first: they are sorted by
+// their reflections, so the strongest come when the sum's rounding matters least.
+// Bound by the FP32 pipe, about eleven operations a term: F 512, 64 x 256, 63
+// paths per element: 948 us with sincospif per term and an FP64 prologue, 248 us
+// so (258 us with one element per thread and scalar operations, 269 us with every
+// operation packed and the weights doubled in shared memory).
+constexpr int kElF = 16, kElMid = 8, kElPaths = 64, kElMax = 128;
+
+struct ElArgs {
+    int32_t F, Nq, Nt;
+    const int32_t* rx_off;
+    const double* freqs;
+    const float2* g;          // [P][F]
+    const double* L;
+    const float2* dt;         // [P][Nt]
+    float2* H;
+};
+
+__global__ void __launch_bounds__(kElMax) k_synth_el32(const __grid_constant__ ElArgs a) {
+    ::sbr::pdl_wait();
+    __shared__ __align__(16) float2 s_w[kElPaths][kElF];
+    __shared__ df s_f[kElF], s_foc[kElF], s_t[kElPaths];
+    __shared__ float s_step, s_dev;
+    __shared__ df s_mid;
+    const int tid = threadIdx.x;
+    const int32_t f0 = blockIdx.x * kElF, q = blockIdx.y;
+    const int32_t p0 = blockIdx.z * 2 * blockDim.x + tid, p1 = p0 + blockDim.x;   // the two elements
+    const int nf = min(kElF, a.F - f0);
+    const bool act = p0 < a.Nt, two = p1 < a.Nt;
+    if (tid < 32) {   // one warp, at least: the block's frequencies
+        const double fk = a.freqs[f0 + min(tid, nf - 1)];
+        const double first = __shfl_sync(0xffffffffu, fk, 0), last = __shfl_sync(0xffffffffu, fk, nf - 1);
+        const double step = nf > 1 ? (last - first) / (nf - 1) : 0.0;
+        const double mid = nf > kElMid ? __shfl_sync(0xffffffffu, fk, kElMid) : first + kElMid * step;
+        float dev = (float)fabs((fk - mid - (min(tid, nf - 1) - kElMid) * step) * kInvC0);
+        if (!(dev == dev)) dev = INFINITY;
+        for (int o = 16; o; o >>= 1) dev = fmaxf(dev, __shfl_xor_sync(0xffffffffu, dev, o));
+        if (tid < kElF) {
+            s_f[tid] = df_split(fk);
+            s_foc[tid] = df_split(fk * kInvC0);
+        }
+        if (tid == 0) {
+            s_mid = df_split(mid * kInvC0);
+            s_step = (float)(step * kInvC0);
+            s_dev = dev;
+        }
+    }
+    const int32_t a0 = a.rx_off[q], a1 = a.rx_off[q + 1];
+    float2 re[kElF], im[kElF];   // of the two elements
+#pragma unroll
+    for (int k = 0; k < kElF; ++k) re[k] = im[k] = make_float2(0.f, 0.f);
+    for (int32_t n1 = a1; n1 > a0; n1 -= kElPaths) {   // paths [n0, n1)
+        const int cnt = min(kElPaths, n1 - a0);
+        const int32_t n0 = n1 - cnt;
+        __syncthreads();
+        for (int n = tid; n < cnt; n += blockDim.x) s_t[n] = df_split(a.L[n0 + n] * kInvC0);
+        __syncthreads();
+#pragma unroll 4
+        for (int e = tid; e < cnt * kElF; e += blockDim.x) {
+            const int n = e / kElF, k = e % kElF;
+            s_w[n][k] = k < nf ? cmul32(a.g[(int64_t)(n0 + n) * a.F + f0 + k],
+                                        phasor32(df{1.f, 0.f}, make_float2(cycles_mod1(s_f[k], s_t[n]), 0.f)))
+                               : make_float2(0.f, 0.f);
+        }
+        __syncthreads();
+        if (!act) continue;
+        const float2* dt = a.dt + (int64_t)n0 * a.Nt;
+        // delays two paths ahead
+        auto delay = [&](int n, int32_t p) { return __ldg(dt + (int64_t)max(n, 0) * a.Nt + p); };
+        const int32_t pb = two ? p1 : p0;
+        float2 da = delay(cnt - 1, p0), db = delay(cnt - 1, pb), ea = delay(cnt - 2, p0), eb = delay(cnt - 2, pb);
+        for (int n = cnt - 1; n >= 0; --n) {
+            const float2 d0 = da, d1 = db;
+            da = ea, db = eb;
+            ea = delay(n - 2, p0), eb = delay(n - 2, pb);
+            // scalar operations here: packed ones would need every weight twice, from
+            // shared memory (whose loads then bound the loop) or by moves
+            const float4* w4 = reinterpret_cast<const float4*>(s_w[n]);   // weights of two frequencies
+            auto add = [&](int k, float wx, float wy, float2 vx, float2 vy) {
+                re[k].x = fmaf(wx, vx.x, fmaf(-wy, vy.x, re[k].x));
+                re[k].y = fmaf(wx, vx.y, fmaf(-wy, vy.y, re[k].y));
+                im[k].x = fmaf(wx, vy.x, fmaf(wy, vx.x, im[k].x));
+                im[k].y = fmaf(wx, vy.y, fmaf(wy, vx.y, im[k].y));
+            };
+            auto turn = [&](float2& vx, float2& vy, float2 c, float2 sx, float2 sy) {
+                const float2 x = __ffma2_rn(vx, c, __ffma2_rn(vy, sx, vx));
+                vy = __ffma2_rn(vx, sy, __ffma2_rn(vy, c, vy));
+                vx = x;
+            };
+            const float dmax = fmaxf(fabsf(d0.x), fabsf(d1.x));
+            if (fabsf(s_step) * dmax <= 0.0625f && s_dev * dmax <= 3.7252903e-9f) {
+                // rotation by one step: c = cos z - 1, s = -sin z (and the other way round for -z)
+                const float2 z = __fmul2_rn(dup2(6.28318531f * s_step), make_float2(d0.x, d1.x)), z2 = __fmul2_rn(z, z);
+                float2 c = __ffma2_rn(z2, dup2(2.48015873e-5f), dup2(-1.38888889e-3f));
+                c = __ffma2_rn(c, z2, dup2(4.16666667e-2f));
+                c = __fmul2_rn(__ffma2_rn(c, z2, dup2(-0.5f)), z2);
+                float2 s = __ffma2_rn(z2, dup2(-1.98412698e-4f), dup2(8.33333333e-3f));
+                s = __ffma2_rn(s, z2, dup2(-1.66666667e-1f));
+                const float2 sp = __ffma2_rn(__fmul2_rn(s, z2), z, z), sn = make_float2(-sp.x, -sp.y);   // sin z, -sin z
+                const float2 m0 = phasor32(s_mid, d0), m1 = phasor32(s_mid, d1);
+                const float2 mx = make_float2(m0.x, m1.x), my = make_float2(m0.y, m1.y);
+                // upwards and downwards from the middle side by side: two independent chains
+                float2 ux = mx, uy = my, dx = mx, dy = my;
+#pragma unroll
+                for (int k = 0; k < kElMid; k += 2) {
+                    const float4 wu = w4[(kElMid + k) / 2], wd = w4[(kElMid - 2 - k) / 2];
+                    turn(dx, dy, c, sn, sp);
+                    add(kElMid + k, wu.x, wu.y, ux, uy);
+                    turn(ux, uy, c, sp, sn);
+                    add(kElMid - 1 - k, wd.z, wd.w, dx, dy);
+                    turn(dx, dy, c, sn, sp);
+                    add(kElMid + k + 1, wu.z, wu.w, ux, uy);
+                    if (k + 2 < kElMid) turn(ux, uy, c, sp, sn);
+                    add(kElMid - 2 - k, wd.x, wd.y, dx, dy);
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < kElF; ++k) {
+                    const float2 v0 = phasor32(s_foc[k], d0), v1 = phasor32(s_foc[k], d1);
+                    add(k, s_w[n][k].x, s_w[n][k].y, make_float2(v0.x, v1.x), make_float2(v0.y, v1.y));
+                }
+            }
+        }
+    }
+    if (act)
+#pragma unroll
+        for (int k = 0; k < kElF; ++k)
+            if (k < nf) {
+                float2* row = a.H + ((int64_t)(f0 + k) * a.Nq + q) * a.Nt;
+                row[p0] = make_float2(re[k].x, im[k].x);
+                if (two) row[p1] = make_float2(re[k].y, im[k].y);
+            }
+}
+
+// FP64 form: thread per output, every phasor in double-float
+__global__ void __launch_bounds__(kSynthThreads) k_synth_el_df(const __grid_constant__ ElArgs a) {
+    ::sbr::pdl_wait();
+    __shared__ cdf2 s_w[kSynthThreads];
+    const int32_t f = blockIdx.x, q = blockIdx.y, p = blockIdx.z * kSynthThreads + threadIdx.x;
+    const double fr = a.freqs[f];
+    const FormDf::Freq fq = FormDf::freq(fr);
+    const int32_t a0 = a.rx_off[q], a1 = a.rx_off[q + 1];
+    cdf2 acc = FormDf::zero();
     for (int32_t n0 = a0; n0 < a1; n0 += kSynthThreads) {
-        int32_t n = n0 + threadIdx.x;
-        if (n < a1) s_w[threadIdx.x] = w[(int64_t)f * P + n];
+        const int cnt = min(kSynthThreads, a1 - n0);
         __syncthreads();
-        int32_t cnt = min(kSynthThreads, a1 - n0);
-        if (act) {
-            for (int32_t k = 0; k < cnt; ++k) {
-                R s, c;
-                sincospi_((R)-2 * foc * dt[(int64_t)(n0 + k) * Nt + p], &s, &c);
-                C2 ww = s_w[k];
-                acc_re += ww.x * c - ww.y * s;
-                acc_im += ww.x * s + ww.y * c;
-            }
-        }
+        if ((int)threadIdx.x < cnt)
+            s_w[threadIdx.x] = FormDf::weight(a.g[(int64_t)(n0 + threadIdx.x) * a.F + f], fq, fr, a.L[n0 + threadIdx.x]);
         __syncthreads();
+        if (p < a.Nt)
+            for (int k = 0; k < cnt; ++k)
+                cdf2_mac(acc, s_w[k], cdf2_j(s_w[k]), FormDf::phasor(fq, __ldg(a.dt + (int64_t)(n0 + k) * a.Nt + p)));
     }
-    if (act) H[((int64_t)f * Nq + q) * Nt + p] = make_float2((float)acc_re, (float)acc_im);
+    if (p < a.Nt) a.H[((int64_t)f * a.Nq + q) * a.Nt + p] = acc.h;
 }
 
 }  // namespace
 
 sbr_status synth_elements_run(const sbr_path_list* pl, const float2* g, const double* freqs, int32_t F,
                               const double* tx_elem, int32_t Nt, bool fp64, float2* H, cudaStream_t s) {
-    const int64_t P = pl->P;
-    const int32_t Nq = pl->n_rx;
-    const int64_t Pp = std::max<int64_t>(P, 1);
-    double* dt;
-    double2* w;
-    SBR_TRY(dalloc_n(&dt, (size_t)Pp * Nt, s));
-    SBR_TRY(dalloc_n(&w, (size_t)Pp * F, s));
-    if (P > 0) {
-        d3 T0 = mk3(pl->tx[0], pl->tx[1], pl->tx[2]);
-        ::sbr::note_launch(), k_el_delays<<<nb256(P * Nt), 256, 0, s>>>(P, pl->rx, pl->nb, pl->pts, pl->L, T0,
-                                                                       pl->rx_xyz, tx_elem, Nt, dt);
-        ::sbr::note_launch(), k_prep_w<<<nb256(P * F), 256, 0, s>>>((int32_t)P, F, g, pl->L, freqs, w);
-        SBR_TRY_CUDA(cudaGetLastError());
+    DelayArgs d{};
+    d.P = pl->P;
+    d.nb = pl->nb;
+    d.pts = pl->pts;
+    d.rx = pl->rx;
+    d.rx_xyz = pl->rx_xyz;
+    d.T0 = mk3(pl->tx[0], pl->tx[1], pl->tx[2]);
+    d.tx_elem = tx_elem;
+    d.Nt = Nt;
+    SBR_TRY(dalloc_n(&d.dt, (size_t)pl->P * Nt, s));
+    sbr_status st = delays_run(d, s);
+    if (st == SBR_OK) {
+        const ElArgs a{F, pl->n_rx, Nt, pl->rx_off, freqs, g, pl->L, d.dt, H};
+        // FP32: two elements per thread, blocks as wide as the array up to kElMax threads
+        const int width = fp64 ? kSynthThreads : std::min(kElMax, ((Nt + 1) / 2 + 31) / 32 * 32), per = fp64 ? width : 2 * width;
+        const dim3 grid((unsigned)(fp64 ? F : (F + kElF - 1) / kElF), (unsigned)pl->n_rx, (unsigned)((Nt + per - 1) / per));
+        ::sbr::note_launch();
+        const cudaError_t e = fp64 ? ::sbr::launch_pdl(k_synth_el_df, grid, dim3(width), 0, s, a)
+                                   : ::sbr::launch_pdl(k_synth_el32, grid, dim3(width), 0, s, a);
+        if (e != cudaSuccess) {
+            set_error("per-element synthesis: %s", cudaGetErrorString(e));
+            st = SBR_ERR_CUDA;
+        }
     }
-    dim3 grid((unsigned)((Nt + kSynthThreads - 1) / kSynthThreads), (unsigned)Nq, (unsigned)F);
-    if (fp64) {
-        ::sbr::note_launch(), k_synth_el<double><<<grid, kSynthThreads, 0, s>>>(F, Nq, Nt, Pp, pl->rx_off, freqs, w,
-                                                                               dt, H);
-    } else {
-        float* dtf;
-        float2* wf;
-        SBR_TRY(dalloc_n(&dtf, (size_t)Pp * Nt, s));
-        SBR_TRY(dalloc_n(&wf, (size_t)Pp * F, s));
-        ::sbr::note_launch(), k_convert<float><<<nb256(Pp * Nt), 256, 0, s>>>(dt, dtf, Pp * Nt);
-        ::sbr::note_launch(), k_convert2<float><<<nb256(Pp * F), 256, 0, s>>>(w, wf, Pp * F);
-        ::sbr::note_launch(), k_synth_el<float><<<grid, kSynthThreads, 0, s>>>(F, Nq, Nt, Pp, pl->rx_off, freqs, wf,
-                                                                              dtf, H);
-        dfree(dtf, s);
-        dfree(wf, s);
-    }
-    SBR_TRY_CUDA(cudaGetLastError());
-    dfree(dt, s);
-    dfree(w, s);
-    return SBR_OK;
-}
-
-sbr_status synth_prepare(const sbr_path_list* pl, const float2* g, const double* freqs, int32_t F,
-                         const double* tx_elem, int32_t Nt, const double* rx_elem, int32_t Nr,
-                         int32_t rx_index, SynthPrep* sp, cudaStream_t s) {
-    const int32_t o0 = pl->h_rx_off[rx_index], o1 = pl->h_rx_off[rx_index + 1];
-    sp->Pr = o1 - o0;
-    sp->off = o0;
-    // the LoS path (no reflection) sorts first among a receiver's paths; the
-    // kernels read its reflection count and the receiver reference on the device
-    sp->nb0 = pl->nb + o0;
-    const int32_t Pr = std::max(sp->Pr, 1);
-    d3 T0 = mk3(pl->tx[0], pl->tx[1], pl->tx[2]);
-    const double* R0 = pl->rx_xyz + 3 * rx_index;
-    SBR_TRY(dalloc_n(&sp->dt, (size_t)Pr * Nt, s));
-    SBR_TRY(dalloc_n(&sp->dr, (size_t)Pr * Nr, s));
-    SBR_TRY(dalloc_n(&sp->w, (size_t)Pr * F, s));
-    SBR_TRY(dalloc_n(&sp->dlos, (size_t)Nr * Nt, s));
-    if (sp->Pr > 0) {
-        int64_t ne = (int64_t)sp->Pr * (Nt + Nr);
-        ::sbr::note_launch(), k_prep_delays<<<nb256(ne), 256, 0, s>>>(sp->Pr, pl->nb + o0, pl->pts + (int64_t)o0 * kKmax * 3,
-                                                T0, R0, tx_elem, Nt, rx_elem, Nr, sp->dt, sp->dr);
-        ::sbr::note_launch(), k_prep_w<<<nb256((int64_t)sp->Pr * F), 256, 0, s>>>(sp->Pr, F, g + (int64_t)o0 * F,
-                                                            pl->L + o0, freqs, sp->w);
-    }
-    ::sbr::note_launch(), k_prep_los<<<nb256((int64_t)Nr * Nt), 256, 0, s>>>(T0, R0, tx_elem, Nt, rx_elem, Nr, sp->dlos);
-    SBR_TRY_CUDA(cudaGetLastError());
-    return SBR_OK;
-}
-
-void synth_release(SynthPrep* sp, cudaStream_t s) {
-    if (sp->dt) dfree(sp->dt, s);
-    if (sp->dr) dfree(sp->dr, s);
-    if (sp->w) dfree(sp->w, s);
-    if (sp->dlos) dfree(sp->dlos, s);
-    *sp = SynthPrep{};
+    dfree(d.dt, s);
+    return st;
 }
 
 sbr_status synth_simt_run(const sbr_path_list* pl, const float2* g, const double* freqs, int32_t F,
                           const double* tx_elem, int32_t Nt, const double* rx_elem, int32_t Nr,
                           int32_t rx_index, bool fp64, float2* H, cudaStream_t s) {
-    SynthPrep sp;
-    SBR_TRY(synth_prepare(pl, g, freqs, F, tx_elem, Nt, rx_elem, Nr, rx_index, &sp, s));
-    dim3 grid((unsigned)((Nt + kSynthThreads - 1) / kSynthThreads), (unsigned)Nr, (unsigned)F);
-    const int32_t Pr = std::max(sp.Pr, 1);
-    if (fp64) {
-        ::sbr::note_launch(), k_synth<double><<<grid, kSynthThreads, 0, s>>>(F, Nr, Nt, sp.Pr, sp.nb0, freqs, sp.w, sp.dt,
-                                                       sp.dr, sp.dlos, H);
-        SBR_TRY_CUDA(cudaGetLastError());
-    } else {
-        float *dt, *dr, *dl;
-        float2* w;
-        SBR_TRY(dalloc_n(&dt, (size_t)Pr * Nt, s));
-        SBR_TRY(dalloc_n(&dr, (size_t)Pr * Nr, s));
-        SBR_TRY(dalloc_n(&dl, (size_t)Nr * Nt, s));
-        SBR_TRY(dalloc_n(&w, (size_t)Pr * F, s));
-        ::sbr::note_launch(), k_convert<float><<<nb256((int64_t)Pr * Nt), 256, 0, s>>>(sp.dt, dt, (int64_t)Pr * Nt);
-        ::sbr::note_launch(), k_convert<float><<<nb256((int64_t)Pr * Nr), 256, 0, s>>>(sp.dr, dr, (int64_t)Pr * Nr);
-        ::sbr::note_launch(), k_convert<float><<<nb256((int64_t)Nr * Nt), 256, 0, s>>>(sp.dlos, dl, (int64_t)Nr * Nt);
-        ::sbr::note_launch(), k_convert2<float><<<nb256((int64_t)Pr * F), 256, 0, s>>>(sp.w, w, (int64_t)Pr * F);
-        ::sbr::note_launch(), k_synth<float><<<grid, kSynthThreads, 0, s>>>(F, Nr, Nt, sp.Pr, sp.nb0, freqs, w, dt, dr, dl, H);
-        SBR_TRY_CUDA(cudaGetLastError());
-        dfree(dt, s); dfree(dr, s); dfree(dl, s); dfree(w, s);
+    const int32_t o0 = pl->h_rx_off[rx_index], Pr = pl->h_rx_off[rx_index + 1] - o0;
+    DelayArgs d{};
+    d.P = Pr;
+    d.nb = pl->nb + o0;
+    d.pts = pl->pts + (int64_t)o0 * kKmax * 3;
+    d.R0 = pl->rx_xyz + 3 * (int64_t)rx_index;
+    d.T0 = mk3(pl->tx[0], pl->tx[1], pl->tx[2]);
+    d.tx_elem = tx_elem;
+    d.rx_elem = rx_elem;
+    d.Nt = Nt;
+    d.Nr = Nr;
+    // the three tables in one allocation
+    const size_t nt = (size_t)Pr * Nt, nr = (size_t)Pr * Nr, nl = (size_t)Nr * Nt;
+    SBR_TRY(dalloc_n(&d.dt, nt + nr + nl, s));
+    d.dr = d.dt + nt;
+    d.dlos = d.dr + nr;
+    sbr_status st = delays_run(d, s);
+    if (st == SBR_OK) {
+        // the LoS path (no reflection) sorts first among a receiver's paths; the
+        // kernel reads its reflection count on the device
+        const SynthArgs a{F, Nr, Nt, Pr, d.nb, freqs, g + (int64_t)o0 * F, pl->L + o0, d.dt, d.dr, d.dlos, H};
+        if (fp64)
+            st = Nr <= 8 ? synth_launch<FormDf, 1>(a, s) : (Nr <= 16 ? synth_launch<FormDf, 2>(a, s) : synth_launch<FormDf, 4>(a, s));
+        else
+            st = Nr <= 8 ? synth_launch<Form32, 1>(a, s)
+                         : (Nr <= 16 ? synth_launch<Form32, 2>(a, s)
+                                     : (Nr <= 32 ? synth_launch<Form32, 4>(a, s) : synth_launch<Form32, 8>(a, s)));
     }
-    synth_release(&sp, s);
-    return SBR_OK;
+    dfree(d.dt, s);
+    return st;
 }
 
 }  // namespace sbr

@@ -34,7 +34,6 @@
 #include "batch.cuh"
 #include "tcgen05.cuh"
 #include "sbr_internal.cuh"
-#include "synth_common.cuh"
 #include "synth_ops.cuh"
 
 namespace sbr {
