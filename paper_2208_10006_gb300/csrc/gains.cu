@@ -13,7 +13,7 @@ namespace {
 // for 102,400 paths of up to two reflections x 8 frequencies: 2517 us in FP64
 // with eight lanes per item (one reflection each; idle lanes of an FP64 warp
 // instruction cost as much as busy ones); with the targets of the same receivers
-// (1436 us more) the two take 100 us now.
+// (1436 us more) the two take 103 us now.
 constexpr int kGainThreads = 64;
 
 __global__ void __launch_bounds__(kGainThreads)

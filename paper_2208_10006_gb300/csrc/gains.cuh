@@ -130,25 +130,29 @@ __device__ __forceinline__ cdf cdf_inv(cdf a) {
 __device__ __forceinline__ df df_scale2(df a, float s) { return df{a.hi * s, a.lo * s}; }   // s a power of two
 
 // e^x = m 2^n with m in [0.7, 1.42]: Cody-Waite reduction by ln 2 (double-float)
-// and the Taylor series on |r| <= 0.35, whose terms from r^2 on are below 0.07 of
-// the sum, so that FP32 carries them to 2^-27 of it. |x| beyond 400 saturates n.
+// and the Taylor series on |r| <= 0.35, through r^5 in double-float; the terms from
+// r^6 on are below 3e-6 of the sum, so that FP32 carries them to 2^-42 of it.
+// |x| beyond 400 saturates n.
 __device__ __forceinline__ df df_exp_parts(df x, int& n) {
     const float xh = fminf(fmaxf(x.hi, -400.f), 400.f);
     const float k = rintf(__fmul_rn(xh, 1.44269504f));
     const df p = two_prod(k, 0.693147182f);               // ln 2 = 0.693147182 - 1.9046543e-9
     const float lo = xh == x.hi ? x.lo : 0.f;
     const df r = two_sum(__fsub_rn(xh, p.hi), __fadd_rn(__fsub_rn(lo, p.lo), __fmul_rn(k, 1.9046543e-9f)));
-    float q = 1.f / 40320.f;
+    float q = 1.f / 479001600.f;
+    q = __fmaf_rn(q, r.hi, 1.f / 39916800.f);
+    q = __fmaf_rn(q, r.hi, 1.f / 3628800.f);
+    q = __fmaf_rn(q, r.hi, 1.f / 362880.f);
+    q = __fmaf_rn(q, r.hi, 1.f / 40320.f);
     q = __fmaf_rn(q, r.hi, 1.f / 5040.f);
     q = __fmaf_rn(q, r.hi, 1.f / 720.f);
-    q = __fmaf_rn(q, r.hi, 1.f / 120.f);
-    q = __fmaf_rn(q, r.hi, 1.f / 24.f);
-    q = __fmaf_rn(q, r.hi, 1.f / 6.f);
-    q = __fmaf_rn(q, r.hi, 0.5f);
-    q = __fmul_rn(q, __fmul_rn(r.hi, r.hi));
-    const df s = fast_two_sum(1.f, r.hi), t = two_sum(s.hi, q);
+    constexpr double c5 = 1.0 / 120.0, c4 = 1.0 / 24.0, c3 = 1.0 / 6.0;
+    df t = df_fma(df{(float)c5, (float)(c5 - (double)(float)c5)}, r, df{q, 0.f});
+    t = df_fma(df{(float)c4, (float)(c4 - (double)(float)c4)}, r, t);
+    t = df_fma(df{(float)c3, (float)(c3 - (double)(float)c3)}, r, t);
+    t = df_fma(df{0.5f, 0.f}, r, t);
     n = (int)k;
-    return fast_two_sum(t.hi, __fadd_rn(__fadd_rn(s.lo, t.lo), __fmaf_rn(r.lo, r.hi, r.lo)));
+    return df_add(df{1.f, 0.f}, df_fma(r, r, df_mul(r, t)));
 }
 
 // m reflections off surfaces surf[0..m), unfolded length Lp, polarimetric

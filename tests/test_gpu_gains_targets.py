@@ -46,6 +46,30 @@ def test_gains_over_materials(sbr, sigma, rough):
     assert (np.abs(g - go) <= 1e-6 * np.abs(go) + 2e-45).all(), np.nanmax(np.abs(g - go) / np.abs(go))
 
 
+@pytest.mark.parametrize("gamma", [0.0, 3e2, 3e4])   # dB/km: absorption exponents to 0, 0.1 and 10 a path
+@pytest.mark.parametrize("rough", [0.0, 2e-4])
+def test_gains_round_as_in_fp64(sbr, gamma, rough):
+    """The delay and angle statistics are FP64 sums over the gains, so the gains have to
+    be the FP32 rounding of the exact value: double-float errors (2^-42 with the
+    cancellations of most paths) move 2^-17 of the parts to the neighbouring number.
+    Bound: 1e-3 of them (an exponential in FP32 terms moves several in a hundred)."""
+    sc = scenes.shoebox(N=60, K=3)
+    sc["materials"] = np.array([[5.31, 0.1, rough], [2.0, 0.01, rough], [3.0, 1.0, rough]] * 2)
+    sc["freqs"] = np.geomspace(1e9, 300e9, 64)
+    sc["gamma_db_km"] = np.full(64, gamma, np.float32)
+    sc["disp_deg_km"] = np.zeros(64, np.float32)
+    r = sbr.run_scene(sc)
+    ex = {k: v.cpu().numpy() for k, v in r["export"].items()}
+    o = oracle.run(sc)
+    key = lambda p, i: (int(p["rx"][i]), tuple(p["seq"][i][: p["nb"][i]]))
+    at = {key(o["paths"], i): i for i in range(len(o["paths"]["rx"]))}
+    g = r["g"].cpu().numpy()
+    go = o["g"][[at[key(ex, i)] for i in range(len(g))]].astype(np.complex64)
+    parts, want = g.view(np.float32), go.view(np.float32)
+    assert parts.size > 2 * 60 * 64
+    assert (parts != want).mean() <= 1e-3, (parts != want).mean()
+
+
 @pytest.mark.parametrize("F", [1, 2, 5, 8, 31, 33])
 @pytest.mark.parametrize("n_taps", [1, 7, 32])
 def test_targets_over_ragged_sizes(sbr, F, n_taps):
