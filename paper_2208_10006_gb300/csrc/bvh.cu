@@ -229,7 +229,7 @@ __device__ __forceinline__ int32_t child_ref(int32_t c, const int32_t* __restric
 __global__ void k_emit(int64_t n, const int32_t* __restrict__ left, const int32_t* __restrict__ right,
                        const int32_t* __restrict__ span, int leaf_max,
                        const float* __restrict__ lbox, const float* __restrict__ ibox, float pad,
-                       float4* __restrict__ nodes, float* __restrict__ root) {
+                       float4* __restrict__ nodes, float4* __restrict__ root) {
     ::sbr::pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int64_t nn = n > 1 ? n - 1 : 1;
@@ -255,14 +255,17 @@ __global__ void k_emit(int64_t n, const int32_t* __restrict__ left, const int32_
         b0[k] = pad_lo(b0[k], pad); b0[3 + k] = pad_hi(b0[3 + k], pad);
         b1[k] = pad_lo(b1[k], pad); b1[3 + k] = pad_hi(b1[3 + k], pad);
     }
-    float4* o = nodes + 4 * i;
-    o[0] = make_float4(b0[0], b0[1], b0[2], b0[3]);
-    o[1] = make_float4(b0[4], b0[5], b1[0], b1[1]);
-    o[2] = make_float4(b1[2], b1[3], b1[4], b1[5]);
-    o[3] = make_float4(__int_as_float(r0), __int_as_float(r1), 0.f, 0.f);
+    node_store(nodes + 4 * i, b0, b1, r0, r1);
     if (i == 0) {
         const float* rb = n > 1 ? ibox : lbox;
-        for (int k = 0; k < 3; ++k) { root[k] = pad_lo(rb[k], pad); root[3 + k] = pad_hi(rb[3 + k], pad); }
+        float c[3], h[3];
+        for (int k = 0; k < 3; ++k) {
+            const float lo = pad_lo(rb[k], pad), hi = pad_hi(rb[3 + k], pad);
+            c[k] = 0.5f * lo + 0.5f * hi;
+            h[k] = half_extent(lo, hi, c[k]);
+        }
+        root[0] = make_float4(c[0], c[1], c[2], sqrtf(h[0] * h[0] + h[1] * h[1] + h[2] * h[2]));
+        root[1] = make_float4(h[0], h[1], h[2], 0.f);
     }
 }
 
@@ -311,7 +314,8 @@ __global__ void k_top_cut(int64_t nn, const int32_t* __restrict__ span, const in
     const float4* nd = nodes + 4 * i;
     const float4 n0 = nd[0], n1 = nd[1], n2 = nd[2], n3 = nd[3];
     const int32_t r[2] = {__float_as_int(n3.x), __float_as_int(n3.y)};
-    const float bx[2][6] = {{n0.x, n0.y, n0.z, n0.w, n1.x, n1.y}, {n1.z, n1.w, n2.x, n2.y, n2.z, n2.w}};
+    float bx[2][6];
+    node_boxes(n0, n1, n2, bx[0], bx[1]);
     for (int c = 0; c < 2; ++c) {
         if (span_size(span, r[c]) > lim) continue;
         const int e = atomicAdd(n_cut, 1);
@@ -363,11 +367,7 @@ __device__ void top_emit(const TopTask& tk, int nl, const float* sl, const float
             next[atomicAdd(s_next, 1)] = TopTask{cb[c], cn[c], ref[c], tk.depth + 1};
         }
     }
-    float4* o = nodes + 4 * (int64_t)tk.slot;
-    o[0] = make_float4(sl[0], sl[1], sl[2], sl[3]);
-    o[1] = make_float4(sl[4], sl[5], sr[0], sr[1]);
-    o[2] = make_float4(sr[2], sr[3], sr[4], sr[5]);
-    o[3] = make_float4(__int_as_float(ref[0]), __int_as_float(ref[1]), 0.f, 0.f);
+    node_store(nodes + 4 * (int64_t)tk.slot, sl, sr, ref[0], ref[1]);
 }
 
 // float <-> int with the same order (for shared-memory atomicMin / atomicMax
@@ -698,7 +698,7 @@ sbr_status build_lbvh(const float* prim_box, int64_t n, float pad_rel, int leaf_
     SBR_TRY(dalloc_n(&lbox, 6 * n, s));
     SBR_TRY(dalloc_n(&ibox, 6 * nn, s));
     SBR_TRY(dalloc_n(&out->nodes, 4 * nn, s));
-    SBR_TRY(dalloc_n(&out->d_root, 6, s));
+    SBR_TRY(dalloc_n(&out->d_root, 2, s));
     const int nparts = (int)std::min<int64_t>(std::max<int64_t>(1, (n + 255) / 256), 2 * (int64_t)sm_count());
     ::sbr::note_launch(), (void)::sbr::launch_pdl(k_bounds, dim3(nparts), dim3(256), 0, s, prim_box, n, part);
     ::sbr::note_launch(), (void)::sbr::launch_pdl(k_bounds_final, dim3(1), dim3(256), 0, s, part, nparts, bnd);

@@ -119,8 +119,8 @@ struct RefineScene {
 // (the caller then scans the surface).
 constexpr int kFindStack = 64;
 
-__device__ __forceinline__ bool in_box(float3 p, float lx, float ly, float lz, float hx, float hy, float hz) {
-    return p.x >= lx && p.x <= hx && p.y >= ly && p.y <= hy && p.z >= lz && p.z <= hz;
+__device__ __forceinline__ bool in_box(float3 p, float cx, float cy, float cz, float hx, float hy, float hz) {
+    return fabsf(p.x - cx) <= hx && fabsf(p.y - cy) <= hy && fabsf(p.z - cz) <= hz;
 }
 
 __device__ int32_t bvh_find_face(const RefineScene& sc, int s, d3 P) {
@@ -134,8 +134,8 @@ __device__ int32_t bvh_find_face(const RefineScene& sc, int s, d3 P) {
             const float4* nd = sc.nodes + 4 * (int64_t)ref;
             const float4 n0 = __ldg(nd), n1 = __ldg(nd + 1), n2 = __ldg(nd + 2), n3 = __ldg(nd + 3);
             const int32_t r0 = __float_as_int(n3.x), r1 = __float_as_int(n3.y);
-            const bool h0 = in_box(pf, n0.x, n0.y, n0.z, n0.w, n1.x, n1.y);
-            const bool h1 = in_box(pf, n1.z, n1.w, n2.x, n2.y, n2.z, n2.w) && r1 != r0;
+            const bool h0 = in_box(pf, n0.x, n0.y, n2.x, n1.x, n1.y, n2.z);
+            const bool h1 = in_box(pf, n0.z, n0.w, n2.y, n1.z, n1.w, n2.w) && r1 != r0;
             if (h0 && h1) {
                 if (sp == kFindStack) return -2;
                 stack[sp++] = r1;

@@ -123,13 +123,17 @@ sbr_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, int64_t n, int bits,
 sbr_status exclusive_scan_u32(uint32_t* data, int64_t n, uint32_t* total, cudaStream_t s);
 
 // ---------------------------------------------------------------- BVH
-// Node: 4 x float4 = child 0 box, child 1 box, refs. ref >= 0 internal node,
-// ref < 0 leaf holding sorted primitive ~ref.
+// Node: 4 x float4, the boxes of its two children as centre c and half extent h
+// (the packed slab test of the traversal wants them so, x and y of a child in one
+// pair, the z of both in another):
+//   (c0x, c0y, c1x, c1y), (h0x, h0y, h1x, h1y), (c0z, c1z, h0z, h1z), (ref0, ref1, 0, 0)
+// ref >= 0 internal node, ref < 0 leaf holding sorted primitive ~ref. The half
+// extents are rounded up: c -+ h covers the box.
 struct BvhNodes {
     float4* nodes = nullptr;   // [n_nodes * 4]
     int32_t* order = nullptr;  // [n] sorted position -> primitive index
     int32_t n_nodes = 0;       // internal nodes (>= 1 when n >= 1)
-    float* d_root = nullptr;   // [6] root bounds on the device
+    float4* d_root = nullptr;  // [2] root box on the device: (centre, half diagonal), (half extents, 0)
 };
 // Build over n primitives given by boxes [n*6] (lo xyz, hi xyz) on the device.
 // pad_rel: relative padding added to every child box (covers FP32 rounding).
@@ -279,6 +283,31 @@ sbr_status capacity_noalloc_run(const float2* H, int32_t F, int32_t Nr, int32_t 
 // ---------------------------------------------------------------- device helpers
 #ifdef __CUDACC__
 namespace sbr {
+__device__ __forceinline__ float half_extent(float lo, float hi, float c) {
+    return fmaxf(__fsub_ru(hi, c), __fsub_ru(c, lo));
+}
+// a node from its children's boxes (lo xyz, hi xyz) and references
+__device__ __forceinline__ void node_store(float4* o, const float* b0, const float* b1, int32_t r0, int32_t r1) {
+    float c[2][3], h[2][3];
+    for (int k = 0; k < 3; ++k) {
+        c[0][k] = 0.5f * b0[k] + 0.5f * b0[3 + k];
+        c[1][k] = 0.5f * b1[k] + 0.5f * b1[3 + k];
+        h[0][k] = half_extent(b0[k], b0[3 + k], c[0][k]);
+        h[1][k] = half_extent(b1[k], b1[3 + k], c[1][k]);
+    }
+    o[0] = make_float4(c[0][0], c[0][1], c[1][0], c[1][1]);
+    o[1] = make_float4(h[0][0], h[0][1], h[1][0], h[1][1]);
+    o[2] = make_float4(c[0][2], c[1][2], h[0][2], h[1][2]);
+    o[3] = make_float4(__int_as_float(r0), __int_as_float(r1), 0.f, 0.f);
+}
+// bounds of the stored child boxes, rounded outward
+__device__ __forceinline__ void node_boxes(float4 n0, float4 n1, float4 n2, float* b0, float* b1) {
+    const float c[2][3] = {{n0.x, n0.y, n2.x}, {n0.z, n0.w, n2.y}}, h[2][3] = {{n1.x, n1.y, n2.z}, {n1.z, n1.w, n2.w}};
+    for (int k = 0; k < 3; ++k) {
+        b0[k] = __fsub_rd(c[0][k], h[0][k]); b0[3 + k] = __fadd_ru(c[0][k], h[0][k]);
+        b1[k] = __fsub_rd(c[1][k], h[1][k]); b1[3 + k] = __fadd_ru(c[1][k], h[1][k]);
+    }
+}
 struct d3 {
     double x, y, z;
 };
