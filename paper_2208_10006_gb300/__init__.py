@@ -47,8 +47,10 @@ def _check(st: int):
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    # the current stream's handle without a Stream object around it (3 us)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _ptr(t):
@@ -58,7 +60,7 @@ def _ptr(t):
         raise ValueError("expected a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError("expected a contiguous tensor")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _ptr_or_pinned(t):
@@ -66,12 +68,12 @@ def _ptr_or_pinned(t):
     if t is not None and not t.is_cuda:
         if not t.is_pinned() or not t.is_contiguous():
             raise ValueError("expected a CUDA tensor or a contiguous pinned host tensor")
-        return C.c_void_p(t.data_ptr())
+        return t.data_ptr()
     return _ptr(t)
 
 
 def _dev():
-    if not torch.cuda.is_available():
+    if not torch.cuda.is_initialized() and not torch.cuda.is_available():
         raise RuntimeError("no CUDA device: the SBR library has no CPU path")
     return torch.device("cuda", torch.cuda.current_device())
 
@@ -570,6 +572,7 @@ class MLP:
         h = C.c_void_p()
         _check(_L().sbr_mlp_create(C.byref(c), p(lw), p(sh), p(sc), C.byref(h), _stream(stream)))
         self._h = h
+        self._n_params = int(_L().sbr_mlp_param_count(h))
 
     def train_step(self, x: torch.Tensor, y: torch.Tensor, loss: torch.Tensor = None, stream=None):
         assert x.dtype == torch.float32 and y.dtype == torch.float32
@@ -586,7 +589,7 @@ class MLP:
 
     def params(self, mode: int = 0, values: torch.Tensor = None, stream=None) -> torch.Tensor:
         """mode 0: parameters, 2: last gradients (flat float32); mode 1 loads `values`."""
-        n = int(_L().sbr_mlp_param_count(self._h))
+        n = self._n_params
         buf = values if mode == 1 else torch.empty(n, dtype=torch.float32, device=_dev())
         _check(_L().sbr_mlp_params(self._h, _ptr(buf), int(mode), _stream(stream)))
         return buf

@@ -178,8 +178,7 @@ void sbr_bvh_free(sbr_bvh* b) {
     if (!b) return;
     cudaStream_t s = b->stream;
     free_lbvh(&b->tree, s);
-    dfree(b->tri_rot, s); dfree(b->plane_sorted, s); dfree(b->tri, s); dfree(b->surf, s);
-    dfree(b->nrm, s); dfree(b->s_off, s); dfree(b->s_tri, s); dfree(b->d_depth, s);
+    dfree(b->mem, s);
     delete b;
 }
 
@@ -236,9 +235,11 @@ sbr_status sbr_trace(const sbr_bvh* b, const sbr_trace_params* p, sbr_trace_resu
         while (lg < 26 && ((int64_t)1 << lg) < (int64_t)p->n_rx * 512) ++lg;
         tr->table_log2 = lg;
     }
-    sbr_status st = SBR_OK;
+    Arena in;
+    if (tr->n_rx > 0) in.add(&tr->rx, 3 * (size_t)tr->n_rx);
+    in.add(&tr->d_alpha, 1);
+    sbr_status st = in.take(&tr->mem_in, s);
     if (tr->n_rx > 0) {
-        st = dalloc_n(&tr->rx, 3 * (size_t)tr->n_rx, s);
         if (st == SBR_OK &&
             cudaMemcpyAsync(tr->rx, p->rx_xyz, sizeof(double) * 3 * tr->n_rx, cudaMemcpyDeviceToDevice,
                             s) != cudaSuccess) {
@@ -246,7 +247,6 @@ sbr_status sbr_trace(const sbr_bvh* b, const sbr_trace_params* p, sbr_trace_resu
             st = SBR_ERR_CUDA;
         }
     }
-    if (st == SBR_OK) st = dalloc_n(&tr->d_alpha, 1, s);
     // a given alpha is stored by the trace's set-up launch; the default one
     // (alpha = 0) is computed from the launch grid first
     if (st == SBR_OK && !(p->alpha > 0.0)) st = launch_alpha_fast(p->subdiv_N, tr->d_alpha, s);
@@ -343,9 +343,11 @@ sbr_status sbr_trace_merge(const sbr_trace_params* p, const uint32_t* keys, cons
         while (lg < 28 && ((int64_t)1 << lg) < 2 * n) ++lg;   // load factor <= 1/2
         tr->table_log2 = lg;
     }
-    sbr_status st = SBR_OK;
+    Arena in;
+    if (tr->n_rx > 0) in.add(&tr->rx, 3 * (size_t)tr->n_rx);
+    in.add(&tr->d_alpha, 1);
+    sbr_status st = in.take(&tr->mem_in, s);
     if (tr->n_rx > 0) {
-        st = dalloc_n(&tr->rx, 3 * (size_t)tr->n_rx, s);
         if (st == SBR_OK &&
             cudaMemcpyAsync(tr->rx, p->rx_xyz, sizeof(double) * 3 * tr->n_rx, cudaMemcpyDeviceToDevice,
                             s) != cudaSuccess) {
@@ -353,7 +355,6 @@ sbr_status sbr_trace_merge(const sbr_trace_params* p, const uint32_t* keys, cons
             st = SBR_ERR_CUDA;
         }
     }
-    if (st == SBR_OK) st = dalloc_n(&tr->d_alpha, 1, s);
     if (st == SBR_OK && !(p->alpha > 0.0)) st = launch_alpha_fast(p->subdiv_N, tr->d_alpha, s);
     if (st == SBR_OK) st = trace_merge_run(tr, keys, reinterpret_cast<const unsigned long long*>(vals), n, s);
     if (st != SBR_OK) {
@@ -367,8 +368,8 @@ sbr_status sbr_trace_merge(const sbr_trace_params* p, const uint32_t* keys, cons
 void sbr_trace_free(sbr_trace_result* tr) {
     if (!tr) return;
     cudaStream_t s = tr->stream;
-    dfree(tr->seqf, s); dfree(tr->rx, s); dfree(tr->d_alpha, s); dfree(tr->ht_state, s); dfree(tr->ht_key, s);
-    dfree(tr->ht_val, s); dfree(tr->cnt, s);
+    dfree(tr->mem_in, s);
+    dfree(tr->mem, s);
     for (auto& e : tr->ev)
         if (e) cudaEventDestroy(e);
     delete tr;
@@ -456,9 +457,8 @@ sbr_status sbr_path_export(const sbr_path_list* pl, int32_t* rx, int32_t* n_boun
 void sbr_path_list_free(sbr_path_list* pl) {
     if (!pl) return;
     cudaStream_t s = pl->stream;
-    dfree(pl->rx_xyz, s); dfree(pl->rx, s); dfree(pl->nb, s); dfree(pl->surf, s); dfree(pl->face, s);
-    dfree(pl->pts, s); dfree(pl->L, s); dfree(pl->aod, s); dfree(pl->aoa, s); dfree(pl->ray, s);
-    dfree(pl->dist, s); dfree(pl->jones, s); dfree(pl->rx_off, s); dfree(pl->d_status, s);
+    dfree(pl->mem, s);
+    dfree(pl->mem_paths, s);
     delete[] pl->h_rx_off;
     delete pl;
 }

@@ -682,23 +682,35 @@ sbr_status build_lbvh(const float* prim_box, int64_t n, float pad_rel, int leaf_
     uint32_t *code, *idx;
     int32_t *left, *right, *pint, *pleaf, *flag, *span;
     float *lbox, *ibox;
-    SBR_TRY(dalloc_n(&bnd, 12, s));
     float* part;
-    SBR_TRY(dalloc_n(&part, 12 * 2 * (size_t)sm_count(), s));
     int32_t* hd;
-    SBR_TRY(dalloc_n(&hd, nn, s));
-    SBR_TRY(dalloc_n(&code, n, s));
-    SBR_TRY(dalloc_n(&idx, n, s));
-    SBR_TRY(dalloc_n(&left, nn, s));
-    SBR_TRY(dalloc_n(&right, nn, s));
-    SBR_TRY(dalloc_n(&pint, nn, s));
-    SBR_TRY(dalloc_n(&pleaf, n, s));
-    SBR_TRY(dalloc_n(&flag, nn, s));
-    SBR_TRY(dalloc_n(&span, 2 * nn, s));
-    SBR_TRY(dalloc_n(&lbox, 6 * n, s));
-    SBR_TRY(dalloc_n(&ibox, 6 * nn, s));
-    SBR_TRY(dalloc_n(&out->nodes, 4 * nn, s));
-    SBR_TRY(dalloc_n(&out->d_root, 2, s));
+    TopElem* E;
+    int32_t* slots;
+    int* cnt;
+    Arena keep, scratch;
+    keep.add(&idx, n);
+    keep.add(&out->nodes, 4 * nn);
+    keep.add(&out->d_root, 2);
+    scratch.add(&bnd, 12);
+    scratch.add(&part, 12 * 2 * (size_t)sm_count());
+    scratch.add(&hd, nn);
+    scratch.add(&code, n);
+    scratch.add(&left, nn);
+    scratch.add(&right, nn);
+    scratch.add(&pint, nn);
+    scratch.add(&pleaf, n);
+    scratch.add(&flag, nn);
+    scratch.add(&span, 2 * nn);
+    scratch.add(&lbox, 6 * n);
+    scratch.add(&ibox, 6 * nn);
+    if (top_sah) {
+        scratch.add(&E, kTopCap);
+        scratch.add(&slots, kTopCap);
+        scratch.add(&cnt, 2);
+    }
+    void* tmp;
+    SBR_TRY(keep.take(&out->mem, s));
+    SBR_TRY(scratch.take(&tmp, s));
     const int nparts = (int)std::min<int64_t>(std::max<int64_t>(1, (n + 255) / 256), 2 * (int64_t)sm_count());
     ::sbr::note_launch(), (void)::sbr::launch_pdl(k_bounds, dim3(nparts), dim3(256), 0, s, prim_box, n, part);
     ::sbr::note_launch(), (void)::sbr::launch_pdl(k_bounds_final, dim3(1), dim3(256), 0, s, part, nparts, bnd);
@@ -717,30 +729,20 @@ sbr_status build_lbvh(const float* prim_box, int64_t n, float pad_rel, int leaf_
     if (top_sah && n > lim) {
         static std::atomic<unsigned long long> attr{0};
         SBR_TRY(set_smem_once((const void*)k_top_sah, kTopSmem, &attr));
-        TopElem* E;
-        int32_t* slots;
-        int* cnt;
-        SBR_TRY(dalloc_n(&E, kTopCap, s));
-        SBR_TRY(dalloc_n(&slots, kTopCap, s));
-        SBR_TRY(dalloc_n(&cnt, 2, s));
         SBR_TRY_CUDA(cudaMemsetAsync(cnt, 0, 2 * sizeof(int), s));
         ::sbr::note_launch(), k_top_cut<<<blocks_for(nn), kThreads, 0, s>>>(nn, span, hd, out->nodes, (int)lim, E, cnt,
                                                                           slots, cnt + 1);
         ::sbr::note_launch(), k_top_sah<<<1, 32 * kTopWarps, kTopSmem, s>>>(out->nodes, E, slots, cnt, cnt + 1, d_depth);
         SBR_TRY_CUDA(cudaGetLastError());
-        dfree(E, s); dfree(slots, s); dfree(cnt, s);
     }
     out->order = reinterpret_cast<int32_t*>(idx);
     out->n_nodes = (int32_t)nn;
-    dfree(bnd, s); dfree(part, s); dfree(hd, s); dfree(code, s); dfree(left, s); dfree(right, s); dfree(pint, s);
-    dfree(pleaf, s); dfree(flag, s); dfree(span, s); dfree(lbox, s); dfree(ibox, s);
+    dfree(tmp, s);
     return SBR_OK;
 }
 
 void free_lbvh(BvhNodes* b, cudaStream_t s) {
-    if (b->nodes) dfree(b->nodes, s);
-    if (b->order) dfree(b->order, s);
-    if (b->d_root) dfree(b->d_root, s);
+    dfree(b->mem, s);
     *b = BvhNodes{};
 }
 
@@ -759,24 +761,31 @@ sbr_status bvh_build(const float* tri, const int32_t* surf, int64_t T, int32_t S
                      bool sah_top) {
     b->T = T;
     b->S = S;
-    SBR_TRY(dalloc_n(&b->d_depth, 1, s));
-    SBR_TRY(dalloc_n(&b->s_off, (size_t)S + 1, s));
+    Arena keep;
+    keep.add(&b->d_depth, 1);
+    keep.add(&b->s_off, (size_t)S + 1);
+    if (T > 0) {
+        keep.add(&b->tri, 9 * T);
+        keep.add(&b->surf, T);
+        keep.add(&b->nrm, 3 * T);
+        keep.add(&b->tri_rot, 9 * T);
+        keep.add(&b->plane_sorted, 2 * T);
+        keep.add(&b->s_tri, T);
+    }
+    SBR_TRY(keep.take(&b->mem, s));
     if (T == 0) {
         SBR_TRY_CUDA(cudaMemsetAsync(b->d_depth, 0, sizeof(int32_t), s));
         SBR_TRY_CUDA(cudaMemsetAsync(b->s_off, 0, sizeof(int32_t) * ((size_t)S + 1), s));
         return SBR_OK;
     }
-    SBR_TRY(dalloc_n(&b->tri, 9 * T, s));
-    SBR_TRY(dalloc_n(&b->surf, T, s));
-    SBR_TRY(dalloc_n(&b->nrm, 3 * T, s));
-    SBR_TRY(dalloc_n(&b->tri_rot, 9 * T, s));
     b->tri_sorted = b->tri_rot + 6 * T;
-    SBR_TRY(dalloc_n(&b->plane_sorted, 2 * T, s));
-    SBR_TRY(dalloc_n(&b->s_tri, T, s));
     float* box;
     uint32_t *key, *val;
-    SBR_TRY(dalloc_n(&box, 6 * T, s));
-    SBR_TRY(dalloc_n(&key, T, s));
+    Arena scratch;
+    void* tmp;
+    scratch.add(&box, 6 * T);
+    scratch.add(&key, T);
+    SBR_TRY(scratch.take(&tmp, s));
     val = reinterpret_cast<uint32_t*>(b->s_tri);
     HostFlag* hf;
     SBR_TRY(host_flag(&hf));
@@ -797,8 +806,7 @@ sbr_status bvh_build(const float* tri, const int32_t* surf, int64_t T, int32_t S
     SBR_TRY_CUDA(cudaGetLastError());
     SBR_TRY_CUDA(cudaEventSynchronize(hf->ev));
     const unsigned h_status = *(volatile unsigned*)hf->h;
-    dfree(box, s);
-    dfree(key, s);
+    dfree(tmp, s);
     if (h_status) {
         set_error("sbr_build_bvh: degenerate triangle or surface id out of range");
         return SBR_ERR_INVALID_ARG;

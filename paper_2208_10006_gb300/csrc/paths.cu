@@ -267,14 +267,20 @@ sbr_status paths_run(const sbr_trace_result* tr, const sbr_bvh* b, sbr_path_list
     pl->n_rx = tr->n_rx;
     pl->K = K;
     for (int k = 0; k < 3; ++k) pl->tx[k] = tr->params.tx[k];
-    SBR_TRY(dalloc_n(&pl->rx_xyz, 3 * (size_t)std::max(1, tr->n_rx), s));
+    unsigned int* count;
+    uint32_t* idx;
+    Arena per_rx, table;
+    per_rx.add(&pl->rx_xyz, 3 * (size_t)std::max(1, tr->n_rx));
+    per_rx.add(&pl->rx_off, (size_t)tr->n_rx + 1);
+    per_rx.add(&pl->d_status, 1);
+    table.add(&count, 1);
+    table.add(&idx, cap);
+    void *tmp, *tmp_n;
+    SBR_TRY(per_rx.take(&pl->mem, s));
+    SBR_TRY(table.take(&tmp, s));
     if (tr->n_rx > 0)
         SBR_TRY_CUDA(cudaMemcpyAsync(pl->rx_xyz, tr->rx, sizeof(double) * 3 * tr->n_rx,
                                      cudaMemcpyDeviceToDevice, s));
-    unsigned int* count;
-    uint32_t* idx;
-    SBR_TRY(dalloc_n(&count, 1, s));
-    SBR_TRY(dalloc_n(&idx, cap, s));
     SBR_TRY_CUDA(cudaMemsetAsync(count, 0, sizeof(unsigned), s));
     char *hm, *dm;
     SBR_TRY(mapped_buf(sizeof(MappedHead) + sizeof(int32_t) * (1 + (size_t)tr->n_rx), &hm, &dm));
@@ -294,16 +300,32 @@ sbr_status paths_run(const sbr_trace_result* tr, const sbr_bvh* b, sbr_path_list
     // a trace that ended with an error (full dedup table, stack overflow, ...)
     // yields no path list; the table was read only as plain memory
     if (const sbr_status ts = status_from_bits(h_trace); ts != SBR_OK) {
-        dfree(count, s);
-        dfree(idx, s);
+        dfree(tmp, s);
         return ts;
     }
     const int64_t n = *h_count;
     pl->n_keys = n;
     // sort keys: least significant word first (stable LSD over words)
-    uint32_t *perm, *word;
-    SBR_TRY(dalloc_n(&perm, std::max<int64_t>(n, 1), s));
-    SBR_TRY(dalloc_n(&word, std::max<int64_t>(n, 1), s));
+    uint32_t *perm, *word, *valid, *pos;
+    RefineArgs a{};
+    const int64_t nn = std::max<int64_t>(n, 1);
+    Arena raw;
+    raw.add(&perm, nn);
+    raw.add(&word, nn);
+    raw.add(&valid, nn);
+    raw.add(&pos, nn);
+    raw.add(&a.rx_o, nn);
+    raw.add(&a.nb_o, nn);
+    raw.add(&a.surf_o, nn * kKmax);
+    raw.add(&a.face_o, nn * kKmax);
+    raw.add(&a.pts_o, nn * kKmax * 3);
+    raw.add(&a.L_o, nn);
+    raw.add(&a.aod_o, nn * 2);
+    raw.add(&a.aoa_o, nn * 2);
+    raw.add(&a.ray_o, nn);
+    raw.add(&a.dist_o, nn);
+    raw.add(&a.jones_o, nn * kJones);
+    SBR_TRY(raw.take(&tmp_n, s));
     ::sbr::note_launch(), (void)::sbr::launch_pdl(k_iota, dim3(nblk(n)), dim3(kThreads), 0, s, perm, n);
     // key fields from the least significant (the last surface) to the most
     // (the receiver), packed greedily into 32-bit sort words; a stable LSD pass
@@ -328,7 +350,6 @@ sbr_status paths_run(const sbr_trace_result* tr, const sbr_bvh* b, sbr_path_list
         SBR_TRY(radix_sort_pairs(word, perm, n, bits, s));
     }
     // refine into raw (key-order) buffers
-    RefineArgs a{};
     a.key = tr->ht_key;
     a.val = tr->ht_val;
     a.idx = idx;
@@ -346,22 +367,6 @@ sbr_status paths_run(const sbr_trace_result* tr, const sbr_bvh* b, sbr_path_list
     a.seqf = tr->seqf;
     a.R = tr->Rr;
     a.ray0 = tr->ray0;
-    int64_t nn = std::max<int64_t>(n, 1);
-    uint32_t* valid;
-    uint32_t* pos;
-    SBR_TRY(dalloc_n(&valid, nn, s));
-    SBR_TRY(dalloc_n(&pos, nn, s));
-    SBR_TRY(dalloc_n(&a.rx_o, nn, s));
-    SBR_TRY(dalloc_n(&a.nb_o, nn, s));
-    SBR_TRY(dalloc_n(&a.surf_o, nn * kKmax, s));
-    SBR_TRY(dalloc_n(&a.face_o, nn * kKmax, s));
-    SBR_TRY(dalloc_n(&a.pts_o, nn * kKmax * 3, s));
-    SBR_TRY(dalloc_n(&a.L_o, nn, s));
-    SBR_TRY(dalloc_n(&a.aod_o, nn * 2, s));
-    SBR_TRY(dalloc_n(&a.aoa_o, nn * 2, s));
-    SBR_TRY(dalloc_n(&a.ray_o, nn, s));
-    SBR_TRY(dalloc_n(&a.dist_o, nn, s));
-    SBR_TRY(dalloc_n(&a.jones_o, nn * kJones, s));
     a.valid = valid;
     if (n > 0) {
         if (a.seqf)
@@ -375,20 +380,19 @@ sbr_status paths_run(const sbr_trace_result* tr, const sbr_bvh* b, sbr_path_list
     SBR_TRY(exclusive_scan_u32(pos, n, count, s));
     // the list is sized for every key (P <= n), so compaction and the receiver
     // offsets run before the host learns P: one wait for P and the offsets
-    const int64_t Pp = nn;
-    SBR_TRY(dalloc_n(&pl->rx, Pp, s));
-    SBR_TRY(dalloc_n(&pl->nb, Pp, s));
-    SBR_TRY(dalloc_n(&pl->surf, Pp * kKmax, s));
-    SBR_TRY(dalloc_n(&pl->face, Pp * kKmax, s));
-    SBR_TRY(dalloc_n(&pl->pts, Pp * kKmax * 3, s));
-    SBR_TRY(dalloc_n(&pl->L, Pp, s));
-    SBR_TRY(dalloc_n(&pl->aod, Pp * 2, s));
-    SBR_TRY(dalloc_n(&pl->aoa, Pp * 2, s));
-    SBR_TRY(dalloc_n(&pl->ray, Pp, s));
-    SBR_TRY(dalloc_n(&pl->dist, Pp, s));
-    SBR_TRY(dalloc_n(&pl->jones, Pp * kJones, s));
-    SBR_TRY(dalloc_n(&pl->rx_off, (size_t)tr->n_rx + 1, s));
-    SBR_TRY(dalloc_n(&pl->d_status, 1, s));
+    Arena list;
+    list.add(&pl->rx, nn);
+    list.add(&pl->nb, nn);
+    list.add(&pl->surf, nn * kKmax);
+    list.add(&pl->face, nn * kKmax);
+    list.add(&pl->pts, nn * kKmax * 3);
+    list.add(&pl->L, nn);
+    list.add(&pl->aod, nn * 2);
+    list.add(&pl->aoa, nn * 2);
+    list.add(&pl->ray, nn);
+    list.add(&pl->dist, nn);
+    list.add(&pl->jones, nn * kJones);
+    SBR_TRY(list.take(&pl->mem_paths, s));
     SBR_TRY_CUDA(cudaMemsetAsync(pl->d_status, 0, sizeof(unsigned), s));
     if (n > 0) {
         CompactArgs c{};
@@ -414,10 +418,8 @@ sbr_status paths_run(const sbr_trace_result* tr, const sbr_bvh* b, sbr_path_list
     const int64_t P = *h_count;
     pl->P = P;
     pl->n_invalid = n - P;
-    dfree(count, s); dfree(idx, s); dfree(perm, s); dfree(word, s); dfree(valid, s); dfree(pos, s);
-    dfree(a.rx_o, s); dfree(a.nb_o, s); dfree(a.surf_o, s); dfree(a.face_o, s); dfree(a.pts_o, s);
-    dfree(a.L_o, s); dfree(a.aod_o, s); dfree(a.aoa_o, s); dfree(a.ray_o, s); dfree(a.dist_o, s);
-    dfree(a.jones_o, s);
+    dfree(tmp, s);
+    dfree(tmp_n, s);
     return SBR_OK;
 }
 

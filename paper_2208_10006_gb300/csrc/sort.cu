@@ -415,22 +415,26 @@ sbr_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, int64_t n, int bits,
     if (coop_tiles > 0 && rounds <= kCoopMaxRounds) {
         int grid = (int)coop_tiles, r = (int)rounds;
         uint32_t *k2, *v2, *hist;
-        SBR_TRY(dalloc_n(&k2, n, s));
-        SBR_TRY(dalloc_n(&v2, n, s));
-        SBR_TRY(dalloc_n(&hist, (size_t)256 * grid, s));
+        Arena buf;
+        void* tmp;
+        buf.add(&k2, n);
+        buf.add(&v2, n);
+        buf.add(&hist, (size_t)256 * grid);
+        SBR_TRY(buf.take(&tmp, s));
         void* args[] = {&keys, &vals, &k2, &v2, &n, &passes, &r, &hist};
         ::sbr::note_launch();
         SBR_TRY_CUDA(cudaLaunchCooperativeKernel((const void*)k_sort_coop, dim3(grid), dim3(kSortThreads), args, 0, s));
-        dfree(k2, s);
-        dfree(v2, s);
-        dfree(hist, s);
+        dfree(tmp, s);
         return SBR_OK;
     }
     int nblocks = (int)((n + kSortTile - 1) / kSortTile);
     uint32_t *k2, *v2, *hist;
-    SBR_TRY(dalloc_n(&k2, n, s));
-    SBR_TRY(dalloc_n(&v2, n, s));
-    SBR_TRY(dalloc_n(&hist, (size_t)256 * nblocks, s));
+    Arena buf;
+    void* tmp;
+    buf.add(&k2, n);
+    buf.add(&v2, n);
+    buf.add(&hist, (size_t)256 * nblocks);
+    SBR_TRY(buf.take(&tmp, s));
     uint32_t *ka = keys, *va = vals, *kb = k2, *vb = v2;
     sbr_status st = SBR_OK;
     for (int p = 0; p < passes && st == SBR_OK; ++p) {
@@ -449,9 +453,7 @@ sbr_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, int64_t n, int bits,
         cudaMemcpyAsync(keys, ka, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
         cudaMemcpyAsync(vals, va, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
     }
-    dfree(k2, s);
-    dfree(v2, s);
-    dfree(hist, s);
+    dfree(tmp, s);
     return st;
 }
 

@@ -1212,21 +1212,35 @@ sbr_status trace_run(const sbr_bvh* b, sbr_trace_result* tr, cudaStream_t s) {
     const int K = p.max_bounces;
     const int64_t R = tr->Rr;   // rays traced: the id range [ray0, ray0 + Rr)
     size_t cap = (size_t)1 << tr->table_log2;
-    SBR_TRY(dalloc_n(&tr->ht_state, cap, s));
-    SBR_TRY(dalloc_n(&tr->ht_key, cap * kKeyWords, s));
-    SBR_TRY(dalloc_n(&tr->ht_val, cap, s));
-    SBR_TRY(dalloc_n(&tr->cnt, 1, s));
     BvhNodes rxb;
     float* rxbox = nullptr;
     int32_t* rx_depth = nullptr;
     float4* rx_df = nullptr;
     float4* alpha_df = nullptr;
-    SBR_TRY(dalloc_n(&alpha_df, 1, s));
+    RayRec *q0 = nullptr, *q1 = nullptr;
+    int32_t* seq = nullptr;
+    Arena keep, scratch;
+    keep.add(&tr->ht_state, cap);
+    keep.add(&tr->ht_key, cap * kKeyWords);
+    keep.add(&tr->ht_val, cap);
+    keep.add(&tr->cnt, 1);
+    scratch.add(&alpha_df, 1);
     if (tr->n_rx > 0) {
-        SBR_TRY(dalloc_n(&rxbox, 6 * (size_t)tr->n_rx, s));
-        SBR_TRY(dalloc_n(&rx_depth, 1, s));
-        SBR_TRY(dalloc_n(&rx_df, 2 * (size_t)tr->n_rx, s));
+        scratch.add(&rxbox, 6 * (size_t)tr->n_rx);
+        scratch.add(&rx_depth, 1);
+        scratch.add(&rx_df, 2 * (size_t)tr->n_rx);
     }
+    if (K > 0) {
+        if (tr->df_from > 0) {   // ray queues of the breadth-first bounces
+            scratch.add(&q0, (size_t)R);
+            scratch.add(&q1, (size_t)R);
+        }
+        scratch.add(&seq, (size_t)R * K);
+        keep.add(&tr->seqf, (size_t)R * K);
+    }
+    void* tmp;
+    SBR_TRY(keep.take(&tr->mem, s));
+    SBR_TRY(scratch.take(&tmp, s));
     {
         const size_t n_set = std::max<size_t>(std::max<size_t>(cap, (size_t)tr->n_rx), sizeof(TraceCountersDev) / 8);
         ::sbr::note_launch(), (void)::sbr::launch_pdl(k_trace_setup, dim3((unsigned)((n_set + 255) / 256)), dim3(256), 0, s,
@@ -1236,16 +1250,6 @@ sbr_status trace_run(const sbr_bvh* b, sbr_trace_result* tr, cudaStream_t s) {
     }
     // receiver BVH
     if (tr->n_rx > 0) SBR_TRY(build_lbvh(rxbox, tr->n_rx, 0.0f, 1, &rxb, rx_depth, s));
-    RayRec *q0 = nullptr, *q1 = nullptr;
-    int32_t* seq = nullptr;
-    if (K > 0) {
-        if (tr->df_from > 0) {   // ray queues of the breadth-first bounces
-            SBR_TRY(dalloc_n(&q0, (size_t)R, s));
-            SBR_TRY(dalloc_n(&q1, (size_t)R, s));
-        }
-        SBR_TRY(dalloc_n(&seq, (size_t)R * K, s));
-        SBR_TRY(dalloc_n(&tr->seqf, (size_t)R * K, s));
-    }
     TraceArgs a{};
     a.nodes = b->tree.nodes;
     a.tris = b->tri_sorted;
@@ -1315,16 +1319,8 @@ sbr_status trace_run(const sbr_bvh* b, sbr_trace_result* tr, cudaStream_t s) {
         SBR_TRY_CUDA(cudaGetLastError());
         if (timing) SBR_TRY_CUDA(cudaEventRecord(tr->ev[bnc + 1], s));
     }
-    if (q0) dfree(q0, s);
-    if (q1) dfree(q1, s);
-    if (seq) dfree(seq, s);
-    if (tr->n_rx > 0) {
-        free_lbvh(&rxb, s);
-        dfree(rxbox, s);
-        dfree(rx_depth, s);
-        dfree(rx_df, s);
-    }
-    dfree(alpha_df, s);
+    free_lbvh(&rxb, s);
+    dfree(tmp, s);
     return SBR_OK;
 }
 
@@ -1359,10 +1355,12 @@ sbr_status trace_entries_run(const sbr_trace_result* tr, uint32_t* keys, unsigne
 sbr_status trace_merge_run(sbr_trace_result* tr, const uint32_t* keys, const unsigned long long* vals, int64_t n,
                            cudaStream_t s) {
     const size_t cap = (size_t)1 << tr->table_log2;
-    SBR_TRY(dalloc_n(&tr->ht_state, cap, s));
-    SBR_TRY(dalloc_n(&tr->ht_key, cap * kKeyWords, s));
-    SBR_TRY(dalloc_n(&tr->ht_val, cap, s));
-    SBR_TRY(dalloc_n(&tr->cnt, 1, s));
+    Arena keep;
+    keep.add(&tr->ht_state, cap);
+    keep.add(&tr->ht_key, cap * kKeyWords);
+    keep.add(&tr->ht_val, cap);
+    keep.add(&tr->cnt, 1);
+    SBR_TRY(keep.take(&tr->mem, s));
     SBR_TRY_CUDA(cudaMemsetAsync(tr->cnt, 0, sizeof(TraceCountersDev), s));
     ::sbr::note_launch(), (void)::sbr::launch_pdl(k_init_table, dim3((unsigned)((cap + 255) / 256)), dim3(256), 0, s, tr->ht_state, tr->ht_val, cap);
     SBR_TRY_CUDA(cudaGetLastError());
