@@ -95,6 +95,49 @@ int sm_count() {
 }
 
 namespace {
+// whether [p, p + bytes) is device memory of device dev inside one allocation
+// (what a copy to it would check; anything else is left to the copy)
+bool device_range(const void* p, size_t bytes, int dev) {
+    using Range = int (*)(unsigned long long*, size_t*, unsigned long long);   // cuMemGetAddressRange
+    static const Range range = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            fn = nullptr;
+        return reinterpret_cast<Range>(fn);
+    }();
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    if (!range || at.type != cudaMemoryTypeDevice || at.device != dev || ((uintptr_t)p & 3)) return false;
+    unsigned long long base = 0;
+    size_t size = 0;
+    if (range(&base, &size, (unsigned long long)(uintptr_t)p) != 0) return false;
+    return (uintptr_t)p >= base && (uintptr_t)p + bytes <= base + size;
+}
+// the fields of a path list into the caller's arrays: 16-byte words where both
+// sides allow them, 4-byte words otherwise and at the end
+struct ExportArgs {
+    int n;
+    uint32_t* dst[10];
+    const uint32_t* src[10];
+    int64_t words[10];
+};
+__global__ void k_export(const __grid_constant__ ExportArgs a) {
+    ::sbr::pdl_wait();
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    for (int f = 0; f < a.n; ++f) {
+        uint32_t* d = a.dst[f];
+        const uint32_t* s = a.src[f];
+        const int64_t n = a.words[f];
+        const int64_t n4 = (((uintptr_t)d | (uintptr_t)s) & 15) == 0 ? n / 4 : 0;
+        for (int64_t i = t; i < n4; i += step) reinterpret_cast<uint4*>(d)[i] = __ldg(reinterpret_cast<const uint4*>(s) + i);
+        for (int64_t i = 4 * n4 + t; i < n; i += step) d[i] = __ldg(s + i);
+    }
+}
 __global__ void k_set_u64(unsigned long long* dst, unsigned long long v) { *dst = v; }
 }  // namespace
 
@@ -247,9 +290,7 @@ sbr_status sbr_trace(const sbr_bvh* b, const sbr_trace_params* p, sbr_trace_resu
             st = SBR_ERR_CUDA;
         }
     }
-    // a given alpha is stored by the trace's set-up launch; the default one
-    // (alpha = 0) is computed from the launch grid first
-    if (st == SBR_OK && !(p->alpha > 0.0)) st = launch_alpha_fast(p->subdiv_N, tr->d_alpha, s);
+    // alpha, given or that of the launch grid, is stored by the trace's set-up launch
     if (st == SBR_OK) st = trace_run(b, tr, s);
     if (st != SBR_OK) {
         sbr_trace_free(tr);
@@ -435,22 +476,42 @@ sbr_status sbr_path_export(const sbr_path_list* pl, int32_t* rx, int32_t* n_boun
     cudaStream_t s = (cudaStream_t)stream;
     const size_t P = (size_t)pl->P;
     if (P == 0) return SBR_OK;
-    auto cp = [&](void* dst, const void* src, size_t bytes) -> sbr_status {
-        if (!dst) return SBR_OK;
-        // device or (pinned) host destination, resolved by unified addressing
-        SBR_TRY_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, s));
-        return SBR_OK;
-    };
-    SBR_TRY(cp(rx, pl->rx, P * sizeof(int32_t)));
-    SBR_TRY(cp(n_bounce, pl->nb, P * sizeof(int32_t)));
-    SBR_TRY(cp(surf_seq, pl->surf, P * kKmax * sizeof(int32_t)));
-    SBR_TRY(cp(face_seq, pl->face, P * kKmax * sizeof(int32_t)));
-    SBR_TRY(cp(pts, pl->pts, P * kKmax * 3 * sizeof(double)));
-    SBR_TRY(cp(length, pl->L, P * sizeof(double)));
-    SBR_TRY(cp(aod, pl->aod, P * 2 * sizeof(double)));
-    SBR_TRY(cp(aoa, pl->aoa, P * 2 * sizeof(double)));
-    SBR_TRY(cp(ray_id, pl->ray, P * sizeof(uint32_t)));
-    SBR_TRY(cp(dist, pl->dist, P * sizeof(float)));
+    struct Field {
+        void* dst;
+        const void* src;
+        size_t bytes;
+    } f[] = {{rx, pl->rx, P * sizeof(int32_t)},
+             {n_bounce, pl->nb, P * sizeof(int32_t)},
+             {surf_seq, pl->surf, P * kKmax * sizeof(int32_t)},
+             {face_seq, pl->face, P * kKmax * sizeof(int32_t)},
+             {pts, pl->pts, P * kKmax * 3 * sizeof(double)},
+             {length, pl->L, P * sizeof(double)},
+             {aod, pl->aod, P * 2 * sizeof(double)},
+             {aoa, pl->aoa, P * 2 * sizeof(double)},
+             {ray_id, pl->ray, P * sizeof(uint32_t)},
+             {dist, pl->dist, P * sizeof(float)}};
+    // Destinations in this device's memory are filled by one launch instead of a copy
+    // each (3 us of host time and a gap on the device); any other (pinned host, another
+    // device), resolved by unified addressing, by a copy.
+    ExportArgs a{};
+    int dev = -1;
+    SBR_TRY_CUDA(cudaGetDevice(&dev));
+    for (const Field& x : f) {
+        if (!x.dst) continue;
+        if (device_range(x.dst, x.bytes, dev)) {
+            a.dst[a.n] = static_cast<uint32_t*>(x.dst);
+            a.src[a.n] = static_cast<const uint32_t*>(x.src);
+            a.words[a.n++] = (int64_t)(x.bytes / 4);
+        } else {
+            SBR_TRY_CUDA(cudaMemcpyAsync(x.dst, x.src, x.bytes, cudaMemcpyDefault, s));
+        }
+    }
+    if (a.n) {
+        const int64_t quads = (int64_t)P * kKmax * 3 * 2 / 4;   // of the largest field
+        const unsigned grid = (unsigned)std::min<int64_t>((quads + 255) / 256, 8 * (int64_t)sm_count());
+        ::sbr::note_launch(), (void)::sbr::launch_pdl(k_export, dim3(grid), dim3(256), 0, s, a);
+        SBR_TRY_CUDA(cudaGetLastError());
+    }
     return SBR_OK;
 }
 

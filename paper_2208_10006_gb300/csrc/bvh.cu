@@ -88,6 +88,18 @@ __device__ __forceinline__ uint32_t expand_bits(uint32_t x) {
     return x;
 }
 
+__device__ __forceinline__ uint32_t morton_code(const float* box, int64_t i, const float* bnd) {
+    uint32_t q[3];
+    for (int a = 0; a < 3; ++a) {
+        float c = 0.5f * (box[6 * i + a] + box[6 * i + 3 + a]);
+        float ext = bnd[3 + a] - bnd[a];
+        float u = ext > 0.f ? (c - bnd[a]) / ext : 0.f;
+        u = fminf(fmaxf(u * 1024.f, 0.f), 1023.f);
+        q[a] = (uint32_t)u;
+    }
+    return (expand_bits(q[0]) << 2) | (expand_bits(q[1]) << 1) | expand_bits(q[2]);
+}
+
 // Also clears the refit's arrival flags (nn of them, nn <= n) and the depth.
 __global__ void k_morton(const float* __restrict__ box, int64_t n, const float* __restrict__ bnd,
                          uint32_t* __restrict__ code, uint32_t* __restrict__ idx, int32_t* __restrict__ flag,
@@ -97,20 +109,12 @@ __global__ void k_morton(const float* __restrict__ box, int64_t n, const float* 
     if (i >= n) return;
     if (i < nn) flag[i] = 0;
     if (i == 0) *depth = 0;
-    uint32_t q[3];
-    for (int a = 0; a < 3; ++a) {
-        float c = 0.5f * (box[6 * i + a] + box[6 * i + 3 + a]);
-        float ext = bnd[3 + a] - bnd[a];
-        float u = ext > 0.f ? (c - bnd[a]) / ext : 0.f;
-        u = fminf(fmaxf(u * 1024.f, 0.f), 1023.f);
-        q[a] = (uint32_t)u;
-    }
-    code[i] = (expand_bits(q[0]) << 2) | (expand_bits(q[1]) << 1) | expand_bits(q[2]);
+    code[i] = morton_code(box, i, bnd);
     idx[i] = (uint32_t)i;
 }
 
 // longest common prefix of the (code, index) keys of sorted positions i and j
-__device__ __forceinline__ int delta(const uint32_t* __restrict__ code, int64_t n, int64_t i,
+__device__ __forceinline__ int delta(const uint32_t* code, int64_t n, int64_t i,
                                      int64_t j) {
     if (j < 0 || j >= n) return -1;
     uint64_t a = ((uint64_t)code[i] << 32) | (uint64_t)(uint32_t)i;
@@ -118,12 +122,8 @@ __device__ __forceinline__ int delta(const uint32_t* __restrict__ code, int64_t 
     return __clzll((long long)(a ^ b));
 }
 
-__global__ void k_karras(const uint32_t* __restrict__ code, int64_t n, int32_t* __restrict__ left,
-                         int32_t* __restrict__ right, int32_t* __restrict__ parent_int,
-                         int32_t* __restrict__ parent_leaf, int32_t* __restrict__ span) {
-    ::sbr::pdl_wait();
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n - 1) return;
+__device__ __forceinline__ void karras_node(const uint32_t* code, int64_t n, int64_t i, int32_t* left, int32_t* right,
+                                            int32_t* parent_int, int32_t* parent_leaf, int32_t* span) {
     int d = (delta(code, n, i, i + 1) - delta(code, n, i, i - 1)) >= 0 ? 1 : -1;
     int dmin = delta(code, n, i, i - d);
     int64_t lmax = 2;
@@ -159,20 +159,23 @@ __global__ void k_karras(const uint32_t* __restrict__ code, int64_t n, int32_t* 
     if (i == 0) parent_int[0] = -1;
 }
 
+__global__ void k_karras(const uint32_t* __restrict__ code, int64_t n, int32_t* __restrict__ left,
+                         int32_t* __restrict__ right, int32_t* __restrict__ parent_int,
+                         int32_t* __restrict__ parent_leaf, int32_t* __restrict__ span) {
+    ::sbr::pdl_wait();
+    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n - 1) karras_node(code, n, i, left, right, parent_int, parent_leaf, span);
+}
+
 __device__ __forceinline__ void ld_box(const float* p, float b[6]) {
     const volatile float* q = p;
     for (int k = 0; k < 6; ++k) b[k] = q[k];
 }
 
-__global__ void k_refit(const float* __restrict__ prim_box, const int32_t* __restrict__ order,
-                        int64_t n, const int32_t* __restrict__ left,
-                        const int32_t* __restrict__ right, const int32_t* __restrict__ parent_int,
-                        const int32_t* __restrict__ parent_leaf, int32_t* __restrict__ flag,
-                        float* lbox, float* ibox, int32_t* hd, int32_t* __restrict__ depth) {
-    ::sbr::pdl_wait();
-    int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    const float* src = prim_box + 6 * (int64_t)order[j];
+__device__ __forceinline__ void refit_climb(const float* src, int64_t n, int64_t j, const int32_t* left,
+                                            const int32_t* right, const int32_t* parent_int,
+                                            const int32_t* parent_leaf, int32_t* flag, float* lbox, float* ibox,
+                                            int32_t* hd, int32_t* depth) {
     for (int k = 0; k < 6; ++k) lbox[6 * j + k] = src[k];
     if (n < 2) {
         *depth = 1;
@@ -212,6 +215,17 @@ __global__ void k_refit(const float* __restrict__ prim_box, const int32_t* __res
     }
 }
 
+__global__ void k_refit(const float* __restrict__ prim_box, const int32_t* __restrict__ order,
+                        int64_t n, const int32_t* __restrict__ left,
+                        const int32_t* __restrict__ right, const int32_t* __restrict__ parent_int,
+                        const int32_t* __restrict__ parent_leaf, int32_t* __restrict__ flag,
+                        float* lbox, float* ibox, int32_t* hd, int32_t* __restrict__ depth) {
+    ::sbr::pdl_wait();
+    int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < n)
+        refit_climb(prim_box + 6 * (int64_t)order[j], n, j, left, right, parent_int, parent_leaf, flag, lbox, ibox, hd, depth);
+}
+
 __device__ __forceinline__ float pad_lo(float x, float pad) { return x - pad * (fabsf(x) + 1.f); }
 __device__ __forceinline__ float pad_hi(float x, float pad) { return x + pad * (fabsf(x) + 1.f); }
 
@@ -219,21 +233,16 @@ __device__ __forceinline__ float pad_hi(float x, float pad) { return x + pad * (
 // holding `count` consecutive sorted primitives; subtrees of at most leaf_max
 // primitives are emitted as one leaf (their primitives are consecutive in
 // Morton order), so traversal stops above them
-__device__ __forceinline__ int32_t child_ref(int32_t c, const int32_t* __restrict__ span, int leaf_max) {
+__device__ __forceinline__ int32_t child_ref(int32_t c, const int32_t* span, int leaf_max) {
     if (c < 0) return c;  // single primitive ~p (count 1)
     int32_t lo = span[2 * c], hi = span[2 * c + 1];
     if (hi - lo + 1 <= leaf_max) return ~(lo | ((hi - lo) << 28));
     return c;
 }
 
-__global__ void k_emit(int64_t n, const int32_t* __restrict__ left, const int32_t* __restrict__ right,
-                       const int32_t* __restrict__ span, int leaf_max,
-                       const float* __restrict__ lbox, const float* __restrict__ ibox, float pad,
-                       float4* __restrict__ nodes, float4* __restrict__ root) {
-    ::sbr::pdl_wait();
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int64_t nn = n > 1 ? n - 1 : 1;
-    if (i >= nn) return;
+__device__ __forceinline__ void emit_node(int64_t i, int64_t n, const int32_t* left, const int32_t* right,
+                                          const int32_t* span, int leaf_max, const float* lbox, const float* ibox,
+                                          float pad, float4* nodes, float4* root) {
     float b0[6], b1[6];
     int32_t r0, r1;
     if (n == 1) {
@@ -267,6 +276,77 @@ __global__ void k_emit(int64_t n, const int32_t* __restrict__ left, const int32_
         root[0] = make_float4(c[0], c[1], c[2], sqrtf(h[0] * h[0] + h[1] * h[1] + h[2] * h[2]));
         root[1] = make_float4(h[0], h[1], h[2], 0.f);
     }
+}
+
+__global__ void k_emit(int64_t n, const int32_t* __restrict__ left, const int32_t* __restrict__ right,
+                       const int32_t* __restrict__ span, int leaf_max,
+                       const float* __restrict__ lbox, const float* __restrict__ ibox, float pad,
+                       float4* __restrict__ nodes, float4* __restrict__ root) {
+    ::sbr::pdl_wait();
+    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < (n > 1 ? n - 1 : 1)) emit_node(i, n, left, right, span, leaf_max, lbox, ibox, pad, nodes, root);
+}
+
+// The whole tree of a small set in one block and one launch: the phases above over
+// shared memory, one primitive and one node per thread, the Morton order by a
+// bitonic sort of (code, index) - the order of the stable radix sort. A launch of
+// the general build costs more than all its work: trace of 1,024 receivers and few
+// rays 159.5 us with it, 142.0 so; of 64 receivers 87.7 and 69.4.
+// Same nodes, order and depth.
+constexpr int kSmallTree = 1024;
+__host__ __device__ constexpr size_t small_tree_words(int m) { return 22 * (size_t)m + 12; }   // m: primitives padded to a power of two
+
+__global__ void __launch_bounds__(kSmallTree)
+k_tree_small(const float* __restrict__ box, int n, int m, int leaf_max, float pad, uint32_t* __restrict__ order,
+             float4* __restrict__ nodes, float4* __restrict__ root, int32_t* __restrict__ depth) {
+    ::sbr::pdl_wait();
+    extern __shared__ unsigned long long sm64[];
+    __shared__ float red[12][32];
+    unsigned long long* key = sm64;                         // [m]
+    uint32_t* code = reinterpret_cast<uint32_t*>(sm64 + m); // [m] in order
+    float* lbox = reinterpret_cast<float*>(code + m);       // [6 m]
+    float* ibox = lbox + 6 * m;                             // [6 m]
+    int32_t* left = reinterpret_cast<int32_t*>(ibox + 6 * m);
+    int32_t *right = left + m, *pint = left + 2 * m, *pleaf = left + 3 * m, *flag = left + 4 * m;
+    int32_t* span = reinterpret_cast<int32_t*>(key);        // [2 m], once the keys are spent
+    float* bnd = reinterpret_cast<float*>(left + 6 * m);    // [12]
+    int32_t* hd = left + 5 * m;
+    const int i = threadIdx.x;
+    float v[12];
+    for (int a = 0; a < 3; ++a) {
+        const float lo = i < n ? box[6 * i + a] : INFINITY, hi = i < n ? box[6 * i + 3 + a] : -INFINITY;
+        v[a] = i < n ? 0.5f * (lo + hi) : INFINITY; v[3 + a] = i < n ? 0.5f * (lo + hi) : -INFINITY;
+        v[6 + a] = lo; v[9 + a] = hi;
+    }
+    bounds_block_reduce(v, red, bnd);
+    __syncthreads();
+    if (i < m) {
+        key[i] = i < n ? ((unsigned long long)morton_code(box, i, bnd) << 32) | (unsigned)i : ~0ull;
+        flag[i] = 0;
+    }
+    if (i == 0) *depth = 0;
+    __syncthreads();
+    for (int k = 2; k <= m; k <<= 1)
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            const int o = i ^ j;
+            if (i < m && o > i) {
+                const unsigned long long x = key[i], y = key[o];
+                if ((x > y) == ((i & k) == 0)) { key[i] = y; key[o] = x; }
+            }
+            __syncthreads();
+        }
+    uint32_t id = 0;
+    if (i < n) {
+        code[i] = (uint32_t)(key[i] >> 32);
+        id = (uint32_t)key[i];
+        order[i] = id;
+    }
+    __syncthreads();
+    if (i < n - 1) karras_node(code, n, i, left, right, pint, pleaf, span);
+    __syncthreads();
+    if (i < n) refit_climb(box + 6 * (int64_t)id, n, i, left, right, pint, pleaf, flag, lbox, ibox, hd, depth);
+    __syncthreads();
+    if (i < (n > 1 ? n - 1 : 1)) emit_node(i, n, left, right, span, leaf_max, lbox, ibox, pad, nodes, root);
 }
 
 // ---------------------------------------------------------------- SAH top levels
@@ -710,6 +790,21 @@ sbr_status build_lbvh(const float* prim_box, int64_t n, float pad_rel, int leaf_
     }
     void* tmp;
     SBR_TRY(keep.take(&out->mem, s));
+    out->order = reinterpret_cast<int32_t*>(idx);
+    out->n_nodes = (int32_t)nn;
+    // SBR_BVH_PHASES=1 keeps to the launches per phase (a test hook)
+    const char* phases = getenv("SBR_BVH_PHASES");
+    if (n <= kSmallTree && !top_sah && !(phases && phases[0] == '1')) {
+        int m = 32;
+        while (m < n) m <<= 1;
+        const size_t smem = 4 * small_tree_words(m);
+        static std::atomic<unsigned long long> attr{0};
+        SBR_TRY(set_smem_once((const void*)k_tree_small, (int)(4 * small_tree_words(kSmallTree)), &attr));
+        ::sbr::note_launch(), (void)::sbr::launch_pdl(k_tree_small, dim3(1), dim3(m), smem, s, prim_box, (int)n, m, leaf_max, pad_rel, idx,
+                                                      out->nodes, out->d_root, d_depth);
+        SBR_TRY_CUDA(cudaGetLastError());
+        return SBR_OK;
+    }
     SBR_TRY(scratch.take(&tmp, s));
     const int nparts = (int)std::min<int64_t>(std::max<int64_t>(1, (n + 255) / 256), 2 * (int64_t)sm_count());
     ::sbr::note_launch(), (void)::sbr::launch_pdl(k_bounds, dim3(nparts), dim3(256), 0, s, prim_box, n, part);
@@ -735,8 +830,6 @@ sbr_status build_lbvh(const float* prim_box, int64_t n, float pad_rel, int leaf_
         ::sbr::note_launch(), k_top_sah<<<1, 32 * kTopWarps, kTopSmem, s>>>(out->nodes, E, slots, cnt, cnt + 1, d_depth);
         SBR_TRY_CUDA(cudaGetLastError());
     }
-    out->order = reinterpret_cast<int32_t*>(idx);
-    out->n_nodes = (int32_t)nn;
     dfree(tmp, s);
     return SBR_OK;
 }

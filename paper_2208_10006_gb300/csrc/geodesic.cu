@@ -177,23 +177,25 @@ __global__ void k_alpha_df(const __grid_constant__ IcoLattice t, int N, int64_t 
     if ((threadIdx.x & 31) == 0) atomicMax(best, (unsigned long long)__double_as_longlong(df_to_double(m)));
 }
 
-__global__ void k_alpha_df_store(const unsigned long long* best, double* alpha) {
+__global__ void k_alpha_df_store(double* alpha) {
     ::sbr::pdl_wait();
-    const double c2 = __longlong_as_double((long long)*best);
-    *alpha = 2.0 * asin(0.5 * sqrt(c2));
+    *alpha = chord_angle(*alpha);
 }
 }  // namespace
 
-sbr_status launch_alpha_fast(int32_t N, double* alpha, cudaStream_t s) {
+sbr_status launch_chord_fast(int32_t N, double* chord2, cudaStream_t s) {
     const int64_t per_face = (int64_t)N * (N + 1) / 2;
-    unsigned long long* best;
-    SBR_TRY(dalloc_n(&best, 1, s));
-    SBR_TRY_CUDA(cudaMemsetAsync(best, 0, sizeof(unsigned long long), s));
+    SBR_TRY_CUDA(cudaMemsetAsync(chord2, 0, sizeof(double), s));
     ::sbr::note_launch(), (void)::sbr::launch_pdl(k_alpha_df, dim3((unsigned)((per_face + 255) / 256)), dim3(256), 0, s, make_ico_lattice(), N,
-                                                                                          per_face, best);
-    ::sbr::note_launch(), (void)::sbr::launch_pdl(k_alpha_df_store, dim3(1), dim3(1), 0, s, best, alpha);
+                                                  per_face, reinterpret_cast<unsigned long long*>(chord2));
     SBR_TRY_CUDA(cudaGetLastError());
-    dfree(best, s);
+    return SBR_OK;
+}
+
+sbr_status launch_alpha_fast(int32_t N, double* alpha, cudaStream_t s) {
+    SBR_TRY(launch_chord_fast(N, alpha, s));
+    ::sbr::note_launch(), (void)::sbr::launch_pdl(k_alpha_df_store, dim3(1), dim3(1), 0, s, alpha);
+    SBR_TRY_CUDA(cudaGetLastError());
     return SBR_OK;
 }
 

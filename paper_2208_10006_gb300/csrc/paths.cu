@@ -11,6 +11,7 @@
 // artefacts near edges) are dropped and counted; the rest keep key order.
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <vector>
 
@@ -23,41 +24,72 @@ namespace {
 constexpr int kThreads = 256;
 inline unsigned nblk(int64_t n) { return (unsigned)std::max<int64_t>(1, (n + kThreads - 1) / kThreads); }
 
+// Layout of the host-mapped words of one path-list build: the key count (later
+// P), the trace's alpha and final counters, then the receiver offsets.
+struct MappedHead {
+    unsigned count;
+    unsigned pad;
+    double alpha;
+    TraceCountersDev cnt;
+};
+static_assert(sizeof(MappedHead) % 8 == 0 && sizeof(TraceCountersDev) % 8 == 0, "64-bit words");
+
+// the list's own copy of the receivers, and its counters cleared (count: keys
+// collected and blocks done)
+__global__ void k_paths_init(const double* __restrict__ rx, int n3, double* __restrict__ rx_xyz, unsigned* count,
+                             unsigned* status) {
+    ::sbr::pdl_wait();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n3) rx_xyz[i] = rx[i];
+    if (i < 2) count[i] = 0u;
+    if (i == 0) *status = 0u;
+}
+
+// the used slots of the table in idx[0..count[0]), any order; the block that ends
+// last (count[1]) stores the count, alpha and the trace's counters to the
+// host-mapped head
 __global__ void k_collect(const uint32_t* __restrict__ state, size_t cap, uint32_t* __restrict__ idx,
-                          unsigned int* __restrict__ count) {
+                          unsigned int* __restrict__ count, const double* __restrict__ alpha,
+                          const TraceCountersDev* __restrict__ cnt, MappedHead* h) {
     ::sbr::pdl_wait();
     size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     bool ready = s < cap && state[s] == 2u;
     unsigned m = __ballot_sync(0xffffffffu, ready);
-    if (!m) return;
-    unsigned base = 0;
-    int lane = threadIdx.x & 31;
-    if (lane == 0) base = atomicAdd(count, (unsigned)__popc(m));
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (ready) idx[base + __popc(m & ((1u << lane) - 1u))] = (uint32_t)s;
+    const int lane = threadIdx.x & 31;
+    if (m) {
+        unsigned base = 0;
+        if (lane == 0) base = atomicAdd(count, (unsigned)__popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (ready) idx[base + __popc(m & ((1u << lane) - 1u))] = (uint32_t)s;
+    }
+    // this block's additions before its ticket; the last block's read after it
+    __shared__ unsigned last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(count + 1, 1u) == gridDim.x - 1 ? 1u : 0u;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int i = threadIdx.x;
+    constexpr int kWords = (int)(sizeof(TraceCountersDev) / 8);
+    if (i < kWords)
+        reinterpret_cast<volatile unsigned long long*>(&h->cnt)[i] =
+            reinterpret_cast<const unsigned long long*>(cnt)[i];
+    if (i == 0) {
+        *(volatile unsigned*)&h->count = *(volatile unsigned*)count;
+        *(volatile double*)&h->alpha = *alpha;
+    }
 }
+static_assert(sizeof(TraceCountersDev) / 8 <= 256, "one block of k_collect stores the counters");
 
-// one 32-bit sort word of slot idx[perm[i]]: the key words w[0..nf) placed at
-// bit shifts sh[0..nf), surface ids shifted by one so that the -1 padding sorts
-// first (the fields of one word are consecutive in significance)
-struct PackWord {
-    int nf;
-    int w[kKeyWords];
-    int sh[kKeyWords];
-};
+// one 32-bit sort word of slot idx[perm[i]]
 __global__ void k_key_pack(const uint32_t* __restrict__ key, const uint32_t* __restrict__ idx,
                            const uint32_t* __restrict__ perm, int64_t n, const __grid_constant__ PackWord pw,
                            uint32_t* __restrict__ out) {
     ::sbr::pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const uint32_t* k = key + (size_t)idx[perm[i]] * kKeyWords;
-    uint32_t v = 0;
-    for (int f = 0; f < pw.nf; ++f) {
-        uint32_t x = k[pw.w[f]];
-        v |= (pw.w[f] >= 2 ? x + 1u : x) << pw.sh[f];
-    }
-    out[i] = v;
+    out[i] = pack_word(pw, key + (size_t)idx[perm[i]] * kKeyWords);
 }
 
 __global__ void k_iota(uint32_t* p, int64_t n) {
@@ -86,6 +118,7 @@ struct RefineArgs {
     int64_t ray0;          // first ray id of the trace
     // raw outputs, key order
     uint32_t* valid;
+    uint32_t* pos;      // the same, scanned in place afterwards
     int32_t* rx_o;
     int32_t* nb_o;
     int32_t* surf_o;
@@ -116,7 +149,7 @@ __global__ void k_refine(const __grid_constant__ RefineArgs a) {
     const RefineOut o{a.nb_o, a.surf_o, a.face_o, a.pts_o, a.L_o, a.aod_o, a.aoa_o, a.ray_o, a.dist_o, a.jones_o};
     bool ok = refine_key<false>(lane, m, seq, v, sc, mk3(a.tx[0], a.tx[1], a.tx[2]), ld3(a.rx + 3 * rx_id), o, i);
     if (lane != 0) return;
-    a.valid[i] = ok ? 1u : 0u;
+    a.valid[i] = a.pos[i] = ok ? 1u : 0u;
     if (ok) a.rx_o[i] = rx_id;
 }
 
@@ -145,7 +178,7 @@ __global__ void k_refine_solo(const __grid_constant__ RefineArgs a) {
     const d3 Rx = have ? ld3(a.rx + 3 * rx_id) : mk3(0, 0, 0);
     bool ok = refine_key<true>(lane, m, seq, v, sc, mk3(a.tx[0], a.tx[1], a.tx[2]), Rx, o, have ? i : 0, hint, a.R);
     if (!have) return;
-    a.valid[i] = ok ? 1u : 0u;
+    a.valid[i] = a.pos[i] = ok ? 1u : 0u;
     if (ok) a.rx_o[i] = rx_id;
 }
 
@@ -188,31 +221,6 @@ __global__ void k_rx_offsets(const int32_t* __restrict__ rx, const unsigned* __r
     }
     off[r] = (int32_t)lo;
     *(volatile int32_t*)(h_off + r) = (int32_t)lo;
-}
-
-// Layout of the host-mapped words of one path-list build: the key count (later
-// P), the trace's alpha and final counters, then the receiver offsets.
-struct MappedHead {
-    unsigned count;
-    unsigned pad;
-    double alpha;
-    TraceCountersDev cnt;
-};
-static_assert(sizeof(MappedHead) % 8 == 0 && sizeof(TraceCountersDev) % 8 == 0, "64-bit words");
-
-// the key count, alpha and the trace's counters, stored to the host-mapped head
-__global__ void k_peek_counts(const unsigned* __restrict__ count, const double* __restrict__ alpha,
-                              const TraceCountersDev* __restrict__ cnt, MappedHead* h) {
-    ::sbr::pdl_wait();
-    const int i = threadIdx.x;
-    constexpr int kWords = (int)(sizeof(TraceCountersDev) / 8);
-    if (i < kWords)
-        reinterpret_cast<volatile unsigned long long*>(&h->cnt)[i] =
-            reinterpret_cast<const unsigned long long*>(cnt)[i];
-    if (i == 0) {
-        *(volatile unsigned*)&h->count = *count;
-        *(volatile double*)&h->alpha = *alpha;
-    }
 }
 
 // A pinned, device-mapped host buffer per thread and device. The small
@@ -273,23 +281,20 @@ sbr_status paths_run(const sbr_trace_result* tr, const sbr_bvh* b, sbr_path_list
     per_rx.add(&pl->rx_xyz, 3 * (size_t)std::max(1, tr->n_rx));
     per_rx.add(&pl->rx_off, (size_t)tr->n_rx + 1);
     per_rx.add(&pl->d_status, 1);
-    table.add(&count, 1);
+    table.add(&count, 2);
     table.add(&idx, cap);
     void *tmp, *tmp_n;
     SBR_TRY(per_rx.take(&pl->mem, s));
     SBR_TRY(table.take(&tmp, s));
-    if (tr->n_rx > 0)
-        SBR_TRY_CUDA(cudaMemcpyAsync(pl->rx_xyz, tr->rx, sizeof(double) * 3 * tr->n_rx,
-                                     cudaMemcpyDeviceToDevice, s));
-    SBR_TRY_CUDA(cudaMemsetAsync(count, 0, sizeof(unsigned), s));
+    ::sbr::note_launch(), (void)::sbr::launch_pdl(k_paths_init, dim3(nblk(3 * (int64_t)tr->n_rx)), dim3(kThreads), 0, s, tr->rx,
+                                                  3 * tr->n_rx, pl->rx_xyz, count, pl->d_status);
     char *hm, *dm;
     SBR_TRY(mapped_buf(sizeof(MappedHead) + sizeof(int32_t) * (1 + (size_t)tr->n_rx), &hm, &dm));
     MappedHead* hh = reinterpret_cast<MappedHead*>(hm);
     volatile unsigned* h_count = &hh->count;
     int32_t* h_off = reinterpret_cast<int32_t*>(hm + sizeof(MappedHead));
-    ::sbr::note_launch(), (void)::sbr::launch_pdl(k_collect, dim3((unsigned)((cap + 255) / 256)), dim3(256), 0, s, tr->ht_state, cap, idx, count);
-    ::sbr::note_launch(), (void)::sbr::launch_pdl(k_peek_counts, dim3(1), dim3(32), 0, s, count, tr->d_alpha, tr->cnt,
-                                                          reinterpret_cast<MappedHead*>(dm));
+    ::sbr::note_launch(), (void)::sbr::launch_pdl(k_collect, dim3((unsigned)((cap + 255) / 256)), dim3(256), 0, s, tr->ht_state, cap, idx, count,
+                                                  tr->d_alpha, tr->cnt, reinterpret_cast<MappedHead*>(dm));
     SBR_TRY_CUDA(cudaGetLastError());
     SBR_TRY_CUDA(cudaStreamSynchronize(s));
     // the trace has ended: its counters are final and are kept on the host
@@ -326,7 +331,6 @@ sbr_status paths_run(const sbr_trace_result* tr, const sbr_bvh* b, sbr_path_list
     raw.add(&a.dist_o, nn);
     raw.add(&a.jones_o, nn * kJones);
     SBR_TRY(raw.take(&tmp_n, s));
-    ::sbr::note_launch(), (void)::sbr::launch_pdl(k_iota, dim3(nblk(n)), dim3(kThreads), 0, s, perm, n);
     // key fields from the least significant (the last surface) to the most
     // (the receiver), packed greedily into 32-bit sort words; a stable LSD pass
     // per word, least significant word first, gives the lexicographic order
@@ -334,20 +338,30 @@ sbr_status paths_run(const sbr_trace_result* tr, const sbr_bvh* b, sbr_path_list
     for (int k = K - 1; k >= 0; --k) fields.push_back({2 + k, bits_for((int64_t)b->S)});
     fields.push_back({1, bits_for(K)});
     fields.push_back({0, bits_for(std::max(1, tr->n_rx - 1))});
-    size_t f0 = 0;
-    while (f0 < fields.size()) {
+    std::vector<PackWord> words;
+    for (size_t f0 = 0; f0 < fields.size();) {
         PackWord pw{};
-        int bits = 0;
-        while (f0 < fields.size() && bits + fields[f0].second <= 32) {
+        while (f0 < fields.size() && pw.bits + fields[f0].second <= 32) {
             pw.w[pw.nf] = fields[f0].first;
-            pw.sh[pw.nf] = bits;
-            bits += fields[f0].second;
+            pw.sh[pw.nf] = pw.bits;
+            pw.bits += fields[f0].second;
             ++pw.nf;
             ++f0;
         }
+        words.push_back(pw);
+    }
+    // SBR_SORT_PHASES=1 keeps to the per-word launches (a test hook, as in the sort)
+    const char* phases = getenv("SBR_SORT_PHASES");
+    if (sort_keys_fits(n) && !(phases && phases[0] == '1')) {
+        SBR_TRY(sort_keys_small(tr->ht_key, idx, n, words.data(), (int)words.size(), perm, s));
+        words.clear();
+    } else {
+        ::sbr::note_launch(), (void)::sbr::launch_pdl(k_iota, dim3(nblk(n)), dim3(kThreads), 0, s, perm, n);
+    }
+    for (const PackWord& pw : words) {
         ::sbr::note_launch(), (void)::sbr::launch_pdl(k_key_pack, dim3(nblk(n)), dim3(kThreads), 0, s, tr->ht_key, idx, perm, n, pw, word);
         SBR_TRY_CUDA(cudaGetLastError());
-        SBR_TRY(radix_sort_pairs(word, perm, n, bits, s));
+        SBR_TRY(radix_sort_pairs(word, perm, n, pw.bits, s));
     }
     // refine into raw (key-order) buffers
     a.key = tr->ht_key;
@@ -368,6 +382,7 @@ sbr_status paths_run(const sbr_trace_result* tr, const sbr_bvh* b, sbr_path_list
     a.R = tr->Rr;
     a.ray0 = tr->ray0;
     a.valid = valid;
+    a.pos = pos;
     if (n > 0) {
         if (a.seqf)
             // one warp per block: the keys spread over every SM (latency-bound FP64 chains)
@@ -375,7 +390,6 @@ sbr_status paths_run(const sbr_trace_result* tr, const sbr_bvh* b, sbr_path_list
         else
             ::sbr::note_launch(), (void)::sbr::launch_pdl(k_refine, dim3(nblk(32 * n)), dim3(kThreads), 0, s, a);
         SBR_TRY_CUDA(cudaGetLastError());
-        SBR_TRY_CUDA(cudaMemcpyAsync(pos, valid, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s));
     }
     SBR_TRY(exclusive_scan_u32(pos, n, count, s));
     // the list is sized for every key (P <= n), so compaction and the receiver
@@ -393,7 +407,6 @@ sbr_status paths_run(const sbr_trace_result* tr, const sbr_bvh* b, sbr_path_list
     list.add(&pl->dist, nn);
     list.add(&pl->jones, nn * kJones);
     SBR_TRY(list.take(&pl->mem_paths, s));
-    SBR_TRY_CUDA(cudaMemsetAsync(pl->d_status, 0, sizeof(unsigned), s));
     if (n > 0) {
         CompactArgs c{};
         c.valid = valid;

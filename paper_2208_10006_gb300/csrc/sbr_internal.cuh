@@ -142,6 +142,29 @@ Ico make_ico();
 // Stable LSD radix sort of (key, value) pairs on the low `bits` bits of key.
 // keys/vals are sorted in place; tmp buffers are allocated on the stream.
 sbr_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, int64_t n, int bits, cudaStream_t s);
+// One sort word of a path key: the key words w[0..nf) placed at bit shifts
+// sh[0..nf), surface ids shifted by one so that the -1 padding sorts first (the
+// fields of one word are consecutive in significance).
+struct PackWord {
+    int nf, bits;
+    int w[kKeyWords];
+    int sh[kKeyWords];
+};
+__device__ __forceinline__ uint32_t pack_word(const PackWord& pw, const uint32_t* __restrict__ k) {
+    uint32_t v = 0;
+    for (int f = 0; f < pw.nf; ++f) {
+        const uint32_t x = k[pw.w[f]];
+        v |= (pw.w[f] >= 2 ? x + 1u : x) << pw.sh[f];
+    }
+    return v;
+}
+// Lexicographic order of the n keys at key[idx[i] * kKeyWords], sort words
+// pw[0..n_words) from the least significant: perm[r] = i of the r-th. In one
+// launch while the keys fit one block (sort_keys_fits); for the rest see the
+// caller (a pack and a radix sort per word).
+bool sort_keys_fits(int64_t n);
+sbr_status sort_keys_small(const uint32_t* key, const uint32_t* idx, int64_t n, const PackWord* pw, int n_words,
+                           uint32_t* perm, cudaStream_t s);
 // Exclusive prefix sum of n uint32 values, in place; *total (device, may be
 // NULL) receives the sum.
 sbr_status exclusive_scan_u32(uint32_t* data, int64_t n, uint32_t* total, cudaStream_t s);
@@ -278,6 +301,8 @@ sbr_status launch_alpha(int32_t N, double* alpha, cudaStream_t s);
 // the same alpha from one face of the lattice in double-float (the form a trace
 // computes when it is given no alpha): ~1e-15 relative of the FP64 form
 sbr_status launch_alpha_fast(int32_t N, double* alpha, cudaStream_t s);
+// its first part alone: the largest squared chord, of which chord_angle is alpha
+sbr_status launch_chord_fast(int32_t N, double* chord2, cudaStream_t s);
 sbr_status bvh_build(const float* tri, const int32_t* surf, int64_t T, int32_t S, sbr_bvh* b, cudaStream_t s,
                      bool sah_top);
 sbr_status trace_run(const sbr_bvh* b, sbr_trace_result* tr, cudaStream_t s);
@@ -313,6 +338,7 @@ sbr_status capacity_noalloc_run(const float2* H, int32_t F, int32_t Nr, int32_t 
 // ---------------------------------------------------------------- device helpers
 #ifdef __CUDACC__
 namespace sbr {
+__device__ __forceinline__ double chord_angle(double chord2) { return 2.0 * asin(0.5 * sqrt(chord2)); }
 __device__ __forceinline__ float half_extent(float lo, float hi, float c) {
     return fmaxf(__fsub_ru(hi, c), __fsub_ru(c, lo));
 }

@@ -143,12 +143,6 @@ __global__ void k_add_offsets(uint32_t* data, int64_t n, const uint32_t* offs) {
     if (i < n) data[i] += offs[blockIdx.x];
 }
 
-__global__ void k_total(const uint32_t* scanned, const uint32_t* last_in, int64_t n,
-                        uint32_t* total) {
-    ::sbr::pdl_wait();
-    *total = n > 0 ? scanned[n - 1] + *last_in : 0u;
-}
-
 // The sort of a mid-sized array in one cooperative launch (every block is
 // resident), one tile of 256 x rounds keys per block and one chunk of
 // 32 x rounds keys per warp. Per 8-bit pass: each warp counts the digits of
@@ -243,11 +237,11 @@ k_sort_coop(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, int64_t n, i
         }
 }
 
-sbr_status scan_rec(uint32_t* data, int64_t n, cudaStream_t s) {
+sbr_status scan_rec(uint32_t* data, int64_t n, uint32_t* total, cudaStream_t s) {
     if (n <= 0) return SBR_OK;
     int64_t nb = (n + kScanBlock - 1) / kScanBlock;
     if (nb == 1) {
-        ::sbr::note_launch(), (void)::sbr::launch_pdl(k_scan_blocks, dim3(1), dim3(kScanBlock), 0, s, data, n, nullptr);
+        ::sbr::note_launch(), (void)::sbr::launch_pdl(k_scan_blocks, dim3(1), dim3(kScanBlock), 0, s, data, n, total);
         SBR_TRY_CUDA(cudaGetLastError());
         return SBR_OK;
     }
@@ -255,7 +249,7 @@ sbr_status scan_rec(uint32_t* data, int64_t n, cudaStream_t s) {
     SBR_TRY(dalloc_n(&sums, nb, s));
     ::sbr::note_launch(), (void)::sbr::launch_pdl(k_scan_blocks, dim3((unsigned)nb), dim3(kScanBlock), 0, s, data, n, sums);
     SBR_TRY_CUDA(cudaGetLastError());
-    sbr_status st = scan_rec(sums, nb, s);
+    sbr_status st = scan_rec(sums, nb, total, s);
     if (st == SBR_OK) {
         ::sbr::note_launch(), (void)::sbr::launch_pdl(k_add_offsets, dim3((unsigned)nb), dim3(kScanBlock), 0, s, data, n, sums);
         if (cudaGetLastError() != cudaSuccess) st = SBR_ERR_CUDA;
@@ -274,22 +268,15 @@ constexpr int kSmallThreads = 1024;
 constexpr int kSmallWarps = kSmallThreads / 32;
 constexpr int kSmallMax = 12288;  // 2 x 2 x 4 B x 12288 = 192 KB of shared memory
 
-__global__ void __launch_bounds__(kSmallThreads)
-k_sort_small(uint32_t* __restrict__ keys, uint32_t* __restrict__ vals, int n, int passes) {
-    ::sbr::pdl_wait();
-    extern __shared__ uint32_t sm[];
-    uint32_t* ka = sm;
-    uint32_t* va = sm + kSmallMax;
-    uint32_t* kb = sm + 2 * kSmallMax;
-    uint32_t* vb = sm + 3 * kSmallMax;
+// passes over the keys ka and values va in shared memory, swapping them with kb, vb
+__device__ __forceinline__ void sort_in_block(uint32_t*& ka, uint32_t*& va, uint32_t*& kb, uint32_t*& vb, int n,
+                                              int passes) {
     __shared__ uint32_t s_cnt[kSmallWarps][256];   // per warp and digit: count, then output position
     __shared__ uint32_t s_wsum[8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const int chunk = ((n + kSmallWarps - 1) / kSmallWarps + 31) & ~31;
     const int c0 = min(n, warp * chunk), c1 = min(n, c0 + chunk);
-    for (int i = tid; i < n; i += kSmallThreads) { ka[i] = keys[i]; va[i] = vals[i]; }
-    __syncthreads();
     for (int p = 0; p < passes; ++p) {
         const int shift = 8 * p;
         for (int d = lane; d < 256; d += 32) s_cnt[warp][d] = 0;
@@ -343,7 +330,46 @@ k_sort_small(uint32_t* __restrict__ keys, uint32_t* __restrict__ vals, int n, in
         uint32_t* t = ka; ka = kb; kb = t;
         t = va; va = vb; vb = t;
     }
-    for (int i = tid; i < n; i += kSmallThreads) { keys[i] = ka[i]; vals[i] = va[i]; }
+}
+
+__global__ void __launch_bounds__(kSmallThreads)
+k_sort_small(uint32_t* __restrict__ keys, uint32_t* __restrict__ vals, int n, int passes) {
+    ::sbr::pdl_wait();
+    extern __shared__ uint32_t sm[];
+    uint32_t *ka = sm, *va = sm + kSmallMax, *kb = sm + 2 * kSmallMax, *vb = sm + 3 * kSmallMax;
+    for (int i = threadIdx.x; i < n; i += kSmallThreads) { ka[i] = keys[i]; va[i] = vals[i]; }
+    __syncthreads();
+    sort_in_block(ka, va, kb, vb, n, passes);
+    for (int i = threadIdx.x; i < n; i += kSmallThreads) { keys[i] = ka[i]; vals[i] = va[i]; }
+}
+
+// The order of n multi-word keys in one launch: per sort word, least significant
+// first, the packed words in the current order and their stable passes. Before, a
+// launch for the first order, one to pack and one to sort per word, each of which
+// costs more than its work on the few keys of a small scene. The gather of the key
+// words from one SM is what more keys wait for: 380 keys of 7 words 176 us (a launch
+// per pack and sort: 179; whole path list), 939 183 (181), 3,886 236 (214).
+constexpr int kKeysMax = 512;
+struct SortWords {
+    PackWord pw[kKeyWords];
+    int n;
+};
+__global__ void __launch_bounds__(kSmallThreads)
+k_sort_keys(const uint32_t* __restrict__ key, const uint32_t* __restrict__ idx, int n,
+            const __grid_constant__ SortWords a, uint32_t* __restrict__ perm) {
+    ::sbr::pdl_wait();
+    __shared__ uint32_t sm[4 * kKeysMax];
+    uint32_t *ka = sm, *va = sm + kKeysMax, *kb = sm + 2 * kKeysMax, *vb = sm + 3 * kKeysMax;
+    for (int i = threadIdx.x; i < n; i += kSmallThreads) va[i] = (uint32_t)i;
+    for (int w = 0; w < a.n; ++w) {
+        // a thread packs the entries it reads itself in the first pass's order only
+        // after the barrier that ended the last one
+        for (int i = threadIdx.x; i < n; i += kSmallThreads)
+            ka[i] = pack_word(a.pw[w], key + (size_t)idx[va[i]] * kKeyWords);
+        __syncthreads();
+        sort_in_block(ka, va, kb, vb, n, (a.pw[w].bits + 7) / 8);
+    }
+    for (int i = threadIdx.x; i < n; i += kSmallThreads) perm[i] = va[i];
 }
 
 }  // namespace
@@ -353,19 +379,7 @@ sbr_status exclusive_scan_u32(uint32_t* data, int64_t n, uint32_t* total, cudaSt
         if (total) SBR_TRY_CUDA(cudaMemsetAsync(total, 0, sizeof(uint32_t), s));
         return SBR_OK;
     }
-    uint32_t* last = nullptr;
-    if (total) {
-        SBR_TRY(dalloc_n(&last, 1, s));
-        SBR_TRY_CUDA(cudaMemcpyAsync(last, data + n - 1, sizeof(uint32_t),
-                                     cudaMemcpyDeviceToDevice, s));
-    }
-    sbr_status st = scan_rec(data, n, s);
-    if (st == SBR_OK && total) {
-        ::sbr::note_launch(), (void)::sbr::launch_pdl(k_total, dim3(1), dim3(1), 0, s, data, last, n, total);
-        if (cudaGetLastError() != cudaSuccess) st = SBR_ERR_CUDA;
-    }
-    if (last) dfree(last, s);
-    return st;
+    return scan_rec(data, n, total, s);   // the last level's one block knows the total
 }
 
 // blocks of k_sort_coop that fit on the current device at once (0: no
@@ -386,6 +400,19 @@ static sbr_status coop_blocks(int* out) {
         cache[dev].store(c);
     }
     *out = c - 1;
+    return SBR_OK;
+}
+
+bool sort_keys_fits(int64_t n) { return n <= kKeysMax; }
+
+sbr_status sort_keys_small(const uint32_t* key, const uint32_t* idx, int64_t n, const PackWord* pw, int n_words,
+                           uint32_t* perm, cudaStream_t s) {
+    if (n <= 0) return SBR_OK;
+    SortWords a{};
+    a.n = n_words;
+    for (int w = 0; w < n_words; ++w) a.pw[w] = pw[w];
+    ::sbr::note_launch(), (void)::sbr::launch_pdl(k_sort_keys, dim3(1), dim3(kSmallThreads), 0, s, key, idx, (int)n, a, perm);
+    SBR_TRY_CUDA(cudaGetLastError());
     return SBR_OK;
 }
 
@@ -439,7 +466,7 @@ sbr_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, int64_t n, int bits,
     sbr_status st = SBR_OK;
     for (int p = 0; p < passes && st == SBR_OK; ++p) {
         ::sbr::note_launch(), (void)::sbr::launch_pdl(k_hist, dim3(nblocks), dim3(kSortThreads), 0, s, ka, n, 8 * p, hist, nblocks);
-        st = scan_rec(hist, (int64_t)256 * nblocks, s);
+        st = scan_rec(hist, (int64_t)256 * nblocks, nullptr, s);
         if (st != SBR_OK) break;
         ::sbr::note_launch(), (void)::sbr::launch_pdl(k_scatter, dim3(nblocks), dim3(kSortThreads), 0, s, ka, va, kb, vb, n, 8 * p, hist, nblocks);
         if (cudaGetLastError() != cudaSuccess) {

@@ -1062,9 +1062,9 @@ __global__ void k_trace_setup(TraceCountersDev* __restrict__ cnt, unsigned long 
         rx_df[2 * i + 1] = make_float4(x.lo, y.lo, z.lo, 0.f);
     }
     if (i == 0) {
-        double al = alpha_in;
-        if (al > 0.0) *alpha = al;
-        else al = *alpha;
+        // a given alpha, or that of the largest squared chord found before
+        const double al = alpha_in > 0.0 ? alpha_in : chord_angle(*alpha);
+        *alpha = al;
         df a1 = df_from_double(al), a2 = df_from_double(al * al / 3.0);
         *alpha_df = make_float4(a1.hi, a1.lo, a2.hi, a2.lo);
     }
@@ -1241,6 +1241,7 @@ sbr_status trace_run(const sbr_bvh* b, sbr_trace_result* tr, cudaStream_t s) {
     void* tmp;
     SBR_TRY(keep.take(&tr->mem, s));
     SBR_TRY(scratch.take(&tmp, s));
+    if (!(p.alpha > 0.0)) SBR_TRY(launch_chord_fast(p.subdiv_N, tr->d_alpha, s));
     {
         const size_t n_set = std::max<size_t>(std::max<size_t>(cap, (size_t)tr->n_rx), sizeof(TraceCountersDev) / 8);
         ::sbr::note_launch(), (void)::sbr::launch_pdl(k_trace_setup, dim3((unsigned)((n_set + 255) / 256)), dim3(256), 0, s,
