@@ -225,11 +225,11 @@ __global__ void __launch_bounds__(kBThreads) k_batch_gains(const __grid_constant
     }
 }
 
-// element delays of the synthesis (Eq. 13-14 near field; synth_ops.cuh), FP64
+// element delays of the synthesis (Eq. 13-14 near field; synth_ops.cuh), double-float
 // then FP32, transposed per element over the reflected paths (padded slots up
 // to the next multiple of 8 zeroed):
 //   dt[p][n] = |T_p - P1| - |T_0 - P1|, dr[q][n] = |R_q - Pm| - |R_0 - Pm|;
-//   dl[q][p] = |T_p - R_q| - |T_0 - R_0|
+//   dl[dl_index(q, p)] = |T_p - R_q| - |T_0 - R_0|
 __global__ void __launch_bounds__(kBThreads) k_batch_delays(const BatchJobDev* __restrict__ jobs,
                                                             const int32_t* __restrict__ np, BatchPathsDev paths,
                                                             int32_t path_cap, float* __restrict__ dt,
@@ -251,8 +251,8 @@ __global__ void __launch_bounds__(kBThreads) k_batch_delays(const BatchJobDev* _
         if (n < nrefl) {
             const int64_t slot = J->path_base + n + n0;
             const int m = paths.nb[slot];
-            const d3 Pk = ld3(paths.pts + (slot * kKmax + (tx ? 0 : m - 1)) * 3);
-            const double ref = dist_rn(tx ? T0 : R0, Pk);
+            const df3 Pk = df3_of(ld3(paths.pts + (slot * kKmax + (tx ? 0 : m - 1)) * 3));
+            const df ref = dist_df(df3_of(tx ? T0 : R0), Pk);
             const double* el = tx ? J->tx_elem : J->rx_elem;
             for (int e = e0; e < e1; ++e) dst[(int64_t)e * 4] = el_delay(el + 3 * e, Pk, ref);
         } else {
@@ -260,10 +260,10 @@ __global__ void __launch_bounds__(kBThreads) k_batch_delays(const BatchJobDev* _
         }
     }
     (void)ne;
-    const double ref = dist_rn(T0, R0);
+    const df ref = dist_df(df3_of(T0), df3_of(R0));
     for (int it = threadIdx.x; it < Nr * Nt; it += kBThreads) {
         const int q = it / Nt, p = it - q * Nt;
-        dl[J->dl_base + it] = el_delay(J->tx_elem + 3 * p, ld3(J->rx_elem + 3 * q), ref);
+        dl[J->dl_base + dl_index(q, p, Nt)] = el_delay(J->tx_elem + 3 * p, df3_of(ld3(J->rx_elem + 3 * q)), ref);
     }
 }
 
@@ -673,7 +673,7 @@ sbr_status create(const sbr_bvh* const* scenes, const sbr_material* const* mats,
             J.dr_base = odr;
             odr += (int64_t)synth_stride(c.path_cap) * jb.Nr;
             J.dl_base = odl;
-            odl += (int64_t)jb.Nr * jb.Nt;
+            odl += dl_size(jb.Nr, jb.Nt);
             ray_off.push_back(r0);
             r0 += R;
             item_off.push_back(it0);

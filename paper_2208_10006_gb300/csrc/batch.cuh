@@ -46,7 +46,7 @@ struct BatchJobDev {
     // synthesis operands (wave scratch), rows of ps = the path capacity rounded up to 8
     int64_t w_base;              // first reflected-path weight, frequency-major [F][ps]
     int64_t wl_base;             // first LoS weight and FP16 scale, [F] each
-    int64_t dt_base, dr_base, dl_base;   // element delays, [Nt][ps], [Nr][ps], [Nr][Nt]
+    int64_t dt_base, dr_base, dl_base;   // element delays, [Nt][ps], [Nr][ps], [dl_size(Nr, Nt)]
 };
 
 // Path records of the batch, SoA over path slots (job j owns slots

@@ -10,35 +10,42 @@
 //                        max_n max(|Re w|, |Im w|) into [1/2, 1) (1 if all zero)
 //   dtT [Pp/4][Nt][4] float   |T_p - P1| - |T_0 - P1|   (P1 first interaction point)
 //   drT [Pp/4][Nr][4] float   |R_q - Pm| - |R_0 - Pm|   (Pm last interaction point)
-//   dl  [Nr][Nt] float   |T_p - R_q| - |T_0 - R_0|
+//   dl  [dl_size(Nr, Nt)] float, element (q, p) at dl_index: |T_p - R_q| - |T_0 - R_0|,
+//                        in blocks of 8 receive x 16 transmit elements as the epilogue
+//                        reads them (a lane's four of a block in 16 bytes, a warp's in 512)
 // (the delay tables in groups of 4 paths, element-major within a group, so
 // that consecutive threads, on consecutive elements, read consecutive 16-byte
 // groups)
 #pragma once
+#include "dfloat.cuh"
 #include "sbr_internal.cuh"
 
 namespace sbr {
 
 constexpr double kInvC0 = 1.0 / kC0;
 
-// g exp(-j 2 pi f L / c). The phase f L / c (up to ~1e6 cycles at THz) is
-// reduced exactly in FP64 to its fraction r in [0, 1); r = hi + lo with hi the
-// FP32 rounding of r and |lo| <= 2^-25; exp(-j 2 pi r) = exp(-j 2 pi hi)
-// (1 - j 2 pi lo) to second order in lo (< 1e-13), with the FP32 sine and
-// cosine of pi x (sincospif) for the hi part. FP64 is used for 7 operations
-// only: this GPU's FP64 rate is a small fraction of its FP32 rate.
+__host__ __device__ __forceinline__ int64_t dl_size(int64_t Nr, int64_t Nt) { return ((Nr + 7) / 8) * ((Nt + 15) / 16) * 128; }
+// within a block: lane 4 (q % 8) + (p % 8) / 2 holds the pairs of columns p % 16 and p % 16 + 8
+__host__ __device__ __forceinline__ int64_t dl_index(int q, int p, int Nt) {
+    return ((int64_t)(q >> 3) * ((Nt + 15) / 16) + (p >> 4)) * 128 + ((q & 7) * 4 + ((p & 7) >> 1)) * 4 + ((p >> 3) & 1) * 2 + (p & 1);
+}
+
+// g exp(-j 2 pi f L / c). The phase f L / c (up to ~1e6 cycles at THz) is formed in
+// double-float, its integer part removed exactly; the rest r = hi + lo with hi the
+// FP32 rounding of r; exp(-j 2 pi r) = exp(-j 2 pi hi) (1 - j 2 pi lo) to second
+// order in lo (< 1e-13), with the FP32 sine and cosine of pi x (sincospif) for the
+// hi part. No FP64 operation: one takes as long as some 70 FP32 ones on this GPU.
 //
 // Every operation is written with an explicit rounding intrinsic, so that the
 // compiler cannot contract a multiply and an add differently in the kernels
 // that share these functions (their results must agree bit for bit).
 __device__ __forceinline__ float2 synth_weight(float2 g, double f, double L) {
-    const double cyc = __dmul_rn(__dmul_rn(f, L), kInvC0);
-    const double r = __dsub_rn(cyc, floor(cyc));
-    const float hi = __double2float_rn(r);
-    const float lo = __double2float_rn(__dsub_rn(r, (double)hi));
+    const df fd = df_split(f), t = df_mul(df_split(L), df{(float)kInvC0, (float)(kInvC0 - (double)(float)kInvC0)});
+    const df p = two_prod(fd.hi, t.hi);
+    const df r = two_sum(__fsub_rn(p.hi, rintf(p.hi)), __fmaf_rn(fd.hi, t.lo, __fmaf_rn(fd.lo, t.hi, p.lo)));
     float s, c;
-    sincospif(__fmul_rn(-2.0f, hi), &s, &c);
-    const float d = __fmul_rn(-6.283185307179586f, lo);   // exp(j d) ~ 1 + j d
+    sincospif(__fmul_rn(-2.0f, r.hi), &s, &c);
+    const float d = __fmul_rn(-6.283185307179586f, r.lo);   // exp(j d) ~ 1 + j d
     const float cr = __fmaf_rn(-s, d, c), ci = __fmaf_rn(c, d, s);
     return make_float2(__fmaf_rn(g.x, cr, __fmul_rn(-g.y, ci)), __fmaf_rn(g.x, ci, __fmul_rn(g.y, cr)));
 }
@@ -51,16 +58,18 @@ __device__ __forceinline__ float synth_scale(float m) {
     return ldexpf(1.f, -e);
 }
 
-// |a - b| in FP64 with a fixed operation sequence
-__device__ __forceinline__ double dist_rn(d3 a, d3 b) {
-    const double x = __dsub_rn(a.x, b.x), y = __dsub_rn(a.y, b.y), z = __dsub_rn(a.z, b.z);
-    return __dsqrt_rn(__fma_rn(z, z, __fma_rn(y, y, __dmul_rn(x, x))));
+// |a - b| in double-float (relative error about 2^-45)
+__device__ __forceinline__ df3 df3_of(d3 v) { return df3{df_split(v.x), df_split(v.y), df_split(v.z)}; }
+__device__ __forceinline__ df dist_df(const df3& a, const df3& b) {
+    const df3 v = df3_sub(a, b);
+    const df n2 = df3_dot(v, v);
+    return n2.hi > 0.f ? df_sqrt(n2) : df{0.f, 0.f};
 }
 
-// element delay |E - P| - ref, ref = |E0 - P| = dist_rn(E0, P) computed once
-// per path (FP64, then rounded to FP32)
-__device__ __forceinline__ float el_delay(const double* elem, d3 P, double ref) {
-    return __double2float_rn(__dsub_rn(dist_rn(ld3(elem), P), ref));
+// element delay |E - P| - ref, ref = |E0 - P| = dist_df(E0, P) computed once
+// per path, rounded to FP32
+__device__ __forceinline__ float el_delay(const double* elem, const df3& P, df ref) {
+    return df_sub(dist_df(df3_of(ld3(elem)), P), ref).hi;
 }
 
 }  // namespace sbr

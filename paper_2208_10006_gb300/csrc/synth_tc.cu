@@ -18,20 +18,21 @@
 // relative, with 5 exponent bits: A' is scaled per frequency by a power of two
 // that brings max_n |w_n| into [1/2, 1), and the accumulator is scaled back,
 // both exactly). The phasors are generated on chip
-// (FP32 phase from the FP64-prepared delays) straight into 128-byte-swizzled
-// K-major shared-memory tiles; one thread issues tcgen05.mma (M=128, N=256,
+// (FP32 phase from the prepared delays) straight into 128-byte-swizzled
+// K-major shared-memory tiles; one thread of a warp of its own issues tcgen05.mma (M=128, N=256,
 // K=16) and commits to an mbarrier; the epilogue reads TMEM with tcgen05.ld
 // in the 16-lane shape that gives each thread the real and the imaginary row
 // of one receive element, adds the exact per-element LoS term and stores
 // complex64.
 //
-// Every wait on the mbarrier is bounded; on expiry the CTA records
+// Every wait on an mbarrier is bounded; on expiry the CTA records
 // ST_TIMEOUT, releases its tensor memory and returns.
 #include <algorithm>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include "batch.cuh"
+#include "dfloat.cuh"
 #include "tcgen05.cuh"
 #include "sbr_internal.cuh"
 #include "synth_ops.cuh"
@@ -41,8 +42,12 @@ namespace {
 
 using namespace tc;
 
-constexpr int kTcThreads = 512;  // 16 warps, one CTA per SM
-constexpr int kTcWarps = kTcThreads / 32;
+// One CTA per SM: warps [0, 16) generate the operands, [16, 24) are the epilogue,
+// the last one issues the MMAs.
+constexpr int kGenWarps = 16, kEpiWarps = 8;
+constexpr int kGenThreads = 32 * kGenWarps;
+constexpr int kMmaWarp = kGenWarps + kEpiWarps;
+constexpr int kTcThreads = 32 * (kMmaWarp + 1);
 constexpr int kChunkP = 32;      // paths per K-chunk (K = 64 16-bit values = one 128-byte row)
 constexpr int kABytes = kTileM * 128;  // 16 KB: 2 x 64 receive elements
 
@@ -59,12 +64,17 @@ struct TcShape {
     static constexpr int kTmemCols = 2 * kTileN;                    // two accumulators
 };
 
-// exp(-j 2 pi c) for a phase of c cycles: reduce to [-1/2, 1/2] exactly, then
+// exp(-j 2 pi c) for two phases of c cycles: reduce to [-1/2, 1/2] exactly, then
 // the hardware sine/cosine, whose absolute error on [-pi, pi] (below 1e-6) is
-// well under the 2^-16 resolution of the BF16 hi/lo operands
-__device__ __forceinline__ void phasor(float cycles, float& s, float& c) {
-    float r = cycles - rintf(cycles);
-    __sincosf(-6.283185307179586f * r, &s, &c);
+// well under the 2^-16 resolution of the BF16 hi/lo operands. The nearest integer
+// comes from adding and taking away 1.5 2^23 (rintf is an instruction of the narrow
+// pipe that the sine and cosine need); packed operations up to the sine and cosine.
+__device__ __forceinline__ void phasor2(float2 cycles, float2& s, float2& c) {
+    const float2 m = __fadd2_rn(cycles, make_float2(12582912.f, 12582912.f));
+    const float2 k = __fadd2_rn(m, make_float2(-12582912.f, -12582912.f));
+    const float2 z = __fmul2_rn(sub2(cycles, k), make_float2(-6.283185307179586f, -6.283185307179586f));
+    __sincosf(z.x, &s.x, &c.x);
+    __sincosf(z.y, &s.y, &c.y);
 }
 
 // Operands of the tensor-core forms (layouts in synth_ops.cuh): reflected
@@ -83,7 +93,7 @@ struct TcArgs {
     const float2* w;           // [F][Pp]
     const float2* wl;          // [F]
     const float* sc;           // [F]
-    const float* dlos;         // [Nr][Nt]
+    const float* dlos;         // [dl_size(Nr, Nt)]
     float2* H;
     unsigned int* status;
     int inject_timeout;        // test-only: wait on a barrier nothing arrives at
@@ -172,7 +182,9 @@ __device__ __forceinline__ TcItem tc_item(const TcArgs& a, int64_t it) {
     x.p0 = (int)(rem - qt * ntiles) * kTileN;
     x.los = Pr > 0 && *nb0 == 0;
     x.nrefl = Pr - (x.los ? 1 : 0);
-    x.foc = (float)(freqs[x.f] * kInvC0);
+    // f / c in double-float, rounded once (an FP64 product in every thread costs 20
+    // clocks a warp on the narrow pipe)
+    x.foc = df_mul(df_split(freqs[x.f]), df{(float)kInvC0, (float)(kInvC0 - (double)(float)kInvC0)}).hi;
     x.wf = w + (int64_t)x.f * x.Pp;
     x.wl = wl[x.f];
     x.sc = sc[x.f];
@@ -214,13 +226,12 @@ __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, ui
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d));
 }
 
-// what the epilogue of a tile needs once its MMAs have been issued
+// what the epilogue of a tile needs
 struct TcEpi {
     int q0, p0, Nr, Nt, acc;
     bool los;
     bool full;                 // whole tile inside H, even Nt, aligned rows: no per-output checks
     bool mma;                  // the tile has reflected paths (an accumulator to read)
-    uint32_t acc_parity;       // phase of acc_full[acc] that completes this tile
     float foc, isc;
     float2 wl;                 // LoS weight (unscaled)
     const float* dlos;
@@ -233,143 +244,111 @@ struct TcEpi {
 // 16-lane tensor-memory load hands each thread both parts of one output
 __device__ __forceinline__ int acc_row(int ql, int part) { return 16 * (ql >> 3) + 8 * part + (ql & 7); }
 
-// Epilogue of one tile: warp w reads TMEM lanes [32 (w % 4), + 32) (receive
-// elements [16 (w % 4), + 16) of the tile) over its N / 4 columns, 16 lanes
-// (8 receive elements) x 32 columns at a time; thread t receives, for 8
-// consecutive columns, (Re, Im) of receive element t / 4 at transmit elements
+// two outputs, (Re, Im) each, from the accumulator words (re, re, im, im)
+template <bool kF16, bool kLos>
+__device__ __forceinline__ float4 tc_out(const TcEpi& e, const uint32_t* v, float2 dl) {
+    float2 re = make_float2(__uint_as_float(v[0]), __uint_as_float(v[1]));
+    float2 im = make_float2(__uint_as_float(v[2]), __uint_as_float(v[3]));
+    if (kF16) {
+        re = __fmul2_rn(re, dup2(e.isc));
+        im = __fmul2_rn(im, dup2(e.isc));
+    }
+    if (kLos) {
+        float2 sn, cs;
+        phasor2(__fmul2_rn(dup2(e.foc), dl), sn, cs);
+        re = __ffma2_rn(dup2(e.wl.x), cs, __ffma2_rn(dup2(-e.wl.y), sn, re));
+        im = __ffma2_rn(dup2(e.wl.x), sn, __ffma2_rn(dup2(e.wl.y), cs, im));
+    }
+    return make_float4(re.x, im.x, re.y, im.y);
+}
+
+// Epilogue of one tile in blocks of 16 lanes (8 receive elements) x 32 columns:
+// epilogue warp w reads TMEM lanes [32 (w % 4), + 32) (receive elements
+// [16 (w % 4), + 16) of the tile), every second block of them; thread t receives,
+// for 8 consecutive columns, (Re, Im) of receive element t / 4 at transmit elements
 // 2 (t % 4) and + 1. It scales back (FP16 form), adds the exact per-element
 // LoS term and writes them as one 16-byte store (four lanes write 64
 // contiguous bytes of a row of H).
-template <bool kF16, int kTileN>
+template <bool kF16, int kTileN, bool kFull, bool kLos>
 __device__ __forceinline__ void tc_epilogue(const TcEpi& e, uint32_t tmem, int warp, int lane) {
-    const int lg = warp & 3, cg = warp >> 2;   // TMEM lane quarter, column group
-    constexpr int kCols = kTileN / 4;          // columns of one warp
-    constexpr int kRep = kCols >= 32 ? 4 : kCols / 8;   // 8-column repeats per load
-    constexpr int kBlkCols = 8 * kRep;
-    constexpr int kJ = kCols / kBlkCols;       // column blocks per 16-lane half
-    constexpr int kBlocks = 2 * kJ;
+    constexpr int kJ = kTileN / 32, kBlocks = 2 * kJ, kBs = kEpiWarps / 4;   // blocks; warps that share a quarter's
+    const int lg = warp & 3, b0 = warp >> 2;
     const int qa = lane >> 2, pc = 2 * (lane & 3);
-    const uint32_t tacc = tmem + (uint32_t)(e.acc * kTileN);
-    if (e.full) {
-        // every output of the tile exists: no per-output checks. 32-bit element
-        // offsets within frequency f's H and LoS delays (Nr * Nt < 2^31 for a
-        // full tile); the LoS delays of block b + 1 are requested while block b
-        // is processed
-        auto offset = [&](int b, int k) {
-            const int h = b / kJ, jj = b % kJ;
-            const uint32_t q = (uint32_t)(e.q0 + 16 * lg + 8 * h + qa);
-            return q * (uint32_t)e.Nt + (uint32_t)(e.p0 + cg * kCols + kBlkCols * jj + 8 * k + pc);
-        };
-        float2 dl_next[kRep];
-        if (e.los) {
+    const uint32_t tacc = tmem + (uint32_t)(e.acc * kTileN) + ((uint32_t)(32 * lg) << 16);
+    const int nt16 = (e.Nt + 15) / 16, nr8 = (e.Nr + 7) / 8;
+    // LoS delays of a block (dl_index): two 16-byte loads, column pairs 0, 8 and 16, 24
+    const float4* dl0 = reinterpret_cast<const float4*>(e.dlos) + ((int64_t)(e.q0 / 8 + 2 * lg) * nt16 + e.p0 / 16) * 32 + lane;
+    auto load_dl = [&](int b, float4 (&dl)[2]) {
+        const int h = b / kJ, j2 = 2 * (b % kJ);
+        const bool rows = kFull || (e.q0 + 16 * lg) / 8 + h < nr8;
 #pragma unroll
-            for (int k = 0; k < kRep; ++k) dl_next[k] = __ldg(reinterpret_cast<const float2*>(e.dlos + offset(0, k)));
-        }
-#pragma unroll
-        for (int b = 0; b < kBlocks; ++b) {
-            const int h = b / kJ, jj = b % kJ;
-            float2 dl[kRep];
-            if (e.los) {
-#pragma unroll
-                for (int k = 0; k < kRep; ++k) dl[k] = dl_next[k];
-                if (b + 1 < kBlocks) {
-#pragma unroll
-                    for (int k = 0; k < kRep; ++k)
-                        dl_next[k] = __ldg(reinterpret_cast<const float2*>(e.dlos + offset(b + 1, k)));
-                }
-            }
-            uint32_t v[4 * kRep];
-            if (e.mma) {
-                tmem_ld_16x256b<kRep>(tacc + ((uint32_t)(32 * lg + 16 * h) << 16) + (uint32_t)(cg * kCols + kBlkCols * jj), v);
-            } else {
-#pragma unroll
-                for (int k = 0; k < 4 * kRep; ++k) v[k] = 0u;
-            }
-#pragma unroll
-            for (int k = 0; k < kRep; ++k) {
-                const float re0 = __uint_as_float(v[4 * k]), re1 = __uint_as_float(v[4 * k + 1]);
-                const float im0 = __uint_as_float(v[4 * k + 2]), im1 = __uint_as_float(v[4 * k + 3]);
-                float4 o = kF16 ? make_float4(re0 * e.isc, im0 * e.isc, re1 * e.isc, im1 * e.isc)
-                                : make_float4(re0, im0, re1, im1);
-                if (e.los) {
-                    float sn, cs;
-                    phasor(e.foc * dl[k].x, sn, cs);
-                    o.x = fmaf(e.wl.x, cs, fmaf(-e.wl.y, sn, o.x));
-                    o.y = fmaf(e.wl.x, sn, fmaf(e.wl.y, cs, o.y));
-                    phasor(e.foc * dl[k].y, sn, cs);
-                    o.z = fmaf(e.wl.x, cs, fmaf(-e.wl.y, sn, o.z));
-                    o.w = fmaf(e.wl.x, sn, fmaf(e.wl.y, cs, o.w));
-                }
-                *reinterpret_cast<float4*>(e.Hf + offset(b, k)) = o;
-            }
-        }
-        return;
-    }
-#pragma unroll 1
-    for (int b = 0; b < kBlocks; ++b) {
+        for (int k = 0; k < 2; ++k)
+            dl[k] = kFull || (rows && e.p0 / 16 + j2 + k < nt16) ? __ldg(dl0 + (h * nt16 + j2 + k) * 32) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    float2* out = e.Hf + (int64_t)(e.q0 + 16 * lg + qa) * e.Nt + e.p0 + pc;
+    float4 next[2];
+    if (kLos) load_dl(b0, next);
+#pragma unroll 4
+    for (int b = b0; b < kBlocks; b += kBs) {
         const int h = b / kJ, jj = b % kJ;
-        const int q = e.q0 + 16 * lg + 8 * h + qa;
-        const int pb = e.p0 + cg * kCols + kBlkCols * jj + pc;
-        // LoS delays of this lane's outputs, requested before the tensor-memory
-        // load so that their latency overlaps it
-        float2 dl[kRep];
-#pragma unroll
-        for (int k = 0; k < kRep; ++k) {
-            const int p = pb + 8 * k;
-            dl[k] = make_float2(0.f, 0.f);
-            if (e.los && q < e.Nr && p < e.Nt) {
-                const float* src = e.dlos + (int64_t)q * e.Nt + p;
-                if (p + 1 < e.Nt && ((((uintptr_t)src) & 7) == 0)) dl[k] = __ldg(reinterpret_cast<const float2*>(src));
-                else dl[k] = make_float2(__ldg(src), p + 1 < e.Nt ? __ldg(src + 1) : 0.f);
-            }
+        // the delays of the next block are requested while this one is processed
+        float4 dl[2];
+        if (kLos) {
+            dl[0] = next[0]; dl[1] = next[1];
+            if (b + kBs < kBlocks) load_dl(b + kBs, next);
         }
-        uint32_t v[4 * kRep];
+        uint32_t v[16];
         if (e.mma) {
-            tmem_ld_16x256b<kRep>(tacc + ((uint32_t)(32 * lg + 16 * h) << 16) + (uint32_t)(cg * kCols + kBlkCols * jj), v);
+            tmem_ld_16x256b<4>(tacc + ((uint32_t)(16 * h) << 16) + (uint32_t)(32 * jj), v);
         } else {
 #pragma unroll
-            for (int k = 0; k < 4 * kRep; ++k) v[k] = 0u;
+            for (int k = 0; k < 16; ++k) v[k] = 0u;
         }
+        const int q = e.q0 + 16 * lg + 8 * h + qa, p0 = e.p0 + 32 * jj + pc;
+        float2* row = out + (8 * h * e.Nt + 32 * jj);
 #pragma unroll
-        for (int k = 0; k < kRep; ++k) {
-            const int p = pb + 8 * k;
-            const float re0 = __uint_as_float(v[4 * k]), re1 = __uint_as_float(v[4 * k + 1]);
-            const float im0 = __uint_as_float(v[4 * k + 2]), im1 = __uint_as_float(v[4 * k + 3]);
-            float4 o = make_float4(re0 * e.isc, im0 * e.isc, re1 * e.isc, im1 * e.isc);
-            if (e.los) {
-                float sn, cs;
-                phasor(e.foc * dl[k].x, sn, cs);
-                o.x = fmaf(e.wl.x, cs, fmaf(-e.wl.y, sn, o.x));
-                o.y = fmaf(e.wl.x, sn, fmaf(e.wl.y, cs, o.y));
-                phasor(e.foc * dl[k].y, sn, cs);
-                o.z = fmaf(e.wl.x, cs, fmaf(-e.wl.y, sn, o.z));
-                o.w = fmaf(e.wl.x, sn, fmaf(e.wl.y, cs, o.w));
-            }
-            if (q < e.Nr && p < e.Nt) {
-                float2* dst = e.Hf + (int64_t)q * e.Nt + p;
-                if (p + 1 < e.Nt && ((((uintptr_t)dst) & 15) == 0)) {
+        for (int k = 0; k < 4; ++k) {
+            const float4 d4 = dl[k / 2];
+            const float4 o = tc_out<kF16, kLos>(e, v + 4 * k, k & 1 ? make_float2(d4.z, d4.w) : make_float2(d4.x, d4.y));
+            float2* dst = row + 8 * k;
+            if (kFull) {   // whole tile inside H, even Nt, aligned rows: no per-output checks
+                *reinterpret_cast<float4*>(dst) = o;
+            } else if (q < e.Nr && p0 + 8 * k < e.Nt) {
+                const bool two = p0 + 8 * k + 1 < e.Nt;
+                if (two && ((((uintptr_t)dst) & 15) == 0)) {
                     *reinterpret_cast<float4*>(dst) = o;
                 } else {
                     dst[0] = make_float2(o.x, o.y);
-                    if (p + 1 < e.Nt) dst[1] = make_float2(o.z, o.w);
+                    if (two) dst[1] = make_float2(o.z, o.w);
                 }
             }
         }
     }
 }
 
+// The roles meet at mbarriers only: the generating warps fill the two operand
+// stages (full), the MMA warp consumes them into one of two accumulators (empty,
+// acc_full), the epilogue warps empty those (acc_free), so phasors, MMAs and
+// output of different tiles run side by side and each role's latencies (loads,
+// sine and cosine, shared memory) are covered by the others' work. With all 16
+// warps first generating, then writing out, a block barrier per K-chunk between,
+// 42% of the issue slots were used. H [1024, 64, 256] from 45 reflected paths and the
+// LoS path, whole call: 68.5 us then, 59 with the roles side by side, 55 with packed
+// phasors and the operand prologue in double-float, 48 with the LoS delays in the
+// epilogue's order and an epilogue per kind of tile. It is the epilogue that bounds
+// it (32 us without; 47 without the B' phasors; 42 without the stores): 16 + 8 warps
+// are the split that leaves it 72 registers (8 + 16: 63 us, 16 + 12 with 64: 50).
 template <bool kF16, bool kBatch, int kTileN>
 __global__ void __launch_bounds__(kTcThreads, 1) k_synth_tc(const __grid_constant__ TcArgs a) {
     using Sh = TcShape<kTileN>;
-    static_assert(kTcThreads % kTileN == 0 && 64 * (kChunkP / 4) <= kTcThreads, "generation units");
+    static_assert(kGenThreads % kTileN == 0 && 64 * (kChunkP / 4) <= kGenThreads, "generation units");
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t* bars = (uint64_t*)(smem + 2 * Sh::kStage);
-    // bars: mma_done[0..1] (per operand stage), acc_full[0..1] (per accumulator),
-    // never (injected fault), drain (final wait before the tensor memory is freed)
+    enum { kFull = 0, kEmpty = 2, kAccFull = 4, kAccFree = 6, kNever = 8, kDrain = 9, kBars = 10 };
     const uint32_t bar0 = smem_u32(bars);
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
-    uint32_t* tmem_slot = (uint32_t*)(bars + 6);
+    uint32_t* tmem_slot = (uint32_t*)(bars + kBars);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (warp == 0) {
@@ -379,7 +358,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_synth_tc(const __grid_constan
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
-        for (int i = 0; i < 6; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar(i)), "r"(1));
+        for (int i = 0; i < kBars; ++i)
+            mbar_init(bar(i), i < kEmpty ? kGenWarps : i >= kAccFree && i < kNever ? kEpiWarps : 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -390,98 +370,88 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_synth_tc(const __grid_constan
     // prologue above overlaps its tail; its results are read only after this
     // (a no-op for an ordinary launch)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    bool failed = false;
+    bool ok = true;
     // injected fault: the first phase of `never` never completes; the bounded
     // wait gives up and the CTA takes the same exit as a real timeout
-    if (a.inject_timeout) failed = __syncthreads_or(!mbar_wait(bar(4), 0u, 1u << 12)) != 0;
+    if (a.inject_timeout) ok = __syncthreads_or(!mbar_wait(bar(kNever), 0u, 1u << 12)) == 0;
 
     const int64_t items = kBatch ? a.items
                                  : (int64_t)a.F * ((a.Nr + 63) / 64) * ((a.Nt + kTileN - 1) / kTileN);
-    uint32_t stage_uses0 = 0u, stage_uses1 = 0u;   // chunks issued per operand stage
-    uint32_t acc_uses0 = 0u, acc_uses1 = 0u;       // tiles with MMAs per accumulator
-    uint32_t chunk_all = 0;
-    TcEpi prev{};
-    bool have_prev = false;
-    bool epi_ok = true;   // this thread's last epilogue wait succeeded (folded into the next barrier)
-    int local = 0;
-    for (int64_t it = blockIdx.x; it < items && !failed; it += gridDim.x, ++local) {
-        const TcItem x = tc_item<kBatch, kTileN>(a, it);
-        const int acc = local & 1;
-        const int nch = (x.nrefl + kChunkP - 1) / kChunkP;
-        // FP16 form: the power-of-two scale of this frequency's weights (exact)
-        const float sc = kF16 ? x.sc : 1.f;
-        for (int c = 0; c < nch; ++c) {
-            const int st = chunk_all & 1;
-            unsigned char* sA_hi = smem + st * Sh::kStage;
-            unsigned char* sA_lo = sA_hi + kABytes;
-            unsigned char* sB_hi = sA_hi + 2 * kABytes;
-            unsigned char* sB_lo = sB_hi + Sh::kBBytes;
-            bool ok = true;
-            // the stage is free once the MMAs of its previous chunk have completed
-            const uint32_t su = st ? stage_uses1 : stage_uses0;
-            if (su > 0) ok = mbar_wait(bar(st), (su - 1u) & 1u);
-            const int nb = c * kChunkP;
-            const int cnt = min(kChunkP, x.nrefl - nb);
-            const int nks = (cnt + 7) >> 3;        // MMA K-steps (8 paths each)
-            const int n16 = 2 * nks;               // 16-byte chunks per row (4 paths each)
-            if (ok) {
+    auto wait = [&](int i, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait(bar(i), parity)) != 0; };
+    uint32_t chunk = 0;   // chunks so far (operand stage and its phase)
+    uint32_t tile = 0;    // tiles with MMAs so far (accumulator and its phase)
+    if (warp < kGenWarps) {
+        for (int64_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
+            const TcItem x = tc_item<kBatch, kTileN>(a, it);
+            // FP16 form: the power-of-two scale of this frequency's weights (exact)
+            const float sc = kF16 ? x.sc : 1.f;
+            for (int nb = 0; nb < x.nrefl; nb += kChunkP, ++chunk) {
+                const int st = chunk & 1;
+                const uint32_t sA_hi = smem_u32(smem) + st * Sh::kStage, sA_lo = sA_hi + kABytes;
+                const uint32_t sB_hi = sA_hi + 2 * kABytes, sB_lo = sB_hi + Sh::kBBytes;
+                const int cnt = min(kChunkP, x.nrefl - nb);
+                const int n16 = 2 * ((cnt + 7) >> 3);   // 16-byte chunks per row (4 paths each), whole MMA K-steps
                 // B' (stored N x K): transmit element p, paths nb + 4 c16 .. + 3
                 // (padded paths have zero weight, so their phasors are harmless);
-                // kTcThreads is a multiple of N, so a thread keeps its element and
-                // steps through the chunks
-                {
-                    const int pl = tid % kTileN;
-                    const int p = x.p0 + pl;
-                    // [Pp / 4][Nt] groups of 4 paths: consecutive lanes read
-                    // consecutive 16-byte groups
-                    const float4* src = reinterpret_cast<const float4*>(x.dtT) + (int64_t)(nb >> 2) * x.Nt + (p < x.Nt ? p : 0);
-                    const uint32_t b_hi = smem_u32(sB_hi) + (uint32_t)pl * 128u;
-                    const uint32_t b_lo = smem_u32(sB_lo) + (uint32_t)pl * 128u;
-#pragma unroll 2
-                    for (int c16 = tid / kTileN; c16 < n16; c16 += kTcThreads / kTileN) {
-                        float4 d4 = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (p < x.Nt) d4 = __ldg(src + (int64_t)c16 * x.Nt);
-                        float vr[4], vi[4];
-                        phasor(x.foc * d4.x, vi[0], vr[0]);
-                        phasor(x.foc * d4.y, vi[1], vr[1]);
-                        phasor(x.foc * d4.z, vi[2], vr[2]);
-                        phasor(x.foc * d4.w, vi[3], vr[3]);
+                // kGenThreads is a multiple of N, so a thread keeps its element and
+                // steps through the chunks. [Pp / 4][Nt] groups of 4 paths:
+                // consecutive lanes read consecutive 16-byte groups
+                constexpr int kStep = kGenThreads / kTileN, kUnits = 8 / kStep;
+                const int pl = tid % kTileN, p = x.p0 + pl;
+                const float4* src = reinterpret_cast<const float4*>(x.dtT) + (int64_t)(nb >> 2) * x.Nt + (p < x.Nt ? p : 0);
+                // A': receive element q, paths nb + 4 c16 .. + 3 (at most 64 x 8
+                // units: one per thread); consecutive lanes take consecutive receive
+                // elements (rows r(q) & 7 = q & 7), so that a quarter warp's 16-byte
+                // stores land in 8 distinct bank groups of the swizzled rows and a
+                // warp shares its weights
+                const int ql = tid & 63, qc = tid >> 6, q = x.q0 + ql, n = nb + 4 * qc;
+                // every load of the chunk before the wait for its stage
+                float4 dt[kUnits], dr = make_float4(0.f, 0.f, 0.f, 0.f), w01 = dr, w23 = dr;
+#pragma unroll
+                for (int u = 0; u < kUnits; ++u) {
+                    const int c16 = tid / kTileN + u * kStep;
+                    dt[u] = p < x.Nt && c16 < n16 ? __ldg(src + (int64_t)c16 * x.Nt) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+                if (qc < n16 && q < x.Nr) {
+                    dr = __ldg(reinterpret_cast<const float4*>(x.drT) + (int64_t)(n >> 2) * x.Nr + q);
+                    w01 = __ldg(reinterpret_cast<const float4*>(x.wf + n));
+                    w23 = __ldg(reinterpret_cast<const float4*>(x.wf + n + 2));
+                }
+                // the stage is free once the MMAs of its previous chunk have completed
+                if (chunk >= 2 && !(ok = wait(kEmpty + st, (chunk / 2 - 1) & 1u))) break;
+#pragma unroll
+                for (int u = 0; u < kUnits; ++u) {
+                    const int c16 = tid / kTileN + u * kStep;
+                    if (c16 < n16) {
                         uint32_t h[4], l[4];
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) split2<kF16>(vr[k], vi[k], h[k], l[k]);
-                        const uint32_t o = (uint32_t)(c16 ^ (pl & 7)) << 4;   // chunk_off(pl, c16) - pl * 128
-                        sts128(b_hi + o, h[0], h[1], h[2], h[3]);
-                        sts128(b_lo + o, l[0], l[1], l[2], l[3]);
+                        for (int k = 0; k < 4; k += 2) {
+                            float2 sn, cs;
+                            phasor2(__fmul2_rn(dup2(x.foc), k ? make_float2(dt[u].z, dt[u].w) : make_float2(dt[u].x, dt[u].y)), sn, cs);
+                            split2<kF16>(cs.x, sn.x, h[k], l[k]);
+                            split2<kF16>(cs.y, sn.y, h[k + 1], l[k + 1]);
+                        }
+                        const uint32_t o = chunk_off(pl, c16);
+                        sts128(sB_hi + o, h[0], h[1], h[2], h[3]);
+                        sts128(sB_lo + o, l[0], l[1], l[2], l[3]);
                     }
                 }
-                // A': receive element q, paths nb + 4 c16 .. + 3, as the two rows
-                // r(q) (Re A, -Im A) and i(q) (Im A, Re A); consecutive lanes take
-                // consecutive receive elements (rows r(q) & 7 = q & 7), so that a
-                // quarter warp's 16-byte stores land in 8 distinct bank groups of
-                // the swizzled rows and a warp shares its weights (at most 64 x 8
-                // units: one per thread)
-                const int v = tid;
-                if (v < 64 * n16) {
-                    const int ql = v & 63, c16 = v >> 6;
-                    const int q = x.q0 + ql;
-                    const int n = nb + 4 * c16;
-                    float4 d4 = make_float4(0.f, 0.f, 0.f, 0.f);
-                    float4 w01 = d4, w23 = d4;
-                    if (q < x.Nr) {
-                        d4 = __ldg(reinterpret_cast<const float4*>(x.drT) + (int64_t)(n >> 2) * x.Nr + q);
-                        w01 = __ldg(reinterpret_cast<const float4*>(x.wf + n));
-                        w23 = __ldg(reinterpret_cast<const float4*>(x.wf + n + 2));
+                // A' as the two rows r(q) (Re A, -Im A) and i(q) (Im A, Re A)
+                if (qc < n16) {
+                    float sn[4], cs[4];
+#pragma unroll
+                    for (int k = 0; k < 4; k += 2) {
+                        float2 s2, c2;
+                        phasor2(__fmul2_rn(dup2(x.foc), k ? make_float2(dr.z, dr.w) : make_float2(dr.x, dr.y)), s2, c2);
+                        sn[k] = s2.x; sn[k + 1] = s2.y; cs[k] = c2.x; cs[k + 1] = c2.y;
                     }
-                    const float dd[4] = {d4.x, d4.y, d4.z, d4.w};
                     const float wr[4] = {w01.x, w01.z, w23.x, w23.z};
                     const float wi[4] = {w01.y, w01.w, w23.y, w23.w};
                     uint32_t h0[4], l0[4], h1[4], l1[4];
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        float sn, cs;
-                        phasor(x.foc * dd[k], sn, cs);
-                        const float ar = (wr[k] * cs - wi[k] * sn) * sc;
-                        const float ai = (wr[k] * sn + wi[k] * cs) * sc;
+                        const float ar = (wr[k] * cs[k] - wi[k] * sn[k]) * sc;
+                        const float ai = (wr[k] * sn[k] + wi[k] * cs[k]) * sc;
                         split2<kF16>(ar, -ai, h0[k], l0[k]);
                         // row i(q) holds (Im A, Re A): the same halves swapped, with
                         // the sign of -Im A flipped (rounding to nearest is symmetric,
@@ -489,82 +459,92 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_synth_tc(const __grid_constan
                         h1[k] = __byte_perm(h0[k], 0u, 0x1032) ^ 0x8000u;
                         l1[k] = __byte_perm(l0[k], 0u, 0x1032) ^ 0x8000u;
                     }
-                    const uint32_t o0 = chunk_off(acc_row(ql, 0), c16), o1 = chunk_off(acc_row(ql, 1), c16);
-                    sts128(smem_u32(sA_hi) + o0, h0[0], h0[1], h0[2], h0[3]);
-                    sts128(smem_u32(sA_lo) + o0, l0[0], l0[1], l0[2], l0[3]);
-                    sts128(smem_u32(sA_hi) + o1, h1[0], h1[1], h1[2], h1[3]);
-                    sts128(smem_u32(sA_lo) + o1, l1[0], l1[1], l1[2], l1[3]);
+                    const uint32_t o0 = chunk_off(acc_row(ql, 0), qc), o1 = chunk_off(acc_row(ql, 1), qc);
+                    sts128(sA_hi + o0, h0[0], h0[1], h0[2], h0[3]);
+                    sts128(sA_lo + o0, l0[0], l0[1], l0[2], l0[3]);
+                    sts128(sA_hi + o1, h1[0], h1[1], h1[2], h1[3]);
+                    sts128(sA_lo + o1, l1[0], l1[1], l1[2], l1[3]);
                 }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(kFull + st));
             }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            // one decision for the whole CTA (this chunk's wait and the last epilogue's)
-            failed = __syncthreads_or(!(ok && epi_ok)) != 0;
-            if (failed) break;
-            if (tid == 0) {
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint64_t dAh = make_desc(smem_u32(sA_hi)), dAl = make_desc(smem_u32(sA_lo));
-                const uint64_t dBh = make_desc(smem_u32(sB_hi)), dBl = make_desc(smem_u32(sB_lo));
-                const uint32_t d = tmem + (uint32_t)(acc * kTileN);
-                for (int ks = 0; ks < nks; ++ks) {
-                    const uint64_t off = (uint64_t)(ks * 32) >> 4;  // 16 K values
-                    mma_16<kF16, kTileN>(d, dAh + off, dBh + off, (c > 0 || ks > 0) ? 1u : 0u);
-                    mma_16<kF16, kTileN>(d, dAh + off, dBl + off, 1u);
-                    mma_16<kF16, kTileN>(d, dAl + off, dBh + off, 1u);
-                }
-                mma_commit(bar(st));
-                if (c == nch - 1) mma_commit(bar(2 + acc));
-            }
-            if (st) stage_uses1 += 1u; else stage_uses0 += 1u;
-            chunk_all += 1u;
         }
-        if (failed) break;
-        TcEpi cur;
-        cur.q0 = x.q0; cur.p0 = x.p0; cur.Nr = x.Nr; cur.Nt = x.Nt; cur.los = x.los; cur.acc = acc;
-        cur.mma = nch > 0;
-        cur.acc_parity = (acc ? acc_uses1 : acc_uses0) & 1u;
-        if (nch > 0) {
-            if (acc) acc_uses1 += 1u; else acc_uses0 += 1u;
-        }
-        cur.foc = x.foc;
-        cur.isc = kF16 ? 1.f / sc : 1.f;   // exact: sc is a power of two
-        cur.wl = x.wl;
-        cur.dlos = x.dlos; cur.Hf = x.Hf;
-        cur.full = x.q0 + 64 <= x.Nr && x.p0 + kTileN <= x.Nt && (x.Nt & 1) == 0 &&
-                   (int64_t)x.Nr * x.Nt < ((int64_t)1 << 31) &&   // 32-bit offsets in the fast epilogue
-                   ((((uintptr_t)x.Hf) & 15) == 0) && (!x.los || ((((uintptr_t)x.dlos) & 7) == 0));
-        // the previous tile's epilogue runs while this tile's MMAs do; no
-        // barrier follows it: the next tile's first chunk barrier carries its
-        // status, and its accumulator is written again only after that barrier
-        if (have_prev) {
-            bool ok = true;
-            if (prev.mma) {
-                ok = __all_sync(0xffffffffu, mbar_wait(bar(2 + prev.acc), prev.acc_parity));
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            }
-            if (ok) tc_epilogue<kF16, kTileN>(prev, tmem, warp, lane);
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            epi_ok = epi_ok && ok;
-        }
-        prev = cur;
-        have_prev = true;
-    }
-    if (!failed && have_prev) {
-        bool ok = true;
-        if (prev.mma) {
-            ok = __all_sync(0xffffffffu, mbar_wait(bar(2 + prev.acc), prev.acc_parity));
+    } else if (warp == kMmaWarp) {
+        // the whole warp walks the loop, so that descriptors and addresses stay in
+        // uniform registers; one elected lane issues
+        const bool lead = elect_one();
+        const uint64_t dA = make_desc(smem_u32(smem)), dB = make_desc(smem_u32(smem) + 2 * kABytes);
+        for (int64_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
+            const TcItem x = tc_item<kBatch, kTileN>(a, it);
+            if (x.nrefl <= 0) continue;
+            const int acc = tile & 1;
+            const uint32_t d = tmem + (uint32_t)(acc * kTileN);
+            // the accumulator is free once the epilogue of its previous tile has read it
+            if (tile >= 2 && !(ok = wait(kAccFree + acc, (tile / 2 - 1) & 1u))) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int nb = 0; nb < x.nrefl; nb += kChunkP, ++chunk) {
+                const int st = chunk & 1;
+                const int nks = (min(kChunkP, x.nrefl - nb) + 7) >> 3;   // MMA K-steps (8 paths each)
+                if (!(ok = wait(kFull + st, (chunk / 2) & 1u))) break;
+                // the generating warps' stores become visible to the tensor core by one
+                // proxy fence here, on the path from them to its reads
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                if (lead) {
+                    const uint64_t so = (uint64_t)(st * (Sh::kStage >> 4));
+                    for (int ks = 0; ks < nks; ++ks) {
+                        const uint64_t o = so + (uint64_t)(2 * ks);   // 16 K values
+                        mma_16<kF16, kTileN>(d, dA + o, dB + o, (nb > 0 || ks > 0) ? 1u : 0u);
+                        mma_16<kF16, kTileN>(d, dA + o, dB + o + (Sh::kBBytes >> 4), 1u);
+                        mma_16<kF16, kTileN>(d, dA + o + (kABytes >> 4), dB + o, 1u);
+                    }
+                    mma_commit(bar(kEmpty + st));
+                    if (nb + kChunkP >= x.nrefl) mma_commit(bar(kAccFull + acc));
+                }
+                __syncwarp();
+            }
+            ++tile;
         }
-        if (ok) tc_epilogue<kF16, kTileN>(prev, tmem, warp, lane);
-        epi_ok = epi_ok && ok;
+    } else {
+        for (int64_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
+            const TcItem x = tc_item<kBatch, kTileN>(a, it);
+            TcEpi e;
+            e.q0 = x.q0; e.p0 = x.p0; e.Nr = x.Nr; e.Nt = x.Nt; e.los = x.los;
+            e.acc = tile & 1;
+            e.mma = x.nrefl > 0;
+            e.foc = x.foc;
+            e.isc = kF16 ? 1.f / x.sc : 1.f;   // exact: sc is a power of two
+            e.wl = x.wl;
+            e.dlos = x.dlos; e.Hf = x.Hf;
+            e.full = x.q0 + 64 <= x.Nr && x.p0 + kTileN <= x.Nt && (x.Nt & 1) == 0 && (((uintptr_t)x.Hf) & 15) == 0 &&
+                     x.Nt < (1 << 26);   // 32-bit offsets within the tile
+            if (e.mma) {
+                if (!(ok = wait(kAccFull + e.acc, (tile / 2) & 1u))) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            }
+            if (!e.full) {
+                if (e.los) tc_epilogue<kF16, kTileN, false, true>(e, tmem, warp - kGenWarps, lane);
+                else tc_epilogue<kF16, kTileN, false, false>(e, tmem, warp - kGenWarps, lane);
+            } else {
+                if (e.los) tc_epilogue<kF16, kTileN, true, true>(e, tmem, warp - kGenWarps, lane);
+                else tc_epilogue<kF16, kTileN, true, false>(e, tmem, warp - kGenWarps, lane);
+            }
+            if (e.mma) {
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(kAccFree + e.acc));
+                ++tile;
+            }
+        }
     }
-    failed = __syncthreads_or(failed || !epi_ok) != 0;
+    const bool failed = __syncthreads_or(!ok) != 0;
     // every MMA this CTA issued has completed before its tensor memory is freed
     // (bounded wait; on a normal exit the last epilogue has already seen them)
-    if (tid == 0) {
-        mma_commit(bar(5));
-        if (!mbar_wait(bar(5), 0u)) failed = true;
+    if (warp == kMmaWarp) {
+        if (elect_one()) mma_commit(bar(kDrain));
+        __syncwarp();
+        const bool drained = wait(kDrain, 0u);
+        if ((failed || !drained) && lane == 0) atomicOr(a.status, (unsigned)ST_TIMEOUT);
     }
-    if (failed && tid == 0) atomicOr(a.status, (unsigned)ST_TIMEOUT);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0) {
@@ -577,8 +557,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_synth_tc(const __grid_constan
 // is that warp's maximum); the other blocks compute the element delays, one
 // thread per path and group of kPrepG elements (per transmit element and
 // group of kPrepG receive elements for the LoS delays), the reference
-// distance once per thread. Blocks of kPrepThreads threads spread the FP64
-// work (square roots above all) over every SM.
+// distance once per thread. Double-float throughout: it is a chain of latencies,
+// so blocks of kPrepThreads threads spread it over every SM.
 constexpr int kPrepThreads = 128;
 constexpr int kPrepG = 2;
 struct TcPrep {
@@ -643,8 +623,8 @@ __global__ void k_tc_prep(const __grid_constant__ TcPrep a) {
             float* dst = (tx ? a.dtT : a.drT) + (int64_t)(n >> 2) * ne * 4 + (n & 3);
             if (n < nrefl) {
                 const int i = n + n0, m = a.nb[i];
-                const d3 P = ld3(a.pts + ((int64_t)i * kKmax + (tx ? 0 : m - 1)) * 3);
-                const double ref = dist_rn(tx ? a.T0 : ld3(a.R0), P);
+                const df3 P = df3_of(ld3(a.pts + ((int64_t)i * kKmax + (tx ? 0 : m - 1)) * 3));
+                const df ref = dist_df(df3_of(tx ? a.T0 : ld3(a.R0)), P);
 #pragma unroll
                 for (int k = 0; k < kPrepG; ++k)
                     if (e0 + k < ne) dst[(int64_t)(e0 + k) * 4] = el_delay(elem + 3 * (e0 + k), P, ref);
@@ -656,11 +636,11 @@ __global__ void k_tc_prep(const __grid_constant__ TcPrep a) {
         } else {
             const int64_t u = t - n_dt - n_dr;
             const int p = (int)(u % a.Nt), q0 = (int)(u / a.Nt) * kPrepG;
-            const double ref = dist_rn(a.T0, ld3(a.R0));
+            const df ref = dist_df(df3_of(a.T0), df3_of(ld3(a.R0)));
 #pragma unroll
             for (int k = 0; k < kPrepG; ++k)
                 if (q0 + k < a.Nr)
-                    a.dlos[(int64_t)(q0 + k) * a.Nt + p] = el_delay(a.tx_elem + 3 * p, ld3(a.rx_elem + 3 * (q0 + k)), ref);
+                    a.dlos[dl_index(q0 + k, p, a.Nt)] = el_delay(a.tx_elem + 3 * p, df3_of(ld3(a.rx_elem + 3 * (q0 + k))), ref);
         }
     }
 }
@@ -680,7 +660,7 @@ sbr_status synth_tc_run(const sbr_path_list* pl, const float2* g, const double* 
     // elements) first, then sc, dtT, drT, dlos
     const size_t n_w = (size_t)Pp * F, n_wl = ((size_t)F + 1) & ~(size_t)1;
     const size_t n_sc = ((size_t)F + 3) & ~(size_t)3;
-    const size_t n_f = n_sc + (size_t)Pp * Nt + (size_t)Pp * Nr + (((size_t)Nr * Nt + 3) & ~(size_t)3);
+    const size_t n_f = n_sc + (size_t)Pp * Nt + (size_t)Pp * Nr + (size_t)dl_size(Nr, Nt);
     float2* w;
     SBR_TRY(dalloc_n(&w, n_w + n_wl + (n_f + 1) / 2, s));
     float2* wl = w + n_w;

@@ -83,3 +83,27 @@ def test_per_element_steps_of_many_turns(sbr, room):
     Ho = oracle.synth_H_elements(to_numpy(r["export"]), g.astype(np.complex128), f, sc["tx"], te, sc["rx"])
     H = sbr.synthesize_H_elements(r["paths"], torch.as_tensor(g, device="cuda"), dev(f), dev(te), sbr.SYNTH_FP32).cpu().numpy()
     assert np.abs(H - Ho).max() < 2e-5 * np.abs(Ho).max()   # an aperture of 1 m: phases of 60 cycles in FP32
+
+
+@pytest.mark.parametrize("K", [0, 1, 2, 3])   # paths: LoS alone, one K-step, one chunk and more than a chunk of 32
+@pytest.mark.parametrize("Nr,Nt,F", [(1, 1, 1), (7, 15, 3), (8, 17, 2), (63, 255, 2), (64, 256, 3), (65, 257, 2), (64, 514, 160), (130, 30, 200)])
+def test_tensor_core_tiles(sbr, K, Nr, Nt, F):
+    """Both tensor-core forms against the oracle. Per term: three FP32 roundings of a
+    phase of at most `cycles` (delay, f / c, product), the hardware sine and cosine
+    (1e-6 each) and the dropped lo-lo products (2^-22 FP16, 2^-16 BF16); bound: that,
+    times the sum of the path magnitudes."""
+    sc = scenes.shoebox(N=60, K=K, n_rx=2)
+    r = sbr.run_scene(sc)
+    f = grid(F, "odd")
+    te, re = scenes.upa_yz(sc["tx"], Nt, 1, 2.5e-3), scenes.ula_y(sc["rx"][1], Nr, 2.5e-3)
+    g = gains(r["paths"].n, F)
+    ex = to_numpy(r["export"])
+    on = ex["rx"] == 1
+    paths = {k: v[on] for k, v in ex.items()}
+    Ho = oracle.synth_H(paths, g[on].astype(np.complex128), f, sc["tx"], sc["rx"][1], te, re, rx_index=1)
+    aperture = np.linalg.norm(te - sc["tx"], axis=1).max() + np.linalg.norm(re - sc["rx"][1], axis=1).max()
+    phase = 3 * 2 * np.pi * aperture * f.max() / 299792458.0 * 2.0 ** -24
+    scale = np.abs(g[on]).sum(0).max()
+    for precision, split in ((sbr.SYNTH_FP16X3, 2.0 ** -20), (sbr.SYNTH_BF16X3, 2.0 ** -14)):
+        H = sbr.synthesize_H(r["paths"], torch.as_tensor(g, device="cuda"), dev(f), dev(te), dev(re), 1, precision).cpu().numpy()
+        assert np.abs(H - Ho).max() < (phase + 4e-6 + split) * scale, (precision, np.abs(H - Ho).max() / scale)
