@@ -187,13 +187,20 @@ struct EntryDf {
         const df cd = df_from_double(c);
         v = cdf2_make(df_add(df{one, 0.f}, df_mul_f(cd, w.x)), df_mul_f(cd, w.y));
     }
-    __device__ __forceinline__ double real() const { return (double)v.h.x + (double)v.l.x; }
-    struct Inv { df v; };
-    __device__ __forceinline__ Inv inverse() const { return Inv{df_rcp(df{v.h.x, v.l.x})}; }
-    __device__ __forceinline__ Row row(const Inv& inv) const {
-        const df r = df_mul(df{v.h.x, v.l.x}, inv.v), m = df_mul(df{v.h.y, v.l.y}, inv.v);
-        return Row{cdf2_make(df_neg(r), df_neg(m)), cdf2_make(df_neg(m), r)};
+    // a pivot as kept in shared memory, and its value
+    __device__ __forceinline__ double raw() const { return __hiloint2double(__float_as_int(v.h.x), __float_as_int(v.l.x)); }
+    static __device__ __forceinline__ double value(double raw) {
+        return (double)__int_as_float(__double2hiint(raw)) + (double)__int_as_float(__double2loint(raw));
     }
+    struct Inv { df v; };
+    __device__ __forceinline__ Inv inverse(unsigned mask, int lane) const {   // that of the given lane's entry
+        const df r = df_rcp(df{v.h.x, v.l.x});
+        return Inv{df{__shfl_sync(mask, r.hi, lane), __shfl_sync(mask, r.lo, lane)}};
+    }
+    __device__ __forceinline__ EntryDf scaled(const Inv& inv) const {   // minus the entry over the pivot
+        return EntryDf{cdf2_make(df_neg(df_mul(df{v.h.x, v.l.x}, inv.v)), df_neg(df_mul(df{v.h.y, v.l.y}, inv.v)))};
+    }
+    __device__ __forceinline__ Row row() const { return Row{v, cdf2{make_float2(v.h.y, -v.h.x), make_float2(v.l.y, -v.l.x)}}; }
     __device__ __forceinline__ void update(const Row& u, const EntryDf& k) { cdf2_mac(v, u.u, u.ju, k.v); }
 };
 
@@ -202,9 +209,11 @@ struct EntryF64 {
     struct Row { double re, im; };
     struct Inv { double v; };
     __device__ __forceinline__ void set(double c, float2 w, float one) { re = one + c * w.x; im = c * w.y; }
-    __device__ __forceinline__ double real() const { return re; }
-    __device__ __forceinline__ Inv inverse() const { return Inv{1.0 / re}; }
-    __device__ __forceinline__ Row row(const Inv& inv) const { return Row{re * inv.v, im * inv.v}; }
+    __device__ __forceinline__ double raw() const { return re; }
+    static __device__ __forceinline__ double value(double raw) { return raw; }
+    __device__ __forceinline__ Inv inverse(unsigned mask, int lane) const { return Inv{__shfl_sync(mask, 1.0 / re, lane)}; }
+    __device__ __forceinline__ EntryF64 scaled(const Inv& inv) const { return EntryF64{re * inv.v, im * inv.v}; }
+    __device__ __forceinline__ Row row() const { return Row{re, im}; }
     __device__ __forceinline__ void update(const Row& u, const EntryF64& k) {
         re -= u.re * k.re + u.im * k.im;
         im -= u.im * k.re - u.re * k.im;
@@ -214,35 +223,42 @@ static_assert(sizeof(EntryDf) == 16 && sizeof(EntryF64) == 16, "one shared-memor
 
 __host__ __device__ constexpr int cap_blk(int a, int b) { return a * (a + 1) / 2 + b; }   // block (a, b), a >= b
 
+// column `16 b + (tk = c)` of the block, as its 16 owners (a half warp) publish it for
+// the step that eliminates it: the entries, minus the entries over the pivot, the pivot
+template <int NB, int b, class E>
+__device__ __forceinline__ void ldl_publish(const E (&A)[cap_blk(NB, 0)], int c, E* col, E* row, double* piv) {
+    const int ti = threadIdx.x & 15, half = threadIdx.x & 16;
+    const typename E::Inv inv = A[cap_blk(b, b)].inverse(0xffffu << half, half | c);
+#pragma unroll
+    for (int a = b; a < NB; ++a) {
+        col[ti + 16 * a] = A[cap_blk(a, b)];
+        row[ti + 16 * a] = A[cap_blk(a, b)].scaled(inv);
+    }
+    if (ti == c) piv[16 * b + c] = A[cap_blk(b, b)].raw();
+}
+
 // the columns of block jb (16 jb ...), then those of the blocks after it
 template <int NB, int jb, class E>
 __device__ __forceinline__ void ldl_block(int n, E (&A)[cap_blk(NB, 0)], E* s_col, double* piv) {
     constexpr int N = 16 * NB;
-    const int ti = threadIdx.x >> 4, tk = threadIdx.x & 15;
+    const int ti = threadIdx.x & 15, tk = threadIdx.x >> 4;
     for (int jj = 0; jj < 16 && 16 * jb + jj < n; ++jj) {
         const int j = 16 * jb + jj;
-        const E* col = s_col + (j & 1) * N;
-        E* next = s_col + ((j + 1) & 1) * N;
-        const E d = col[j];
-        if (threadIdx.x == 0) piv[j] = d.real();
-        const typename E::Inv inv = d.inverse();
+        const E *col = s_col + (j & 1) * 2 * N, *row = col + N;
+        E* next = s_col + ((j + 1) & 1) * 2 * N;
         typename E::Row u[NB];
 #pragma unroll
-        for (int a = jb; a < NB; ++a) u[a] = col[ti + 16 * a].row(inv);
+        for (int a = jb; a < NB; ++a) u[a] = row[ti + 16 * a].row();
 #pragma unroll
         for (int b = jb; b < NB; ++b) {
+            if (b == jb && (tk | 1) <= jj) continue;   // both columns of this warp are done
             const E k = col[tk + 16 * b];
 #pragma unroll
             for (int a = b; a < NB; ++a) A[cap_blk(a, b)].update(u[a], k);
         }
         if (tk == ((jj + 1) & 15)) {
-            if (jj < 15) {
-#pragma unroll
-                for (int a = jb; a < NB; ++a) next[ti + 16 * a] = A[cap_blk(a, jb)];
-            } else if constexpr (jb + 1 < NB) {
-#pragma unroll
-                for (int a = jb + 1; a < NB; ++a) next[ti + 16 * a] = A[cap_blk(a, jb + 1)];
-            }
+            if (jj < 15) ldl_publish<NB, jb>(A, tk, next, next + N, piv);
+            else if constexpr (jb + 1 < NB) ldl_publish<NB, jb + 1>(A, tk, next, next + N, piv);
         }
         __syncthreads();
     }
@@ -251,13 +267,13 @@ __device__ __forceinline__ void ldl_block(int n, E (&A)[cap_blk(NB, 0)], E* s_co
 
 // Pivots of the L D L^H factorisation of I + c ws W into piv[0 .. n). Thread
 // (ti, tk) of 16 x 16 holds entries (ti + 16 a, tk + 16 b), a >= b, in
-// registers; per column one barrier, after which every thread reads the column
-// and updates its entries (those left of the column or above the diagonal are
-// updated too: nothing reads them).
+// registers; per column one barrier, after which every thread reads the column and
+// its scaled form and updates its entries (those above the diagonal and, in a block
+// off the column's, left of it are updated too: nothing reads them).
 template <int NB, class E>
 __device__ __forceinline__ void ldl_pivots(int n, double c, const float2* s_w, float ws, E* s_col, double* piv) {
     constexpr int N = 16 * NB;
-    const int ti = threadIdx.x >> 4, tk = threadIdx.x & 15;
+    const int ti = threadIdx.x & 15, tk = threadIdx.x >> 4;
     E A[cap_blk(NB, 0)];
 #pragma unroll
     for (int a = 0; a < NB; ++a)
@@ -266,9 +282,7 @@ __device__ __forceinline__ void ldl_pivots(int n, double c, const float2* s_w, f
             const float2 w = s_w[cap_blk(a, b) * kCapThreads + threadIdx.x];
             A[cap_blk(a, b)].set(c, make_float2(w.x * ws, w.y * ws), a == b && ti == tk ? 1.f : 0.f);
         }
-    if (tk == 0)
-#pragma unroll
-        for (int a = 0; a < NB; ++a) s_col[ti + 16 * a] = A[cap_blk(a, 0)];
+    if (tk == 0) ldl_publish<NB, 0>(A, 0, s_col, s_col + N, piv);
     __syncthreads();
     ldl_block<NB, 0>(n, A, s_col, piv);
 }
@@ -289,14 +303,19 @@ __device__ __forceinline__ void ldl_pivots(int n, double c, const float2* s_w, f
 // the smallest pivot (>= 1), far inside what the FP32 entries of W carry. Above
 // (SNRs beyond about 45 dB) it runs in FP64.
 // H [1024, 64, 256], seven SNRs, the whole call: 15.4 ms with an FP64 Cholesky
-// in shared memory (three barriers per column), 1.87 ms so; the packed
-// instructions alone take 1.1 ms.
+// in shared memory (three barriers per column); 1.84 ms with a thread's columns
+// across its warp, a reciprocal of the pivot and scaled entries in every thread and
+// two blocks an SM; 1.53 with a warp owning two columns, so that it skips the ones
+// that are done, and three blocks; 1.35 with the reciprocal by the pivot's owner;
+// 1.31 with the scaled column by its owners; 1.29 with four blocks (64 registers).
+// The packed instructions left (15 block updates of 64 columns in place of 20) take
+// 0.85 ms.
 constexpr int kCapRun = 32;
 
 template <int NB>
 struct CapShared {
     float2 h[kCapRun][16 * NB + 1];
-    float4 col[2 * 16 * NB];
+    float4 col[4 * 16 * NB];
     float2 w[cap_blk(NB, 0) * kCapThreads];
     double piv[16 * NB];
     double scale;
@@ -307,7 +326,7 @@ struct CapShared {
 template <int NB, bool kWide>
 __device__ __forceinline__ void gram(const float2* __restrict__ h, int Nt, int n, int len, CapShared<NB>& sh) {
     constexpr int N = 16 * NB, kBlk = cap_blk(NB, 0), kLoad = kCapRun * N / kCapThreads;
-    const int tid = threadIdx.x, ti = tid >> 4, tk = tid & 15;
+    const int tid = threadIdx.x, ti = tid & 15, tk = tid >> 4;
     // entry e of a run is (p, row), consecutive threads along the rows of H
     float2 v[kLoad];
     auto load = [&](int p0) {
@@ -361,13 +380,13 @@ __device__ __forceinline__ void gram(const float2* __restrict__ h, int Nt, int n
 }
 
 template <int NB>
-__global__ void __launch_bounds__(kCapThreads, 2)
+__global__ void __launch_bounds__(kCapThreads, 4)
 k_capacity(const float2* __restrict__ H, int32_t Nr, int32_t Nt, const __grid_constant__ SnrList snr, int32_t n_snr,
            const double* __restrict__ part, int32_t n_part, double* __restrict__ ld) {
     ::sbr::pdl_wait();
     extern __shared__ __align__(16) unsigned char smem[];
     CapShared<NB>& sh = *reinterpret_cast<CapShared<NB>*>(smem);
-    const int tid = threadIdx.x, ti = tid >> 4, tk = tid & 15;
+    const int tid = threadIdx.x, ti = tid & 15, tk = tid >> 4;
     const int n = min(Nr, Nt);
     const float2* h = H + (int64_t)blockIdx.x * Nr * Nt;
     if (tid < 32) {   // Qbar = mean over f of ||H_f||^2, from the partial sums of all of H
@@ -397,17 +416,16 @@ k_capacity(const float2* __restrict__ H, int32_t Nr, int32_t Nt, const __grid_co
 #pragma unroll
             for (int a = 0; a < NB; ++a)
                 large |= ti + 16 * a < n && !(1.0 + c * (sh.w[cap_blk(a, a) * kCapThreads + tid].x * ws) <= 65536.0);
-        if (__syncthreads_or(large))
-            ldl_pivots<NB>(n, c, sh.w, ws, reinterpret_cast<EntryF64*>(sh.col), sh.piv);
-        else
-            ldl_pivots<NB>(n, c, sh.w, ws, reinterpret_cast<EntryDf*>(sh.col), sh.piv);
-        // thread 0 alone writes piv, and its warp alone reads it
+        const bool wide = __syncthreads_or(large) != 0;
+        if (wide) ldl_pivots<NB>(n, c, sh.w, ws, reinterpret_cast<EntryF64*>(sh.col), sh.piv);
+        else ldl_pivots<NB>(n, c, sh.w, ws, reinterpret_cast<EntryDf*>(sh.col), sh.piv);
+        // the first warp reads the pivots; the next SNR's are written after a barrier
+        // (the first of them by thread 0, of this warp)
         if (tid < 32) {
-            __syncwarp();
             double s = 0.0;
             bool bad = false;
             for (int j = tid; j < n; j += 32) {
-                const double d = sh.piv[j];
+                const double d = wide ? sh.piv[j] : EntryDf::value(sh.piv[j]);
                 bad |= !(d > 0.0);
                 s += log(d);
             }
@@ -481,7 +499,7 @@ __device__ __forceinline__ float ratio_db(double a, double b) {
 // (nine operations per path and frequency). 4096 receivers x 25 paths x 8
 // frequencies: 1436 us with a warp per (receiver, frequency) and butterflies
 // over 35 FP64 sums; with the gains of the same paths (2517 us more) the two
-// take 100 us now.
+// take 103 us now.
 constexpr int kTgtWarps = 4;
 
 __global__ void __launch_bounds__(32 * kTgtWarps)
