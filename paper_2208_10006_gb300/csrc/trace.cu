@@ -447,6 +447,20 @@ __device__ __forceinline__ bool rx_accept(const df3& o, const df3& d, df L, df t
     return true;
 }
 
+// FP32 form of the same test with the margins of the receiver walk's (relative 1e-4
+// of the radius, 1e-5 of the coordinates): false only where rx_accept is false. Most
+// segments of a batched job pass far from its one receiver and cost a fifth so.
+__device__ __forceinline__ bool rx_near(float3 o, float3 d, float L, float t_hit, bool hit, float4 R, float alpha) {
+    const float vx = R.x - o.x, vy = R.y - o.y, vz = R.z - o.z;
+    const float ts = fmaf(vx, d.x, fmaf(vy, d.y, vz * d.z));
+    const float slack = 1e-5f * (fabsf(o.x) + fabsf(o.y) + fabsf(o.z) + fabsf(R.x) + fabsf(R.y) + fabsf(R.z) + L + fabsf(ts));
+    if (ts < -slack || (hit && ts > t_hit + slack)) return false;
+    const float wx = fmaf(-ts, d.x, vx), wy = fmaf(-ts, d.y, vy), wz = fmaf(-ts, d.z, vz);
+    const float rad = alpha * (L + fmaxf(ts, 0.f)) * 0.57735027f * (1.f + 1e-4f) + slack;
+    return !(wx * wx + wy * wy + wz * wz > rad * rad);
+}
+__device__ __forceinline__ df3 job_rx(float4 h, float4 l) { return df3{df_make(h.x, l.x), df_make(h.y, l.y), df_make(h.z, l.z)}; }
+
 // Receivers near the segment come from a BVH over the receiver points whose
 // boxes are grown by the largest sphere radius on the segment (FP32,
 // conservative); each is then tested exactly in double-float:
@@ -944,9 +958,15 @@ __global__ void __launch_bounds__(kTraceThreads) k_trace_batch(const __grid_cons
 // eight 128-thread blocks per SM (64 registers), as the single-job depth-first
 // kernel: the walks are latency-bound and gain more from resident warps than
 // they lose to spills (4096-job batch: 2.07 s at 96 registers and 4 blocks,
-// 1.64 s here)
+// 1.64 s here). The FP32 reception test ahead of the exact one, the job's pointers
+// read again after the walk and the rays per bounce counted per block took a batch
+// of 24 jobs from 7.69 to 7.44 ms.
 __global__ void __launch_bounds__(kTraceThreads, 8) k_trace_batch_df(const __grid_constant__ BatchTraceArgs a) {
     int stack[kStack];
+    // rays entering each bounce, counted per block and added up once at the end
+    __shared__ unsigned s_queue[kKmax + 2];
+    if (threadIdx.x < kKmax + 2) s_queue[threadIdx.x] = 0u;
+    __syncthreads();
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned long long n_in = (unsigned long long)a.R_total;
@@ -993,12 +1013,15 @@ __global__ void __launch_bounds__(kTraceThreads, 8) k_trace_batch_df(const __gri
             df t = df_make(INFINITY, 0.f), nd = df_make(0.f, 0.f);
             Trav tv;
             int32_t j = traverse32<false>(sc, r, prev, tv, stack, nullptr, nullptr);
-            j = settle_hit(sc, o, d, prev, tv, j, stack, t, nd);
+            // the job's pointers are read again after the walk rather than kept through it
+            J = a.jobs + job;
+            asm volatile("" : "+l"(J));
+            j = settle_hit(JobScene{J->nodes, J->tris, J->plane, a.cnt, J->rot_stride}, o, d, prev, tv, j, stack, t, nd);
             {
-                const float4 rh = J->rx_h, rl = J->rx_l, al = J->alpha;
-                const df3 Rx{df_make(rh.x, rl.x), df_make(rh.y, rl.y), df_make(rh.z, rl.z)};
+                const float4 rh = J->rx_h, al = J->alpha;
                 float dist;
-                if (rx_accept(o, d, L, t, j >= 0, Rx, df_make(al.z, al.w), dist)) {
+                if (rx_near(df3_hi(o), df3_hi(d), L.hi, t.hi, j >= 0, rh, al.x) &&
+                    rx_accept(o, d, L, t, j >= 0, job_rx(rh, J->rx_l), df_make(al.z, al.w), dist)) {
                     uint32_t key[kKeyWords];
                     key[0] = (uint32_t)job;
                     key[1] = (uint32_t)bounce;
@@ -1027,9 +1050,11 @@ __global__ void __launch_bounds__(kTraceThreads, 8) k_trace_batch_df(const __gri
             }
         }
         const unsigned grp = __match_any_sync(FULL, entered);
-        if (entered >= 0 && lane == __ffs(grp) - 1)
-            atomicAdd(&a.cnt->queue[entered], (unsigned long long)__popc(grp));
+        if (entered >= 0 && lane == __ffs(grp) - 1) atomicAdd(&s_queue[entered], (unsigned)__popc(grp));
     }
+    __syncthreads();   // every warp of the block leaves the loop above (no early return)
+    if (threadIdx.x < kKmax + 2 && s_queue[threadIdx.x])
+        atomicAdd(&a.cnt->queue[threadIdx.x], (unsigned long long)s_queue[threadIdx.x]);
 }
 
 // Set-up of one trace in one launch: zeroed counters with queue[0] = R, an
