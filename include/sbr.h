@@ -54,7 +54,7 @@ typedef enum {
 #define SBR_POL_H 1         /* phi-hat polarisation at both ends                 */
 
 /* precision of sbr_synthesize_H */
-#define SBR_SYNTH_FP64 0    /* FP64 CUDA-core summation                          */
+#define SBR_SYNTH_FP64 0    /* CUDA cores, double-float sum (48 bits)             */
 #define SBR_SYNTH_FP32 1    /* FP32 CUDA-core summation, FP64 delay phase        */
 #define SBR_SYNTH_BF16X3 2  /* tcgen05 BF16 hi/lo split (3 products), FP32 TMEM  */
 #define SBR_SYNTH_FP16X3 3  /* tcgen05 FP16 hi/lo split (3 products), weights scaled
