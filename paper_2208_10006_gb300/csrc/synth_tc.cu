@@ -28,6 +28,7 @@
 // Every wait on an mbarrier is bounded; on expiry the CTA records
 // ST_TIMEOUT, releases its tensor memory and returns.
 #include <algorithm>
+#include <type_traits>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -275,7 +276,9 @@ __device__ __forceinline__ void tc_epilogue(const TcEpi& e, uint32_t tmem, int w
     const int lg = warp & 3, b0 = warp >> 2;
     const int qa = lane >> 2, pc = 2 * (lane & 3);
     const uint32_t tacc = tmem + (uint32_t)(e.acc * kTileN) + ((uint32_t)(32 * lg) << 16);
-    const int nt16 = (e.Nt + 15) / 16, nr8 = (e.Nr + 7) / 8;
+    using Off = typename std::conditional<kFull, int, int64_t>::type;   // a full tile's offsets fit 32 bits
+    const Off nt16 = ((Off)e.Nt + 15) / 16;
+    const int nr8 = (int)(((int64_t)e.Nr + 7) / 8);
     // LoS delays of a block (dl_index): two 16-byte loads, column pairs 0, 8 and 16, 24
     const float4* dl0 = reinterpret_cast<const float4*>(e.dlos) + ((int64_t)(e.q0 / 8 + 2 * lg) * nt16 + e.p0 / 16) * 32 + lane;
     auto load_dl = [&](int b, float4 (&dl)[2]) {
@@ -305,7 +308,7 @@ __device__ __forceinline__ void tc_epilogue(const TcEpi& e, uint32_t tmem, int w
             for (int k = 0; k < 16; ++k) v[k] = 0u;
         }
         const int q = e.q0 + 16 * lg + 8 * h + qa, p0 = e.p0 + 32 * jj + pc;
-        float2* row = out + (8 * h * e.Nt + 32 * jj);
+        float2* row = out + ((Off)(8 * h) * e.Nt + 32 * jj);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const float4 d4 = dl[k / 2];
@@ -334,8 +337,9 @@ __device__ __forceinline__ void tc_epilogue(const TcEpi& e, uint32_t tmem, int w
 // warps first generating, then writing out, a block barrier per K-chunk between,
 // 42% of the issue slots were used. H [1024, 64, 256] from 45 reflected paths and the
 // LoS path, whole call: 68.5 us then, 59 with the roles side by side, 55 with packed
-// phasors and the operand prologue in double-float, 48 with the LoS delays in the
-// epilogue's order and an epilogue per kind of tile. It is the epilogue that bounds
+// phasors and the operand prologue in double-float, 50 with the LoS delays in the
+// epilogue's order and an epilogue per kind of tile (48 before edge tiles had 64-bit
+// offsets, for rows of 2^28 elements and more). It is the epilogue that bounds
 // it (32 us without; 47 without the B' phasors; 42 without the stores): 16 + 8 warps
 // are the split that leaves it 72 registers (8 + 16: 63 us, 16 + 12 with 64: 50).
 template <bool kF16, bool kBatch, int kTileN>
