@@ -108,9 +108,13 @@ sbr_status delays_run(const DelayArgs& a, cudaStream_t s) {
     const int64_t y = (a.P + kDelayPaths - 1) / kDelayPaths + (a.R0 ? (a.Nr + kDelayPaths - 1) / kDelayPaths : 0);
     if (y == 0) return SBR_OK;
     // path groups in slices of at most 65535 (P up to 2^31)
+    if (a.R0 && a.Nr > 65535) {
+        set_error("synthesis: more than 65535 receive elements");
+        return SBR_ERR_CUDA;
+    }
     if (y > 65535) {
         DelayArgs part = a;
-        const int64_t step = 32768 * (int64_t)kDelayPaths;
+        const int64_t step = 16384 * (int64_t)kDelayPaths;   // with 32768 groups of receive elements at most
         const double* r0 = a.R0;
         for (int64_t n = 0; n < a.P; n += step) {
             part.P = std::min(step, a.P - n);
@@ -269,6 +273,7 @@ struct SynthArgs {
     const double* L;
     const float2 *dt, *dr, *dlos;
     float2* H;
+    int32_t p_base;   // first transmit element of this launch
 };
 
 template <class M, int RQ, int G>
@@ -282,7 +287,7 @@ __global__ void __launch_bounds__(kSynthThreads* G) k_synth(const __grid_constan
     C* s_a = s_mem;                    // [NCG][QT]
     C* s_v = s_mem + NCG * QT;         // [NCG][kSynthPT]
     const int tid = threadIdx.x, tp = tid & 15, tq = (tid >> 4) & 7, grp = tid / kSynthThreads;
-    const int32_t f = blockIdx.x, p0 = blockIdx.y * kSynthPT, q0 = blockIdx.z * QT;
+    const int32_t f = blockIdx.x, p0 = a.p_base + blockIdx.y * kSynthPT, q0 = blockIdx.z * QT;
     const double fr = a.freqs[f];
     const typename M::Freq fq = M::freq(fr);
     const int los = a.Pr > 0 && *a.nb0 == 0 ? 1 : 0;
@@ -371,19 +376,23 @@ __global__ void __launch_bounds__(kSynthThreads* G) k_synth(const __grid_constan
 }
 
 template <class M, int RQ>
-sbr_status synth_launch(const SynthArgs& a, cudaStream_t s) {
-    const dim3 grid((unsigned)a.F, (unsigned)((a.Nt + kSynthPT - 1) / kSynthPT), (unsigned)((a.Nr + 8 * RQ - 1) / (8 * RQ)));
-    // groups: 32 warps per SM are wanted, a block of one group has four
-    const int64_t want = 8 * (int64_t)sm_count() / ((int64_t)grid.x * grid.y * grid.z);
-    ::sbr::note_launch();
-    if constexpr (RQ <= 2) {   // (48 KB of shared memory)
-        if (want >= 4) {
-            SBR_TRY_CUDA(::sbr::launch_pdl(k_synth<M, RQ, 4>, grid, dim3(4 * kSynthThreads), 0, s, a));
-            return SBR_OK;
+sbr_status synth_launch(SynthArgs a, cudaStream_t s) {
+    const int64_t cols = ((int64_t)a.Nt + kSynthPT - 1) / kSynthPT;
+    for (int64_t c = 0; c < cols; c += 65535) {   // (a grid's y dimension)
+        a.p_base = (int32_t)(c * kSynthPT);
+        const dim3 grid((unsigned)a.F, (unsigned)std::min<int64_t>(65535, cols - c), (unsigned)((a.Nr + 8 * RQ - 1) / (8 * RQ)));
+        // groups: 32 warps per SM are wanted, a block of one group has four
+        const int64_t want = 8 * (int64_t)sm_count() / ((int64_t)grid.x * grid.y * grid.z);
+        ::sbr::note_launch();
+        if constexpr (RQ <= 2) {   // (48 KB of shared memory)
+            if (want >= 4) {
+                SBR_TRY_CUDA(::sbr::launch_pdl(k_synth<M, RQ, 4>, grid, dim3(4 * kSynthThreads), 0, s, a));
+                continue;
+            }
         }
+        if (want >= 2) SBR_TRY_CUDA(::sbr::launch_pdl(k_synth<M, RQ, 2>, grid, dim3(2 * kSynthThreads), 0, s, a));
+        else SBR_TRY_CUDA(::sbr::launch_pdl(k_synth<M, RQ, 1>, grid, dim3(kSynthThreads), 0, s, a));
     }
-    if (want >= 2) SBR_TRY_CUDA(::sbr::launch_pdl(k_synth<M, RQ, 2>, grid, dim3(2 * kSynthThreads), 0, s, a));
-    else SBR_TRY_CUDA(::sbr::launch_pdl(k_synth<M, RQ, 1>, grid, dim3(kSynthThreads), 0, s, a));
     return SBR_OK;
 }
 
@@ -413,6 +422,7 @@ struct ElArgs {
     const double* L;
     const float2* dt;         // [P][Nt]
     float2* H;
+    int32_t p_base;   // first transmit element of this launch
 };
 
 __global__ void __launch_bounds__(kElMax) k_synth_el32(const __grid_constant__ ElArgs a) {
@@ -423,7 +433,7 @@ __global__ void __launch_bounds__(kElMax) k_synth_el32(const __grid_constant__ E
     __shared__ df s_mid;
     const int tid = threadIdx.x;
     const int32_t f0 = blockIdx.x * kElF, q = blockIdx.y;
-    const int32_t p0 = blockIdx.z * 2 * blockDim.x + tid, p1 = p0 + blockDim.x;   // the two elements
+    const int32_t p0 = a.p_base + blockIdx.z * 2 * blockDim.x + tid, p1 = p0 + blockDim.x;   // the two elements
     const int nf = min(kElF, a.F - f0);
     const bool act = p0 < a.Nt, two = p1 < a.Nt;
     if (tid < 32) {   // one warp, at least: the block's frequencies
@@ -535,7 +545,7 @@ __global__ void __launch_bounds__(kElMax) k_synth_el32(const __grid_constant__ E
 __global__ void __launch_bounds__(kSynthThreads) k_synth_el_df(const __grid_constant__ ElArgs a) {
     ::sbr::pdl_wait();
     __shared__ cdf2 s_w[kSynthThreads];
-    const int32_t f = blockIdx.x, q = blockIdx.y, p = blockIdx.z * kSynthThreads + threadIdx.x;
+    const int32_t f = blockIdx.x, q = blockIdx.y, p = a.p_base + blockIdx.z * kSynthThreads + threadIdx.x;
     const double fr = a.freqs[f];
     const FormDf::Freq fq = FormDf::freq(fr);
     const int32_t a0 = a.rx_off[q], a1 = a.rx_off[q + 1];
@@ -569,16 +579,20 @@ sbr_status synth_elements_run(const sbr_path_list* pl, const float2* g, const do
     SBR_TRY(dalloc_n(&d.dt, (size_t)pl->P * Nt, s));
     sbr_status st = delays_run(d, s);
     if (st == SBR_OK) {
-        const ElArgs a{F, pl->n_rx, Nt, pl->rx_off, freqs, g, pl->L, d.dt, H};
+        ElArgs a{F, pl->n_rx, Nt, pl->rx_off, freqs, g, pl->L, d.dt, H, 0};
         // FP32: two elements per thread, blocks as wide as the array up to kElMax threads
         const int width = fp64 ? kSynthThreads : std::min(kElMax, ((Nt + 1) / 2 + 31) / 32 * 32), per = fp64 ? width : 2 * width;
-        const dim3 grid((unsigned)(fp64 ? F : (F + kElF - 1) / kElF), (unsigned)pl->n_rx, (unsigned)((Nt + per - 1) / per));
-        ::sbr::note_launch();
-        const cudaError_t e = fp64 ? ::sbr::launch_pdl(k_synth_el_df, grid, dim3(width), 0, s, a)
-                                   : ::sbr::launch_pdl(k_synth_el32, grid, dim3(width), 0, s, a);
-        if (e != cudaSuccess) {
-            set_error("per-element synthesis: %s", cudaGetErrorString(e));
-            st = SBR_ERR_CUDA;
+        const int64_t cols = ((int64_t)Nt + per - 1) / per;
+        for (int64_t c = 0; c < cols && st == SBR_OK; c += 65535) {   // (a grid's z dimension)
+            a.p_base = (int32_t)(c * per);
+            const dim3 grid((unsigned)(fp64 ? F : (F + kElF - 1) / kElF), (unsigned)pl->n_rx, (unsigned)std::min<int64_t>(65535, cols - c));
+            ::sbr::note_launch();
+            const cudaError_t e = fp64 ? ::sbr::launch_pdl(k_synth_el_df, grid, dim3(width), 0, s, a)
+                                       : ::sbr::launch_pdl(k_synth_el32, grid, dim3(width), 0, s, a);
+            if (e != cudaSuccess) {
+                set_error("per-element synthesis: %s", cudaGetErrorString(e));
+                st = SBR_ERR_CUDA;
+            }
         }
     }
     dfree(d.dt, s);
@@ -608,7 +622,7 @@ sbr_status synth_simt_run(const sbr_path_list* pl, const float2* g, const double
     if (st == SBR_OK) {
         // the LoS path (no reflection) sorts first among a receiver's paths; the
         // kernel reads its reflection count on the device
-        const SynthArgs a{F, Nr, Nt, Pr, d.nb, freqs, g + (int64_t)o0 * F, pl->L + o0, d.dt, d.dr, d.dlos, H};
+        const SynthArgs a{F, Nr, Nt, Pr, d.nb, freqs, g + (int64_t)o0 * F, pl->L + o0, d.dt, d.dr, d.dlos, H, 0};
         if (fp64)
             st = Nr <= 8 ? synth_launch<FormDf, 1>(a, s) : (Nr <= 16 ? synth_launch<FormDf, 2>(a, s) : synth_launch<FormDf, 4>(a, s));
         else

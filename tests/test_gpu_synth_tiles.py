@@ -107,3 +107,26 @@ def test_tensor_core_tiles(sbr, K, Nr, Nt, F):
     for precision, split in ((sbr.SYNTH_FP16X3, 2.0 ** -20), (sbr.SYNTH_BF16X3, 2.0 ** -14)):
         H = sbr.synthesize_H(r["paths"], torch.as_tensor(g, device="cuda"), dev(f), dev(te), dev(re), 1, precision).cpu().numpy()
         assert np.abs(H - Ho).max() < (phase + 4e-6 + split) * scale, (precision, np.abs(H - Ho).max() / scale)
+
+
+@pytest.mark.parametrize("form,Nt", [("reference", 65535 * 64 + 100), ("elements", 65535 * 256 + 100)])
+def test_more_columns_than_one_grid(sbr, form, Nt):
+    """Arrays past the 65,535 column blocks of one launch: the last elements and those
+    around the seam against a call with these alone (the same terms, summed in another
+    order of path groups: 1e-6 of max |H|)."""
+    sc = scenes.shoebox(N=40, K=1, n_rx=1)
+    r = sbr.run_scene(sc)
+    n = r["paths"].n
+    assert 1 <= n <= 7
+    f = grid(1, "even")
+    g = torch.as_tensor(gains(n, 1), device="cuda")
+    te = torch.zeros((Nt, 3), dtype=torch.float64, device="cuda") + torch.as_tensor(np.asarray(sc["tx"], np.float64), device="cuda")
+    te[:, 1] += torch.linspace(-0.2, 0.2, Nt, dtype=torch.float64, device="cuda")
+    seam = Nt - 100
+    pick = torch.cat([torch.arange(0, 64), torch.arange(seam - 64, Nt)]).cuda()
+    if form == "reference":
+        call = lambda t: sbr.synthesize_H(r["paths"], g, dev(f), t, dev(np.asarray(sc["rx"])[:1]), 0, sbr.SYNTH_FP32)
+    else:
+        call = lambda t: sbr.synthesize_H_elements(r["paths"], g, dev(f), t, sbr.SYNTH_FP32)
+    big, small = call(te.contiguous()), call(te[pick].contiguous())
+    assert (big[..., pick] - small).abs().max() <= 1e-6 * small.abs().max() and small.abs().max() > 0
