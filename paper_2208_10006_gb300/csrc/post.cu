@@ -364,8 +364,13 @@ __device__ __forceinline__ void gram(const float2* __restrict__ h, int Nt, int n
             for (int a = 0; a < NB; ++a)
 #pragma unroll
                 for (int b = 0; b <= a; ++b) {
-                    sr[cap_blk(a, b)] += x[a].x * y[b].x + x[a].y * y[b].y;
-                    si[cap_blk(a, b)] += kWide ? x[a].y * y[b].x - x[a].x * y[b].y : x[a].x * y[b].y - x[a].y * y[b].x;
+                    // one fused operation a term, then the sum: with every rounding written out,
+                    // since a compiler free to choose the product that is fused chose another
+                    // in one of the eight forms (C in the ninth digit of a few antennas)
+                    float &r = sr[cap_blk(a, b)], &i = si[cap_blk(a, b)];
+                    r = __fadd_rn(r, __fmaf_rn(x[a].x, y[b].x, __fmul_rn(x[a].y, y[b].y)));
+                    i = __fadd_rn(i, kWide ? __fmaf_rn(x[a].y, y[b].x, -__fmul_rn(x[a].x, y[b].y))
+                                           : __fmaf_rn(x[a].x, y[b].y, -__fmul_rn(x[a].y, y[b].x)));
                 }
         }
 #pragma unroll
