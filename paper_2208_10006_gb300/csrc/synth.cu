@@ -412,7 +412,10 @@ sbr_status synth_launch(SynthArgs a, cudaStream_t s) {
 // paths per element: 948 us with sincospif per term and an FP64 prologue, 248 us
 // so (258 us with one element per thread and scalar operations, 269 us with every
 // operation packed and the weights doubled in shared memory).
-constexpr int kElF = 16, kElMid = 8, kElPaths = 64, kElMax = 128;
+// A launch of few warps waits for the chain of one element's paths (0.45 us a path):
+// there G groups of 32 threads take a part of the paths each, from the weakest to the
+// strongest, and their sums are added at the end.
+constexpr int kElF = 16, kElMid = 8, kElPaths = 64, kElMax = 128, kElGroups = 8;
 
 struct ElArgs {
     int32_t F, Nq, Nt;
@@ -425,15 +428,18 @@ struct ElArgs {
     int32_t p_base;   // first transmit element of this launch
 };
 
-__global__ void __launch_bounds__(kElMax) k_synth_el32(const __grid_constant__ ElArgs a) {
+// block (elements / 2, G)
+template <int G>
+__global__ void __launch_bounds__(G > 1 ? 32 * G : kElMax) k_synth_el32(const __grid_constant__ ElArgs a) {
     ::sbr::pdl_wait();
     __shared__ __align__(16) float2 s_w[kElPaths][kElF];
+    __shared__ float s_sum[G > 1 ? G / 2 : 1][4 * kElF][G > 1 ? 32 : 1];
     __shared__ df s_f[kElF], s_foc[kElF], s_t[kElPaths];
     __shared__ float s_step, s_dev;
     __shared__ df s_mid;
-    const int tid = threadIdx.x;
+    const int grp = G > 1 ? threadIdx.y : 0, tid = grp * blockDim.x + threadIdx.x, threads = G * blockDim.x;
     const int32_t f0 = blockIdx.x * kElF, q = blockIdx.y;
-    const int32_t p0 = a.p_base + blockIdx.z * 2 * blockDim.x + tid, p1 = p0 + blockDim.x;   // the two elements
+    const int32_t p0 = a.p_base + blockIdx.z * 2 * blockDim.x + threadIdx.x, p1 = p0 + blockDim.x;   // the two elements
     const int nf = min(kElF, a.F - f0);
     const bool act = p0 < a.Nt, two = p1 < a.Nt;
     if (tid < 32) {   // one warp, at least: the block's frequencies
@@ -462,10 +468,10 @@ __global__ void __launch_bounds__(kElMax) k_synth_el32(const __grid_constant__ E
         const int cnt = min(kElPaths, n1 - a0);
         const int32_t n0 = n1 - cnt;
         __syncthreads();
-        for (int n = tid; n < cnt; n += blockDim.x) s_t[n] = df_split(a.L[n0 + n] * kInvC0);
+        for (int n = tid; n < cnt; n += threads) s_t[n] = df_split(a.L[n0 + n] * kInvC0);
         __syncthreads();
 #pragma unroll 4
-        for (int e = tid; e < cnt * kElF; e += blockDim.x) {
+        for (int e = tid; e < cnt * kElF; e += threads) {
             const int n = e / kElF, k = e % kElF;
             s_w[n][k] = k < nf ? cmul32(a.g[(int64_t)(n0 + n) * a.F + f0 + k],
                                         phasor32(df{1.f, 0.f}, make_float2(cycles_mod1(s_f[k], s_t[n]), 0.f)))
@@ -474,11 +480,14 @@ __global__ void __launch_bounds__(kElMax) k_synth_el32(const __grid_constant__ E
         __syncthreads();
         if (!act) continue;
         const float2* dt = a.dt + (int64_t)n0 * a.Nt;
+        // this group's paths [c0, c1) of the chunk
+        const int part = (cnt + G - 1) / G, c0 = grp * part, c1 = min(cnt, c0 + part);
+        if (c0 >= c1) continue;
         // delays two paths ahead
-        auto delay = [&](int n, int32_t p) { return __ldg(dt + (int64_t)max(n, 0) * a.Nt + p); };
+        auto delay = [&](int n, int32_t p) { return __ldg(dt + (int64_t)max(n, c0) * a.Nt + p); };
         const int32_t pb = two ? p1 : p0;
-        float2 da = delay(cnt - 1, p0), db = delay(cnt - 1, pb), ea = delay(cnt - 2, p0), eb = delay(cnt - 2, pb);
-        for (int n = cnt - 1; n >= 0; --n) {
+        float2 da = delay(c1 - 1, p0), db = delay(c1 - 1, pb), ea = delay(c1 - 2, p0), eb = delay(c1 - 2, pb);
+        for (int n = c1 - 1; n >= c0; --n) {
             const float2 d0 = da, d1 = db;
             da = ea, db = eb;
             ea = delay(n - 2, p0), eb = delay(n - 2, pb);
@@ -531,6 +540,28 @@ __global__ void __launch_bounds__(kElMax) k_synth_el32(const __grid_constant__ E
             }
         }
     }
+    if constexpr (G > 1) {   // the sums of the groups, pairwise
+#pragma unroll 1
+        for (int h = G / 2; h >= 1; h /= 2) {
+            __syncthreads();
+            if (grp >= h && grp < 2 * h)
+#pragma unroll
+                for (int k = 0; k < kElF; ++k) {
+                    float(*o)[32] = &s_sum[grp - h][4 * k];
+                    o[0][threadIdx.x] = re[k].x; o[1][threadIdx.x] = re[k].y;
+                    o[2][threadIdx.x] = im[k].x; o[3][threadIdx.x] = im[k].y;
+                }
+            __syncthreads();
+            if (grp < h)
+#pragma unroll
+                for (int k = 0; k < kElF; ++k) {
+                    const float(*o)[32] = &s_sum[grp][4 * k];
+                    re[k].x += o[0][threadIdx.x]; re[k].y += o[1][threadIdx.x];
+                    im[k].x += o[2][threadIdx.x]; im[k].y += o[3][threadIdx.x];
+                }
+        }
+        if (grp > 0) return;
+    }
     if (act)
 #pragma unroll
         for (int k = 0; k < kElF; ++k)
@@ -580,15 +611,24 @@ sbr_status synth_elements_run(const sbr_path_list* pl, const float2* g, const do
     sbr_status st = delays_run(d, s);
     if (st == SBR_OK) {
         ElArgs a{F, pl->n_rx, Nt, pl->rx_off, freqs, g, pl->L, d.dt, H, 0};
-        // FP32: two elements per thread, blocks as wide as the array up to kElMax threads
-        const int width = fp64 ? kSynthThreads : std::min(kElMax, ((Nt + 1) / 2 + 31) / 32 * 32), per = fp64 ? width : 2 * width;
+        // FP32: two elements per thread; blocks as wide as the array up to kElMax threads, or of
+        // 32 in 2, 4 or 8 groups while the launch has fewer than four warps per scheduler.
+        // Whole call, 63 paths per element, warps without groups: 1 to 76 warps 39 us with one
+        // group, 24 with two, 16.5 (the host's time) with four or eight (33 to 41 before the
+        // rotations, a thread per output then); 304: 39.8, 24.7, 18.5, 17.7; 608: 41.1, 29.7,
+        // 26.8, 31.4; 912: 43.7, 37.1, 37.8, 43.8.
+        const int64_t warps = ((int64_t)F + kElF - 1) / kElF * pl->n_rx * (((int64_t)Nt + 63) / 64);
+        int groups = 1;
+        while (!fp64 && groups < kElGroups && warps * groups < 16 * (int64_t)sm_count()) groups *= 2;
+        const int width = fp64 ? kSynthThreads : groups > 1 ? 32 : std::min(kElMax, ((Nt + 1) / 2 + 31) / 32 * 32), per = fp64 ? width : 2 * width;
         const int64_t cols = ((int64_t)Nt + per - 1) / per;
         for (int64_t c = 0; c < cols && st == SBR_OK; c += 65535) {   // (a grid's z dimension)
             a.p_base = (int32_t)(c * per);
             const dim3 grid((unsigned)(fp64 ? F : (F + kElF - 1) / kElF), (unsigned)pl->n_rx, (unsigned)std::min<int64_t>(65535, cols - c));
             ::sbr::note_launch();
+            const auto kern = groups == 1 ? k_synth_el32<1> : groups == 2 ? k_synth_el32<2> : groups == 4 ? k_synth_el32<4> : k_synth_el32<8>;
             const cudaError_t e = fp64 ? ::sbr::launch_pdl(k_synth_el_df, grid, dim3(width), 0, s, a)
-                                       : ::sbr::launch_pdl(k_synth_el32, grid, dim3(width), 0, s, a);
+                                       : ::sbr::launch_pdl(kern, grid, dim3(width, groups), 0, s, a);
             if (e != cudaSuccess) {
                 set_error("per-element synthesis: %s", cudaGetErrorString(e));
                 st = SBR_ERR_CUDA;
