@@ -300,6 +300,7 @@ __device__ __forceinline__ void tc_epilogue(const TcEpi& e, uint32_t tmem, int w
             dl[0] = next[0]; dl[1] = next[1];
             if (b + kBs < kBlocks) load_dl(b + kBs, next);
         }
+        if (!kFull && (e.q0 + 16 * lg + 8 * h >= e.Nr || e.p0 + 32 * jj >= e.Nt)) continue;   // all outside H
         uint32_t v[16];
         if (e.mma) {
             tmem_ld_16x256b<4>(tacc + ((uint32_t)(16 * h) << 16) + (uint32_t)(32 * jj), v);
@@ -342,6 +343,9 @@ __device__ __forceinline__ void tc_epilogue(const TcEpi& e, uint32_t tmem, int w
 // offsets, for rows of 2^28 elements and more). It is the epilogue that bounds
 // it (32 us without; 47 without the B' phasors; 42 without the stores): 16 + 8 warps
 // are the split that leaves it 72 registers (8 + 16: 63 us, 16 + 12 with 64: 50).
+// Small arrays at 1024 frequencies, where a tile is mostly outside H: 1 x 1 from 6
+// reflected paths 39 us with whole tiles generated and written out (29 before the roles), 24
+// with what is outside skipped; 13 x 63 from 128 paths 63 (97), 51.
 template <bool kF16, bool kBatch, int kTileN>
 __global__ void __launch_bounds__(kTcThreads, 1) k_synth_tc(const __grid_constant__ TcArgs a) {
     using Sh = TcShape<kTileN>;
@@ -396,7 +400,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_synth_tc(const __grid_constan
                 const int cnt = min(kChunkP, x.nrefl - nb);
                 const int n16 = 2 * ((cnt + 7) >> 3);   // 16-byte chunks per row (4 paths each), whole MMA K-steps
                 // B' (stored N x K): transmit element p, paths nb + 4 c16 .. + 3
-                // (padded paths have zero weight, so their phasors are harmless);
+                // (padded paths have zero weight, so their phasors are harmless; elements
+                // past Nt or Nr are left as they are: their row of an operand reaches only
+                // their own row or column of the accumulator, which nothing stores);
                 // kGenThreads is a multiple of N, so a thread keeps its element and
                 // steps through the chunks. [Pp / 4][Nt] groups of 4 paths:
                 // consecutive lanes read consecutive 16-byte groups
@@ -426,7 +432,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_synth_tc(const __grid_constan
 #pragma unroll
                 for (int u = 0; u < kUnits; ++u) {
                     const int c16 = tid / kTileN + u * kStep;
-                    if (c16 < n16) {
+                    if (c16 < n16 && p < x.Nt) {
                         uint32_t h[4], l[4];
 #pragma unroll
                         for (int k = 0; k < 4; k += 2) {
@@ -441,7 +447,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_synth_tc(const __grid_constan
                     }
                 }
                 // A' as the two rows r(q) (Re A, -Im A) and i(q) (Im A, Re A)
-                if (qc < n16) {
+                if (qc < n16 && q < x.Nr) {
                     float sn[4], cs[4];
 #pragma unroll
                     for (int k = 0; k < 4; k += 2) {
