@@ -132,8 +132,9 @@ struct SnrList {
 // sum of |h|^2 over this block's share of H, in double-float: an FP64 addition
 // costs some 70 FP32 ones on this GPU, a double-float one about ten, so the
 // pass runs at memory speed (H [1024, 64, 256]: 167 us with FP64 sums, 28 us).
-// A share with an entry that is not finite, above 2^60, or with none above
-// 2^-40 (where an FP32 product could leave the normal range) is summed in FP64.
+// A share with an entry that is not finite, above 2^40 (a thread's sum of 2^47 squares
+// stays in the FP32 range), or with none above 2^-40 (where an FP32 product could leave
+// the normal range) is summed in FP64.
 __global__ void __launch_bounds__(kCapThreads)
 k_frob(const float2* __restrict__ H, int64_t n, double* __restrict__ part) {
     ::sbr::pdl_wait();
@@ -148,7 +149,7 @@ k_frob(const float2* __restrict__ H, int64_t n, double* __restrict__ part) {
         const df t = two_sum(s.hi, p.hi);
         s = fast_two_sum(t.hi, __fadd_rn(s.lo, __fadd_rn(t.lo, p.lo)));
         top = fmaxf(top, fabsf(x));
-        wild |= !(fabsf(x) < 1.1529215e18f);
+        wild |= !(fabsf(x) < 1.0995116e12f);
     };
     // 16-byte loads of two entries where H starts on 16 bytes
     const bool pairs = (reinterpret_cast<uintptr_t>(H) & 15) == 0;
