@@ -410,10 +410,11 @@ k_capacity(const float2* __restrict__ H, int32_t Nr, int32_t Nt, const __grid_co
 #pragma unroll
         for (int a = 0; a < NB; ++a) atomicMax(&sh.top, __float_as_uint(sh.w[cap_blk(a, a) * kCapThreads + tid].x));
     __syncthreads();
-    // W in units of 2^e, its largest entry in [1, 2), so that neither it nor the
-    // factor of an SNR leaves the normal FP32 range whatever the scale of H
+    // W in units of 2^e, its largest entry in [1, 2) (below 1 where it is subnormal), so that
+    // neither it nor the factor of an SNR leaves the normal FP32 range whatever the scale of
+    // H; as it is where it is zero or not finite
     const int e = (int)((sh.top >> 23) & 0xffu) - 127;
-    const float ws = e > -127 && e < 127 ? ldexpf(1.f, -e) : 1.f;
+    const float ws = sh.top && e < 128 ? ldexpf(1.f, -e) : 1.f;
     const double scale = sh.scale;
     for (int si = blockIdx.y; si < n_snr; si += gridDim.y) {
         const double c = snr.lin[si] / Nt * scale / ws;

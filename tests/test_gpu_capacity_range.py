@@ -7,6 +7,8 @@ import numpy as np
 import pytest
 import torch
 
+from test_gpu_capacity_roundings import reference
+
 pytestmark = pytest.mark.gpu
 
 
@@ -23,3 +25,23 @@ def test_many_large_entries():
     C = sbr.capacity(H, [0.0, 20.0]).cpu().numpy()
     Cs = sbr.capacity(H.mul_(2.0 ** 59), [0.0, 20.0]).cpu().numpy()
     assert np.isfinite(Cs).all() and (np.abs(C - Cs) < 1e-12 * C).all(), (C, Cs)
+
+
+def test_gram_at_the_top_of_the_range():
+    # diagonal of W 2^127.8
+    import paper_2208_10006_gb300 as sbr
+    H = signs((3, 8, 16), 2)
+    C = sbr.capacity(H, [0.0, 20.0]).cpu().numpy()
+    Cs = sbr.capacity(H * 2.0 ** 61, [0.0, 20.0]).cpu().numpy()
+    assert (np.abs(C - Cs) < 1e-12 * C).all(), (C, Cs)
+
+
+@pytest.mark.parametrize("n", [1, 8, 20])
+def test_subnormal_gram(n):
+    # entries of W of 2^-140 to 2^-127: against the same FP32 roundings on the host
+    import paper_2208_10006_gb300 as sbr
+    rng = np.random.default_rng(n)
+    H = ((rng.normal(size=(3, n, 24)) + 1j * rng.normal(size=(3, n, 24))) * 2.0 ** -67).astype(np.complex64)
+    C = sbr.capacity(torch.as_tensor(H, device="cuda"), [0.0, 20.0]).cpu().numpy()
+    R = reference(H, [0.0, 20.0])
+    assert (np.abs(C - R) < 1e-12 * R).all(), C / R - 1
