@@ -123,6 +123,8 @@ __device__ __forceinline__ df df_sqrt(df a) {
     const float r = __fadd_rn(__fmaf_rn(-s, s, a.hi), a.lo);
     return fast_two_sum(s, __fmul_rn(__fmul_rn(0.5f, y), r));
 }
+// length from its square: zero below the normal range (1e-19), where the two above fail
+__device__ __forceinline__ df df_length(df n2) { return n2.hi >= 1.17549435e-38f ? df_sqrt(n2) : df{0.f, 0.f}; }
 // log2 of a positive normal double: exponent and 2 atanh((m - 1) / (m + 1)) of
 // the mantissa m in [0.71, 1.42); absolute error below 1e-9
 __device__ __forceinline__ df df_log2(double x) {

@@ -162,7 +162,8 @@ __device__ __forceinline__ float2 path_gain(int m, const int32_t* __restrict__ s
                                             int32_t S, double f, const float* gamma, const float* disp, int pol) {
     const int pb = pol == SBR_POL_V ? 0 : 2;
     const df fd = df_split(f), Ld = df_split(Lp);
-    // FP32 carries the squares below for f in [1, 1e18] Hz, L in [1e-9, 1e15] m, |eta| < 1e15
+    // FP32 carries the squares below for f in [1, 1e18] Hz, L in [1e-9, 1e15] m, |eta| < 1e15,
+    // |eta - sin^2| > 1e-15
     bool wide = !(fd.hi >= 1.f && fd.hi <= 1e18f && Ld.hi >= 1e-9f && Ld.hi <= 1e15f) ||
                 (gamma && !(fabsf(*gamma) < 1e15f));
     const df fi = df_rcp(fd);
@@ -183,16 +184,13 @@ __device__ __forceinline__ float2 path_gain(int m, const int32_t* __restrict__ s
         const df c2 = df_mul(c, c);
         const df zr = df_add(er, df_sub(c2, df{1.f, 0.f}));
         const df z2 = df_dot2(zr, zr, ei, ei);
-        df r{0.f, 0.f}, ur{0.f, 0.f}, ui{0.f, 0.f};
-        if (z2.hi > 0.f) {
-            r = df_sqrt(z2);
-            const bool neg = zr.hi < 0.f;
-            const df u = df_sqrt(df_scale2(df_add(r, neg ? df_neg(zr) : zr), 0.5f));
-            const df v = df_mul(df_scale2(ei, 0.5f), df_rcp(u));   // signed as Im z
-            const df um = ei.hi < 0.f ? df_neg(u) : u;
-            ur = neg ? (v.hi < 0.f ? df_neg(v) : v) : u;
-            ui = neg ? um : v;
-        }
+        wide |= !(z2.hi >= 1e-30f);   // |z| < 1e-15: grazing incidence on eta = 1
+        const df r = df_sqrt(z2);
+        const bool neg = zr.hi < 0.f;
+        const df u = df_sqrt(df_scale2(df_add(r, neg ? df_neg(zr) : zr), 0.5f));
+        const df v = df_mul(df_scale2(ei, 0.5f), df_rcp(u));   // signed as Im z
+        const df um = ei.hi < 0.f ? df_neg(u) : u;
+        const df ur = neg ? (v.hi < 0.f ? df_neg(v) : v) : u, ui = neg ? um : v;
         // (a - root) / (a + root) = (a^2 - root^2) / (a + root)^2 with the numerator in
         // factors free of cancellation: 1 - eta for a = cos (TE), (eta - 1)(cos^2 (1 + eta) - 1)
         // for a = eta cos (TM)

@@ -30,16 +30,11 @@ namespace {
 // difference; e and b in double-float
 __device__ __forceinline__ df length_change(const df3& b, df b_norm, const df3& e) {
     const df3 a = df3_add(b, e), s = df3_add(a, b);
-    const df n2 = df3_dot(a, a);
-    const df n = n2.hi > 0.f ? df_sqrt(n2) : df{0.f, 0.f};
-    const df den = df_add(n, b_norm);
+    const df den = df_add(df_length(df3_dot(a, a)), b_norm);
     return den.hi > 0.f ? df_mul(df3_dot(e, s), df_rcp(den)) : df{0.f, 0.f};
 }
 __device__ __forceinline__ df3 df3_from(d3 v) { return df3{df_split(v.x), df_split(v.y), df_split(v.z)}; }
-__device__ __forceinline__ df df3_norm(const df3& v) {
-    const df n2 = df3_dot(v, v);
-    return n2.hi > 0.f ? df_sqrt(n2) : df{0.f, 0.f};
-}
+__device__ __forceinline__ df df3_norm(const df3& v) { return df_length(df3_dot(v, v)); }
 
 // Element delays of the paths as (hi, lo): an FP32 delay alone would carry 6e-8 of
 // its cycles into the phase. Thread per element over kDelayPaths paths: the element's offset from its array's reference

@@ -62,8 +62,7 @@ __device__ __forceinline__ float synth_scale(float m) {
 __device__ __forceinline__ df3 df3_of(d3 v) { return df3{df_split(v.x), df_split(v.y), df_split(v.z)}; }
 __device__ __forceinline__ df dist_df(const df3& a, const df3& b) {
     const df3 v = df3_sub(a, b);
-    const df n2 = df3_dot(v, v);
-    return n2.hi > 0.f ? df_sqrt(n2) : df{0.f, 0.f};
+    return df_length(df3_dot(v, v));
 }
 
 // element delay |E - P| - ref, ref = |E0 - P| = dist_df(E0, P) computed once
