@@ -130,15 +130,24 @@ sbr_status delays_run(const DelayArgs& a, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------- phasors
+// cycles f L / c modulo 1 from double-float factors, in [-0.5, 0.5] and a bit:
+// absolute error about 4e-15 of the product (1e6 cycles: 4e-9)
+__device__ __forceinline__ float cycles_mod1(df f, df t) {
+    const df p = two_prod(f.hi, t.hi);
+    const float k = rintf(p.hi);
+    return __fadd_rn(__fsub_rn(p.hi, k), __fmaf_rn(f.hi, t.lo, __fmaf_rn(f.lo, t.hi, p.lo)));
+}
 // exp(-j 2 pi x) for x = foc d cycles (foc = f / c), FP32: the nearest multiple of
 // a quarter turn is removed exactly (foc d - k / 4 in one fused operation, plus the
-// terms of the low words), sine and cosine of the rest (|z| <= pi / 4) from their Taylor
-// series (remainders below 2e-9). Phases beyond 2^19 turns take sincospif.
+// terms of the low words), sine and cosine of the rest (|z| <= pi / 4, up to 0.89 next to
+// 2^19 turns, where k comes from a product rounded to 1/8) from their Taylor series
+// (remainders below 2e-9, there 8e-9). Phases beyond 2^19 turns are reduced to a turn by
+// cycles_mod1.
 __device__ __forceinline__ float2 phasor32(df foc, float2 d) {
     const float x4 = 4.f * __fmul_rn(foc.hi, d.x);
     if (!(fabsf(x4) < 2097152.f)) {
         float s, c;
-        sincospif(-2.f * (foc.hi * d.x), &s, &c);
+        sincospif(-2.f * cycles_mod1(foc, df{d.x, d.y}), &s, &c);
         return make_float2(c, s);
     }
     const float m = __fadd_rn(x4, 12582912.f);   // 1.5 2^23: the sum's low bits are the integer
@@ -190,13 +199,6 @@ __device__ __forceinline__ cdf2 phasor_df(df x) {
     return cdf2_make(a, b);
 }
 
-// cycles f L / c modulo 1 from double-float factors, in [-0.5, 0.5] and a bit:
-// absolute error about 4e-15 of the product (1e6 cycles: 4e-9)
-__device__ __forceinline__ float cycles_mod1(df f, df t) {
-    const df p = two_prod(f.hi, t.hi);
-    const float k = rintf(p.hi);
-    return __fadd_rn(__fsub_rn(p.hi, k), __fmaf_rn(f.hi, t.lo, __fmaf_rn(f.lo, t.hi, p.lo)));
-}
 __device__ __forceinline__ float2 cmul32(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
