@@ -54,8 +54,8 @@ typedef enum {
 #define SBR_POL_H 1         /* phi-hat polarisation at both ends                 */
 
 /* precision of sbr_synthesize_H */
-#define SBR_SYNTH_FP64 0    /* CUDA cores, double-float sum (48 bits)             */
-#define SBR_SYNTH_FP32 1    /* FP32 CUDA-core summation, FP64 delay phase        */
+#define SBR_SYNTH_FP64 0    /* FP64 CUDA-core summation                          */
+#define SBR_SYNTH_FP32 1    /* FP32 CUDA-core summation, double-float delays      */
 #define SBR_SYNTH_BF16X3 2  /* tcgen05 BF16 hi/lo split (3 products), FP32 TMEM  */
 #define SBR_SYNTH_FP16X3 3  /* tcgen05 FP16 hi/lo split (3 products), weights scaled
                                per frequency by a power of two, FP32 TMEM          */
@@ -314,8 +314,7 @@ sbr_status sbr_path_gains(const sbr_path_list* pl, const sbr_material* mats, int
  * T_0 = the trace's tx, R_0 = rx_xyz[rx_index]; a LoS path uses the exact
  * |T_p - R_q| in its phase. gains: dev complex64 [P*F] from sbr_path_gains (NULL when P = 0).
  * tx_elem: dev double [Nt*3]; rx_elem: dev double [Nr*3].
- * precision: SBR_SYNTH_FP64 / FP32 (CUDA cores; the FP64 form sums in
- * double-float, 48 bits: its error is the rounding of H) or SBR_SYNTH_BF16X3 /
+ * precision: SBR_SYNTH_FP64 / FP32 (CUDA cores) or SBR_SYNTH_BF16X3 /
  * SBR_SYNTH_FP16X3 (tcgen05 tensor cores, U diag(w) V^T contraction, FP32
  * accumulation; FP16X3 keeps ~2^-22 of each operand where BF16X3 keeps ~2^-16).
  * H: dev complex64 [F*Nr*Nt], element (f, q, p) at (f*Nr + q)*Nt + p.
@@ -335,10 +334,10 @@ sbr_status sbr_synthesize_H(const sbr_path_list* pl, const void* gains, const do
  * Unlike sbr_synthesize_H no Rx-side correction is applied: the element is
  * the traced point. gains: dev complex64 [P*F] (NULL when P = 0);
  * freqs_hz: dev double [F]; tx_elem: dev double [Nt*3].
- * precision: SBR_SYNTH_FP64 (sums in double-float, 48 bits) or SBR_SYNTH_FP32;
- * element delays are double-float in both.
+ * precision: SBR_SYNTH_FP64 (delays, phases and sums in FP64) or SBR_SYNTH_FP32 (the
+ * phase f L_n / c and the element delays in double-float, 48 bits, the rest in FP32).
  * H: dev complex64 [F*n_rx*Nt], element (f, q, p) at (f*n_rx + q)*Nt + p.
- * F, n_rx <= 65535. Device scratch: P*Nt pairs of floats.
+ * F, n_rx <= 65535. Device scratch: P*Nt doubles.
  */
 sbr_status sbr_synthesize_H_elements(const sbr_path_list* pl, const void* gains, const double* freqs_hz,
                                      int32_t F, const double* tx_elem, int32_t Nt, int32_t precision,

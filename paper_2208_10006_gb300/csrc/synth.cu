@@ -11,11 +11,10 @@
 // cosines per path and one complex multiply-add per term.
 //
 // The FP32 form computes in FP32 with phases reduced from double-float
-// frequencies. The FP64 form computes in double-float (48 bits): an FP64
-// operation takes as long as 71 FP32 ones on this GPU, and the result is rounded
-// to FP32 (its error against 64 bits, 4e-8, is that rounding in either
-// arithmetic).
+// frequencies, the FP64 form in FP64 throughout (an operation of which takes as long
+// as 71 FP32 ones on this GPU).
 #include <algorithm>
+#include <type_traits>
 
 #include "dfloat.cuh"
 #include "sbr_internal.cuh"
@@ -36,10 +35,12 @@ __device__ __forceinline__ df length_change(const df3& b, df b_norm, const df3& 
 __device__ __forceinline__ df3 df3_from(d3 v) { return df3{df_split(v.x), df_split(v.y), df_split(v.z)}; }
 __device__ __forceinline__ df df3_norm(const df3& v) { return df_length(df3_dot(v, v)); }
 
-// Element delays of the paths as (hi, lo): an FP32 delay alone would carry 6e-8 of
-// its cycles into the phase. Thread per element over kDelayPaths paths: the element's offset from its array's reference
-// and each path's vector from the reference to its point are differences taken in
-// FP64, the rest is double-float.
+// Element delays of the paths: FP64 (D = double), or as (hi, lo) for the FP32 form,
+// where an FP32 delay alone would carry 6e-8 of its cycles into the phase. Thread per
+// element over kDelayPaths paths. Double-float: the element's offset from its array's
+// reference and each path's vector from the reference to its point are differences
+// taken in FP64, the rest is double-float.
+template <class D>
 struct DelayArgs {
     int64_t P;                // paths
     const int32_t* nb;
@@ -51,16 +52,18 @@ struct DelayArgs {
     const double* tx_elem;
     const double* rx_elem;    // reference-point form
     int32_t Nt, Nr;
-    float2 *dt, *dr, *dlos;   // [P][Nt], [P][Nr], [Nr][Nt]
+    D *dt, *dr, *dlos;        // [P][Nt], [P][Nr], [Nr][Nt]
 };
 constexpr int kDelayThreads = 128, kDelayPaths = 2;
 
 // path blocks in y (then, reference-point form, receive elements in groups of
 // kDelayPaths for dlos), elements (transmit, then receive) in x
-__global__ void __launch_bounds__(kDelayThreads) k_delays(const __grid_constant__ DelayArgs a) {
+template <class D>
+__global__ void __launch_bounds__(kDelayThreads) k_delays(const __grid_constant__ DelayArgs<D> a) {
     ::sbr::pdl_wait();
-    __shared__ df3 s_b[2][kDelayPaths];
-    __shared__ df s_n[2][kDelayPaths];
+    constexpr bool kF64 = std::is_same<D, double>::value;
+    __shared__ typename std::conditional<kF64, d3, df3>::type s_b[2][kDelayPaths];   // FP64: the points themselves
+    __shared__ typename std::conditional<kF64, double, df>::type s_n[2][kDelayPaths];
     const int64_t blocks = (a.P + kDelayPaths - 1) / kDelayPaths;
     const bool los = (int64_t)blockIdx.y >= blocks;
     const int64_t n0 = ((int64_t)blockIdx.y - (los ? blocks : 0)) * kDelayPaths;
@@ -70,35 +73,55 @@ __global__ void __launch_bounds__(kDelayThreads) k_delays(const __grid_constant_
         const int64_t n = n0 + k;
         if (n < a.P) {
             const int m = a.nb[n];
-            d3 b = mk3(0, 0, 0);
-            if (m > 0) b = rx_side ? R0 - ld3(a.pts + (n * kKmax + m - 1) * 3) : a.T0 - ld3(a.pts + n * kKmax * 3);
-            else if (a.rx) b = a.T0 - ld3(a.rx_xyz + 3 * (int64_t)a.rx[n]);   // LoS of the path's own receiver
-            s_b[rx_side][k] = df3_from(b);
-            s_n[rx_side][k] = df3_norm(s_b[rx_side][k]);
+            const d3 ref = rx_side ? R0 : a.T0;
+            d3 at = ref;
+            if (m > 0) at = ld3(a.pts + (n * kKmax + (rx_side ? m - 1 : 0)) * 3);
+            else if (a.rx && !rx_side) at = ld3(a.rx_xyz + 3 * (int64_t)a.rx[n]);   // LoS of the path's own receiver
+            if constexpr (kF64) {
+                s_b[rx_side][k] = at;
+                s_n[rx_side][k] = norm(ref - at);
+            } else {
+                s_b[rx_side][k] = df3_from(ref - at);
+                s_n[rx_side][k] = df3_norm(s_b[rx_side][k]);
+            }
         }
     }
     __syncthreads();
     const int64_t e = (int64_t)blockIdx.x * kDelayThreads + threadIdx.x;
     const bool rx_side = e >= a.Nt;
     if (e >= (int64_t)a.Nt + (a.R0 && !los ? a.Nr : 0)) return;
-    const df3 off = df3_from(rx_side ? ld3(a.rx_elem + 3 * (e - a.Nt)) - R0 : ld3(a.tx_elem + 3 * e) - a.T0);
+    const d3 el = rx_side ? ld3(a.rx_elem + 3 * (e - a.Nt)) : ld3(a.tx_elem + 3 * e);
+    df3 off, b;   // double-float: the element's offset, the arrays' distance
+    df bn;
+    if constexpr (!kF64) off = df3_from(el - (rx_side ? R0 : a.T0));
     if (los) {   // |T_p - R_q| - |T_0 - R_0|
-        const df3 b = df3_from(a.T0 - R0);
-        const df bn = df3_norm(b);
+        if constexpr (!kF64) b = df3_from(a.T0 - R0), bn = df3_norm(b);
         for (int64_t q = n0; q < n0 + kDelayPaths && q < a.Nr; ++q) {
-            const df v = length_change(b, bn, df3_sub(off, df3_from(ld3(a.rx_elem + 3 * q) - R0)));
-            a.dlos[q * a.Nt + e] = make_float2(v.hi, v.lo);
+            const d3 r = ld3(a.rx_elem + 3 * q);
+            if constexpr (kF64) {
+                a.dlos[q * a.Nt + e] = norm(el - r) - norm(a.T0 - R0);
+            } else {
+                const df v = length_change(b, bn, df3_sub(off, df3_from(r - R0)));
+                a.dlos[q * a.Nt + e] = make_float2(v.hi, v.lo);
+            }
         }
         return;
     }
     for (int k = 0; k < kDelayPaths && n0 + k < a.P; ++k) {
+        D* out = rx_side ? a.dr + (n0 + k) * a.Nr + (e - a.Nt) : a.dt + (n0 + k) * a.Nt + e;
         // a LoS path of the reference-point form takes its delay from dlos
-        const df v = a.nb[n0 + k] > 0 || a.rx ? length_change(s_b[rx_side][k], s_n[rx_side][k], off) : df{0.f, 0.f};
-        (rx_side ? a.dr + (n0 + k) * a.Nr + (e - a.Nt) : a.dt + (n0 + k) * a.Nt + e)[0] = make_float2(v.hi, v.lo);
+        const bool on = a.nb[n0 + k] > 0 || a.rx;
+        if constexpr (kF64) {
+            *out = on ? norm(el - s_b[rx_side][k]) - s_n[rx_side][k] : 0.0;
+        } else {
+            const df v = on ? length_change(s_b[rx_side][k], s_n[rx_side][k], off) : df{0.f, 0.f};
+            *out = make_float2(v.hi, v.lo);
+        }
     }
 }
 
-sbr_status delays_run(const DelayArgs& a, cudaStream_t s) {
+template <class D>
+sbr_status delays_run(const DelayArgs<D>& a, cudaStream_t s) {
     const int64_t e = (int64_t)a.Nt + (a.R0 ? a.Nr : 0);
     const int64_t y = (a.P + kDelayPaths - 1) / kDelayPaths + (a.R0 ? (a.Nr + kDelayPaths - 1) / kDelayPaths : 0);
     if (y == 0) return SBR_OK;
@@ -108,7 +131,7 @@ sbr_status delays_run(const DelayArgs& a, cudaStream_t s) {
         return SBR_ERR_CUDA;
     }
     if (y > 65535) {
-        DelayArgs part = a;
+        DelayArgs<D> part = a;
         const int64_t step = 16384 * (int64_t)kDelayPaths;   // with 32768 groups of receive elements at most
         const double* r0 = a.R0;
         for (int64_t n = 0; n < a.P; n += step) {
@@ -124,7 +147,7 @@ sbr_status delays_run(const DelayArgs& a, cudaStream_t s) {
         return SBR_OK;
     }
     ::sbr::note_launch();
-    SBR_TRY_CUDA(::sbr::launch_pdl(k_delays, dim3((unsigned)((e + kDelayThreads - 1) / kDelayThreads), (unsigned)y),
+    SBR_TRY_CUDA(::sbr::launch_pdl(k_delays<D>, dim3((unsigned)((e + kDelayThreads - 1) / kDelayThreads), (unsigned)y),
                                    dim3(kDelayThreads), 0, s, a));
     return SBR_OK;
 }
@@ -171,41 +194,14 @@ __device__ __forceinline__ float2 phasor32(df foc, float2 d) {
     return make_float2(re, im);
 }
 
-// the same in double-float: the leading terms of the series in double-float, the
-// later ones (below 4e-7 of the sum) in FP32
-__device__ __forceinline__ cdf2 phasor_df(df x) {
-    const float k = rintf(4.f * x.hi);
-    const df r = df_add(df{__fmaf_rn(-0.25f, k, x.hi), 0.f}, df{x.lo, 0.f});
-    const df z = df_mul(r, df{6.28318548f, -1.74845560e-7f});
-    const df z2 = df_mul(z, z);
-    const float t = z2.hi;
-    float u = fmaf(t, 1.60590438e-10f, -2.50521084e-8f);   // 1/13!, 1/11!
-    u = fmaf(u, t, 2.75573192e-6f);                        // 1/9!
-    df s = df_fma(df{-1.98412701e-4f, 2.7255969e-12f}, z2, df{u, 0.f});       // 1/7!
-    s = df_fma(df{8.33333377e-3f, -4.34617203e-10f}, z2, s);                  // 1/5!
-    s = df_fma(df{-0.166666672f, 4.96705379e-9f}, z2, s);                     // 1/3!
-    s = df_fma(z, df_mul(z, z2), s);
-    u = fmaf(t, -1.14707456e-11f, 2.08767570e-9f);         // 1/14!, 1/12!
-    u = fmaf(u, t, -2.75573192e-7f);                       // 1/10!
-    df c = df_fma(df{2.48015876e-5f, -3.40699612e-13f}, z2, df{u, 0.f});      // 1/8!
-    c = df_fma(df{-1.38888892e-3f, 3.36310929e-11f}, z2, c);                  // 1/6!
-    c = df_fma(df{4.16666679e-2f, -1.24176345e-9f}, z2, c);                   // 1/4!
-    c = df_fma(df{-0.5f, 0.f}, z2, c);
-    c = df_fma(df{1.f, 0.f}, z2, c);
-    const int q = (int)k;
-    df a = (q & 1) ? s : c, b = (q & 1) ? c : s;
-    if ((q + 1) & 2) a = df_neg(a);
-    if (~q & 2) b = df_neg(b);
-    return cdf2_make(a, b);
-}
-
 __device__ __forceinline__ float2 cmul32(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
 
-// the arithmetic of the two forms: C a complex value
+// the arithmetic of the two forms: C a complex value, D an element delay
 struct Form32 {
     using C = float2;
+    using D = float2;
     struct Freq { df f, foc; };
     static __device__ __forceinline__ Freq freq(double f) { return Freq{df_split(f), df_split(f * kInvC0)}; }
     static __device__ __forceinline__ C phasor(const Freq& f, float2 d) { return phasor32(f.foc, d); }
@@ -214,36 +210,37 @@ struct Form32 {
         return cmul32(g, phasor32(df{1.f, 0.f}, make_float2(cycles_mod1(f.f, df_split(L * kInvC0)), 0.f)));
     }
     static __device__ __forceinline__ C mul(C a, C b) { return cmul32(a, b); }
-    static __device__ __forceinline__ void mac(C& acc, const C& a, const C&, const C& v) {
+    static __device__ __forceinline__ void mac(C& acc, const C& a, const C& v) {
         acc.x = fmaf(a.x, v.x, fmaf(-a.y, v.y, acc.x));
         acc.y = fmaf(a.x, v.y, fmaf(a.y, v.x, acc.y));
     }
     static __device__ __forceinline__ C zero() { return make_float2(0.f, 0.f); }
     static __device__ __forceinline__ C add(C a, C b) { return make_float2(a.x + b.x, a.y + b.y); }
-    static __device__ __forceinline__ C turned(const C& a) { return a; }
     static __device__ __forceinline__ float2 out(const C& a) { return a; }
 };
-struct FormDf {
-    using C = cdf2;
-    struct Freq { df foc; };
-    static __device__ __forceinline__ Freq freq(double f) { return Freq{df_split(f / kC0)}; }
-    static __device__ __forceinline__ C phasor(const Freq& f, float2 d) { return phasor_df(df_mul(f.foc, df{d.x, d.y})); }
+struct Form64 {
+    using C = double2;
+    using D = double;
+    struct Freq { double foc; };
+    static __device__ __forceinline__ Freq freq(double f) { return Freq{f / kC0}; }
+    static __device__ __forceinline__ C turn(double cycles) {
+        double s, c;
+        sincospi(-2.0 * cycles, &s, &c);
+        return make_double2(c, s);
+    }
+    static __device__ __forceinline__ C phasor(const Freq& f, double d) { return turn(f.foc * d); }
     static __device__ __forceinline__ C weight(float2 g, const Freq&, double f, double L) {
         const double cyc = f * L / kC0;
-        return mul(C{g, make_float2(0.f, 0.f)}, phasor_df(df_split(cyc - floor(cyc))));
+        return mul(make_double2(g.x, g.y), turn(cyc - floor(cyc)));
     }
-    static __device__ __forceinline__ C mul(const C& a, const C& b) {
-        C r = zero();
-        cdf2_mac(r, a, cdf2_j(a), b);
-        return r;
+    static __device__ __forceinline__ C mul(C a, C b) { return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
+    static __device__ __forceinline__ void mac(C& acc, const C& a, const C& v) {
+        acc.x = fma(a.x, v.x, fma(-a.y, v.y, acc.x));
+        acc.y = fma(a.x, v.y, fma(a.y, v.x, acc.y));
     }
-    static __device__ __forceinline__ void mac(C& acc, const C& a, const C& ja, const C& v) { cdf2_mac(acc, a, ja, v); }
-    static __device__ __forceinline__ C zero() { return C{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
-    static __device__ __forceinline__ C add(const C& a, const C& b) {
-        return cdf2_make(df_add(df{a.h.x, a.l.x}, df{b.h.x, b.l.x}), df_add(df{a.h.y, a.l.y}, df{b.h.y, b.l.y}));
-    }
-    static __device__ __forceinline__ C turned(const C& a) { return cdf2_j(a); }
-    static __device__ __forceinline__ float2 out(const C& a) { return a.h; }
+    static __device__ __forceinline__ C zero() { return make_double2(0.0, 0.0); }
+    static __device__ __forceinline__ C add(C a, C b) { return make_double2(a.x + b.x, a.y + b.y); }
+    static __device__ __forceinline__ float2 out(const C& a) { return make_float2((float)a.x, (float)a.y); }
 };
 
 // ---------------------------------------------------------------- reference-point form
@@ -252,31 +249,34 @@ struct FormDf {
 // chunk's weighted receive phasors and transmit phasors in shared memory (their
 // delays were requested while the previous chunk was summed), then group g runs
 // the outer products of its NC paths; the groups' sums are added at the end. The
-// LoS path (if any, the first) is added per output. Bound by the FP32 pipe: 4
-// operations a term in FP32, 54 in double-float. RQ follows Nr (the smallest of 1,
+// LoS path (if any, the first) is added per output. Bound by the FP32 pipe, 4
+// operations a term, or the FP64 pipe, where what lies outside H is left out (its
+// phasors and terms cost as much as others). RQ follows Nr (the smallest of 1,
 // 2, 4, 8 that covers it: rows past Nr are computed for nothing, and a block
 // shares its transmit phasors among 8 RQ rows); G follows the number of blocks, up
 // to 4, so that few frequencies still fill the SMs with warps.
 // Measured: FP32, F 600, 13 x 63, 129 paths: 156 us with a sine and cosine per
-// term and eight launches, 33 us so; FP64, F 128, 16 x 64, 63 paths: 572 us in
-// FP64, 32 us so.
+// term and eight launches, 33 us so; FP64, F 128, 16 x 64, 63 paths: 572 us with a
+// sine and cosine per term, 125 us so.
 constexpr int kSynthThreads = 128, kSynthPT = 64;
 
+template <class D>
 struct SynthArgs {
     int32_t F, Nr, Nt, Pr;
     const int32_t* nb0;       // reflections of the first path (0: it is the LoS path)
     const double* freqs;
     const float2* g;          // [Pr][F]
     const double* L;
-    const float2 *dt, *dr, *dlos;
+    const D *dt, *dr, *dlos;
     float2* H;
     int32_t p_base;   // first transmit element of this launch
 };
 
 template <class M, int RQ, int G>
-__global__ void __launch_bounds__(kSynthThreads* G) k_synth(const __grid_constant__ SynthArgs a) {
+__global__ void __launch_bounds__(kSynthThreads* G) k_synth(const __grid_constant__ SynthArgs<typename M::D> a) {
     ::sbr::pdl_wait();
     using C = typename M::C;
+    constexpr bool kF64 = std::is_same<M, Form64>::value;
     constexpr int QT = 8 * RQ, NC = sizeof(C) == 8 ? 16 : 8, NT = kSynthThreads * G, NCG = NC * G;
     constexpr int kV = NCG * kSynthPT / NT, kA = (NCG * QT + NT - 1) / NT, kW = 128;   // per thread; NCG divides kW
     constexpr int kPhasors = NCG * (QT + kSynthPT), kSums = G > 1 ? QT * kSynthPT : 0;
@@ -293,8 +293,10 @@ __global__ void __launch_bounds__(kSynthThreads* G) k_synth(const __grid_constan
     for (int i = 0; i < RQ; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = M::zero();
-    float2 dv[kV], da[kA];   // delays of the chunk
+    float2 dv[kV], da[kA];   // delays of the chunk (FP32)
+    const int np = min(kSynthPT, a.Nt - p0), nq = min(QT, a.Nr - q0);   // elements of the tile (FP64)
     auto request = [&](int n0) {
+        if constexpr (!kF64) {
 #pragma unroll
         for (int i = 0; i < kV; ++i) {
             const int e = tid + i * NT, n = n0 + e / kSynthPT, p = p0 + e % kSynthPT;
@@ -305,6 +307,7 @@ __global__ void __launch_bounds__(kSynthThreads* G) k_synth(const __grid_constan
             const int e = tid + i * NT, n = n0 + e / QT, q = q0 + e % QT;
             da[i] = e < NCG * QT && n < a.Pr && q < a.Nr ? __ldg(a.dr + (int64_t)n * a.Nr + q) : make_float2(0.f, 0.f);
         }
+        }
     };
     request(los);
     for (int n0 = los; n0 < a.Pr; n0 += NCG) {
@@ -314,12 +317,22 @@ __global__ void __launch_bounds__(kSynthThreads* G) k_synth(const __grid_constan
             if (tid < kW && n0 + tid < a.Pr) s_w[tid] = M::weight(a.g[(int64_t)(n0 + tid) * a.F + f], fq, fr, a.L[n0 + tid]);
         }
         if (n0 == los || w0 == 0) __syncthreads();
+        if constexpr (kF64) {   // no lane without a phasor: a sine and cosine of one lane take the pipe for a warp's
+            for (int e = tid; e < cnt * (np + nq); e += NT) {
+                const bool tx = e < cnt * np;
+                const int u = tx ? e : e - cnt * np, k = u / (tx ? np : nq), x = u - k * (tx ? np : nq);
+                const C v = M::phasor(fq, tx ? __ldg(a.dt + (int64_t)(n0 + k) * a.Nt + p0 + x) : __ldg(a.dr + (int64_t)(n0 + k) * a.Nr + q0 + x));
+                if (tx) s_v[k * kSynthPT + x] = v;
+                else s_a[k * QT + x] = M::mul(s_w[w0 + k], v);
+            }
+        } else {
 #pragma unroll
         for (int i = 0; i < kV; ++i)
             if ((tid + i * NT) / kSynthPT < cnt) s_v[tid + i * NT] = M::phasor(fq, dv[i]);
 #pragma unroll
         for (int i = 0; i < kA; ++i)
             if ((tid + i * NT) / QT < cnt) s_a[tid + i * NT] = M::mul(s_w[w0 + (tid + i * NT) / QT], M::phasor(fq, da[i]));
+        }
         __syncthreads();
         if (n0 + NCG < a.Pr) request(n0 + NCG);
         for (int k = grp * NC; k < min(cnt, grp * NC + NC); ++k) {
@@ -328,9 +341,11 @@ __global__ void __launch_bounds__(kSynthThreads* G) k_synth(const __grid_constan
             for (int j = 0; j < 4; ++j) v[j] = s_v[k * kSynthPT + tp + 16 * j];
 #pragma unroll
             for (int i = 0; i < RQ; ++i) {
-                const C x = s_a[k * QT + tq + 8 * i], jx = M::turned(x);
+                if (kF64 && tq + 8 * i >= nq) continue;
+                const C x = s_a[k * QT + tq + 8 * i];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) M::mac(acc[i][j], x, jx, v[j]);
+                for (int j = 0; j < 4; ++j)
+                    if (!kF64 || 16 * j < np) M::mac(acc[i][j], x, v[j]);
             }
         }
         __syncthreads();
@@ -353,14 +368,14 @@ __global__ void __launch_bounds__(kSynthThreads* G) k_synth(const __grid_constan
         if (grp > 0) return;
     }
     if (los) {
-        const C w = M::weight(a.g[f], fq, fr, a.L[0]), jw = M::turned(w);
+        const C w = M::weight(a.g[f], fq, fr, a.L[0]);
 #pragma unroll
         for (int i = 0; i < RQ; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int q = q0 + tq + 8 * i, p = p0 + tp + 16 * j;
                 if (q < a.Nr && p < a.Nt)
-                    M::mac(acc[i][j], w, jw, M::phasor(fq, __ldg(a.dlos + (int64_t)q * a.Nt + p)));
+                    M::mac(acc[i][j], w, M::phasor(fq, __ldg(a.dlos + (int64_t)q * a.Nt + p)));
             }
     }
 #pragma unroll
@@ -373,7 +388,7 @@ __global__ void __launch_bounds__(kSynthThreads* G) k_synth(const __grid_constan
 }
 
 template <class M, int RQ>
-sbr_status synth_launch(SynthArgs a, cudaStream_t s) {
+sbr_status synth_launch(SynthArgs<typename M::D> a, cudaStream_t s) {
     const int64_t cols = ((int64_t)a.Nt + kSynthPT - 1) / kSynthPT;
     for (int64_t c = 0; c < cols; c += 65535) {   // (a grid's y dimension)
         a.p_base = (int32_t)(c * kSynthPT);
@@ -414,20 +429,21 @@ sbr_status synth_launch(SynthArgs a, cudaStream_t s) {
 // strongest, and their sums are added at the end.
 constexpr int kElF = 16, kElMid = 8, kElPaths = 64, kElMax = 128, kElGroups = 8;
 
+template <class D>
 struct ElArgs {
     int32_t F, Nq, Nt;
     const int32_t* rx_off;
     const double* freqs;
     const float2* g;          // [P][F]
     const double* L;
-    const float2* dt;         // [P][Nt]
+    const D* dt;              // [P][Nt]
     float2* H;
     int32_t p_base;   // first transmit element of this launch
 };
 
 // block (elements / 2, G)
 template <int G>
-__global__ void __launch_bounds__(G > 1 ? 32 * G : kElMax) k_synth_el32(const __grid_constant__ ElArgs a) {
+__global__ void __launch_bounds__(G > 1 ? 32 * G : kElMax) k_synth_el32(const __grid_constant__ ElArgs<float2> a) {
     ::sbr::pdl_wait();
     __shared__ __align__(16) float2 s_w[kElPaths][kElF];
     __shared__ float s_sum[G > 1 ? G / 2 : 1][4 * kElF][G > 1 ? 32 : 1];
@@ -569,33 +585,36 @@ __global__ void __launch_bounds__(G > 1 ? 32 * G : kElMax) k_synth_el32(const __
             }
 }
 
-// FP64 form: thread per output, every phasor in double-float
-__global__ void __launch_bounds__(kSynthThreads) k_synth_el_df(const __grid_constant__ ElArgs a) {
+// FP64 form: thread per output, a sine and cosine per term. Blocks no wider than the
+// array, as many of them on an SM as fit: the pipe is kept busy by one warp of each.
+// F 300, 64 x 64, 63 paths per element: 4860 us with phasors and delays in the same
+// arithmetic and the products left to the compiler (six operations), 4645 us with four.
+__global__ void __launch_bounds__(kSynthThreads, 16) k_synth_el64(const __grid_constant__ ElArgs<double> a) {
     ::sbr::pdl_wait();
-    __shared__ cdf2 s_w[kSynthThreads];
-    const int32_t f = blockIdx.x, q = blockIdx.y, p = a.p_base + blockIdx.z * kSynthThreads + threadIdx.x;
+    __shared__ double2 s_w[kSynthThreads];
+    const int32_t f = blockIdx.x, q = blockIdx.y, p = a.p_base + blockIdx.z * blockDim.x + threadIdx.x;
     const double fr = a.freqs[f];
-    const FormDf::Freq fq = FormDf::freq(fr);
+    const Form64::Freq fq = Form64::freq(fr);
     const int32_t a0 = a.rx_off[q], a1 = a.rx_off[q + 1];
-    cdf2 acc = FormDf::zero();
+    double2 acc = Form64::zero();
     for (int32_t n0 = a0; n0 < a1; n0 += kSynthThreads) {
         const int cnt = min(kSynthThreads, a1 - n0);
         __syncthreads();
-        if ((int)threadIdx.x < cnt)
-            s_w[threadIdx.x] = FormDf::weight(a.g[(int64_t)(n0 + threadIdx.x) * a.F + f], fq, fr, a.L[n0 + threadIdx.x]);
+        for (int k = threadIdx.x; k < cnt; k += blockDim.x)
+            s_w[k] = Form64::weight(a.g[(int64_t)(n0 + k) * a.F + f], fq, fr, a.L[n0 + k]);
         __syncthreads();
         if (p < a.Nt)
             for (int k = 0; k < cnt; ++k)
-                cdf2_mac(acc, s_w[k], cdf2_j(s_w[k]), FormDf::phasor(fq, __ldg(a.dt + (int64_t)(n0 + k) * a.Nt + p)));
+                Form64::mac(acc, s_w[k], Form64::phasor(fq, __ldg(a.dt + (int64_t)(n0 + k) * a.Nt + p)));
     }
-    if (p < a.Nt) a.H[((int64_t)f * a.Nq + q) * a.Nt + p] = acc.h;
+    if (p < a.Nt) a.H[((int64_t)f * a.Nq + q) * a.Nt + p] = Form64::out(acc);
 }
 
-}  // namespace
-
-sbr_status synth_elements_run(const sbr_path_list* pl, const float2* g, const double* freqs, int32_t F,
-                              const double* tx_elem, int32_t Nt, bool fp64, float2* H, cudaStream_t s) {
-    DelayArgs d{};
+template <class D>
+sbr_status elements_form(const sbr_path_list* pl, const float2* g, const double* freqs, int32_t F,
+                         const double* tx_elem, int32_t Nt, float2* H, cudaStream_t s) {
+    constexpr bool fp64 = std::is_same<D, double>::value;
+    DelayArgs<D> d{};
     d.P = pl->P;
     d.nb = pl->nb;
     d.pts = pl->pts;
@@ -607,7 +626,7 @@ sbr_status synth_elements_run(const sbr_path_list* pl, const float2* g, const do
     SBR_TRY(dalloc_n(&d.dt, (size_t)pl->P * Nt, s));
     sbr_status st = delays_run(d, s);
     if (st == SBR_OK) {
-        ElArgs a{F, pl->n_rx, Nt, pl->rx_off, freqs, g, pl->L, d.dt, H, 0};
+        ElArgs<D> a{F, pl->n_rx, Nt, pl->rx_off, freqs, g, pl->L, d.dt, H, 0};
         // FP32: two elements per thread; blocks as wide as the array up to kElMax threads, or of
         // 32 in 2, 4 or 8 groups while the launch has fewer than four warps per scheduler.
         // Whole call, 63 paths per element, warps without groups: 1 to 76 warps 39 us with one
@@ -617,15 +636,19 @@ sbr_status synth_elements_run(const sbr_path_list* pl, const float2* g, const do
         const int64_t warps = ((int64_t)F + kElF - 1) / kElF * pl->n_rx * (((int64_t)Nt + 63) / 64);
         int groups = 1;
         while (!fp64 && groups < kElGroups && warps * groups < 16 * (int64_t)sm_count()) groups *= 2;
-        const int width = fp64 ? kSynthThreads : groups > 1 ? 32 : std::min(kElMax, ((Nt + 1) / 2 + 31) / 32 * 32), per = fp64 ? width : 2 * width;
+        const int width = fp64 ? std::min(kSynthThreads, (Nt + 31) / 32 * 32) : groups > 1 ? 32 : std::min(kElMax, ((Nt + 1) / 2 + 31) / 32 * 32), per = fp64 ? width : 2 * width;
         const int64_t cols = ((int64_t)Nt + per - 1) / per;
         for (int64_t c = 0; c < cols && st == SBR_OK; c += 65535) {   // (a grid's z dimension)
             a.p_base = (int32_t)(c * per);
             const dim3 grid((unsigned)(fp64 ? F : (F + kElF - 1) / kElF), (unsigned)pl->n_rx, (unsigned)std::min<int64_t>(65535, cols - c));
             ::sbr::note_launch();
-            const auto kern = groups == 1 ? k_synth_el32<1> : groups == 2 ? k_synth_el32<2> : groups == 4 ? k_synth_el32<4> : k_synth_el32<8>;
-            const cudaError_t e = fp64 ? ::sbr::launch_pdl(k_synth_el_df, grid, dim3(width), 0, s, a)
-                                       : ::sbr::launch_pdl(kern, grid, dim3(width, groups), 0, s, a);
+            cudaError_t e;
+            if constexpr (fp64) {
+                e = ::sbr::launch_pdl(k_synth_el64, grid, dim3(width), 0, s, a);
+            } else {
+                const auto kern = groups == 1 ? k_synth_el32<1> : groups == 2 ? k_synth_el32<2> : groups == 4 ? k_synth_el32<4> : k_synth_el32<8>;
+                e = ::sbr::launch_pdl(kern, grid, dim3(width, groups), 0, s, a);
+            }
             if (e != cudaSuccess) {
                 set_error("per-element synthesis: %s", cudaGetErrorString(e));
                 st = SBR_ERR_CUDA;
@@ -636,11 +659,12 @@ sbr_status synth_elements_run(const sbr_path_list* pl, const float2* g, const do
     return st;
 }
 
-sbr_status synth_simt_run(const sbr_path_list* pl, const float2* g, const double* freqs, int32_t F,
+template <class D>
+sbr_status reference_form(const sbr_path_list* pl, const float2* g, const double* freqs, int32_t F,
                           const double* tx_elem, int32_t Nt, const double* rx_elem, int32_t Nr,
-                          int32_t rx_index, bool fp64, float2* H, cudaStream_t s) {
+                          int32_t rx_index, float2* H, cudaStream_t s) {
     const int32_t o0 = pl->h_rx_off[rx_index], Pr = pl->h_rx_off[rx_index + 1] - o0;
-    DelayArgs d{};
+    DelayArgs<D> d{};
     d.P = Pr;
     d.nb = pl->nb + o0;
     d.pts = pl->pts + (int64_t)o0 * kKmax * 3;
@@ -659,9 +683,9 @@ sbr_status synth_simt_run(const sbr_path_list* pl, const float2* g, const double
     if (st == SBR_OK) {
         // the LoS path (no reflection) sorts first among a receiver's paths; the
         // kernel reads its reflection count on the device
-        const SynthArgs a{F, Nr, Nt, Pr, d.nb, freqs, g + (int64_t)o0 * F, pl->L + o0, d.dt, d.dr, d.dlos, H, 0};
-        if (fp64)
-            st = Nr <= 8 ? synth_launch<FormDf, 1>(a, s) : (Nr <= 16 ? synth_launch<FormDf, 2>(a, s) : synth_launch<FormDf, 4>(a, s));
+        const SynthArgs<D> a{F, Nr, Nt, Pr, d.nb, freqs, g + (int64_t)o0 * F, pl->L + o0, d.dt, d.dr, d.dlos, H, 0};
+        if constexpr (std::is_same<D, double>::value)
+            st = Nr <= 8 ? synth_launch<Form64, 1>(a, s) : (Nr <= 16 ? synth_launch<Form64, 2>(a, s) : synth_launch<Form64, 4>(a, s));
         else
             st = Nr <= 8 ? synth_launch<Form32, 1>(a, s)
                          : (Nr <= 16 ? synth_launch<Form32, 2>(a, s)
@@ -669,6 +693,21 @@ sbr_status synth_simt_run(const sbr_path_list* pl, const float2* g, const double
     }
     dfree(d.dt, s);
     return st;
+}
+
+}  // namespace
+
+sbr_status synth_elements_run(const sbr_path_list* pl, const float2* g, const double* freqs, int32_t F,
+                              const double* tx_elem, int32_t Nt, bool fp64, float2* H, cudaStream_t s) {
+    return fp64 ? elements_form<double>(pl, g, freqs, F, tx_elem, Nt, H, s)
+                : elements_form<float2>(pl, g, freqs, F, tx_elem, Nt, H, s);
+}
+
+sbr_status synth_simt_run(const sbr_path_list* pl, const float2* g, const double* freqs, int32_t F,
+                          const double* tx_elem, int32_t Nt, const double* rx_elem, int32_t Nr,
+                          int32_t rx_index, bool fp64, float2* H, cudaStream_t s) {
+    return fp64 ? reference_form<double>(pl, g, freqs, F, tx_elem, Nt, rx_elem, Nr, rx_index, H, s)
+                : reference_form<float2>(pl, g, freqs, F, tx_elem, Nt, rx_elem, Nr, rx_index, H, s);
 }
 
 }  // namespace sbr

@@ -4,7 +4,8 @@ way, against the oracle's FP64 sum over the same path list.
 
 Tolerance, of the sum of the path magnitudes: an element delay to 2^-46 of the
 distance and its product with f / c to 2^-45 (d, f, at 2^25 turns: 2e-6 of a turn,
-1e-5 rad), the FP32 phase, sine and cosine 4e-7 and the FP32 sum.
+1e-5 rad), the FP32 phase, sine and cosine 4e-7 and the FP32 sum. The
+FP64 form is below the same bound.
 """
 import numpy as np
 import pytest
@@ -33,7 +34,7 @@ def test_far_elements(form, metres):
     turns = 1.03 * metres * f.max() / 299792458.0
     tol = 2 * np.pi * turns * 2.0 ** -44 + 2e-6
     G = torch.as_tensor(g, device="cuda")
-    for p in (sbr.SYNTH_FP32,):
+    for p in (sbr.SYNTH_FP32, sbr.SYNTH_FP64):
         if form == "elements":
             H = sbr.synthesize_H_elements(r["paths"], G, dev(f), dev(te), p).cpu().numpy()
             Ho = oracle.synth_H_elements(ex, g.astype(np.complex128), f, sc["tx"], te, sc["rx"])
