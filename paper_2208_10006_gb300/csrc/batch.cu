@@ -239,13 +239,13 @@ __global__ void __launch_bounds__(kBThreads) k_batch_delays(const BatchJobDev* _
     const d3 T0 = mk3(J->tx[0], J->tx[1], J->tx[2]), R0 = mk3(J->rx[0], J->rx[1], J->rx[2]);
     const int n0 = (P > 0 && paths.nb[J->path_base] == 0) ? 1 : 0;
     const int nrefl = P - n0, npad = (nrefl + 7) & ~7;
-    const int ne = Nt + Nr;
     // one thread per (path, element side, run of up to 8 elements)
-    const int gt = (Nt + 7) / 8, gr = (Nr + 7) / 8;
-    for (int it = threadIdx.x; it < npad * (gt + gr); it += kBThreads) {
-        const int n = it % npad, g = it / npad;
+    const int64_t gt = tiles_of(Nt, 8), gr = tiles_of(Nr, 8);
+    for (int64_t it = threadIdx.x; it < npad * (gt + gr); it += kBThreads) {
+        const int64_t g = it / npad;
+        const int n = (int)(it - g * npad);
         const bool tx = g < gt;
-        const int e0 = (tx ? g : g - gt) * 8, e1 = min(tx ? Nt : Nr, e0 + 8);
+        const int64_t e0 = (tx ? g : g - gt) * 8, e1 = min((int64_t)(tx ? Nt : Nr), e0 + 8);
         // element e, path n at [n / 4][e][n % 4] (layout in synth_ops.cuh)
         float* dst = (tx ? dt + J->dt_base : dr + J->dr_base) + (int64_t)(n >> 2) * (tx ? Nt : Nr) * 4 + (n & 3);
         if (n < nrefl) {
@@ -254,16 +254,15 @@ __global__ void __launch_bounds__(kBThreads) k_batch_delays(const BatchJobDev* _
             const df3 Pk = df3_of(ld3(paths.pts + (slot * kKmax + (tx ? 0 : m - 1)) * 3));
             const df ref = dist_df(df3_of(tx ? T0 : R0), Pk);
             const double* el = tx ? J->tx_elem : J->rx_elem;
-            for (int e = e0; e < e1; ++e) dst[(int64_t)e * 4] = el_delay(el + 3 * e, Pk, ref);
+            for (int64_t e = e0; e < e1; ++e) dst[e * 4] = el_delay(el + xyz_at(e), Pk, ref);
         } else {
-            for (int e = e0; e < e1; ++e) dst[(int64_t)e * 4] = 0.f;
+            for (int64_t e = e0; e < e1; ++e) dst[e * 4] = 0.f;
         }
     }
-    (void)ne;
     const df ref = dist_df(df3_of(T0), df3_of(R0));
-    for (int it = threadIdx.x; it < Nr * Nt; it += kBThreads) {
-        const int q = it / Nt, p = it - q * Nt;
-        dl[J->dl_base + dl_index(q, p, Nt)] = el_delay(J->tx_elem + 3 * p, df3_of(ld3(J->rx_elem + 3 * q)), ref);
+    for (int64_t it = threadIdx.x; it < (int64_t)Nr * Nt; it += kBThreads) {
+        const int q = (int)(it / Nt), p = (int)(it - (int64_t)q * Nt);
+        dl[J->dl_base + dl_index(q, p, Nt)] = el_delay(J->tx_elem + xyz_at(p), df3_of(ld3(J->rx_elem + xyz_at(q))), ref);
     }
 }
 

@@ -3,6 +3,7 @@
 #pragma once
 #include "geodesic_df.cuh"
 #include "sbr_internal.cuh"
+#include "synth_index.cuh"
 
 namespace sbr {
 
@@ -110,7 +111,7 @@ struct BatchSynthWave {
 };
 // tiles of one job for a tile width (64 receive elements x tile_n transmit elements per frequency)
 inline int64_t batch_synth_items(int32_t F, int32_t Nr, int32_t Nt, int tile_n) {
-    return (int64_t)F * ((Nr + 63) / 64) * ((Nt + tile_n - 1) / tile_n);
+    return (int64_t)F * tiles_of(Nr, 64) * tiles_of(Nt, tile_n);
 }
 sbr_status batch_synth_prepare(bool f16, int tile_n);   // kernel attributes; call before capture
 sbr_status batch_synth_tc(const BatchSynthWave& w, bool f16, int tile_n, cudaStream_t s);

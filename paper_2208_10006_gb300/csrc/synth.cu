@@ -294,18 +294,18 @@ __global__ void __launch_bounds__(kSynthThreads* G) k_synth(const __grid_constan
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = M::zero();
     float2 dv[kV], da[kA];   // delays of the chunk (FP32)
-    const int np = min(kSynthPT, a.Nt - p0), nq = min(QT, a.Nr - q0);   // elements of the tile (FP64)
+    const int np = min(kSynthPT, a.Nt - p0), nq = min(QT, a.Nr - q0);   // elements of the tile
     auto request = [&](int n0) {
         if constexpr (!kF64) {
 #pragma unroll
         for (int i = 0; i < kV; ++i) {
-            const int e = tid + i * NT, n = n0 + e / kSynthPT, p = p0 + e % kSynthPT;
-            dv[i] = n < a.Pr && p < a.Nt ? __ldg(a.dt + (int64_t)n * a.Nt + p) : make_float2(0.f, 0.f);
+            const int e = tid + i * NT, n = n0 + e / kSynthPT, x = e % kSynthPT;
+            dv[i] = n < a.Pr && x < np ? __ldg(a.dt + (int64_t)n * a.Nt + (p0 + x)) : make_float2(0.f, 0.f);
         }
 #pragma unroll
         for (int i = 0; i < kA; ++i) {
-            const int e = tid + i * NT, n = n0 + e / QT, q = q0 + e % QT;
-            da[i] = e < NCG * QT && n < a.Pr && q < a.Nr ? __ldg(a.dr + (int64_t)n * a.Nr + q) : make_float2(0.f, 0.f);
+            const int e = tid + i * NT, n = n0 + e / QT, x = e % QT;
+            da[i] = e < NCG * QT && n < a.Pr && x < nq ? __ldg(a.dr + (int64_t)n * a.Nr + (q0 + x)) : make_float2(0.f, 0.f);
         }
         }
     };
@@ -373,17 +373,17 @@ __global__ void __launch_bounds__(kSynthThreads* G) k_synth(const __grid_constan
         for (int i = 0; i < RQ; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const int q = q0 + tq + 8 * i, p = p0 + tp + 16 * j;
-                if (q < a.Nr && p < a.Nt)
-                    M::mac(acc[i][j], w, M::phasor(fq, __ldg(a.dlos + (int64_t)q * a.Nt + p)));
+                const int q = tq + 8 * i, p = tp + 16 * j;
+                if (q < nq && p < np)
+                    M::mac(acc[i][j], w, M::phasor(fq, __ldg(a.dlos + (int64_t)(q0 + q) * a.Nt + (p0 + p))));
             }
     }
 #pragma unroll
     for (int i = 0; i < RQ; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int q = q0 + tq + 8 * i, p = p0 + tp + 16 * j;
-            if (q < a.Nr && p < a.Nt) a.H[((int64_t)f * a.Nr + q) * a.Nt + p] = M::out(acc[i][j]);
+            const int q = tq + 8 * i, p = tp + 16 * j;
+            if (q < nq && p < np) a.H[((int64_t)f * a.Nr + (q0 + q)) * a.Nt + (p0 + p)] = M::out(acc[i][j]);
         }
 }
 
@@ -452,9 +452,9 @@ __global__ void __launch_bounds__(G > 1 ? 32 * G : kElMax) k_synth_el32(const __
     __shared__ df s_mid;
     const int grp = G > 1 ? threadIdx.y : 0, tid = grp * blockDim.x + threadIdx.x, threads = G * blockDim.x;
     const int32_t f0 = blockIdx.x * kElF, q = blockIdx.y;
-    const int32_t p0 = a.p_base + blockIdx.z * 2 * blockDim.x + threadIdx.x, p1 = p0 + blockDim.x;   // the two elements
+    const uint32_t p0 = a.p_base + blockIdx.z * 2 * blockDim.x + threadIdx.x, p1 = p0 + blockDim.x;   // the two elements (unsigned: past Nt, up to 2^31 and some)
     const int nf = min(kElF, a.F - f0);
-    const bool act = p0 < a.Nt, two = p1 < a.Nt;
+    const bool act = p0 < (uint32_t)a.Nt, two = p1 < (uint32_t)a.Nt;
     if (tid < 32) {   // one warp, at least: the block's frequencies
         const double fk = a.freqs[f0 + min(tid, nf - 1)];
         const double first = __shfl_sync(0xffffffffu, fk, 0), last = __shfl_sync(0xffffffffu, fk, nf - 1);
@@ -497,8 +497,8 @@ __global__ void __launch_bounds__(G > 1 ? 32 * G : kElMax) k_synth_el32(const __
         const int part = (cnt + G - 1) / G, c0 = grp * part, c1 = min(cnt, c0 + part);
         if (c0 >= c1) continue;
         // delays two paths ahead
-        auto delay = [&](int n, int32_t p) { return __ldg(dt + (int64_t)max(n, c0) * a.Nt + p); };
-        const int32_t pb = two ? p1 : p0;
+        auto delay = [&](int n, uint32_t p) { return __ldg(dt + (int64_t)max(n, c0) * a.Nt + p); };
+        const uint32_t pb = two ? p1 : p0;
         float2 da = delay(c1 - 1, p0), db = delay(c1 - 1, pb), ea = delay(c1 - 2, p0), eb = delay(c1 - 2, pb);
         for (int n = c1 - 1; n >= c0; --n) {
             const float2 d0 = da, d1 = db;
@@ -592,7 +592,8 @@ __global__ void __launch_bounds__(G > 1 ? 32 * G : kElMax) k_synth_el32(const __
 __global__ void __launch_bounds__(kSynthThreads, 16) k_synth_el64(const __grid_constant__ ElArgs<double> a) {
     ::sbr::pdl_wait();
     __shared__ double2 s_w[kSynthThreads];
-    const int32_t f = blockIdx.x, q = blockIdx.y, p = a.p_base + blockIdx.z * blockDim.x + threadIdx.x;
+    const int32_t f = blockIdx.x, q = blockIdx.y;
+    const uint32_t p = a.p_base + blockIdx.z * blockDim.x + threadIdx.x;
     const double fr = a.freqs[f];
     const Form64::Freq fq = Form64::freq(fr);
     const int32_t a0 = a.rx_off[q], a1 = a.rx_off[q + 1];
@@ -603,11 +604,11 @@ __global__ void __launch_bounds__(kSynthThreads, 16) k_synth_el64(const __grid_c
         for (int k = threadIdx.x; k < cnt; k += blockDim.x)
             s_w[k] = Form64::weight(a.g[(int64_t)(n0 + k) * a.F + f], fq, fr, a.L[n0 + k]);
         __syncthreads();
-        if (p < a.Nt)
+        if (p < (uint32_t)a.Nt)
             for (int k = 0; k < cnt; ++k)
                 Form64::mac(acc, s_w[k], Form64::phasor(fq, __ldg(a.dt + (int64_t)(n0 + k) * a.Nt + p)));
     }
-    if (p < a.Nt) a.H[((int64_t)f * a.Nq + q) * a.Nt + p] = Form64::out(acc);
+    if (p < (uint32_t)a.Nt) a.H[((int64_t)f * a.Nq + q) * a.Nt + p] = Form64::out(acc);
 }
 
 template <class D>

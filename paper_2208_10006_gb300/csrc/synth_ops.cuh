@@ -19,16 +19,11 @@
 #pragma once
 #include "dfloat.cuh"
 #include "sbr_internal.cuh"
+#include "synth_index.cuh"
 
 namespace sbr {
 
 constexpr double kInvC0 = 1.0 / kC0;
-
-__host__ __device__ __forceinline__ int64_t dl_size(int64_t Nr, int64_t Nt) { return ((Nr + 7) / 8) * ((Nt + 15) / 16) * 128; }
-// within a block: lane 4 (q % 8) + (p % 8) / 2 holds the pairs of columns p % 16 and p % 16 + 8
-__host__ __device__ __forceinline__ int64_t dl_index(int q, int p, int Nt) {
-    return ((int64_t)(q >> 3) * ((Nt + 15) / 16) + (p >> 4)) * 128 + ((q & 7) * 4 + ((p & 7) >> 1)) * 4 + ((p >> 3) & 1) * 2 + (p & 1);
-}
 
 // g exp(-j 2 pi f L / c). The phase f L / c (up to ~1e6 cycles at THz) is formed in
 // double-float, its integer part removed exactly; the rest r = hi + lo with hi the

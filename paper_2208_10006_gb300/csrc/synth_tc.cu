@@ -173,7 +173,7 @@ __device__ __forceinline__ TcItem tc_item(const TcArgs& a, int64_t it) {
     }
     // 32-bit decode (a job has F * tiles < 2^31 items); every thread of the
     // CTA repeats it, so it stays cheap
-    const uint32_t mtiles = (uint32_t)(x.Nr + 63) / 64u, ntiles = (uint32_t)(x.Nt + kTileN - 1) / (uint32_t)kTileN;
+    const uint32_t mtiles = tiles_of(x.Nr, 64), ntiles = tiles_of(x.Nt, kTileN);
     const uint32_t per_f = mtiles * ntiles, itu = (uint32_t)it;
     const uint32_t fq = per_f == 1u ? itu : itu / per_f;
     const uint32_t rem = itu - fq * per_f;
@@ -277,18 +277,19 @@ __device__ __forceinline__ void tc_epilogue(const TcEpi& e, uint32_t tmem, int w
     const int qa = lane >> 2, pc = 2 * (lane & 3);
     const uint32_t tacc = tmem + (uint32_t)(e.acc * kTileN) + ((uint32_t)(32 * lg) << 16);
     using Off = typename std::conditional<kFull, int, int64_t>::type;   // a full tile's offsets fit 32 bits
-    const Off nt16 = ((Off)e.Nt + 15) / 16;
-    const int nr8 = (int)(((int64_t)e.Nr + 7) / 8);
+    const Off nt16 = (Off)tiles_of(e.Nt, 16);
+    const int nr8 = (int)tiles_of(e.Nr, 8);
+    const int rows = e.Nr - e.q0, cols = e.Nt - e.p0;   // of H from the tile's first on
     // LoS delays of a block (dl_index): two 16-byte loads, column pairs 0, 8 and 16, 24
     const float4* dl0 = reinterpret_cast<const float4*>(e.dlos) + ((int64_t)(e.q0 / 8 + 2 * lg) * nt16 + e.p0 / 16) * 32 + lane;
     auto load_dl = [&](int b, float4 (&dl)[2]) {
         const int h = b / kJ, j2 = 2 * (b % kJ);
-        const bool rows = kFull || (e.q0 + 16 * lg) / 8 + h < nr8;
+        const bool in = kFull || e.q0 / 8 + 2 * lg + h < nr8;
 #pragma unroll
         for (int k = 0; k < 2; ++k)
-            dl[k] = kFull || (rows && e.p0 / 16 + j2 + k < nt16) ? __ldg(dl0 + (h * nt16 + j2 + k) * 32) : make_float4(0.f, 0.f, 0.f, 0.f);
+            dl[k] = kFull || (in && e.p0 / 16 + j2 + k < nt16) ? __ldg(dl0 + (h * nt16 + j2 + k) * 32) : make_float4(0.f, 0.f, 0.f, 0.f);
     };
-    float2* out = e.Hf + (int64_t)(e.q0 + 16 * lg + qa) * e.Nt + e.p0 + pc;
+    float2* out = e.Hf + ((int64_t)e.q0 + 16 * lg + qa) * e.Nt + e.p0 + pc;
     float4 next[2];
     if (kLos) load_dl(b0, next);
 #pragma unroll 4
@@ -300,7 +301,7 @@ __device__ __forceinline__ void tc_epilogue(const TcEpi& e, uint32_t tmem, int w
             dl[0] = next[0]; dl[1] = next[1];
             if (b + kBs < kBlocks) load_dl(b + kBs, next);
         }
-        if (!kFull && (e.q0 + 16 * lg + 8 * h >= e.Nr || e.p0 + 32 * jj >= e.Nt)) continue;   // all outside H
+        if (!kFull && (16 * lg + 8 * h >= rows || 32 * jj >= cols)) continue;   // all outside H
         uint32_t v[16];
         if (e.mma) {
             tmem_ld_16x256b<4>(tacc + ((uint32_t)(16 * h) << 16) + (uint32_t)(32 * jj), v);
@@ -308,7 +309,7 @@ __device__ __forceinline__ void tc_epilogue(const TcEpi& e, uint32_t tmem, int w
 #pragma unroll
             for (int k = 0; k < 16; ++k) v[k] = 0u;
         }
-        const int q = e.q0 + 16 * lg + 8 * h + qa, p0 = e.p0 + 32 * jj + pc;
+        const int q = 16 * lg + 8 * h + qa, p0 = 32 * jj + pc;   // within the tile
         float2* row = out + ((Off)(8 * h) * e.Nt + 32 * jj);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -317,8 +318,8 @@ __device__ __forceinline__ void tc_epilogue(const TcEpi& e, uint32_t tmem, int w
             float2* dst = row + 8 * k;
             if (kFull) {   // whole tile inside H, even Nt, aligned rows: no per-output checks
                 *reinterpret_cast<float4*>(dst) = o;
-            } else if (q < e.Nr && p0 + 8 * k < e.Nt) {
-                const bool two = p0 + 8 * k + 1 < e.Nt;
+            } else if (q < rows && p0 + 8 * k < cols) {
+                const bool two = p0 + 8 * k + 1 < cols;
                 if (two && ((((uintptr_t)dst) & 15) == 0)) {
                     *reinterpret_cast<float4*>(dst) = o;
                 } else {
@@ -384,7 +385,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_synth_tc(const __grid_constan
     if (a.inject_timeout) ok = __syncthreads_or(!mbar_wait(bar(kNever), 0u, 1u << 12)) == 0;
 
     const int64_t items = kBatch ? a.items
-                                 : (int64_t)a.F * ((a.Nr + 63) / 64) * ((a.Nt + kTileN - 1) / kTileN);
+                                 : (int64_t)a.F * tiles_of(a.Nr, 64) * tiles_of(a.Nt, kTileN);
     auto wait = [&](int i, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait(bar(i), parity)) != 0; };
     uint32_t chunk = 0;   // chunks so far (operand stage and its phase)
     uint32_t tile = 0;    // tiles with MMAs so far (accumulator and its phase)
@@ -407,23 +408,25 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_synth_tc(const __grid_constan
                 // steps through the chunks. [Pp / 4][Nt] groups of 4 paths:
                 // consecutive lanes read consecutive 16-byte groups
                 constexpr int kStep = kGenThreads / kTileN, kUnits = 8 / kStep;
-                const int pl = tid % kTileN, p = x.p0 + pl;
-                const float4* src = reinterpret_cast<const float4*>(x.dtT) + (int64_t)(nb >> 2) * x.Nt + (p < x.Nt ? p : 0);
+                const int pl = tid % kTileN;
+                const bool p_in = pl < x.Nt - x.p0;
+                const float4* src = reinterpret_cast<const float4*>(x.dtT) + (int64_t)(nb >> 2) * x.Nt + (p_in ? x.p0 + pl : 0);
                 // A': receive element q, paths nb + 4 c16 .. + 3 (at most 64 x 8
                 // units: one per thread); consecutive lanes take consecutive receive
                 // elements (rows r(q) & 7 = q & 7), so that a quarter warp's 16-byte
                 // stores land in 8 distinct bank groups of the swizzled rows and a
                 // warp shares its weights
-                const int ql = tid & 63, qc = tid >> 6, q = x.q0 + ql, n = nb + 4 * qc;
+                const int ql = tid & 63, qc = tid >> 6, n = nb + 4 * qc;
+                const bool q_in = ql < x.Nr - x.q0;
                 // every load of the chunk before the wait for its stage
                 float4 dt[kUnits], dr = make_float4(0.f, 0.f, 0.f, 0.f), w01 = dr, w23 = dr;
 #pragma unroll
                 for (int u = 0; u < kUnits; ++u) {
                     const int c16 = tid / kTileN + u * kStep;
-                    dt[u] = p < x.Nt && c16 < n16 ? __ldg(src + (int64_t)c16 * x.Nt) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    dt[u] = p_in && c16 < n16 ? __ldg(src + (int64_t)c16 * x.Nt) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
-                if (qc < n16 && q < x.Nr) {
-                    dr = __ldg(reinterpret_cast<const float4*>(x.drT) + (int64_t)(n >> 2) * x.Nr + q);
+                if (qc < n16 && q_in) {
+                    dr = __ldg(reinterpret_cast<const float4*>(x.drT) + (int64_t)(n >> 2) * x.Nr + (x.q0 + ql));
                     w01 = __ldg(reinterpret_cast<const float4*>(x.wf + n));
                     w23 = __ldg(reinterpret_cast<const float4*>(x.wf + n + 2));
                 }
@@ -432,7 +435,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_synth_tc(const __grid_constan
 #pragma unroll
                 for (int u = 0; u < kUnits; ++u) {
                     const int c16 = tid / kTileN + u * kStep;
-                    if (c16 < n16 && p < x.Nt) {
+                    if (c16 < n16 && p_in) {
                         uint32_t h[4], l[4];
 #pragma unroll
                         for (int k = 0; k < 4; k += 2) {
@@ -447,7 +450,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_synth_tc(const __grid_constan
                     }
                 }
                 // A' as the two rows r(q) (Re A, -Im A) and i(q) (Im A, Re A)
-                if (qc < n16 && q < x.Nr) {
+                if (qc < n16 && q_in) {
                     float sn[4], cs[4];
 #pragma unroll
                     for (int k = 0; k < 4; k += 2) {
@@ -525,7 +528,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_synth_tc(const __grid_constan
             e.isc = kF16 ? 1.f / x.sc : 1.f;   // exact: sc is a power of two
             e.wl = x.wl;
             e.dlos = x.dlos; e.Hf = x.Hf;
-            e.full = x.q0 + 64 <= x.Nr && x.p0 + kTileN <= x.Nt && (x.Nt & 1) == 0 && (((uintptr_t)x.Hf) & 15) == 0 &&
+            e.full = x.Nr - x.q0 >= 64 && x.Nt - x.p0 >= kTileN && (x.Nt & 1) == 0 && (((uintptr_t)x.Hf) & 15) == 0 &&
                      x.Nt < (1 << 26);   // 32-bit offsets within the tile
             if (e.mma) {
                 if (!(ok = wait(kAccFull + e.acc, (tile / 2) & 1u))) break;
@@ -597,7 +600,7 @@ __global__ void k_tc_prep(const __grid_constant__ TcPrep a) {
     const int n0 = (a.Pr > 0 && a.nb[0] == 0) ? 1 : 0;   // the LoS path sorts first
     const int nrefl = a.Pr - n0;
     if ((int)blockIdx.x < a.nbw) {
-        const int f = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+        const int f = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
         if (f >= a.F) return;
         const double fr = a.freqs[f];
         float m = 0.f;
@@ -618,7 +621,7 @@ __global__ void k_tc_prep(const __grid_constant__ TcPrep a) {
         return;
     }
     // delays; consecutive threads write consecutive words of a row
-    const int64_t gt = (a.Nt + kPrepG - 1) / kPrepG, gr = (a.Nr + kPrepG - 1) / kPrepG;
+    const int64_t gt = tiles_of(a.Nt, kPrepG), gr = tiles_of(a.Nr, kPrepG);
     const int64_t n_dt = (int64_t)a.Pp * gt, n_dr = (int64_t)a.Pp * gr, n_dl = (int64_t)a.Nt * gr;
     const int64_t total = n_dt + n_dr + n_dl;
     const int64_t stride = (int64_t)(gridDim.x - a.nbw) * blockDim.x;
@@ -627,7 +630,7 @@ __global__ void k_tc_prep(const __grid_constant__ TcPrep a) {
             const bool tx = t < n_dt;
             const int64_t u = tx ? t : t - n_dt;
             const int n = (int)(u % a.Pp), e0 = (int)(u / a.Pp) * kPrepG;
-            const int ne = tx ? a.Nt : a.Nr;
+            const int ne = tx ? a.Nt : a.Nr, left = ne - e0;
             const double* elem = tx ? a.tx_elem : a.rx_elem;
             // element e, path n at [n / 4][e][n % 4]
             float* dst = (tx ? a.dtT : a.drT) + (int64_t)(n >> 2) * ne * 4 + (n & 3);
@@ -637,11 +640,11 @@ __global__ void k_tc_prep(const __grid_constant__ TcPrep a) {
                 const df ref = dist_df(df3_of(tx ? a.T0 : ld3(a.R0)), P);
 #pragma unroll
                 for (int k = 0; k < kPrepG; ++k)
-                    if (e0 + k < ne) dst[(int64_t)(e0 + k) * 4] = el_delay(elem + 3 * (e0 + k), P, ref);
+                    if (k < left) dst[((int64_t)e0 + k) * 4] = el_delay(elem + xyz_at(e0 + k), P, ref);
             } else {
 #pragma unroll
                 for (int k = 0; k < kPrepG; ++k)
-                    if (e0 + k < ne) dst[(int64_t)(e0 + k) * 4] = 0.f;
+                    if (k < left) dst[((int64_t)e0 + k) * 4] = 0.f;
             }
         } else {
             const int64_t u = t - n_dt - n_dr;
@@ -649,8 +652,8 @@ __global__ void k_tc_prep(const __grid_constant__ TcPrep a) {
             const df ref = dist_df(df3_of(a.T0), df3_of(ld3(a.R0)));
 #pragma unroll
             for (int k = 0; k < kPrepG; ++k)
-                if (q0 + k < a.Nr)
-                    a.dlos[dl_index(q0 + k, p, a.Nt)] = el_delay(a.tx_elem + 3 * p, df3_of(ld3(a.rx_elem + 3 * (q0 + k))), ref);
+                if (k < a.Nr - q0)
+                    a.dlos[dl_index(q0 + k, p, a.Nt)] = el_delay(a.tx_elem + xyz_at(p), df3_of(ld3(a.rx_elem + xyz_at(q0 + k))), ref);
         }
     }
 }
@@ -665,7 +668,7 @@ sbr_status synth_tc_run(const sbr_path_list* pl, const float2* g, const double* 
                         const double* tx_elem, int32_t Nt, const double* rx_elem, int32_t Nr,
                         int32_t rx_index, float2* H, bool f16, cudaStream_t s) {
     const int32_t o0 = pl->h_rx_off[rx_index], Pr = pl->h_rx_off[rx_index + 1] - o0;
-    const int32_t Pp = (int32_t)std::max<int64_t>(8, (Pr + 7) & ~7);   // reflected paths, padded
+    const int32_t Pp = (int32_t)std::max<int64_t>(8, ((int64_t)Pr + 7) & ~(int64_t)7);   // reflected paths, padded
     // one buffer for every operand, 16-byte aligned parts: w, wl (8-byte
     // elements) first, then sc, dtT, drT, dlos
     const size_t n_w = (size_t)Pp * F, n_wl = ((size_t)F + 1) & ~(size_t)1;
@@ -685,11 +688,11 @@ sbr_status synth_tc_run(const sbr_path_list* pl, const float2* g, const double* 
     pp.L = pl->L + o0;
     pp.g = g + (int64_t)o0 * F;
     pp.freqs = freqs; pp.tx_elem = tx_elem; pp.rx_elem = rx_elem;
-    pp.R0 = pl->rx_xyz + 3 * rx_index;
+    pp.R0 = pl->rx_xyz + xyz_at(rx_index);
     pp.T0 = mk3(pl->tx[0], pl->tx[1], pl->tx[2]);
     pp.dtT = dtT; pp.drT = drT; pp.dlos = dl; pp.w = w; pp.wl = wl; pp.sc = sc;
     pp.nbw = (int)blocks_of((int64_t)F * 32, kPrepThreads);
-    const int64_t gt = (Nt + kPrepG - 1) / kPrepG, gr = (Nr + kPrepG - 1) / kPrepG;
+    const int64_t gt = tiles_of(Nt, kPrepG), gr = tiles_of(Nr, kPrepG);
     const int64_t n_del = (int64_t)Pp * (gt + gr) + (int64_t)Nt * gr;
     const unsigned nbd = (unsigned)std::min<int64_t>(blocks_of(n_del, kPrepThreads), 32 * (int64_t)sm_count());
     ::sbr::note_launch(), k_tc_prep<<<(unsigned)pp.nbw + nbd, kPrepThreads, 0, s>>>(pp);
@@ -704,7 +707,7 @@ sbr_status synth_tc_run(const sbr_path_list* pl, const float2* g, const double* 
     auto kern = f16 ? k_synth_tc<true, false, 256> : k_synth_tc<false, false, 256>;
     constexpr int kSmemBytes = TcShape<256>::kSmemBytes;
     SBR_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-    int64_t items = (int64_t)F * ((Nr + 63) / 64) * ((Nt + 255) / 256);
+    int64_t items = (int64_t)F * tiles_of(Nr, 64) * tiles_of(Nt, 256);
     // one persistent CTA per SM (two operand stages and two accumulators each),
     // launched as a programmatic dependent of the prologue
     const int grid = (int)std::min<int64_t>(items, (int64_t)sm_count());
