@@ -153,12 +153,11 @@ sbr_status delays_run(const DelayArgs<D>& a, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------- phasors
-// cycles f L / c modulo 1 from double-float factors, in [-0.5, 0.5] and a bit:
+// cycles f t modulo 1 from double-float factors, in [-0.5, 0.5] and a bit:
 // absolute error about 4e-15 of the product (1e6 cycles: 4e-9)
-__device__ __forceinline__ float cycles_mod1(df f, df t) {
+__device__ __forceinline__ df cycles_mod1(df f, df t) {
     const df p = two_prod(f.hi, t.hi);
-    const float k = rintf(p.hi);
-    return __fadd_rn(__fsub_rn(p.hi, k), __fmaf_rn(f.hi, t.lo, __fmaf_rn(f.lo, t.hi, p.lo)));
+    return two_sum(__fsub_rn(p.hi, rintf(p.hi)), __fmaf_rn(f.hi, t.lo, __fmaf_rn(f.lo, t.hi, p.lo)));
 }
 // exp(-j 2 pi x) for x = foc d cycles (foc = f / c), FP32: the nearest multiple of
 // a quarter turn is removed exactly (foc d - k / 4 in one fused operation, plus the
@@ -170,7 +169,7 @@ __device__ __forceinline__ float2 phasor32(df foc, float2 d) {
     const float x4 = 4.f * __fmul_rn(foc.hi, d.x);
     if (!(fabsf(x4) < 2097152.f)) {
         float s, c;
-        sincospif(-2.f * cycles_mod1(foc, df{d.x, d.y}), &s, &c);
+        sincospif(-2.f * cycles_mod1(foc, df{d.x, d.y}).hi, &s, &c);
         return make_float2(c, s);
     }
     const float m = __fadd_rn(x4, 12582912.f);   // 1.5 2^23: the sum's low bits are the integer
@@ -194,6 +193,32 @@ __device__ __forceinline__ float2 phasor32(df foc, float2 d) {
     return make_float2(re, im);
 }
 
+// g exp(-j 2 pi x), x in [-0.5, 0.5] and a bit, rounded once: sine and cosine of the
+// rest to a quarter turn with the leading terms of their series in double-float, the
+// later ones (below 4e-7 of the sum) in FP32
+__device__ __forceinline__ float2 turned(float2 g, df x) {
+    const float k = rintf(4.f * x.hi);
+    const df z = df_mul(df_add(df{__fmaf_rn(-0.25f, k, x.hi), 0.f}, df{x.lo, 0.f}), df{6.28318548f, -1.74845560e-7f});
+    const df z2 = df_mul(z, z);
+    const float t = z2.hi;
+    float u = fmaf(t, -2.50521084e-8f, 2.75573192e-6f);    // 1/11!, 1/9!
+    u = fmaf(u, t, -1.98412698e-4f);                       // 1/7!
+    df s = df_add(df{8.33333377e-3f, -4.34617203e-10f}, two_prod(u, t));      // 1/5!
+    s = df_fma(df{-0.166666672f, 4.96705379e-9f}, z2, s);                     // 1/3!
+    s = df_fma(z, df_mul(z, z2), s);
+    u = fmaf(t, 2.08767570e-9f, -2.75573192e-7f);          // 1/12!, 1/10!
+    u = fmaf(u, t, 2.48015873e-5f);                        // 1/8!
+    df c = df_add(df{-1.38888892e-3f, 3.36310929e-11f}, two_prod(u, t));      // 1/6!
+    c = df_fma(df{4.16666679e-2f, -1.24176345e-9f}, z2, c);                   // 1/4!
+    c = df_fma(df{-0.5f, 0.f}, z2, c);
+    c = df_fma(df{1.f, 0.f}, z2, c);
+    const int q = (int)k;
+    df a = (q & 1) ? s : c, b = (q & 1) ? c : s;
+    if ((q + 1) & 2) a = df_neg(a);
+    if (~q & 2) b = df_neg(b);
+    const df gx{g.x, 0.f}, gy{g.y, 0.f};
+    return make_float2(df_dot2(gx, a, df_neg(gy), b).hi, df_dot2(gx, b, gy, a).hi);
+}
 __device__ __forceinline__ float2 cmul32(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
@@ -207,7 +232,7 @@ struct Form32 {
     static __device__ __forceinline__ C phasor(const Freq& f, float2 d) { return phasor32(f.foc, d); }
     // g exp(-j 2 pi f L / c)
     static __device__ __forceinline__ C weight(float2 g, const Freq& f, double, double L) {
-        return cmul32(g, phasor32(df{1.f, 0.f}, make_float2(cycles_mod1(f.f, df_split(L * kInvC0)), 0.f)));
+        return turned(g, cycles_mod1(f.f, df_split(L * kInvC0)));
     }
     static __device__ __forceinline__ C mul(C a, C b) { return cmul32(a, b); }
     static __device__ __forceinline__ void mac(C& acc, const C& a, const C& v) {
@@ -486,9 +511,7 @@ __global__ void __launch_bounds__(G > 1 ? 32 * G : kElMax) k_synth_el32(const __
 #pragma unroll 4
         for (int e = tid; e < cnt * kElF; e += threads) {
             const int n = e / kElF, k = e % kElF;
-            s_w[n][k] = k < nf ? cmul32(a.g[(int64_t)(n0 + n) * a.F + f0 + k],
-                                        phasor32(df{1.f, 0.f}, make_float2(cycles_mod1(s_f[k], s_t[n]), 0.f)))
-                               : make_float2(0.f, 0.f);
+            s_w[n][k] = k < nf ? turned(a.g[(int64_t)(n0 + n) * a.F + f0 + k], cycles_mod1(s_f[k], s_t[n])) : make_float2(0.f, 0.f);
         }
         __syncthreads();
         if (!act) continue;
