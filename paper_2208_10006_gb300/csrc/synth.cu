@@ -439,16 +439,19 @@ sbr_status synth_launch(SynthArgs<typename M::D> a, cudaStream_t s) {
 // needed. FP32: a thread holds two transmit elements (so that their phasors
 // turn in packed operations: half the issue slots) at kElF consecutive frequencies; the phasor
 // at the middle one comes from phasor32, the others by rotating it with
-// exp(-j 2 pi df d / c) - 1 (precise for the small step between subcarriers, at
-// most eight rotations), four operations each instead of a sine and a cosine. That
-// needs equally spaced frequencies (to 2^-28 of a cycle over the delay) and a step
-// of at most 1/16 cycle, tested per path and element; other grids take phasor32
+// exp(-j 2 pi df d / c) - 1 (precise for the small step between subcarriers) and that
+// of two and four steps, at most three in turn (their roundings add up: eight in turn
+// left 1.15e-7 of H from 7 paths, where a sine and cosine per term leaves 8e-8, as
+// three do), four operations each instead of a sine and a cosine. That needs equally
+// spaced frequencies (to 2^-28 of a cycle over the delay) and a step of at most 1/16
+// cycle, tested per path and element; other grids take phasor32
 // per term. The paths are summed from the last to the first: they are sorted by
 // their reflections, so the strongest come when the sum's rounding matters least.
 // Bound by the FP32 pipe, about eleven operations a term: F 512, 64 x 256, 63
-// paths per element: 948 us with sincospif per term and an FP64 prologue, 248 us
-// so (258 us with one element per thread and scalar operations, 269 us with every
-// operation packed and the weights doubled in shared memory).
+// paths per element: 948 us with sincospif per term and an FP64 prologue, 258 us
+// so (250 us with eight rotations in turn; with those, 10 us more with one element per
+// thread and scalar operations, 21 with every operation packed and the weights doubled
+// in shared memory).
 // A launch of few warps waits for the chain of one element's paths (0.45 us a path):
 // there G groups of 32 threads take a part of the paths each, from the weakest to the
 // strongest, and their sums are added at the end.
@@ -552,20 +555,39 @@ __global__ void __launch_bounds__(G > 1 ? 32 * G : kElMax) k_synth_el32(const __
                 s = __ffma2_rn(s, z2, dup2(-1.66666667e-1f));
                 const float2 sp = __ffma2_rn(__fmul2_rn(s, z2), z, z), sn = make_float2(-sp.x, -sp.y);   // sin z, -sin z
                 const float2 m0 = phasor32(s_mid, d0), m1 = phasor32(s_mid, d1);
-                const float2 mx = make_float2(m0.x, m1.x), my = make_float2(m0.y, m1.y);
-                // upwards and downwards from the middle side by side: two independent chains
-                float2 ux = mx, uy = my, dx = mx, dy = my;
+                // by two and four steps: 2 c (2 + c), 2 s (1 + c)
+                const float2 c2 = __ffma2_rn(__fadd2_rn(c, c), c, __fmul2_rn(c, dup2(4.f)));
+                const float2 sp2 = __ffma2_rn(__fadd2_rn(sp, sp), c, __fadd2_rn(sp, sp)), sn2 = make_float2(-sp2.x, -sp2.y);
+                const float2 c4 = __ffma2_rn(__fadd2_rn(c2, c2), c2, __fmul2_rn(c2, dup2(4.f)));
+                const float2 sp4 = __ffma2_rn(__fadd2_rn(sp2, sp2), c2, __fadd2_rn(sp2, sp2)), sn4 = make_float2(-sp4.x, -sp4.y);
+                float2 bx = make_float2(m0.x, m1.x), by = make_float2(m0.y, m1.y);
+                float2 dx = bx, dy = by;
+                // upwards from the middle (b, b + 4), then downwards: at most three rotations each
 #pragma unroll
-                for (int k = 0; k < kElMid; k += 2) {
-                    const float4 wu = w4[(kElMid + k) / 2], wd = w4[(kElMid - 2 - k) / 2];
-                    turn(dx, dy, c, sn, sp);
-                    add(kElMid + k, wu.x, wu.y, ux, uy);
-                    turn(ux, uy, c, sp, sn);
-                    add(kElMid - 1 - k, wd.z, wd.w, dx, dy);
-                    turn(dx, dy, c, sn, sp);
-                    add(kElMid + k + 1, wu.z, wu.w, ux, uy);
-                    if (k + 2 < kElMid) turn(ux, uy, c, sp, sn);
-                    add(kElMid - 2 - k, wd.x, wd.y, dx, dy);
+                for (int k = 0; k < kElMid; k += 4) {
+                    const float4 w0 = w4[(kElMid + k) / 2], w1 = w4[(kElMid + k) / 2 + 1];
+                    float2 x1 = bx, y1 = by, x2 = bx, y2 = by;
+                    turn(x1, y1, c, sp, sn);
+                    turn(x2, y2, c2, sp2, sn2);
+                    add(kElMid + k, w0.x, w0.y, bx, by);
+                    add(kElMid + k + 1, w0.z, w0.w, x1, y1);
+                    add(kElMid + k + 2, w1.x, w1.y, x2, y2);
+                    turn(x2, y2, c, sp, sn);
+                    if (k + 4 < kElMid) turn(bx, by, c4, sp4, sn4);
+                    add(kElMid + k + 3, w1.z, w1.w, x2, y2);
+                }
+#pragma unroll
+                for (int k = kElMid; k > 0; k -= 4) {   // k - 1 ... k - 4
+                    const float4 w0 = w4[k / 2 - 1], w1 = w4[k / 2 - 2];
+                    float2 x1 = dx, y1 = dy, x2 = dx, y2 = dy;
+                    turn(x1, y1, c, sn, sp);
+                    turn(x2, y2, c2, sn2, sp2);
+                    turn(dx, dy, c4, sn4, sp4);
+                    add(k - 1, w0.z, w0.w, x1, y1);
+                    add(k - 2, w0.x, w0.y, x2, y2);
+                    turn(x2, y2, c, sn, sp);
+                    add(k - 4, w1.x, w1.y, dx, dy);
+                    add(k - 3, w1.z, w1.w, x2, y2);
                 }
             } else {
 #pragma unroll
