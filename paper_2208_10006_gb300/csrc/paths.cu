@@ -47,16 +47,19 @@ __global__ void k_paths_init(const double* __restrict__ rx, int n3, double* __re
 
 // the used slots of the table in idx[0..count[0]), any order; the block that ends
 // last (count[1]) stores the count, alpha and the trace's counters to the
-// host-mapped head
+// host-mapped head. At most kCollectBlocks blocks per SM, each over a run of the table,
+// so that the tickets on that one word stay few whatever the table's size.
+constexpr int kCollectBlocks = 16;
 __global__ void k_collect(const uint32_t* __restrict__ state, size_t cap, uint32_t* __restrict__ idx,
                           unsigned int* __restrict__ count, const double* __restrict__ alpha,
                           const TraceCountersDev* __restrict__ cnt, MappedHead* h) {
     ::sbr::pdl_wait();
-    size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    bool ready = s < cap && state[s] == 2u;
-    unsigned m = __ballot_sync(0xffffffffu, ready);
     const int lane = threadIdx.x & 31;
-    if (m) {
+    for (size_t b = (size_t)blockIdx.x * blockDim.x; b < cap; b += (size_t)gridDim.x * blockDim.x) {
+        const size_t s = b + threadIdx.x;
+        const bool ready = s < cap && state[s] == 2u;
+        const unsigned m = __ballot_sync(0xffffffffu, ready);
+        if (!m) continue;
         unsigned base = 0;
         if (lane == 0) base = atomicAdd(count, (unsigned)__popc(m));
         base = __shfl_sync(0xffffffffu, base, 0);
@@ -293,7 +296,7 @@ sbr_status paths_run(const sbr_trace_result* tr, const sbr_bvh* b, sbr_path_list
     MappedHead* hh = reinterpret_cast<MappedHead*>(hm);
     volatile unsigned* h_count = &hh->count;
     int32_t* h_off = reinterpret_cast<int32_t*>(hm + sizeof(MappedHead));
-    ::sbr::note_launch(), (void)::sbr::launch_pdl(k_collect, dim3((unsigned)((cap + 255) / 256)), dim3(256), 0, s, tr->ht_state, cap, idx, count,
+    ::sbr::note_launch(), (void)::sbr::launch_pdl(k_collect, dim3((unsigned)std::min<size_t>((cap + 255) / 256, (size_t)kCollectBlocks * sm_count())), dim3(256), 0, s, tr->ht_state, cap, idx, count,
                                                   tr->d_alpha, tr->cnt, reinterpret_cast<MappedHead*>(dm));
     SBR_TRY_CUDA(cudaGetLastError());
     SBR_TRY_CUDA(cudaStreamSynchronize(s));
