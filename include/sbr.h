@@ -568,6 +568,8 @@ sbr_status sbr_mlp_create(const sbr_mlp_config* cfg, const float* loss_w, const 
  * (p_e - |p_c - y'_c|)^2 (the head predicts in the normalised units of c,
  * times scale_e + shift_e when predicted). loss: dev
  * float accumulated with atomicAdd (zero it first), or NULL. Asynchronous.
+ * After a bounded tensor-core wait gave up (sbr_mlp_status) this step and the ones
+ * after it leave parameters and moments as they are.
  */
 sbr_status sbr_mlp_train_step(sbr_mlp* m, const float* x, const float* y, int32_t B, float* loss, void* stream);
 /*

@@ -273,6 +273,7 @@ struct NetArgs {
     uint32_t* mask;           // [tile][hidden layer][2][512] ReLU masks
     int n_hidden;
     unsigned int* status;
+    int inject_timeout;       // test-only: wait on a barrier nothing arrives at
 };
 
 struct NetBars {
@@ -280,6 +281,7 @@ struct NetBars {
     uint64_t act[4];          // chunk c of the activations has been written
     uint64_t acc[2];          // accumulator complete
     uint64_t feat_full, feat_free;
+    uint64_t never, drain;
     float oct[kOctaves];      // 2^(k lmax / 15)
     uint32_t tmem;
 };
@@ -422,6 +424,8 @@ __global__ void __launch_bounds__(kNetThreads<kTrain>, 1) k_net(const __grid_con
         for (int k = 0; k < 2; ++k) mbar_init(smem_u32(bar.acc + k), 1);
         mbar_init(smem_u32(&bar.feat_full), kFeatWarps);
         mbar_init(smem_u32(&bar.feat_free), 1);
+        mbar_init(smem_u32(&bar.never), 1);
+        mbar_init(smem_u32(&bar.drain), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (tid < kOctaves) bar.oct[tid] = octave(a.lmax, tid);
@@ -447,6 +451,8 @@ __global__ void __launch_bounds__(kNetThreads<kTrain>, 1) k_net(const __grid_con
     const int ntiles = (a.B + 127) / 128;
     const int my_tiles = (int)blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     bool ok = true;
+    // injected fault: a bounded wait gives up, the CTA takes the exit of a real timeout
+    if (a.inject_timeout) ok = __syncthreads_or(!mbar_wait(smem_u32(&bar.never), 0u, 1u << 12)) == 0;
     if (warp == kLoadWarp) {
         if (lane == 0) {
             uint32_t g = 0;   // chunks staged so far
@@ -460,9 +466,9 @@ __global__ void __launch_bounds__(kNetThreads<kTrain>, 1) k_net(const __grid_con
                         bulk_load(smem_u32(ring + st * kStageBytes), a.op[o].w + (size_t)kc * bytes, bytes, smem_u32(bar.full + st));
                     }
                 }
-            // the copies in flight land before the CTA's shared memory is given up
-            if (!ok)
-                for (uint32_t k = g > kStages ? g - kStages : 0; k < g; ++k) net_wait(bar.full + k % kStages, (k / kStages) & 1u);
+            // the copies in flight land before the CTA's shared memory is given up (another
+            // role's wait may have run out)
+            for (uint32_t k = g > kStages ? g - kStages : 0; k < g; ++k) net_wait(bar.full + k % kStages, (k / kStages) & 1u);
         }
     } else if (warp == kMmaWarp) {
         // the whole warp walks the loop, so that descriptors and addresses stay in
@@ -530,6 +536,11 @@ __global__ void __launch_bounds__(kNetThreads<kTrain>, 1) k_net(const __grid_con
             }
         }
         if (kTrain && lead) bulk_wait_done();
+        if (!ok) {   // the MMAs issued so far complete before their memory is freed
+            if (lead) mma_commit(smem_u32(&bar.drain));
+            __syncwarp();
+            (void)wait(&bar.drain, 0u);
+        }
     } else if (warp >= kEpiWarps) {
         // features of the tiles after the first
         for (int t = 1; t < my_tiles && ok; ++t) {
@@ -723,18 +734,18 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_dw(const __grid_constant__ Dw
     const int t0 = (int)((int64_t)blockIdx.y * a.tiles / a.parts), t1 = (int)((int64_t)(blockIdx.y + 1) * a.tiles / a.parts);
     bool ok = true;
     if (tid == 0) {
+        int staged = 0;
         for (int t = t0; t < t1; ++t) {
             const int k = t - t0, st = k & 1;
-            if (k >= 2 && !net_wait(empty + st, (uint32_t)((k >> 1) - 1) & 1u)) {
-                ok = false;
-                for (int j = k - 2; j < k; ++j) net_wait(full + (j & 1), (uint32_t)(j >> 1) & 1u);
-                break;
-            }
+            if (k >= 2 && !net_wait(empty + st, (uint32_t)((k >> 1) - 1) & 1u)) { ok = false; break; }
+            staged = k + 1;
             const uint32_t sA = smem_u32(smem + st * kDwStage), f = smem_u32(full + st);
             mbar_expect(f, (uint32_t)((2 + nb) * kChunkBytes));
             bulk_load(sA, ly.dH + ((size_t)t * na + 2 * mt) * kChunkBytes, 2 * kChunkBytes, f);
             bulk_load(sA + 2 * kChunkBytes, ly.X + (size_t)t * nb * kChunkBytes, (uint32_t)(nb * kChunkBytes), f);
         }
+        // the copies in flight land before the CTA's shared memory is given up
+        for (int j = staged > 2 ? staged - 2 : 0; j < staged; ++j) net_wait(full + (j & 1), (uint32_t)(j >> 1) & 1u);
     } else if (tid == 32) {
         const uint32_t id = idesc_bf16(ly.n_in, true, true), idb = idesc_bf16(16, true, false);
         const uint64_t d1 = make_desc(smem_u32(ones));
@@ -752,7 +763,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_dw(const __grid_constant__ Dw
             }
             mma_commit(smem_u32(empty + st));
         }
-        if (ok) mma_commit(smem_u32(done));
+        mma_commit(smem_u32(done));   // (after a wait that ran out too: what was issued completes before its memory is freed)
     }
     __syncwarp();
     ok = net_wait(done, 0u) && ok;
@@ -801,17 +812,21 @@ struct AdamArgs {
     int64_t n;
     float *p, *m, *v, *g;
     const float* part;
+    const unsigned int* status;
     float lr, b1, b2, eps, c1, c2;
 };
 
 // four consecutive parameters per thread: the gradient (the sum of its parts, in
 // order), Adam on the FP32 masters, and the BF16 images of the new weights.
-// kStep false: the images alone, from the masters.
+// A step in which a bounded wait gave up changes nothing. kStep false: the images
+// alone, from the masters.
 template <bool kStep>
 __global__ void __launch_bounds__(256) k_adam(const __grid_constant__ AdamArgs a) {
     ::sbr::pdl_wait();
     const int64_t i = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (i >= a.n) return;
+    // a wait that gave up in this step's launches or before: read with the rest, nothing stored
+    const unsigned failed = kStep ? __ldg(a.status) & ST_TIMEOUT : 0u;
     float p[4];
     *reinterpret_cast<float4*>(p) = *reinterpret_cast<const float4*>(a.p + i);
     if (kStep) {
@@ -829,6 +844,7 @@ __global__ void __launch_bounds__(256) k_adam(const __grid_constant__ AdamArgs a
             v[k] = a.b2 * v[k] + (1.f - a.b2) * g[k] * g[k];
             p[k] = p[k] - a.lr * (m[k] / a.c1) / (sqrtf(v[k] / a.c2) + a.eps);
         }
+        if (failed) return;
         *reinterpret_cast<float4*>(a.g + i) = *reinterpret_cast<const float4*>(g);
         *reinterpret_cast<float4*>(a.m + i) = *reinterpret_cast<const float4*>(m);
         *reinterpret_cast<float4*>(a.v + i) = *reinterpret_cast<const float4*>(v);
@@ -990,6 +1006,7 @@ NetArgs net_args(const sbr_mlp* m, const float* x, int B, bool train) {
     a.shift = m->d_shift;
     a.scale = m->d_scale;
     a.status = m->status;
+    a.inject_timeout = fault_mode() == kFaultTimeout ? 1 : 0;
     return a;
 }
 
@@ -1012,6 +1029,7 @@ AdamArgs adam_args(const sbr_mlp* m) {
     a.v = m->v;
     a.g = m->g;
     a.part = m->part;
+    a.status = m->status;
     return a;
 }
 
