@@ -195,8 +195,6 @@ struct cdf2 {
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 __device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
 __device__ __forceinline__ cdf2 cdf2_make(df re, df im) { return cdf2{make_float2(re.hi, im.hi), make_float2(re.lo, im.lo)}; }
-// j u
-__device__ __forceinline__ cdf2 cdf2_j(const cdf2& u) { return cdf2{make_float2(-u.h.y, u.h.x), make_float2(-u.l.y, u.l.x)}; }
 // acc += u k, with ju = j u: the two products and the two sums of each part
 // error-free on the high words, everything below gathered in the low word
 // (27 packed instructions, about 2^-47 of the operands)

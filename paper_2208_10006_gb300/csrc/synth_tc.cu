@@ -304,7 +304,7 @@ __device__ __forceinline__ void tc_epilogue(const TcEpi& e, uint32_t tmem, int w
         if (!kFull && (16 * lg + 8 * h >= rows || 32 * jj >= cols)) continue;   // all outside H
         uint32_t v[16];
         if (e.mma) {
-            tmem_ld_16x256b<4>(tacc + ((uint32_t)(16 * h) << 16) + (uint32_t)(32 * jj), v);
+            tmem_ld_16x256b_x4(tacc + ((uint32_t)(16 * h) << 16) + (uint32_t)(32 * jj), v);
         } else {
 #pragma unroll
             for (int k = 0; k < 16; ++k) v[k] = 0u;

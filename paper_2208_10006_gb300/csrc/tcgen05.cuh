@@ -107,22 +107,6 @@ __device__ __forceinline__ bool mbar_test(uint32_t mbar, uint32_t phase) {
     return done != 0;
 }
 
-// the same wait with a suspend-time hint: a polling thread sleeps up to
-// hint_ns per try instead of spinning; limit tries bound the whole wait
-__device__ __forceinline__ bool mbar_wait_sleep(uint32_t mbar, uint32_t phase, uint32_t hint_ns, uint32_t limit) {
-    for (uint32_t it = 0; it < limit; ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}\n"
-            : "=r"(done)
-            : "r"(mbar), "r"(phase), "r"(hint_ns)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
-}
-
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
@@ -137,34 +121,10 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// 32 lanes x 16 columns of 32 bits (one register per column), then the wait
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-          "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// 16 lanes x (8 kRep) columns of 32 bits starting at lane L of the address:
-// per 8-column repeat k, thread t receives r[4k], r[4k+1] = lane L + t/4,
-// columns 8k + 2(t%4) and + 1, and r[4k+2], r[4k+3] = the same columns of
-// lane L + 8 + t/4; then the wait
-template <int kRep>
-__device__ __forceinline__ void tmem_ld_16x256b(uint32_t taddr, uint32_t* r);
-template <>
-__device__ __forceinline__ void tmem_ld_16x256b<2>(uint32_t taddr, uint32_t* r) {
-    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                   "=r"(r[7])
-                 : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-template <>
-__device__ __forceinline__ void tmem_ld_16x256b<4>(uint32_t taddr, uint32_t* r) {
+// 16 lanes x 32 columns of 32 bits starting at lane L of the address: per 8-column
+// repeat k, thread t receives r[4k], r[4k+1] = lane L + t/4, columns 8k + 2(t%4) and
+// + 1, and r[4k+2], r[4k+3] = the same columns of lane L + 8 + t/4; then the wait
+__device__ __forceinline__ void tmem_ld_16x256b_x4(uint32_t taddr, uint32_t* r) {
     asm volatile(
         "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
         "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
@@ -175,8 +135,9 @@ __device__ __forceinline__ void tmem_ld_16x256b<4>(uint32_t taddr, uint32_t* r) 
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// the 16-column load without its wait, and the wait that makes r readable (other
-// work may come between; r must not be touched until then)
+// 32 lanes x 16 columns of 32 bits (one register per column) without the wait, and the
+// wait that makes r readable (other work may come between; r must not be touched until
+// then)
 __device__ __forceinline__ void tmem_ld16_start(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
