@@ -364,11 +364,14 @@ sbr_status sbr_pdp_angles(const sbr_path_list* pl, const void* gains, int32_t F,
  * sbr_capacity - MIMO capacity (Eq. 15-17). Eq. 16's factor Q = sum |h|^2 is
  * read as a Frobenius normalisation: W_f = (Nr Nt / Qbar) H_f H_f^H
  * (H_f^H H_f when Nt < Nr), Qbar = mean over f of ||H_f||_F^2; SNR linear
- * 10^(dB/10); C = mean_f log2 det(I + SNR/Nt W_f) by an FP64 Cholesky.
+ * 10^(dB/10); C = mean_f log2 det(I + SNR/Nt W_f). W_f is summed in FP32 runs of 32
+ * terms and rounded to FP32; the determinant comes from an L D L^H factorisation, in
+ * double-float (48 bits) while no diagonal entry of I + SNR/Nt W_f exceeds 2^16, in FP64
+ * above.
  * H: dev complex64 [F*Nr*Nt]; snr_db: host double [n_snr], 1 <= n_snr <= 32
  * (read before the call returns); C: dev double [n_snr] (bit/s/Hz).
- * min(Nr, Nt) <= 64 (the n x n Cholesky of one frequency is held in shared
- * memory); larger arrays return SBR_ERR_INVALID_ARG. Asynchronous: returns
+ * min(Nr, Nt) <= 64 (the n x n matrix of one frequency is held in the registers of a
+ * block); larger arrays return SBR_ERR_INVALID_ARG. Asynchronous: returns
  * once the work is enqueued on `stream`.
  */
 sbr_status sbr_capacity(const void* H, int32_t F, int32_t Nr, int32_t Nt, const double* snr_db,
@@ -526,7 +529,8 @@ sbr_status sbr_batch_tune(const sbr_bvh* const* scenes, const sbr_material* cons
  *   k = 2 + i: PDP tap i, 10 log10 of the power with tau_n - tau_min in
  *              [i tap_s, (i + 1) tap_s) over the total (dB), floor_db when
  *              below it or empty.
- * A receiver without paths gets NaN everywhere. FP64 arithmetic, FP32 out.
+ * A receiver without paths gets NaN everywhere. FP64 sums, logarithms in double-float
+ * (1e-10 dB), FP32 out.
  * n_taps in [1, 32]. Asynchronous.
  */
 sbr_status sbr_surrogate_targets(const sbr_path_list* pl, const void* gains, int32_t F, int32_t n_taps,
@@ -575,8 +579,8 @@ sbr_status sbr_mlp_train_step(sbr_mlp* m, const float* x, const float* y, int32_
 /*
  * sbr_mlp_predict - y dev [B*n_out] = outputs for x dev [B*4], in one fused
  * launch (every layer of 128 rows per CTA with the activations kept in shared
- * memory). sbr_mlp_predict_layered: the same outputs through the training
- * path's per-layer GEMMs (activations through device memory), for checking.
+ * memory). sbr_mlp_predict_layered: the same outputs with a GEMM per layer
+ * (activations through device memory), for checking.
  * Asynchronous.
  */
 sbr_status sbr_mlp_predict(const sbr_mlp* m, const float* x, int32_t B, float* y, void* stream);

@@ -149,8 +149,10 @@ __device__ __forceinline__ Ray32 make_ray32(float3 o, float3 d) {
 // within half extent of the centre of an axis for t in c / d - o / d -+ h |1 / d|,
 // so entry and exit of an axis come without the minimum and maximum that a pair of
 // planes needs (they run at half rate; the ALU pipe was the busiest), and the x, y
-// pairs and the two z take nine packed operations. The rounding (~eps |o| in
-// distance) is far inside the relative padding of the BVH boxes. 10 M rays in the
+// pairs and the two z take nine packed operations. The rounding, some eps (|o| + h) in
+// distance, is inside the boxes' padding (2^-20 of |x| + 1) but for large boxes that end
+// next to coordinate 0; it misses as many rays aimed at the edges of such (1e-4 of them,
+// 100 m boxes) as the test with planes. 10 M rays in the
 // urban scene: 2.47 ms with lower and upper planes, 2.22 ms so (18% fewer
 // instructions; the node loads, four register write-back cycles each, now take as
 // long as the issue slots); 4 M rays in the room 2.14 -> 1.93 ms.
@@ -960,7 +962,7 @@ __global__ void __launch_bounds__(kTraceThreads) k_trace_batch(const __grid_cons
 // they lose to spills (4096-job batch: 2.07 s at 96 registers and 4 blocks,
 // 1.64 s here). The FP32 reception test ahead of the exact one, the job's pointers
 // read again after the walk and the rays per bounce counted per block took a batch
-// of 24 jobs from 7.69 to 7.44 ms.
+// of 24 jobs from 7.69 to 7.41 ms.
 __global__ void __launch_bounds__(kTraceThreads, 8) k_trace_batch_df(const __grid_constant__ BatchTraceArgs a) {
     int stack[kStack];
     // rays entering each bounce, counted per block and added up once at the end
