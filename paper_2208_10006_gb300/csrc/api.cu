@@ -492,13 +492,15 @@ sbr_status sbr_path_export(const sbr_path_list* pl, int32_t* rx, int32_t* n_boun
              {dist, pl->dist, P * sizeof(float)}};
     // Destinations in this device's memory are filled by one launch instead of a copy
     // each (3 us of host time and a gap on the device); any other (pinned host, another
-    // device), resolved by unified addressing, by a copy.
+    // device), resolved by unified addressing, by a copy, as everything is when the list
+    // itself is on another device than the current one.
     ExportArgs a{};
     int dev = -1;
     SBR_TRY_CUDA(cudaGetDevice(&dev));
+    const bool here = device_range(pl->rx, P * sizeof(int32_t), dev);
     for (const Field& x : f) {
         if (!x.dst) continue;
-        if (device_range(x.dst, x.bytes, dev)) {
+        if (here && device_range(x.dst, x.bytes, dev)) {
             a.dst[a.n] = static_cast<uint32_t*>(x.dst);
             a.src[a.n] = static_cast<const uint32_t*>(x.src);
             a.words[a.n++] = (int64_t)(x.bytes / 4);
