@@ -285,6 +285,7 @@ struct NetBars {
     float oct[kOctaves];      // 2^(k lmax / 15)
     uint32_t tmem;
 };
+static_assert(sizeof(NetBars) <= 256, "room between the ring and the biases");
 
 // every wait gives up after 2^26 polls (about a second)
 __device__ __forceinline__ bool net_wait(const uint64_t* bar, uint32_t parity) {
