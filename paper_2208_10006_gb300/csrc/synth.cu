@@ -281,7 +281,7 @@ struct Form64 {
 // shares its transmit phasors among 8 RQ rows); G follows the number of blocks, up
 // to 4, so that few frequencies still fill the SMs with warps.
 // Measured: FP32, F 600, 13 x 63, 129 paths: 156 us with a sine and cosine per
-// term and eight launches, 33 us so; FP64, F 128, 16 x 64, 63 paths: 572 us with a
+// term and eight launches, 35 us so; FP64, F 128, 16 x 64, 63 paths: 572 us with a
 // sine and cosine per term, 125 us so.
 constexpr int kSynthThreads = 128, kSynthPT = 64;
 
@@ -323,15 +323,15 @@ __global__ void __launch_bounds__(kSynthThreads* G) k_synth(const __grid_constan
     auto request = [&](int n0) {
         if constexpr (!kF64) {
 #pragma unroll
-        for (int i = 0; i < kV; ++i) {
-            const int e = tid + i * NT, n = n0 + e / kSynthPT, x = e % kSynthPT;
-            dv[i] = n < a.Pr && x < np ? __ldg(a.dt + (int64_t)n * a.Nt + (p0 + x)) : make_float2(0.f, 0.f);
-        }
+            for (int i = 0; i < kV; ++i) {
+                const int e = tid + i * NT, n = n0 + e / kSynthPT, x = e % kSynthPT;
+                dv[i] = n < a.Pr && x < np ? __ldg(a.dt + (int64_t)n * a.Nt + (p0 + x)) : make_float2(0.f, 0.f);
+            }
 #pragma unroll
-        for (int i = 0; i < kA; ++i) {
-            const int e = tid + i * NT, n = n0 + e / QT, x = e % QT;
-            da[i] = e < NCG * QT && n < a.Pr && x < nq ? __ldg(a.dr + (int64_t)n * a.Nr + (q0 + x)) : make_float2(0.f, 0.f);
-        }
+            for (int i = 0; i < kA; ++i) {
+                const int e = tid + i * NT, n = n0 + e / QT, x = e % QT;
+                da[i] = e < NCG * QT && n < a.Pr && x < nq ? __ldg(a.dr + (int64_t)n * a.Nr + (q0 + x)) : make_float2(0.f, 0.f);
+            }
         }
     };
     request(los);
@@ -352,11 +352,11 @@ __global__ void __launch_bounds__(kSynthThreads* G) k_synth(const __grid_constan
             }
         } else {
 #pragma unroll
-        for (int i = 0; i < kV; ++i)
-            if ((tid + i * NT) / kSynthPT < cnt) s_v[tid + i * NT] = M::phasor(fq, dv[i]);
+            for (int i = 0; i < kV; ++i)
+                if ((tid + i * NT) / kSynthPT < cnt) s_v[tid + i * NT] = M::phasor(fq, dv[i]);
 #pragma unroll
-        for (int i = 0; i < kA; ++i)
-            if ((tid + i * NT) / QT < cnt) s_a[tid + i * NT] = M::mul(s_w[w0 + (tid + i * NT) / QT], M::phasor(fq, da[i]));
+            for (int i = 0; i < kA; ++i)
+                if ((tid + i * NT) / QT < cnt) s_a[tid + i * NT] = M::mul(s_w[w0 + (tid + i * NT) / QT], M::phasor(fq, da[i]));
         }
         __syncthreads();
         if (n0 + NCG < a.Pr) request(n0 + NCG);
